@@ -127,6 +127,46 @@ __device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
   return v[0];
 }
 
+// Sum carried as an unevaluated pair hi + lo of FP32 values (Knuth's exact
+// two-term addition): (hi, lo) += x keeps about 2^-46 of the sum.  GB300
+// issues FP64 adds and conversions at 1/64 of the FP32 rate, and these six
+// FP32 additions replace one of each.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x);
+  const float b = __fsub_rn(s, hi);
+  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
+  hi = s;
+  lo = __fadd_rn(lo, e);
+}
+
+// The pair's value (a sum that overflowed leaves NaN in lo: hi has it).
+__device__ __forceinline__ double pair_value(float hi, float lo) {
+  return __fsub_rn(hi, hi) == 0.0f ? (double)hi + (double)lo : (double)hi;
+}
+
+// hi + lo += x^2, the square's rounding error included.
+__device__ __forceinline__ void pair_add_sq(float& hi, float& lo, float x) {
+  const float p = __fmul_rn(x, x);
+  lo = __fadd_rn(lo, __fmaf_rn(x, x, -p));
+  pair_add(hi, lo, p);
+}
+// The warp's lanes' pairs summed and rounded to FP32 (in every lane).
+__device__ __forceinline__ float warp_pair_sum(float hi, float lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
+    lo = __fadd_rn(lo, ol);
+    pair_add(hi, lo, oh);
+  }
+  return __fsub_rn(hi, hi) == 0.0f ? __fadd_rn(hi, lo) : hi;
+}
+
+// (h, l) += a stored pair.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float2 p) {
+  lo = __fadd_rn(lo, p.y);
+  pair_add(hi, lo, p.x);
+}
+
 // Block sum (blockDim.x multiple of 32, <= 1024); result valid in thread 0.
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T* sh /* >= 32 entries */) {

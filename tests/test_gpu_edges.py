@@ -1,0 +1,73 @@
+"""Edges of the tiles, slices and splits of the CUDA kernels against the
+float64 oracle or exact arithmetic: sizes around each boundary, odd counts,
+odd strides, the smallest and the largest of a range."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import spsvm as O
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda"
+
+
+def _t(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+@pytest.fixture(scope="module")
+def sp():
+    import paper_1404_1066_gb300 as m
+    return m
+
+
+def _kmat(sp, K, fmt, odd_plane=False):
+    """A stored kernel matrix of K's values (exact in the format)."""
+    rows, n = K.shape
+    ld = (n + 127) // 128 * 128
+    K32 = _t(K.astype(np.float32))
+    if fmt == "fp32":
+        buf = torch.zeros(rows * ld, dtype=torch.float32, device=DEV)
+        buf.view(rows, ld)[:, :n] = K32
+        return sp.KMat(buf, sp.SPSVM_FP32, n, rows, ld, 0), K32.double().cpu().numpy()
+    plane = rows * ld + (1 if odd_plane else 0)
+    buf = torch.zeros(2 * plane, dtype=torch.bfloat16, device=DEV)
+    hi = K32.to(torch.bfloat16)
+    lo = (K32 - hi.float()).to(torch.bfloat16)
+    buf[:rows * ld].view(rows, ld)[:, :n] = hi
+    buf[plane:plane + rows * ld].view(rows, ld)[:, :n] = lo
+    return sp.KMat(buf, sp.SPSVM_BF16SPLIT, n, rows, ld, plane), (hi.double() + lo.double()).cpu().numpy()
+
+
+# columns taken 128 at a time, at least 1,024 points per slice, rows 4 per warp
+# and 32 per block
+@pytest.mark.parametrize("fmt,kc_fmt", [("fp32", "fp32"), ("fp32", "bf16split"), ("bf16split", "bf16split")])
+@pytest.mark.parametrize("n,m,ns", [(2050, 33, 1025), (2050, 31, 2049), (1024, 4, 1), (4097, 65, 127),
+                                    (4097, 3, 4097), (130, 1, 0), (9001, 5, 129)])
+def test_compaction_edges(sp, fmt, kc_fmt, n, m, ns):
+    """Copies are exact, the tail to 128 is zero, and the weighted sums of ns
+    products are within 32 FP32 roundings of their terms."""
+    g = np.random.default_rng(n + m)
+    km, Kref = _kmat(sp, np.exp(-3 * g.random((m, n))), fmt)
+    S = np.zeros(n, dtype=bool)
+    S[g.choice(n, ns, replace=False)] = True
+    w1, w2 = g.standard_normal((2, n)).astype(np.float32)
+    kc, _ = _kmat(sp, np.zeros((m, km.ld)), kc_fmt, odd_plane=m % 2 == 1)
+    kc.buf.fill_(7.0)
+    a, b, count, pos = sp.spsvm_compact_active(km, _t(S.astype(np.uint8)), _t(w1), _t(w2), kc)
+    assert int(count.item()) == ns
+    np.testing.assert_array_equal(pos.cpu().numpy(), np.cumsum(S) - S)
+    got = kc.to_float().double().cpu().numpy()
+    want = Kref[:, S]
+    if kc_fmt != fmt:
+        w32 = _t(want.astype(np.float32))
+        hi = w32.to(torch.bfloat16)
+        want = (hi.double() + (w32 - hi.float()).to(torch.bfloat16).double()).cpu().numpy()
+    np.testing.assert_array_equal(got[:, :ns], want)
+    end = (ns + 127) // 128 * 128
+    assert np.all(got[:, ns:end] == 0) and np.all(got[:, end:] >= 7.0)
+    for out, w in ((a, w1), (b, w2)):
+        terms = np.abs(Kref[:, S]) @ np.abs(w[S].astype(np.float64))
+        err = np.abs(out.cpu().numpy() - Kref[:, S] @ w[S].astype(np.float64))
+        assert np.all(err <= 32 * 2.0 ** -24 * terms + 1e-300)
