@@ -71,3 +71,29 @@ def test_compaction_edges(sp, fmt, kc_fmt, n, m, ns):
         terms = np.abs(Kref[:, S]) @ np.abs(w[S].astype(np.float64))
         err = np.abs(out.cpu().numpy() - Kref[:, S] @ w[S].astype(np.float64))
         assert np.all(err <= 32 * 2.0 ** -24 * terms + 1e-300)
+
+
+def _points(n, d, seed, pad):
+    """n x d points whose rows are 16-byte aligned, or (pad) are not."""
+    g = np.random.default_rng(seed)
+    X = g.standard_normal((n, d)).astype(np.float32)
+    ld = (d + 3) // 4 * 4 + (1 if pad else 0)
+    buf = torch.zeros((n, ld), dtype=torch.float32, device=DEV)
+    buf[:, :d] = _t(X)
+    return X, buf[:, :d]
+
+
+# four features a lane, 128 a warp step; planes padded to 64 columns
+@pytest.mark.parametrize("pad", [False, True])
+@pytest.mark.parametrize("n,d", [(1, 1), (9, 3), (8, 64), (7, 127), (33, 129), (5, 260)])
+def test_points_norms_and_planes(sp, n, d, pad):
+    """Norms are the FP64 sums rounded once; hi + mid + lo is x exactly."""
+    X, Xt = _points(n, d, n + d, pad)
+    P = sp.spsvm_prepare_points(Xt, "bf16split")
+    want = (X.astype(np.float64) ** 2).sum(1)
+    got = P.norms.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - want) <= 2.0 ** -24 * want * (1 + 2.0 ** -20))
+    planes = [p.float().cpu().numpy() for p in (P.hi, P.mid, P.lo)]
+    np.testing.assert_array_equal(planes[0].astype(np.float64)[:, :d] + planes[1][:, :d] + planes[2][:, :d], X)
+    assert all(np.all(p[:, d:] == 0) for p in planes)
+    np.testing.assert_array_equal(planes[0][:, :d], _t(X).to(torch.bfloat16).float().cpu().numpy())
