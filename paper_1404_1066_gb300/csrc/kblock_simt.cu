@@ -3,156 +3,173 @@
 // ||x - z||^2 = ||x||^2 + ||z||^2 - 2 x^T z; the basis-vector score of
 // Section 4 ("Basis vector selection") fused into the same tile loop.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
+#include "simt_tile.h"
 
 namespace spsvm {
 
 namespace {
 
-constexpr int TM = 128;   // points per tile
-constexpr int TN = 64;    // basis / candidate columns per tile
-constexpr int TK = 16;    // feature chunk
-constexpr int NT = 256;   // threads: 32 (points) x 8 (columns)
+constexpr int64_t PT = 128;   // points per tile
 
-// Accumulates the 128 x 64 tile of x_i^T z_c for points i0.. and columns
-// idx[c0..] into acc[a][b] for point tx + 32a, column ty + 8b.
-__device__ __forceinline__ void dot_tile(const float* __restrict__ X, int64_t n, int64_t d,
-                                         int64_t ldx, const int64_t* __restrict__ zrow,
-                                         int64_t i0, int m_here, float (*Xs)[TM + 4],
-                                         float (*Zs)[TN + 4], float acc[4][8]) {
-  const int t = threadIdx.x, tx = t & 31, ty = t >> 5;
+// Tiles of 64 (or 32) basis rows by 128 points: the points run along the
+// tile's columns, so a warp's kernel values go out as 256 contiguous bytes of
+// a basis row.  FP32 ALU bound for d past about 60: n = 100,000, d = 784, 64
+// rows 0.214 ms (47 TFLOP/s, FMA pipe 69% of active cycles); tiles of 4 x 8
+// outputs with scalar shared loads took 0.540 ms.
+using Wide = simt::Tile<64, 128, 8>;
+using Narrow = simt::Tile<32, 128, 4>;
+
+template <class T, class RA, class RB>
+__device__ __forceinline__ void rbf_rows(const float* __restrict__ X, int64_t n, int64_t ldx,
+                                         const int64_t* __restrict__ idx, int64_t i0, int64_t c0,
+                                         int32_t m, RA (&a)[T::LA], RB (&b)[T::LB]) {
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int u = 0; u < T::LA; ++u) {
+    const int64_t c = c0 + T::load_row(u);
+    a[u].p = c < m ? X + idx[c] * ldx : nullptr;
+  }
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
-  for (int64_t k0 = 0; k0 < d; k0 += TK) {
-    // X tile: 128 rows x 16 features
-#pragma unroll
-    for (int r = 0; r < (TM * TK) / NT; ++r) {
-      const int e = t + NT * r;
-      const int row = e / TK, col = e % TK;
-      const int64_t i = i0 + row, k = k0 + col;
-      Xs[col][row] = (i < n && k < d) ? X[i * ldx + k] : 0.f;
-    }
-#pragma unroll
-    for (int r = 0; r < (TN * TK) / NT; ++r) {
-      const int e = t + NT * r;
-      const int row = e / TK, col = e % TK;
-      const int64_t k = k0 + col;
-      Zs[col][row] = (row < m_here && k < d) ? X[zrow[row] * ldx + k] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      float av[4], bv[8];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = Xs[kk][tx + 32 * a];
-#pragma unroll
-      for (int b = 0; b < 8; ++b) bv[b] = Zs[kk][ty + 8 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
-    }
-    __syncthreads();
+  for (int u = 0; u < T::LB; ++u) {
+    const int64_t i = i0 + T::load_row(u);
+    b[u].p = i < n ? X + i * ldx : nullptr;
   }
 }
 
-__global__ void __launch_bounds__(NT) kernel_block_simt(
+template <class T, bool VEC>
+__global__ void __launch_bounds__(T::NT, 3) kernel_block_simt(
     const float* __restrict__ X, int64_t n, int64_t d, int64_t ldx,
     const float* __restrict__ norms, const int64_t* __restrict__ idx, int32_t m,
     float gamma, void* out, int32_t format, int64_t ld, int64_t plane, int64_t row0) {
-  __shared__ float Xs[TK][TM + 4];
-  __shared__ float Zs[TK][TN + 4];
-  __shared__ int64_t zrow[TN];
-  __shared__ float zn[TN];
-  const int64_t i0 = (int64_t)blockIdx.x * TM;
-  const int c0 = blockIdx.y * TN;
-  const int m_here = min(TN, m - c0);
-  if (threadIdx.x < TN) {
-    const int c = threadIdx.x;
-    const int64_t r = (c < m_here) ? idx[c0 + c] : 0;
-    zrow[c] = r;
-    zn[c] = (c < m_here) ? norms[r] : 0.f;
+  __shared__ typename T::Smem sm;
+  const int64_t i0 = (int64_t)blockIdx.x * T::TN, c0 = (int64_t)blockIdx.y * T::TM;
+  simt::FloatRows<VEC> a[T::LA], b[T::LB];
+  rbf_rows<T>(X, n, ldx, idx, i0, c0, m, a, b);
+  uint64_t acc[T::RM][4];
+  T::product(sm, a, b, 0, d, acc);
+  float xn[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int64_t i = i0 + T::col(c);
+    xn[c] = i < n ? norms[i] : 0.f;
   }
-  __syncthreads();
-  float acc[4][8];
-  dot_tile(X, n, d, ldx, zrow, i0, m_here, Xs, Zs, acc);
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int64_t i = i0 + tx + 32 * a;
-    if (i >= n) continue;
-    const float xn = norms[i];
+  for (int r = 0; r < T::RM; ++r) {
+    const int64_t c = c0 + T::row(r);
+    if (c >= m) continue;
+    const float zn = norms[idx[c]];
 #pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int c = ty + 8 * b;
-      if (c >= m_here) continue;
-      const float v = rbf_from_dot(xn, zn[c], acc[a][b], gamma);
-      kstore(out, format, plane, (row0 + c0 + c) * ld + i, v);
+    for (int h = 0; h < 2; ++h) {
+      const int64_t i = i0 + T::col(4 * h);
+      const float2 lo = simt::unpack2(acc[r][2 * h]), hi = simt::unpack2(acc[r][2 * h + 1]);
+      const float v[4] = {rbf_from_dot(xn[4 * h], zn, lo.x, gamma), rbf_from_dot(xn[4 * h + 1], zn, lo.y, gamma),
+                          rbf_from_dot(xn[4 * h + 2], zn, hi.x, gamma), rbf_from_dot(xn[4 * h + 3], zn, hi.y, gamma)};
+      const int64_t off = (row0 + c) * ld + i;
+      if (format == SPSVM_FP32 && i + 4 <= n) {
+        *reinterpret_cast<float4*>(static_cast<float*>(out) + off) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (i + e < n) kstore(out, format, plane, off + e, v[e]);
+      }
     }
   }
 }
 
 // Per tile of 128 points: partial sums over i in S of (o_i - y_i) K_ic and
-// K_ic^2 for the tile's 64 candidates, written to part[tile][c] (FP64).
-__global__ void __launch_bounds__(NT) score_partials_simt(
+// K_ic^2 for the tile's candidates, written to part[tile][c] (FP64).  A
+// thread sums 4 points at a time in FP32; everything wider is summed as
+// compensated pairs (an FP64 warp sum per candidate would outweigh the tile's
+// product at small d).
+template <class T, bool VEC>
+__global__ void __launch_bounds__(T::NT, 3) score_partials_simt(
     const float* __restrict__ X, int64_t n, int64_t d, int64_t ldx,
     const float* __restrict__ norms, const float* __restrict__ y,
     const float* __restrict__ o, const int64_t* __restrict__ idx, int32_t kappa,
     float gamma, double2* __restrict__ part) {
-  __shared__ float Xs[TK][TM + 4];
-  __shared__ float Zs[TK][TN + 4];
-  __shared__ int64_t zrow[TN];
-  __shared__ float zn[TN];
-  __shared__ double2 red[8][TN];
-  const int64_t i0 = (int64_t)blockIdx.x * TM;
-  const int c0 = blockIdx.y * TN;
-  const int m_here = min(TN, kappa - c0);
-  if (threadIdx.x < TN) {
-    const int c = threadIdx.x;
-    const int64_t r = (c < m_here) ? idx[c0 + c] : 0;
-    zrow[c] = r;
-    zn[c] = (c < m_here) ? norms[r] : 0.f;
-  }
-  __syncthreads();
-  float acc[4][8];
-  dot_tile(X, n, d, ldx, zrow, i0, m_here, Xs, Zs, acc);
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float res[4], act[4], xn[4];
+  __shared__ typename T::Smem sm;
+  const int64_t i0 = (int64_t)blockIdx.x * T::TN, c0 = (int64_t)blockIdx.y * T::TM;
+  simt::FloatRows<VEC> a[T::LA], b[T::LB];
+  rbf_rows<T>(X, n, ldx, idx, i0, c0, kappa, a, b);
+  uint64_t acc[T::RM][4];
+  T::product(sm, a, b, 0, d, acc);
+  float res[8], act[8], xn[8];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int64_t i = i0 + tx + 32 * a;
+  for (int c = 0; c < 8; ++c) {
+    const int64_t i = i0 + T::col(c);
+    res[c] = act[c] = xn[c] = 0.f;
     if (i < n) {
       const float oi = o[i], yi = y[i];
       const bool s = yi * oi < 1.0f;
-      res[a] = s ? (oi - yi) : 0.f;
-      act[a] = s ? 1.f : 0.f;
-      xn[a] = norms[i];
+      res[c] = s ? (oi - yi) : 0.f;
+      act[c] = s ? 1.f : 0.f;
+      xn[c] = norms[i];
+    }
+  }
+  // value 2 r (+ 1): the row's G (H) sum, as a pair
+  constexpr int NV = 2 * T::RM;
+  float hi[NV], lo[NV];
+#pragma unroll
+  for (int r = 0; r < T::RM; ++r) {
+    const int64_t c = c0 + T::row(r);
+    const float zn = c < kappa ? norms[idx[c]] : 0.f;
+    float gs[2] = {0.f, 0.f}, hs[2] = {0.f, 0.f};
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const float2 dot = simt::unpack2(acc[r][p]);
+      const float v0 = rbf_from_dot(xn[2 * p], zn, dot.x, gamma);
+      const float v1 = rbf_from_dot(xn[2 * p + 1], zn, dot.y, gamma);
+      gs[p >> 1] = fmaf(res[2 * p + 1], v1, fmaf(res[2 * p], v0, gs[p >> 1]));
+      hs[p >> 1] = fmaf(act[2 * p + 1] * v1, v1, fmaf(act[2 * p] * v0, v0, hs[p >> 1]));
+    }
+    hi[2 * r] = gs[0];
+    lo[2 * r] = 0.f;
+    pair_add(hi[2 * r], lo[2 * r], gs[1]);
+    hi[2 * r + 1] = hs[0];
+    lo[2 * r + 1] = 0.f;
+    pair_add(hi[2 * r + 1], lo[2 * r + 1], hs[1]);
+  }
+  // sums over the 16 threads of a row group: each exchange halves the values
+  // a thread holds, then (NV < 16) the last lanes combine
+  static_assert(T::TX == 16, "16 threads per row group");
+  const int tx = T::tx();
+  int mine = 0;
+#pragma unroll
+  for (int step = 0; step < 4; ++step) {
+    const int h = 8 >> step, cnt = NV >> (step + 1);
+    const bool up = (tx & h) != 0;
+    if (cnt > 0) {
+#pragma unroll
+      for (int k = 0; k < NV / 2; ++k) {
+        if (k >= cnt) break;
+        const float gh = up ? hi[k] : hi[k + cnt], gl = up ? lo[k] : lo[k + cnt];
+        float kh = up ? hi[k + cnt] : hi[k], kl = up ? lo[k + cnt] : lo[k];
+        pair_add(kh, kl, __shfl_xor_sync(0xffffffffu, gh, h));
+        hi[k] = kh;
+        lo[k] = kl + __shfl_xor_sync(0xffffffffu, gl, h);
+      }
+      mine += up ? cnt : 0;
     } else {
-      res[a] = 0.f; act[a] = 0.f; xn[a] = 0.f;
+      // both lanes end with the same pair: the lower lane's value first
+      const float oh = __shfl_xor_sync(0xffffffffu, hi[0], h), ol = __shfl_xor_sync(0xffffffffu, lo[0], h);
+      float kh = up ? oh : hi[0], kl = up ? ol : lo[0];
+      pair_add(kh, kl, up ? hi[0] : oh);
+      hi[0] = kh;
+      lo[0] = kl + (up ? lo[0] : ol);
     }
   }
-#pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    const int c = ty + 8 * b;
-    float gs = 0.f, hs = 0.f;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const float v = rbf_from_dot(xn[a], zn[c], acc[a][b], gamma);
-      gs = fmaf(res[a], v, gs);
-      hs = fmaf(act[a] * v, v, hs);
-    }
-    double gd = warp_sum((double)gs), hd = warp_sum((double)hs);
-    if (tx == 0) red[ty][c] = make_double2(gd, hd);
-  }
-  __syncthreads();
-  if (threadIdx.x < TN && threadIdx.x < m_here) {
-    const int c = threadIdx.x;
-    // each column c was written by exactly one warp (ty = c % 8)
-    part[(int64_t)blockIdx.x * kappa + c0 + c] = red[c % 8][c];
-  }
+  const int64_t c = c0 + T::row(mine >> 1);
+  if (c < kappa && (NV == 16 || (tx & 1) == 0))
+    reinterpret_cast<double*>(part + (int64_t)blockIdx.x * kappa + c)[mine & 1] = pair_value(hi[0], lo[0]);
+}
+
+// The 32-row tile where it wastes fewer rows, or where 64-row tiles would leave
+// SMs with one block or none (d = 784, 64 rows: n = 20,000 75 us against 83;
+// n = 30,000 110 against 85).
+bool use_narrow(int64_t n, int64_t m) {
+  return m <= 32 || 4 * ceil_div(n, PT) * ceil_div(m, (int64_t)64) < 5 * (int64_t)sm_count();
 }
 
 // g_k = lambda o[c] + sum_tiles G, h_k = lambda + sum_tiles H, delta = g^2/(2h).
@@ -184,11 +201,32 @@ __global__ void score_finish(const double2* __restrict__ part, int64_t tiles, in
 int launch_kernel_block_simt(const spsvm_points* p, const int64_t* idx, int32_t m,
                              float gamma, spsvm_kmat* out, int64_t row0, cudaStream_t s) {
   if (m == 0 || p->n == 0) return SPSVM_OK;
-  dim3 grid((unsigned)ceil_div(p->n, TM), (unsigned)ceil_div(m, TN));
-  kernel_block_simt<<<grid, NT, 0, s>>>(p->X, p->n, p->d, p->ldx, p->norms, idx, m, gamma,
-                                        out->data, out->format, out->ld, out->plane, row0);
+  auto launch = [&](auto tile, auto vec) {
+    using T = decltype(tile);
+    const dim3 grid((unsigned)ceil_div(p->n, PT), (unsigned)ceil_div(m, T::TM));
+    kernel_block_simt<T, decltype(vec)::value><<<grid, T::NT, 0, s>>>(
+        p->X, p->n, p->d, p->ldx, p->norms, idx, m, gamma, out->data, out->format, out->ld,
+        out->plane, row0);
+  };
+  const bool vec = simt::rows_aligned(p->X, p->ldx);
+  if (use_narrow(p->n, m)) vec ? launch(Narrow{}, std::true_type{}) : launch(Narrow{}, std::false_type{});
+  else vec ? launch(Wide{}, std::true_type{}) : launch(Wide{}, std::false_type{});
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
+}
+
+static void launch_score_simt(const spsvm_points* p, const float* y, const float* o,
+                              const int64_t* idx, int32_t kappa, float gamma, double2* part,
+                              cudaStream_t s) {
+  auto launch = [&](auto tile, auto vec) {
+    using T = decltype(tile);
+    const dim3 grid((unsigned)ceil_div(p->n, PT), (unsigned)ceil_div(kappa, T::TM));
+    score_partials_simt<T, decltype(vec)::value><<<grid, T::NT, 0, s>>>(
+        p->X, p->n, p->d, p->ldx, p->norms, y, o, idx, kappa, gamma, part);
+  };
+  const bool vec = simt::rows_aligned(p->X, p->ldx);
+  if (use_narrow(p->n, kappa)) vec ? launch(Narrow{}, std::true_type{}) : launch(Narrow{}, std::false_type{});
+  else vec ? launch(Wide{}, std::true_type{}) : launch(Wide{}, std::false_type{});
 }
 
 }  // namespace spsvm
@@ -233,7 +271,7 @@ namespace {
 // the gathered candidate rows of the tensor-core form
 size_t score_part_bytes(int64_t n, int32_t kappa) {
   // the larger of the two forms' tile counts (both tile 128 points today)
-  const int64_t tiles = std::max<int64_t>(ceil_div(n, TM), score_tc_tiles(n));
+  const int64_t tiles = std::max<int64_t>(ceil_div(n, PT), score_tc_tiles(n));
   return (size_t)round_up(tiles * (int64_t)kappa * (int64_t)sizeof(double2), 256);
 }
 }  // namespace
@@ -260,7 +298,7 @@ extern "C" int spsvm_score_candidates(const spsvm_points* p, const float* y, con
   cudaStream_t s = as_stream(stream);
   ProfScope prof(PROF_SCORE, s, (precision == SPSVM_BF16SPLIT ? 12.0 : 2.0) * (double)p->n * kappa * (double)p->d);
   double2* part = static_cast<double2*>(scratch);
-  int64_t tiles = ceil_div(p->n, TM);
+  int64_t tiles = ceil_div(p->n, PT);
   if (precision == SPSVM_BF16SPLIT) {
     if (!p->hi || !p->mid || !p->lo)
       return set_error(SPSVM_ERR_ARG, "score_candidates: BF16SPLIT needs split planes");
@@ -269,9 +307,7 @@ extern "C" int spsvm_score_candidates(const spsvm_points* p, const float* y, con
     SPSVM_TRY(launch_score_tc(p, y, o, idx, kappa, gamma, part, tiles,
                               static_cast<char*>(scratch) + pb, scratch_bytes - pb, s));
   } else if (precision == SPSVM_FP32) {
-    dim3 grid((unsigned)tiles, (unsigned)ceil_div(kappa, TN));
-    score_partials_simt<<<grid, NT, 0, s>>>(p->X, p->n, p->d, p->ldx, p->norms, y, o, idx,
-                                            kappa, gamma, part);
+    launch_score_simt(p, y, o, idx, kappa, gamma, part, s);
     SPSVM_LAUNCH_CHECK();
   } else {
     return set_error(SPSVM_ERR_ARG, "score_candidates: bad precision");

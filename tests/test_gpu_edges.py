@@ -97,3 +97,33 @@ def test_points_norms_and_planes(sp, n, d, pad):
     np.testing.assert_array_equal(planes[0].astype(np.float64)[:, :d] + planes[1][:, :d] + planes[2][:, :d], X)
     assert all(np.all(p[:, d:] == 0) for p in planes)
     np.testing.assert_array_equal(planes[0][:, :d], _t(X).to(torch.bfloat16).float().cpu().numpy())
+
+
+# tiles of 64 or 32 rows by 128 points, 16 features a step; the wide tile needs
+# 456 tiles of 64 rows
+@pytest.mark.parametrize("pad", [False, True])
+@pytest.mark.parametrize("n,d,m", [(127, 15, 31), (129, 17, 33), (1, 1, 1), (300, 784, 64), (58_500, 33, 65)])
+def test_fp32_block_and_score_edges(sp, n, d, m, pad):
+    """FP32 kernel values, and the scores' sums over 128 points in FP32 terms
+    of four, against float64 from direct differences."""
+    X, Xt = _points(n, d, n + m, pad)
+    g = np.random.default_rng(m)
+    J = g.choice(n, min(m, n), replace=False)
+    gamma = 0.7 / d
+    P = sp.spsvm_prepare_points(Xt, "fp32")
+    out = sp.kmat_empty(n, len(J), "fp32")
+    sp.spsvm_kernel_block(P, _t(J), gamma, "fp32", out)
+    K = O.rbf_kernel(X, X[J], gamma)                # n x m
+    sq = (X.astype(np.float64) ** 2).sum(1)
+    bound = 4 * 2.0 ** -24 * gamma * (sq[:, None] + sq[J][None, :]) + 2e-6
+    assert np.all(np.abs(out.to_float().cpu().numpy().T - K) <= bound)
+
+    y = np.where(g.random(n) < 0.5, 1.0, -1.0).astype(np.float32)
+    o = (y * (1 + 0.5 * g.standard_normal(n))).astype(np.float32)
+    gs, hs, delta = (v.cpu().numpy() for v in sp.spsvm_score_candidates(P, _t(y), _t(o), _t(J), gamma, 1e-3, "fp32"))
+    S = (y * o < 1).astype(np.float64)
+    r = S * (o.astype(np.float64) - y)
+    tol = 4 * 2.0 ** -24
+    assert np.all(np.abs(gs - (1e-3 * o[J] + K.T @ r)) <= (bound + tol * K).T @ np.abs(r) + 1e-9)
+    assert np.all(np.abs(hs - (1e-3 + (K * K).T @ S)) <= (2 * bound * K + tol * K * K).T @ S + 1e-9)
+    np.testing.assert_allclose(delta, gs * gs / (2 * hs), rtol=1e-14)
