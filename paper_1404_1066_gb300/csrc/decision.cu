@@ -1,12 +1,17 @@
 // Decision values f(q) = sum_j beta_j k(q, b_j) (Section 4: the classifier
 // h(x) = w^T phi(x) with w restricted to the basis J), tile by tile, never
 // storing the query-by-basis kernel block.  SPSVM_FP32: plain FP32 SIMT dot
-// products, FP64 accumulation of beta_j k(q, b_j) per tile of 64 basis
-// vectors.  SPSVM_BF16SPLIT: the tensor-core kernel block engine with the
-// basis rows and the queries split into three BF16 planes each, FP32 sums of
-// beta_j k over 32 basis rows per partial, the partials summed in FP64 in a
-// fixed order.
+// products, beta_j k(q, b_j) summed as compensated FP32 pairs and in FP64
+// across threads.  SPSVM_BF16SPLIT: the tensor-core kernel block engine with
+// the basis rows and the queries split into three BF16 planes each, FP32 sums
+// of beta_j k over 32 basis rows per partial, the partials summed as a
+// compensated pair in a fixed order.
+#include <cooperative_groups.h>
+
 #include "internal.h"
+#include "simt_tile.h"
+
+namespace cg = cooperative_groups;
 
 namespace spsvm {
 
@@ -17,124 +22,207 @@ int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes
 
 namespace {
 
-constexpr int QM = 128;   // queries per block
-constexpr int QN = 64;    // basis vectors per tile
-constexpr int QK = 16;
-constexpr int QT = 256;
+// Basis rows by queries.  The wide tile where there are queries enough to fill
+// the SMs; else 32 queries, half the outputs per thread and the
+// features split over four groups of threads: the loop over features is then
+// a latency chain of one warp per sub-partition, which the groups shorten, and
+// blocks that fit an SM twice let every cluster of a small request start at
+// once (with one block per SM not all clusters of 8 found room).
+using Wide = simt::Tile<64, 128, 8>;
+using Small = simt::Tile<64, 32, 4, 4>;
+constexpr int kMaxCluster = 8;
 
 __global__ void row_norms_kernel(const float* __restrict__ A, int64_t m, int64_t d, int64_t lda,
                                  float* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= m) return;
-  double acc = 0.0;
-  for (int64_t k = lane; k < d; k += 32) {
-    const float v = A[i * lda + k];
-    acc += (double)v * (double)v;
-  }
-  acc = warp_sum(acc);
-  if (lane == 0) out[i] = (float)acc;
+  float h = 0.f, l = 0.f;
+#pragma unroll 8
+  for (int64_t k = lane; k < d; k += 32) pair_add_sq(h, l, A[i * lda + k]);
+  const float s = warp_pair_sum(h, l);
+  if (lane == 0) out[i] = s;
 }
 
-__global__ void __launch_bounds__(QT) decision_simt(
+// A cluster of blocks takes one tile of queries; its blocks take the tiles of
+// 64 basis rows in turn and rank 0 adds their sums in rank order, so a small
+// request spreads over the GPU without scratch and its result does not depend
+// on the launch.  beta_j k is summed as compensated pairs with beta_j in two
+// FP32 terms (an FP64 multiply-add and conversion per kernel value, at 1/64 of
+// the FP32 rate, cost more than the dot products at small d).  FP32 ALU bound
+// for many queries, latency of the feature loop for few: 1,000 queries, 512
+// basis rows, d = 784 0.035 ms, where 8 blocks of 128 queries took 0.80 ms.
+template <class T, bool VB, bool VQ>
+__global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
     const float* __restrict__ B, int64_t m, int64_t ldb, const float* __restrict__ bnorm,
     const double* __restrict__ beta, const float* __restrict__ Q, int64_t nq, int64_t ldq,
     int64_t d, float gamma, float* __restrict__ out) {
-  __shared__ float Qs[QK][QM + 4];
-  __shared__ float Bs[QK][QN + 4];
-  __shared__ float qn[QM];
-  __shared__ float bn[QN];
-  __shared__ double bs[QN];
-  __shared__ double red[8][QM];
-  const int t = threadIdx.x, tx = t & 31, ty = t >> 5;
-  const int64_t q0 = (int64_t)blockIdx.x * QM;
-  // query norms (FP64 accumulation), one warp per query
-  for (int r = ty; r < QM; r += 8) {
-    const int64_t q = q0 + r;
-    double acc = 0.0;
-    if (q < nq)
-      for (int64_t k = tx; k < d; k += 32) {
-        const float v = Q[q * ldq + k];
-        acc += (double)v * (double)v;
-      }
-    acc = warp_sum(acc);
-    if (tx == 0) qn[r] = (float)acc;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  typename T::Smem* sm = reinterpret_cast<typename T::Smem*>(dyn);
+  constexpr int W = T::THREADS / 32;
+  __shared__ float qn[T::TN], bn[T::TM], bh[T::TM], bl[T::TM];
+  __shared__ double tot[T::TN];
+  static_assert(sizeof(typename T::Smem) >= sizeof(float2) * W * T::TN, "partial sums fit the stages");
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int64_t q0 = (int64_t)(blockIdx.x / cs) * T::TN;
+  cl.sync();   // every block of the cluster is resident before its shared memory is written
+  // query norms: the rows split over the cluster's warps, each written to every block
+  for (int r = rank * W + w; r < T::TN; r += cs * W) {
+    float h = 0.f, l = 0.f;
+    if (q0 + r < nq) {
+#pragma unroll 8
+      for (int64_t k = lane; k < d; k += 32) pair_add_sq(h, l, Q[(q0 + r) * ldq + k]);
+    }
+    const float s = warp_pair_sum(h, l);
+    if (lane < cs) *cl.map_shared_rank(&qn[r], lane) = s;
   }
-  double accd[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int64_t b0 = 0; b0 < m; b0 += QN) {
-    __syncthreads();
-    if (t < QN) {
-      const int64_t b = b0 + t;
-      bn[t] = (b < m) ? bnorm[b] : 0.f;
-      bs[t] = (b < m) ? beta[b] : 0.0;
+  cl.sync();
+  simt::FloatRows<VB> a[T::LA];
+  simt::FloatRows<VQ> b[T::LB];
+#pragma unroll
+  for (int u = 0; u < T::LB; ++u) {
+    const int64_t q = q0 + T::load_row(u);
+    b[u].p = q < nq ? Q + q * ldq : nullptr;
+  }
+  float sh[8], sl[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) sh[c] = sl[c] = 0.f;
+  // beta_j k(q, b_j) of basis row j (of the tile at b0) into the 8 queries' sums
+  auto add_row = [&](int64_t b0, int j, const float (&dot)[8]) {
+    if (b0 + j >= m) return;
+    const float zn = bn[j], ch = bh[j], cl2 = bl[j];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float k = rbf_from_dot(qn[T::col(c)], zn, dot[c], gamma);
+      const float x = __fmul_rn(ch, k);
+      sl[c] = __fadd_rn(sl[c], __fmaf_rn(cl2, k, __fmaf_rn(ch, k, -x)));
+      pair_add(sh[c], sl[c], x);
     }
-    float acc[4][8];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 8; ++c) acc[a][c] = 0.f;
-    for (int64_t k0 = 0; k0 < d; k0 += QK) {
-#pragma unroll
-      for (int r = 0; r < (QM * QK) / QT; ++r) {
-        const int e = t + QT * r;
-        const int row = e / QK, col = e % QK;
-        const int64_t q = q0 + row, k = k0 + col;
-        Qs[col][row] = (q < nq && k < d) ? Q[q * ldq + k] : 0.f;
-      }
-#pragma unroll
-      for (int r = 0; r < (QN * QK) / QT; ++r) {
-        const int e = t + QT * r;
-        const int row = e / QK, col = e % QK;
-        const int64_t b = b0 + row, k = k0 + col;
-        Bs[col][row] = (b < m && k < d) ? B[b * ldb + k] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < QK; ++kk) {
-        float av[4], bv[8];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) av[a] = Qs[kk][tx + 32 * a];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) bv[c] = Bs[kk][ty + 8 * c];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int c = 0; c < 8; ++c) acc[a][c] = fmaf(av[a], bv[c], acc[a][c]);
-      }
-      __syncthreads();
+  };
+  for (int64_t b0 = (int64_t)rank * T::TM; b0 < m; b0 += (int64_t)cs * T::TM) {
+    __syncthreads();   // the last tile's norms and coefficients have been read
+    if (t < T::TM) {
+      const int64_t j = b0 + t;
+      const double bj = j < m ? beta[j] : 0.0;
+      bn[t] = j < m ? bnorm[j] : 0.f;
+      bh[t] = (float)bj;
+      bl[t] = (float)(bj - (double)bh[t]);
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const float xn = qn[tx + 32 * a];
-      double s = 0.0;
+    for (int u = 0; u < T::LA; ++u) {
+      const int64_t j = b0 + T::load_row(u);
+      a[u].p = j < m ? B + j * ldb : nullptr;
+    }
+    uint64_t acc[T::RM][4];
+    T::block_k(sm, a, b, 0, d, acc);
+    if constexpr (T::KG > 1) {
+      float dot[8];
+      T::combine(sm, acc, dot);
+      add_row(b0, T::row(T::group()), dot);
+    } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int cc = ty + 8 * c;
-        if (b0 + cc < m) s += bs[cc] * (double)rbf_from_dot(xn, bn[cc], acc[a][c], gamma);
+      for (int r = 0; r < T::RM; ++r) {
+        float dot[8];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const float2 v = simt::unpack2(acc[r][p]);
+          dot[2 * p] = v.x;
+          dot[2 * p + 1] = v.y;
+        }
+        add_row(b0, T::row(r), dot);
       }
-      accd[a] += s;
     }
   }
+  // over the rows: the warp's row groups, the warps in order, the ranks in order
+#pragma unroll
+  for (int o = T::TX; o < 32; o <<= 1)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float oh = __shfl_xor_sync(0xffffffffu, sh[c], o), ol = __shfl_xor_sync(0xffffffffu, sl[c], o);
+      sl[c] = __fadd_rn(sl[c], ol);
+      pair_add(sh[c], sl[c], oh);
+    }
   __syncthreads();
+  float2 (*red)[T::TN] = reinterpret_cast<float2 (*)[T::TN]>(dyn);
+  if (lane < T::TX)
 #pragma unroll
-  for (int a = 0; a < 4; ++a) red[ty][tx + 32 * a] = accd[a];
+    for (int c = 0; c < 8; ++c) red[w][T::col(c)] = make_float2(sh[c], sl[c]);
   __syncthreads();
-  if (t < QM) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[w][t];
-    const int64_t q = q0 + t;
-    if (q < nq) out[q] = (float)s;
+  if (t < T::TN) {
+    float h = 0.f, l = 0.f;
+#pragma unroll
+    for (int g = 0; g < W; ++g) {
+      l = __fadd_rn(l, red[g][t].y);
+      pair_add(h, l, red[g][t].x);
+    }
+    tot[t] = pair_value(h, l);
   }
+  cl.sync();
+  if (rank == 0 && t < T::TN && q0 + t < nq) {
+    double s = tot[t];
+    for (int r = 1; r < cs; ++r) s += *cl.map_shared_rank(&tot[t], r);
+    out[q0 + t] = (float)s;
+  }
+  cl.sync();   // no block leaves while rank 0 reads its sums
 }
 
-// out[i] = sum over the P partials of column i, in FP64, in order.
-__global__ void decision_finish(const float* __restrict__ part, int64_t P, int64_t ldp,
-                                int64_t nq, float* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nq) return;
-  double s = 0.0;
-  for (int64_t p = 0; p < P; ++p) s += (double)part[p * ldp + i];
-  out[i] = (float)s;
+template <class T>
+int launch_decision_simt(int cs, const float* B, int64_t m, int64_t ldb, const float* bnorm,
+                         const double* beta, const float* Q, int64_t nq, int64_t ldq, int64_t d,
+                         float gamma, float* out, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(ceil_div(nq, T::TN) * cs));
+  cfg.blockDim = dim3(T::THREADS);
+  cfg.dynamicSmemBytes = T::KG * sizeof(typename T::Smem);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)cs;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const bool vb = simt::rows_aligned(B, ldb), vq = simt::rows_aligned(Q, ldq);
+  auto kern = vb ? (vq ? decision_simt<T, true, true> : decision_simt<T, true, false>)
+                 : (vq ? decision_simt<T, false, true> : decision_simt<T, false, false>);
+  SPSVM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)cfg.dynamicSmemBytes));
+  SPSVM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, B, m, ldb, bnorm, beta, Q, nq, ldq, d, gamma, out));
+  SPSVM_LAUNCH_CHECK();
+  return SPSVM_OK;
+}
+
+// out[i] = sum over the P partials of column i as compensated pairs: each of
+// 8 groups of threads sums every 8th partial of 32 columns, the groups are
+// added in order.  L2 bound: 32,768 columns of 128 partials
+// 9 us; one thread a column in FP64 took 24.
+constexpr int DF_G = 8;
+__global__ void __launch_bounds__(32 * DF_G) decision_finish(const float* __restrict__ part, int64_t P,
+                                                             int64_t ldp, int64_t nq,
+                                                             float* __restrict__ out) {
+  __shared__ float2 sh[DF_G][32];
+  const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t i = (int64_t)blockIdx.x * 32 + c;
+  float h = 0.f, l = 0.f;
+  if (i < nq) {
+    for (int64_t p = g; p < P; p += 8 * DF_G) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = p + u * DF_G < P ? part[(p + u * DF_G) * ldp + i] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) pair_add(h, l, v[u]);
+    }
+  }
+  sh[g][c] = make_float2(h, l);
+  __syncthreads();
+  if (g != 0 || i >= nq) return;
+#pragma unroll
+  for (int u = 1; u < DF_G; ++u) {
+    l = __fadd_rn(l, sh[u][c].y);
+    pair_add(h, l, sh[u][c].x);
+  }
+  out[i] = (float)pair_value(h, l);
 }
 
 // Queries per pass of the tensor-core form (bounds the scratch).
@@ -213,8 +301,8 @@ extern "C" int spsvm_decision(const float* B, int64_t m, int64_t ldb, const doub
                       qp + 2 * L.qc * L.ldh, L.ldh, qp + L.qc * L.ldh};
       SPSVM_TRY(spsvm_prepare_points(&qb, SPSVM_BF16SPLIT, stream));
       SPSVM_TRY(launch_decision_tc(&qb, zp, L.z_bytes, m, zb.norms, beta, gamma, part, L.qc, s));
-      decision_finish<<<(unsigned)ceil_div(cnt, (int64_t)256), 256, 0, s>>>(part, L.parts, L.qc,
-                                                                           cnt, out + q0);
+      decision_finish<<<(unsigned)ceil_div(cnt, (int64_t)32), 32 * DF_G, 0, s>>>(part, L.parts, L.qc,
+                                                                                cnt, out + q0);
       SPSVM_LAUNCH_CHECK();
     }
     return SPSVM_OK;
@@ -225,8 +313,20 @@ extern "C" int spsvm_decision(const float* B, int64_t m, int64_t ldb, const doub
     row_norms_kernel<<<(unsigned)ceil_div(m, 8), 256, 0, s>>>(B, m, d, ldb, bnorm);
     SPSVM_LAUNCH_CHECK();
   }
-  decision_simt<<<(unsigned)ceil_div(nq, QM), QT, 0, s>>>(B, m, ldb, bnorm, beta, Q, nq, ldq, d,
-                                                          gamma, out);
-  SPSVM_LAUNCH_CHECK();
-  return SPSVM_OK;
+  // up to three blocks per SM: first more blocks per query tile (basis rows
+  // split over a cluster); the small tile where that still leaves SMs with one
+  // block or none (512 rows, d = 784: 2,000 queries 70 us against 93; 4,000
+  // queries 120 against 96)
+  const int64_t want = 3 * (int64_t)sm_count(), tiles = ceil_div(nq, (int64_t)Wide::TN);
+  const int64_t basis_tiles = ceil_div(m, (int64_t)Wide::TM);
+  auto cluster = [&](int64_t query_tiles) {
+    int cs = 1;
+    while (2 * cs <= kMaxCluster && 2 * cs <= basis_tiles && query_tiles * cs < want) cs *= 2;
+    return cs;
+  };
+  const int cs = cluster(tiles);
+  if (4 * tiles * cs >= 5 * (int64_t)sm_count())
+    return launch_decision_simt<Wide>(cs, B, m, ldb, bnorm, beta, Q, nq, ldq, d, gamma, out, s);
+  return launch_decision_simt<Small>(cluster(ceil_div(nq, (int64_t)Small::TN)), B, m, ldb, bnorm, beta,
+                                     Q, nq, ldq, d, gamma, out, s);
 }

@@ -127,3 +127,35 @@ def test_fp32_block_and_score_edges(sp, n, d, m, pad):
     assert np.all(np.abs(gs - (1e-3 * o[J] + K.T @ r)) <= (bound + tol * K).T @ np.abs(r) + 1e-9)
     assert np.all(np.abs(hs - (1e-3 + (K * K).T @ S)) <= (2 * bound * K + tol * K * K).T @ S + 1e-9)
     np.testing.assert_allclose(delta, gs * gs / (2 * hs), rtol=1e-14)
+
+
+# query tiles of 128, or 32 with the basis split over 1, 2, 4 or 8 blocks and the
+# features over four groups of threads
+@pytest.mark.parametrize("pad", [False, True])
+@pytest.mark.parametrize("nq,m,d", [(1, 1, 1), (33, 63, 15), (32, 65, 17), (31, 129, 64), (100, 300, 65),
+                                    (129, 520, 31), (58_400, 64, 5)])
+def test_fp32_decision_edges(sp, nq, m, d, pad):
+    """beta_j in FP64 over 12 decades: each kernel value carries its FP32
+    bound, and the sum one FP32 rounding."""
+    X, Xt = _points(nq + m, d, nq, pad)
+    g = np.random.default_rng(d)
+    beta = g.standard_normal(m) * 10.0 ** g.uniform(-6, 6, m)
+    gamma = 0.7 / d
+    f = sp.spsvm_decision(Xt[:m], _t(beta), Xt[m:], gamma, "fp32").cpu().numpy()
+    K = O.rbf_kernel(X[m:], X[:m], gamma)
+    sq = (X.astype(np.float64) ** 2).sum(1)
+    bound = 4 * 2.0 ** -24 * gamma * (sq[m:, None] + sq[None, :m]) + 2e-6
+    ref = K @ beta
+    assert np.all(np.abs(f - ref) <= bound @ np.abs(beta) + 2.0 ** -24 * np.abs(ref))
+
+
+def test_split_decision_sums_in_pairs(sp):
+    """Partials that cancel: 1,024 basis rows (32 partials a query), beta of
+    +-1e6 in pairs on the same point; each partial's 32 terms are FP32."""
+    g = np.random.default_rng(3)
+    B = np.repeat(g.standard_normal((512, 16)), 2, axis=0).astype(np.float32)
+    Q = g.standard_normal((70, 16)).astype(np.float32)
+    beta = np.tile([1e6, -1e6], 512) + g.standard_normal(1024)
+    f = sp.spsvm_decision(_t(B), _t(beta), _t(Q), 0.05, "bf16split").cpu().numpy()
+    K = O.rbf_kernel(Q, B, 0.05)
+    assert np.all(np.abs(f - K @ beta) <= 1e6 * K.sum(1) * 8 * 2.0 ** -24)
