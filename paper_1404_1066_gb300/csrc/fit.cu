@@ -295,8 +295,9 @@ Layout make_layout(int64_t n, int64_t d, int32_t budget, int32_t precision, int3
   sc = std::max(sc, spsvm_kernel_block_scratch_bytes(L.jcap, d, precision));
   sc = std::max(sc, spsvm_reduce_scratch_bytes(n));
   sc = std::max(sc, spsvm_compact_scratch_bytes(n, L.jcap));
-  // the Gram split count depends on |J|: cover every size the fit can reach
-  for (int64_t mm = 1; mm <= L.jcap; ++mm) sc = std::max(sc, gram_part_bytes(mm, n));
+  // the Gram split count depends on |J| (through its tiles of 64 rows and
+  // more): cover every size the fit can reach
+  for (int64_t mm = 64; mm <= L.jcap; mm += 64) sc = std::max(sc, gram_part_bytes(mm, n));
   sc = std::max(sc, spsvm_line_scratch_bytes(n));
   if (score == SPSVM_SCORE_EXACT) sc = std::max(sc, spsvm_score_exact_scratch_bytes(n, d, kappa, precision));
   L.scratch_bytes = al(sc);
@@ -668,7 +669,7 @@ struct Fit {
         SPSVM_TRY(read(&kk, kdev, sizeof(kk)));
         if (kk >= 1 && kk <= kmax) {
           SPSVM_TRY(gram_impl(&Kc, n_active, n, &K, Jd, lambda, op.precision, H, ldH, scratch, sb, s,
-                              st[2], at<double>(L.off_kjj), L.jcap));
+                              (int64_t)st[2], at<double>(L.off_kjj), L.jcap));
           h_fresh = true;
           int32_t* lr_info = reinterpret_cast<int32_t*>(small + 188);
           SPSVM_TRY(spsvm_lowrank_factor(mixw, L.mix_bytes, m, Wt, SPSVM_LOWRANK_KMAX, sgn, kk, lrw,
@@ -700,7 +701,7 @@ struct Fit {
                              "Newton matrix not positive definite up to jitter 1e-2 tr(H)/|J| (|J|=%d)", m);
           if (!h_fresh) {
             SPSVM_TRY(gram_impl(&Kc, n_active, n, &K, Jd, lambda, op.precision, H, ldH, scratch, sb,
-                                s, st[2], at<double>(L.off_kjj), L.jcap));
+                                s, (int64_t)st[2], at<double>(L.off_kjj), L.jcap));
             h_fresh = true;
           }
           if (lv >= 0 && tr < 0.0) {

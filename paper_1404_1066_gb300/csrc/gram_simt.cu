@@ -1,115 +1,143 @@
 // Masked Gram matrix H = lambda K_JJ + K_SJ^T K_SJ (the generalised Hessian
 // of Eq. 4 on the active set S) in FP32 SIMT arithmetic, with FP32 sums per
-// slice of 8192 points promoted to FP64.  Also the FP64 finishing pass
+// 2,048 points added up as compensated pairs.  Also the FP64 finishing pass
 // shared by both arithmetic forms.
 #include "internal.h"
 #include "gram.h"
+#include "simt_tile.h"
 
 namespace spsvm {
 
 namespace {
 
-constexpr int GT = 64;      // output tile
-constexpr int GK = 32;      // points per smem stage
-constexpr int GNT = 256;    // 16 x 16 threads, 4 x 4 outputs each
+constexpr int64_t kChunk = 2048;     // points per FP32 sum
+// Up to this many rows the small tile (m = 512, ns = 20,000: 175 us against 214;
+// m = 700: 318 against 304).
+constexpr int64_t kSmallBasis = 512;
 
-// Maps a linear index to the (ta <= tb) upper-triangular tile pair.
-__device__ __forceinline__ void tri_index(int64_t t, int64_t T, int& ta, int& tb) {
-  // rows of the upper triangle: row a has T - a tiles
-  int a = 0;
-  int64_t rem = t;
-  while (rem >= T - a) { rem -= T - a; ++a; }
-  ta = a;
-  tb = a + (int)rem;
+// Rows a by columns b of the upper triangle.  The wide tile, and for small
+// matrices, whose blocks leave the chain over their points exposed, one with
+// the points split over four groups of threads.
+using Wide = simt::Tile<64, 128, 8>;
+using Small = simt::Tile<64, 64, 4, 4>;
+
+__device__ __forceinline__ void set_row(simt::FloatRows<true>& r, const KView& K, int64_t j, int64_t m) {
+  r.p = j < m ? static_cast<const float*>(K.data) + j * K.ld : nullptr;
+}
+__device__ __forceinline__ void set_row(simt::PlaneRows& r, const KView& K, int64_t j, int64_t m) {
+  r.hi = j < m ? static_cast<const __nv_bfloat16*>(K.data) + j * K.ld : nullptr;
+  r.plane = K.plane;
 }
 
-__global__ void __launch_bounds__(GNT) gram_simt_kernel(
-    KView Kc, int64_t m, const int64_t* __restrict__ ns_dev, int64_t slices_per_split,
-    double* __restrict__ part, int64_t ldp) {
-  __shared__ float As[GK][GT + 1];
-  __shared__ float Bs[GK][GT + 1];
-  const int64_t T = ceil_div(m, (int64_t)GT);
-  int ta, tb;
-  tri_index(blockIdx.x, T, ta, tb);
-  const int64_t a0 = (int64_t)ta * GT, b0 = (int64_t)tb * GT;
+// Column tiles of row tile ta start at the one that holds its diagonal.
+template <class T>
+__host__ __device__ __forceinline__ int64_t first_col(int64_t ta) { return ta * T::TM / T::TN; }
+template <class T>
+int64_t upper_tiles(int64_t m) {   // tiles (ta, tb) with tb >= first_col(ta)
+  const int64_t A = ceil_div(m, (int64_t)T::TM), B = ceil_div(m, (int64_t)T::TN);
+  constexpr int64_t R = T::TN / T::TM;   // row tiles per column tile
+  const int64_t f = A / R, g = A % R;    // sum over ta of ta / R
+  return A * B - (R * (f * (f - 1) / 2) + g * f);
+}
+
+// part[split][a][b] = the split's points' products, for tiles of the upper
+// triangle.  The active points are split evenly over the blocks (their number
+// is read on the device), FP32 sums per 2,048 points.  FP32 ALU bound:
+// ns = 18,000, m = 1,024 0.43 ms (44 TFLOP/s); 64 x 64 tiles of 4 x 4 outputs
+// with scalar shared loads over three slices took 1.77 ms.
+template <class T, class Rows>
+__global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 1) gram_simt_kernel(
+    KView Kc, int64_t m, const int64_t* __restrict__ ns_dev, int64_t splits,
+    float2* __restrict__ part, int64_t ldp) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  typename T::Smem* sm = reinterpret_cast<typename T::Smem*>(dyn);
   const int64_t ns = *ns_dev;
-  const int64_t p_begin = (int64_t)blockIdx.y * slices_per_split * GRAM_SLICE;
-  const int64_t p_end = min(ns, p_begin + slices_per_split * GRAM_SLICE);
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  double accd[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) accd[r][c] = 0.0;
-  for (int64_t s0 = p_begin; s0 < p_end; s0 += GRAM_SLICE) {
-    const int64_t s1 = min(p_end, s0 + GRAM_SLICE);
-    float acc[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-    for (int64_t p0 = s0; p0 < s1; p0 += GK) {
-#pragma unroll
-      for (int r = 0; r < (GT * GK) / GNT; ++r) {
-        const int e = t + GNT * r;
-        const int row = e / GK, col = e % GK;
-        const int64_t p = p0 + col;
-        const bool okp = p < s1;
-        As[col][row] = (okp && a0 + row < m) ? Kc.at(a0 + row, p) : 0.f;
-        Bs[col][row] = (okp && b0 + row < m) ? Kc.at(b0 + row, p) : 0.f;
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int kk = 0; kk < GK; ++kk) {
-        float av[4], bv[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) av[r] = As[kk][ty + 16 * r];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) accd[r][c] += (double)acc[r][c];
+  const int64_t per = gram_split_points(ns, splits, kGramQuantumSimt);
+  const int64_t p_begin = (int64_t)blockIdx.y * per;
+  if (blockIdx.y > 0 && p_begin >= ns) return;   // the finish skips the empty splits
+  const int64_t p_end = min64(ns, p_begin + per);
+  const int64_t nB = ceil_div(m, (int64_t)T::TN);
+  int64_t ta = 0, rem = blockIdx.x;
+  while (rem >= nB - first_col<T>(ta)) {
+    rem -= nB - first_col<T>(ta);
+    ++ta;
   }
-  double* P = part + (int64_t)blockIdx.y * ldp * ldp;
+  const int64_t a0 = ta * T::TM, b0 = (first_col<T>(ta) + rem) * T::TN;
+  Rows a[T::LA], b[T::LB];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int64_t a = a0 + ty + 16 * r;
+  for (int u = 0; u < T::LA; ++u) set_row(a[u], Kc, a0 + T::load_row(u), m);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int64_t b = b0 + tx + 16 * c;
-      if (a < m && b < m) P[a * ldp + b] = accd[r][c];
+  for (int u = 0; u < T::LB; ++u) set_row(b[u], Kc, b0 + T::load_row(u), m);
+  float2* P = part + (int64_t)blockIdx.y * ldp * ldp;
+  int64_t s0 = p_begin;
+  do {
+    uint64_t acc[T::RM][4];
+    T::block_k(sm, a, b, s0, min64(p_end, s0 + kChunk), acc);
+    auto put = [&](int r, const float (&v)[8]) {
+      const int64_t ra = a0 + T::row(r);
+      if (ra >= m) return;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int64_t cb = b0 + T::col(c);
+        if (cb >= m) continue;
+        float2* dst = P + ra * ldp + cb;
+        float2 sum = make_float2(v[c], 0.f);
+        if (s0 != p_begin) {
+          sum = *dst;
+          pair_add(sum.x, sum.y, v[c]);
+        }
+        *dst = sum;
+      }
+    };
+    if constexpr (T::KG > 1) {
+      float v[8];
+      T::combine(sm, acc, v);
+      put(T::group(), v);
+    } else {
+#pragma unroll
+      for (int r = 0; r < T::RM; ++r) {
+        float v[8];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const float2 x = simt::unpack2(acc[r][p]);
+          v[2 * p] = x.x;
+          v[2 * p + 1] = x.y;
+        }
+        put(r, v);
+      }
     }
-  }
+    s0 += kChunk;
+  } while (s0 < p_end);
 }
 
 }  // namespace
 
+// Splits that fill the SMs: the small tile's block has one to itself; the wide
+// tile's share it by threes (m = 1,500, ns = 30,000: 2.05 blocks per SM took
+// 2.14 ms).
 int64_t gram_simt_splits(int64_t m, int64_t ns_max) {
-  const int64_t T = ceil_div(m, (int64_t)GT);
-  const int64_t tiles = T * (T + 1) / 2;
-  const int64_t slices = ceil_div(ns_max > 0 ? ns_max : 1, GRAM_SLICE);
-  int64_t want = ceil_div(2 * (int64_t)sm_count(), tiles > 0 ? tiles : 1);
-  if (want < 1) want = 1;
-  if (want > slices) want = slices;
-  return want;
+  const int64_t sms = sm_count();
+  if (m <= kSmallBasis) return gram_splits(max64(1, upper_tiles<Small>(m)), sms, 1, 0.9, ns_max, kGramQuantumSimt);
+  const int64_t tiles = upper_tiles<Wide>(m);
+  return gram_splits(tiles, sms, ceil_div(5 * sms, 2 * tiles), 0.93, ns_max, kGramQuantumSimt);
 }
 
-int launch_gram_simt(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t ns_max, int64_t m,
-                     double* part, int64_t ldp, int64_t splits, cudaStream_t s) {
-  const int64_t T = ceil_div(m, (int64_t)GT);
-  const int64_t tiles = T * (T + 1) / 2;
-  const int64_t slices = ceil_div(ns_max > 0 ? ns_max : 1, GRAM_SLICE);
-  const int64_t per = ceil_div(slices, splits);
-  dim3 grid((unsigned)tiles, (unsigned)splits);
-  gram_simt_kernel<<<grid, GNT, 0, s>>>(view(Kc), m, ns_dev, per, part, ldp);
+int launch_gram_simt(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t m, float2* part,
+                     int64_t ldp, int64_t splits, cudaStream_t s) {
+  auto launch = [&](auto tile, auto rows) {
+    using T = decltype(tile);
+    const dim3 grid((unsigned)upper_tiles<T>(m), (unsigned)splits);
+    auto kern = gram_simt_kernel<T, decltype(rows)>;
+    const int smem = (int)(T::KG * sizeof(typename T::Smem));
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+      return;   // reported by the launch check
+    kern<<<grid, T::THREADS, smem, s>>>(view(Kc), m, ns_dev, splits, part, ldp);
+  };
+  using F = simt::FloatRows<true>;   // a stored matrix's rows are 16-byte aligned
+  using P = simt::PlaneRows;
+  const bool planes = Kc->format != SPSVM_FP32;
+  if (m <= kSmallBasis) planes ? launch(Small{}, P{}) : launch(Small{}, F{});
+  else planes ? launch(Wide{}, P{}) : launch(Wide{}, F{});
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }
@@ -132,11 +160,15 @@ __global__ void kjj_fill_kernel(KView K, const int64_t* __restrict__ J, int64_t 
 }
 
 // H[a][b] = H[b][a] = lambda K_JJ[a][b] + sum_s part[s][min(a,b)][max(a,b)]
-// over 32 x 32 upper tiles: the partials, K_JJ and both halves of H move
+// over 32 x 32 upper tiles (the partials are compensated FP32 pairs: FP64 adds
+// at 1/64 of the FP32 rate made the sum over 16 splits take 16 us at m = 100,
+// now 9): the partials, K_JJ and both halves of H move
 // through shared memory so that every global access is coalesced.
 constexpr int FT = 32;
-__global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const double* __restrict__ part,
-                                                             int64_t splits, int64_t ldp,
+__global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const float2* __restrict__ part,
+                                                             GramPlan plan,
+                                                             const int64_t* __restrict__ ns_dev,
+                                                             int64_t quantum, int64_t ldp,
                                                              const double* __restrict__ kjj,
                                                              int64_t ldk, int64_t m, double lambda,
                                                              double* __restrict__ H, int64_t ldh) {
@@ -150,17 +182,26 @@ __global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const double* __res
   }
   const int64_t tb = ta + rem;
   const int64_t a0 = ta * FT, b0 = tb * FT;
+  const int64_t ns = *ns_dev;   // the splits that hold points
+  const int64_t splits = max64(1, ceil_div(ns, gram_split_points(ns, plan.splits(ns), quantum)));
   const int c = threadIdx.x;
   const int64_t b = b0 + c;
-  for (int r = threadIdx.y; r < FT; r += 8) {
-    const int64_t a = a0 + r;
-    double sum = 0.0, kv = 0.0;
-    if (a < m && b < m) {
-      for (int64_t k = 0; k < splits; ++k) sum += part[k * ldp * ldp + a * ldp + b];
-      kv = kjj[a * ldk + b];
+  // the thread's four rows together: their partials are independent loads
+  float h[FT / 8], l[FT / 8];
+#pragma unroll
+  for (int u = 0; u < FT / 8; ++u) h[u] = l[u] = 0.f;
+#pragma unroll 4
+  for (int64_t k = 0; k < splits; ++k)
+#pragma unroll
+    for (int u = 0; u < FT / 8; ++u) {
+      const int64_t a = a0 + threadIdx.y + 8 * u;
+      if (a < m && b < m) pair_add(h[u], l[u], part[k * ldp * ldp + a * ldp + b]);
     }
-    P[r][c] = sum;
-    Kt[r][c] = kv;
+#pragma unroll
+  for (int u = 0; u < FT / 8; ++u) {
+    const int r = threadIdx.y + 8 * u;
+    P[r][c] = pair_value(h[u], l[u]);
+    Kt[r][c] = a0 + r < m && b < m ? kjj[(a0 + r) * ldk + b] : 0.0;
   }
   __syncthreads();
   for (int r = threadIdx.y; r < FT; r += 8) {
@@ -180,12 +221,12 @@ __global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const double* __res
   }
 }
 
-int launch_gram_finish(const double* part, int64_t splits, int64_t ldp, const double* kjj,
-                       int64_t ldk, int64_t m, double lambda, double* H, int64_t ldh,
+int launch_gram_finish(const float2* part, const GramPlan& plan, const int64_t* ns_dev, int64_t quantum, int64_t ldp,
+                       const double* kjj, int64_t ldk, int64_t m, double lambda, double* H, int64_t ldh,
                        cudaStream_t s) {
   const int64_t T = ceil_div(m, (int64_t)FT);
-  gram_finish_kernel<<<(unsigned)(T * (T + 1) / 2), dim3(FT, 8), 0, s>>>(part, splits, ldp, kjj,
-                                                                         ldk, m, lambda, H, ldh);
+  gram_finish_kernel<<<(unsigned)(T * (T + 1) / 2), dim3(FT, 8), 0, s>>>(part, plan, ns_dev, quantum, ldp,
+                                                                         kjj, ldk, m, lambda, H, ldh);
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }
@@ -194,9 +235,9 @@ size_t gram_part_bytes(int64_t m, int64_t ns) {
   if (m < 0 || ns < 0) return 0;
   const int64_t ldp = round_up(m > 0 ? m : 1, 64);
   int64_t splits = gram_simt_splits(m, ns);
-  const int64_t tc = gram_tc_splits(m, ns);
+  const int64_t tc = gram_tc_plan(m, ns).most();
   if (tc > splits) splits = tc;
-  return (size_t)(splits * ldp * ldp * (int64_t)sizeof(double));
+  return (size_t)(splits * ldp * ldp * (int64_t)sizeof(float2));
 }
 
 int kjj_fill(const spsvm_kmat* K, const int64_t* J, int64_t m, int64_t row0, double* kjj,
@@ -222,7 +263,7 @@ extern "C" size_t spsvm_gram_scratch_bytes(int64_t m, int64_t ns) {
 namespace spsvm {
 int gram_impl(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t ns_max, const spsvm_kmat* K,
               const int64_t* J, double lambda, int32_t precision, double* H, int64_t ldh,
-              void* scratch, size_t scratch_bytes, cudaStream_t s, double ns_work,
+              void* scratch, size_t scratch_bytes, cudaStream_t s, int64_t ns_hint,
               const double* kjj, int64_t ldk) {
   SPSVM_TRY(check_kmat(Kc, "gram(Kc)"));
   SPSVM_TRY(check_kmat(K, "gram(K)"));
@@ -237,27 +278,29 @@ int gram_impl(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t ns_max, const
   // algorithmic work: one multiply-add per active point per unique entry,
   // times the four plane products of the BF16SPLIT form
   ProfScope prof(PROF_GRAM, s,
-                 (precision == SPSVM_BF16SPLIT ? 4.0 : 1.0) * ns_work * (double)m * (double)(m + 1));
+                 (precision == SPSVM_BF16SPLIT ? 4.0 : 1.0) * (double)(ns_hint >= 0 ? ns_hint : ns_max) * (double)m * (double)(m + 1));
   const int64_t ldp = round_up(m, 64);
-  double* part = static_cast<double*>(scratch);
+  float2* part = static_cast<float2*>(scratch);
   if (!kjj) {   // gather K_JJ into the scratch behind the partial sums
     double* kj = reinterpret_cast<double*>(static_cast<char*>(scratch) + gram_part_bytes(m, ns_max));
     SPSVM_TRY(kjj_fill(K, J, m, 0, kj, ldp, s));
     kjj = kj;
     ldk = ldp;
   }
-  int64_t splits;
+  GramPlan plan{0, 1};
   if (precision == SPSVM_BF16SPLIT) {
     if (Kc->format != SPSVM_BF16SPLIT) return set_error(SPSVM_ERR_ARG, "gram: BF16SPLIT needs split planes");
-    splits = gram_tc_splits(m, ns_max);
-    SPSVM_TRY(launch_gram_tc(Kc, ns_dev, ns_max, m, part, ldp, splits, s));
+    plan = gram_tc_plan(m, ns_max);
+    SPSVM_TRY(launch_gram_tc(Kc, ns_dev, ns_max, ns_hint, m, part, ldp, plan, s));
   } else if (precision == SPSVM_FP32) {
-    splits = gram_simt_splits(m, ns_max);
-    SPSVM_TRY(launch_gram_simt(Kc, ns_dev, ns_max, m, part, ldp, splits, s));
+    plan.s_pair = gram_simt_splits(m, ns_max);
+    SPSVM_TRY(launch_gram_simt(Kc, ns_dev, m, part, ldp, plan.s_pair, s));
   } else {
     return set_error(SPSVM_ERR_ARG, "gram: bad precision");
   }
-  return launch_gram_finish(part, splits, ldp, kjj, ldk, m, lambda, H, ldh, s);
+  return launch_gram_finish(part, plan, ns_dev,
+                            precision == SPSVM_FP32 ? kGramQuantumSimt : kGramQuantumTc, ldp, kjj, ldk,
+                            m, lambda, H, ldh, s);
 }
 }  // namespace spsvm
 
@@ -266,5 +309,5 @@ extern "C" int spsvm_gram(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t n
                           double* H, int64_t ldh, void* scratch, size_t scratch_bytes,
                           void* stream) {
   return gram_impl(Kc, ns_dev, ns_max, K, J, lambda, precision, H, ldh, scratch, scratch_bytes,
-                   as_stream(stream), (double)ns_max, nullptr, 0);
+                   as_stream(stream), -1, nullptr, 0);
 }

@@ -12,8 +12,9 @@
 //   * masked Gram matrix K_SJ^T K_SJ (the Hessian term of Eq. 4 on the
 //     active set): the compact copy split as hi + lo (lo = bf16(x - hi)) and
 //     all four plane products, warp-specialised TMA producer / MMA issuer /
-//     epilogue over 128 x 128 upper-triangular tiles with two TMEM
-//     accumulators, FP32 partial sums per 8192 points promoted to FP64.
+//     epilogue over 256 x 256 upper-triangular tiles of CTA pairs with two
+//     TMEM accumulators, FP32 partial sums per 8,192 points added up as
+//     compensated pairs.
 #include <cudaTypedefs.h>
 
 #include <mutex>
@@ -402,25 +403,69 @@ __global__ void gather_rows_bf16(const uint16_t* __restrict__ Xhi, const uint16_
 }
 
 // ---------------------------------------------------------------------------
-// Masked Gram matrix: P[a][b] (+)= sum_p Kc[a][p] Kc[b][p] over 128 x 128
+// Masked Gram matrix: P[a][b] (+)= sum_p Kc[a][p] Kc[b][p] over 256 x 256
 // upper-triangular tiles, Kc = hi + lo with all four plane products, so P
 // is the Gram matrix of the stored values up to FP32 accumulation rounding
-// (positive semidefinite to that level).  Warp 0: TMEM owner and TMA producer; warp 1: MMA
-// issuer; warps 2-5: epilogue.
+// (positive semidefinite to that level).  A tile belongs to a pair of CTAs
+// (cta_group::2): each stages 128 rows of A and 128 of B, the even CTA issues
+// the 256 x 256 MMAs for both, and each drains its own 128 rows.  Per 64
+// points a CTA then loads 64 KB for 1,024 MMA cycles; a 128 x 128 tile per
+// CTA loads as much for 512, which the path from L2 to the SM cannot carry.
+// ns = 86,000, m = 2,048: 0.764 ms, 1.89 PFLOP/s, tensor pipe 96% of active
+// cycles (128 x 128 tiles: 1.9 ms, 35%).  Warp 0: TMEM owner and TMA producer;
+// warp 1: MMA issuer; warps 2-9: epilogue (warps w and w + 4 share a lane
+// quarter and split the columns).
 // ---------------------------------------------------------------------------
-constexpr int GR_THREADS = 192;
+// 32 FP32 sums into a row of the partial pairs (the first time, as they are);
+// cols: columns left in the matrix; vec: whole vectors fit the row's pitch
+// (columns past the matrix are padding).
+__device__ __forceinline__ void gram_put(float2* __restrict__ row, const float (&v)[32], int64_t cols,
+                                         bool vec, bool first) {
+  if (vec) {
+    float4* r4 = reinterpret_cast<float4*>(row);
+    if (first) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) r4[j] = make_float4(v[2 * j], 0.f, v[2 * j + 1], 0.f);
+      return;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float4 o[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) o[j] = r4[8 * h + j];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        pair_add(o[j].x, o[j].y, v[16 * h + 2 * j]);
+        pair_add(o[j].z, o[j].w, v[16 * h + 2 * j + 1]);
+        r4[8 * h + j] = o[j];
+      }
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 32; ++j) {
+    if (j < cols) {
+      float2 s = first ? make_float2(0.f, 0.f) : row[j];
+      pair_add(s.x, s.y, v[j]);
+      row[j] = s;
+    }
+  }
+}
+
+constexpr int GR_THREADS = 320;
 constexpr int GR_STAGES = 3;
-constexpr int GR_TILE = 128;
-constexpr int GR_PLANE_BYTES = GR_TILE * 128;
+constexpr int GR_TILE = 256;
+constexpr int GR_HALF = GR_TILE / 2;           // rows per CTA
+constexpr int GR_PLANE_BYTES = GR_HALF * 128;
 constexpr int GR_STAGE = 4 * GR_PLANE_BYTES;   // A hi, A lo, B hi, B lo
 constexpr int GR_BAR_OFF = GR_STAGES * GR_STAGE;
 constexpr int GR_SMEM = GR_BAR_OFF + 256 + 1024;
 constexpr int64_t GR_CHUNKS_PER_SLICE = GRAM_SLICE / 64;
 
-__global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_kernel(
+__global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
     const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
-    int64_t m, const int64_t* __restrict__ ns_dev, int64_t slices_per_split,
-    double* __restrict__ part, int64_t ldp, WaitCtx wc) {
+    int64_t m, const int64_t* __restrict__ ns_dev, GramPlan plan, float2* __restrict__ part,
+    int64_t ldp, int vec, WaitCtx wc) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + GR_BAR_OFF);
@@ -428,29 +473,209 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_kernel(
   uint64_t* accf = empty + GR_STAGES;
   uint64_t* acce = accf + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+  uint32_t* bad = tmem_slot + 1;   // [2]: a wait had given up before, as each CTA saw it
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_rank();
+  const int64_t pair = blockIdx.x >> 1;
+  // upper-triangular tile (ta <= tb)
+  const int64_t T = ceil_div(m, (int64_t)GR_TILE);
+  int64_t rem = pair, ta = 0;
+  while (rem >= T - ta) {
+    rem -= T - ta;
+    ++ta;
+  }
+  const int64_t tb = ta + rem;
+  const bool diag = ta == tb;   // the B rows are the A rows
+  const int64_t a0 = ta * GR_TILE + rank * GR_HALF, b0 = tb * GR_TILE + rank * GR_HALF;
+  const int64_t ns = *ns_dev;
+  if (plan.single(ns)) return;   // both CTAs; single CTAs take these points
+  const int64_t per = gram_split_points(ns, plan.s_pair, kGramQuantumTc);
+  const int64_t c_begin = min64(ceil_div(ns, (int64_t)64), (int64_t)blockIdx.y * (per / 64));
+  const int64_t c_end = min64(ceil_div(ns, (int64_t)64), c_begin + per / 64);
+  const int64_t nch = c_end - c_begin;
+  if (blockIdx.y > 0 && nch == 0) return;   // both CTAs; the finish skips the empty splits
+  const int64_t nslices = ceil_div(nch, GR_CHUNKS_PER_SLICE);
+  constexpr uint32_t IDESC = idesc_bf16_f32(GR_TILE, GR_TILE);
+  float2* P = part + (int64_t)blockIdx.y * ldp * ldp;
+
+  if (tid == 0) {
+    for (int s = 0; s < GR_STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&accf[a], 1);
+      mbar_init(&acce[a], 2 * 8);   // one arrival per epilogue warp of the pair
+    }
+    fence_barrier_init();
+    prefetch_tmap(&map_hi);
+    prefetch_tmap(&map_lo);
+  }
+  __syncwarp();
+  cluster_sync();   // both CTAs run, and their barriers are initialised
+  if (tid == 0) {
+    const uint32_t st = *(volatile int*)wc.st != 0 ? 1u : 0u;
+    st_cluster(map_rank(&bad[rank], 0), st);
+    st_cluster(map_rank(&bad[rank], 1), st);
+  }
+  __syncwarp();
+  if (warp == 0) tmem_alloc_pair(tmem_slot, 2 * GR_TILE);
+  fence_before_sync();
+  cluster_sync();
+  fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  const bool live = bad[0] == 0 && bad[1] == 0;   // the same in both CTAs
+
+  if (live && warp == 0 && lane == 0) {
+    // ---- TMA producer: both CTAs' loads complete on the even CTA's barrier
+    const uint32_t bytes = (diag ? 2u : 4u) * GR_PLANE_BYTES;
+    int64_t issued = 0;
+    for (int64_t q = 0; q < nch; ++q) {
+      const int s = (int)(q % GR_STAGES);
+      const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
+      if (!mbar_wait_cluster(&empty[s], ph ^ 1u, wc.st, 11, wc.lim)) break;
+      uint8_t* st = smem + s * GR_STAGE;
+      const int x = (int)((c_begin + q) * 64);
+      if (rank == 0) mbar_expect_tx(&full[s], 2 * bytes);
+      const uint32_t bar = map_rank(&full[s], 0);
+      tma_load_2d_pair(st, &map_hi, x, (int)a0, bar);
+      tma_load_2d_pair(st + GR_PLANE_BYTES, &map_lo, x, (int)a0, bar);
+      if (!diag) {
+        tma_load_2d_pair(st + 2 * GR_PLANE_BYTES, &map_hi, x, (int)b0, bar);
+        tma_load_2d_pair(st + 3 * GR_PLANE_BYTES, &map_lo, x, (int)b0, bar);
+      }
+      issued = q + 1;
+    }
+    // wait for the copies of the last stages so none is in flight at exit
+    if (rank == 0)
+      for (int64_t q = (issued > GR_STAGES ? issued - GR_STAGES : 0); q < issued; ++q)
+        mbar_wait_cluster(&full[q % GR_STAGES], (uint32_t)((q / GR_STAGES) & 1), wc.st, 12, wc.lim);
+  } else if (live && warp == 1 && lane == 0 && rank == 0) {
+    // ---- MMA issuer
+    bool ok = true;
+    for (int64_t t = 0; t < nslices && ok; ++t) {
+      const int acc = (int)(t & 1);
+      const uint32_t use = (uint32_t)((t >> 1) & 1);
+      if (!mbar_wait_cluster(&acce[acc], use ^ 1u, wc.st, 13, wc.lim)) break;
+      fence_after_sync();
+      const uint32_t d = tmem + acc * GR_TILE;
+      const int64_t q0 = t * GR_CHUNKS_PER_SLICE;
+      const int64_t q1 = min64(nch, q0 + GR_CHUNKS_PER_SLICE);
+      for (int64_t q = q0; q < q1; ++q) {
+        const int s = (int)(q % GR_STAGES);
+        const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
+        if (!mbar_wait_cluster(&full[s], ph, wc.st, 14, wc.lim)) {
+          ok = false;
+          break;
+        }
+        fence_after_sync();
+        const uint32_t base = smem_u32(smem + s * GR_STAGE);
+        const uint32_t a_hi = base, a_lo = base + GR_PLANE_BYTES;
+        const uint32_t b_hi = diag ? a_hi : base + 2 * GR_PLANE_BYTES;
+        const uint32_t b_lo = diag ? a_lo : base + 3 * GR_PLANE_BYTES;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t koff = k * 32;
+          mma_bf16_pair(d, desc_sw128(a_hi + koff), desc_sw128(b_hi + koff), IDESC,
+                        (q != q0 || k != 0) ? 1u : 0u);
+          mma_bf16_pair(d, desc_sw128(a_hi + koff), desc_sw128(b_lo + koff), IDESC, 1u);
+          mma_bf16_pair(d, desc_sw128(a_lo + koff), desc_sw128(b_hi + koff), IDESC, 1u);
+          // lo x lo too: without it the sum is (hi + lo)^T (hi + lo) - lo^T lo,
+          // indefinite in the null space of a short K_SJ
+          mma_bf16_pair(d, desc_sw128(a_lo + koff), desc_sw128(b_lo + koff), IDESC, 1u);
+        }
+        mma_commit_pair(&empty[s]);
+      }
+      mma_commit_pair(&accf[acc]);
+    }
+  } else if (live && warp >= 2) {
+    // ---- epilogue: TMEM lanes 32 * (warp % 4) .. + 31, half the columns
+    const int quarter = warp & 3;
+    const int64_t a = a0 + 32 * quarter + lane;
+    const int64_t bc = tb * GR_TILE + (warp >= 6 ? GR_HALF : 0);
+    if (nslices == 0) {
+      if (a < m)
+        for (int64_t b = bc; b < min64(m, bc + GR_HALF); ++b) P[a * ldp + b] = make_float2(0.f, 0.f);
+    }
+    for (int64_t t = 0; t < nslices; ++t) {
+      const int acc = (int)(t & 1);
+      const uint32_t use = (uint32_t)((t >> 1) & 1);
+      if (!mbar_wait_cluster(&accf[acc], use, wc.st, 15, wc.lim)) break;
+      fence_after_sync();
+      const uint32_t tbase = tmem + acc * GR_TILE + (warp >= 6 ? GR_HALF : 0) + ((uint32_t)(32 * quarter) << 16);
+      for (int cc = 0; cc < GR_HALF / 32; ++cc) {
+        const int64_t c0 = bc + cc * 32;
+        if (c0 >= m) break;   // uniform
+        float v[32];
+        __syncwarp();
+        tmem_ld32(tbase + cc * 32, v);
+        if (a < m) gram_put(P + a * ldp + c0, v, m - c0, vec && c0 + 32 <= ldp, t == 0);
+      }
+      __syncwarp();
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(map_rank(&acce[acc], 0));
+    }
+  }
+  fence_before_sync();
+  __syncwarp();
+  cluster_sync();   // no copy, MMA or arrival of the pair is outstanding
+  if (warp == 0) {
+    fence_after_sync();
+    tmem_dealloc_pair(tmem, 2 * GR_TILE);
+  }
+}
+
+// The same over 128 x 128 tiles of single CTAs, for as many points as one wave
+// of such tiles takes in separate slices (GramPlan): a slice then takes 1,160
+// cycles per 64 points, where a pair's 256 x 256 tile takes 2,048 on SMs that
+// would otherwise idle (m = 256, ns = 8,000: 90 us against 148).
+constexpr int GS_THREADS = 192;
+constexpr int GS_STAGES = 3;
+constexpr int GS_TILE = 128;
+constexpr int GS_PLANE_BYTES = GS_TILE * 128;
+constexpr int GS_STAGE = 4 * GS_PLANE_BYTES;   // A hi, A lo, B hi, B lo
+constexpr int GS_BAR_OFF = GS_STAGES * GS_STAGE;
+constexpr int GS_SMEM = GS_BAR_OFF + 256 + 1024;
+
+__global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
+    const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
+    int64_t m, const int64_t* __restrict__ ns_dev, GramPlan plan, float2* __restrict__ part,
+    int64_t ldp, int vec, WaitCtx wc) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align1024(smem_raw);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + GS_BAR_OFF);
+  uint64_t* empty = full + GS_STAGES;
+  uint64_t* accf = empty + GS_STAGES;
+  uint64_t* acce = accf + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (__syncthreads_or(tid == 0 && *(volatile int*)wc.st != 0)) return;
   // upper-triangular tile (ta <= tb)
-  const int64_t T = ceil_div(m, (int64_t)GR_TILE);
+  const int64_t T = ceil_div(m, (int64_t)GS_TILE);
   int64_t rem = blockIdx.x, ta = 0;
   while (rem >= T - ta) {
     rem -= T - ta;
     ++ta;
   }
   const int64_t tb = ta + rem;
-  const int64_t a0 = ta * GR_TILE, b0 = tb * GR_TILE;
+  const int64_t a0 = ta * GS_TILE, b0 = tb * GS_TILE;
   const int64_t ns = *ns_dev;
+  if (!plan.single(ns)) return;   // the pairs take these points
+  const int64_t per = gram_split_points(ns, plan.s_single, kGramQuantumTc);
   const int64_t chunks = ceil_div(ns, (int64_t)64);
-  const int64_t c_begin = min64(chunks, (int64_t)blockIdx.y * slices_per_split * GR_CHUNKS_PER_SLICE);
-  const int64_t c_end = min64(chunks, c_begin + slices_per_split * GR_CHUNKS_PER_SLICE);
+  const int64_t c_begin = min64(chunks, (int64_t)blockIdx.y * (per / 64));
+  const int64_t c_end = min64(chunks, c_begin + per / 64);
   const int64_t nch = c_end - c_begin;
+  if (blockIdx.y > 0 && nch == 0) return;   // the finish skips the empty splits
   const int64_t nslices = ceil_div(nch, GR_CHUNKS_PER_SLICE);
-  constexpr uint32_t IDESC = idesc_bf16_f32(GR_TILE, GR_TILE);
-  double* P = part + (int64_t)blockIdx.y * ldp * ldp;
+  constexpr uint32_t IDESC = idesc_bf16_f32(GS_TILE, GS_TILE);
+  float2* P = part + (int64_t)blockIdx.y * ldp * ldp;
 
   if (tid == 0) {
-    for (int s = 0; s < GR_STAGES; ++s) {
+    for (int s = 0; s < GS_STAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -472,21 +697,21 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_kernel(
     // ---- TMA producer
     int64_t issued = 0;
     for (int64_t q = 0; q < nch; ++q) {
-      const int s = (int)(q % GR_STAGES);
-      const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
+      const int s = (int)(q % GS_STAGES);
+      const uint32_t ph = (uint32_t)((q / GS_STAGES) & 1);
       if (!mbar_wait(&empty[s], ph ^ 1u, wc.st, 11, wc.lim)) break;
-      uint8_t* st = smem + s * GR_STAGE;
+      uint8_t* st = smem + s * GS_STAGE;
       const int x = (int)((c_begin + q) * 64);
-      mbar_expect_tx(&full[s], GR_STAGE);
+      mbar_expect_tx(&full[s], GS_STAGE);
       tma_load_2d(st, &map_hi, x, (int)a0, &full[s]);
-      tma_load_2d(st + GR_PLANE_BYTES, &map_lo, x, (int)a0, &full[s]);
-      tma_load_2d(st + 2 * GR_PLANE_BYTES, &map_hi, x, (int)b0, &full[s]);
-      tma_load_2d(st + 3 * GR_PLANE_BYTES, &map_lo, x, (int)b0, &full[s]);
+      tma_load_2d(st + GS_PLANE_BYTES, &map_lo, x, (int)a0, &full[s]);
+      tma_load_2d(st + 2 * GS_PLANE_BYTES, &map_hi, x, (int)b0, &full[s]);
+      tma_load_2d(st + 3 * GS_PLANE_BYTES, &map_lo, x, (int)b0, &full[s]);
       issued = q + 1;
     }
     // wait for the copies of the last stages so none is in flight at exit
-    for (int64_t q = (issued > GR_STAGES ? issued - GR_STAGES : 0); q < issued; ++q)
-      mbar_wait(&full[q % GR_STAGES], (uint32_t)((q / GR_STAGES) & 1), wc.st, 12, wc.lim);
+    for (int64_t q = (issued > GS_STAGES ? issued - GS_STAGES : 0); q < issued; ++q)
+      mbar_wait(&full[q % GS_STAGES], (uint32_t)((q / GS_STAGES) & 1), wc.st, 12, wc.lim);
   } else if (warp == 1 && lane == 0) {
     // ---- MMA issuer
     bool ok = true;
@@ -495,20 +720,20 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_kernel(
       const uint32_t use = (uint32_t)((t >> 1) & 1);
       if (!mbar_wait(&acce[acc], use ^ 1u, wc.st, 13, wc.lim)) break;
       fence_after_sync();
-      const uint32_t d = tmem + acc * GR_TILE;
+      const uint32_t d = tmem + acc * GS_TILE;
       const int64_t q0 = t * GR_CHUNKS_PER_SLICE;
       const int64_t q1 = min64(nch, q0 + GR_CHUNKS_PER_SLICE);
       for (int64_t q = q0; q < q1; ++q) {
-        const int s = (int)(q % GR_STAGES);
-        const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
+        const int s = (int)(q % GS_STAGES);
+        const uint32_t ph = (uint32_t)((q / GS_STAGES) & 1);
         if (!mbar_wait(&full[s], ph, wc.st, 14, wc.lim)) {
           ok = false;
           break;
         }
         fence_after_sync();
-        const uint32_t base = smem_u32(smem + s * GR_STAGE);
-        const uint32_t a_hi = base, a_lo = base + GR_PLANE_BYTES;
-        const uint32_t b_hi = base + 2 * GR_PLANE_BYTES, b_lo = base + 3 * GR_PLANE_BYTES;
+        const uint32_t base = smem_u32(smem + s * GS_STAGE);
+        const uint32_t a_hi = base, a_lo = base + GS_PLANE_BYTES;
+        const uint32_t b_hi = base + 2 * GS_PLANE_BYTES, b_lo = base + 3 * GS_PLANE_BYTES;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const uint32_t koff = k * 32;
@@ -530,25 +755,23 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_kernel(
     const int64_t a = a0 + 32 * quarter + lane;
     if (nslices == 0) {
       if (a < m)
-        for (int64_t b = b0; b < min64(m, b0 + GR_TILE); ++b) P[a * ldp + b] = 0.0;
+        for (int64_t b = b0; b < min64(m, b0 + GS_TILE); ++b) P[a * ldp + b] = make_float2(0.f, 0.f);
     }
     for (int64_t t = 0; t < nslices; ++t) {
       const int acc = (int)(t & 1);
       const uint32_t use = (uint32_t)((t >> 1) & 1);
       if (!mbar_wait(&accf[acc], use, wc.st, 15, wc.lim)) break;
       fence_after_sync();
-      const uint32_t tbase = tmem + acc * GR_TILE + ((uint32_t)(32 * quarter) << 16);
-      for (int cc = 0; cc < GR_TILE / 32; ++cc) {
+      const uint32_t tbase = tmem + acc * GS_TILE + ((uint32_t)(32 * quarter) << 16);
+      for (int cc = 0; cc < GS_TILE / 32; ++cc) {
+        const int64_t c0 = b0 + cc * 32;
+        if (c0 >= m) break;   // uniform
         float v[32];
+        __syncwarp();
         tmem_ld32(tbase + cc * 32, v);
-        if (a < m) {
-          double* row = P + a * ldp + b0 + cc * 32;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (b0 + cc * 32 + j < m) row[j] = (t == 0) ? (double)v[j] : row[j] + (double)v[j];
-          }
-        }
+        if (a < m) gram_put(P + a * ldp + c0, v, m - c0, vec && c0 + 32 <= ldp, t == 0);
       }
+      __syncwarp();
       fence_before_sync();
       mbar_arrive(&acce[acc]);
     }
@@ -700,36 +923,57 @@ int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes
                               nullptr, 0, const_cast<void*>(zplanes), zbytes, s, da);
 }
 
-int64_t gram_tc_splits(int64_t m, int64_t ns_max) {
-  const int64_t T = ceil_div(m, (int64_t)GR_TILE);
-  const int64_t tiles = T * (T + 1) / 2;
-  const int64_t slices = ceil_div(ns_max > 0 ? ns_max : 1, GRAM_SLICE);
-  int64_t want = ceil_div(2 * (int64_t)sm_count(), tiles > 0 ? tiles : 1);
-  if (want < 1) want = 1;
-  if (want > slices) want = slices;
-  return want;
+GramPlan gram_tc_plan(int64_t m, int64_t ns_max) {
+  const int64_t sms = sm_count();
+  const int64_t T1 = ceil_div(m, (int64_t)GS_TILE), T2 = ceil_div(m, (int64_t)GR_TILE);
+  GramPlan p;
+  p.s_single = min64(sms / max64(1, T1 * (T1 + 1) / 2), min64(kGramMaxSplits, ceil_div(ns_max, kGramQuantumTc)));
+  p.s_pair = gram_splits(max64(1, T2 * (T2 + 1) / 2), max64(1, sms / 2), 1, 0.9, ns_max, kGramQuantumTc);
+  return p;
 }
 
-int launch_gram_tc(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t ns_max, int64_t m,
-                   double* part, int64_t ldp, int64_t splits, cudaStream_t s) {
+// ns_hint: the number of active points when the caller knows it (only the
+// kernel it selects is launched), else -1 (both are, unless ns_max decides;
+// the one not selected returns at once).
+int launch_gram_tc(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t ns_max, int64_t ns_hint,
+                   int64_t m, float2* part, int64_t ldp, const GramPlan& plan, cudaStream_t s) {
   const uint16_t* hi = static_cast<const uint16_t*>(Kc->data);
   const uint16_t* lo = hi + Kc->plane;
-  CUtensorMap mh, ml;
-  SPSVM_TRY(make_map(&mh, hi, Kc->ld, m, Kc->ld, GR_TILE, 64));
-  SPSVM_TRY(make_map(&ml, lo, Kc->ld, m, Kc->ld, GR_TILE, 64));
-  SPSVM_CUDA_TRY(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      GR_SMEM));
-  const int64_t T = ceil_div(m, (int64_t)GR_TILE);
-  const int64_t tiles = T * (T + 1) / 2;
-  const int64_t slices = ceil_div(ns_max > 0 ? ns_max : 1, GRAM_SLICE);
-  const int64_t per = ceil_div(slices, splits);
-  dim3 grid((unsigned)tiles, (unsigned)splits);
+  const int vec = (reinterpret_cast<uintptr_t>(part) & 15) == 0;
+  CUtensorMap mh, ml;   // boxes of 128 rows in both kernels
+  static_assert(GS_TILE == GR_HALF, "one tensor map for both kernels");
+  SPSVM_TRY(make_map(&mh, hi, Kc->ld, m, Kc->ld, GR_HALF, 64));
+  SPSVM_TRY(make_map(&ml, lo, Kc->ld, m, Kc->ld, GR_HALF, 64));
   WaitCtx wc;
   SPSVM_TRY(wait_ctx(s, &wc));
-  gram_tc_kernel<<<grid, GR_THREADS, GR_SMEM, s>>>(mh, ml, m, ns_dev, per, part, ldp, wc);
-  SPSVM_LAUNCH_CHECK();
+  const bool known = ns_hint >= 0;
+  if (known ? plan.single(ns_hint) : plan.s_single > 0) {
+    SPSVM_CUDA_TRY(cudaFuncSetAttribute(gram_tc_single_kernel,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, GS_SMEM));
+    const int64_t T = ceil_div(m, (int64_t)GS_TILE);
+    const dim3 grid((unsigned)(T * (T + 1) / 2), (unsigned)plan.s_single);
+    gram_tc_single_kernel<<<grid, GS_THREADS, GS_SMEM, s>>>(mh, ml, m, ns_dev, plan, part, ldp, vec, wc);
+    SPSVM_LAUNCH_CHECK();
+  }
+  if (known ? !plan.single(ns_hint) : !plan.single(ns_max)) {
+    SPSVM_CUDA_TRY(cudaFuncSetAttribute(gram_tc_pair_kernel,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, GR_SMEM));
+    const int64_t T = ceil_div(m, (int64_t)GR_TILE);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(T * (T + 1)), (unsigned)plan.s_pair);   // two CTAs per tile
+    cfg.blockDim = dim3(GR_THREADS);
+    cfg.dynamicSmemBytes = GR_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    SPSVM_CUDA_TRY(cudaLaunchKernelEx(&cfg, gram_tc_pair_kernel, mh, ml, m, ns_dev, plan, part, ldp, vec, wc));
+    SPSVM_LAUNCH_CHECK();
+  }
   return SPSVM_OK;
 }
 
 }  // namespace spsvm
-

@@ -159,3 +159,28 @@ def test_split_decision_sums_in_pairs(sp):
     f = sp.spsvm_decision(_t(B), _t(beta), _t(Q), 0.05, "bf16split").cpu().numpy()
     K = O.rbf_kernel(Q, B, 0.05)
     assert np.all(np.abs(f - K @ beta) <= 1e6 * K.sum(1) * 8 * 2.0 ** -24)
+
+
+# FP32: 64 x 32 or 64 x 128 tiles, split form: 256 x 256 tiles of CTA pairs;
+# points in splits of at least 128, FP32 sums of 2,048 (8,192) points
+@pytest.mark.parametrize("prec,kfmt", [("fp32", "fp32"), ("fp32", "bf16split"), ("bf16split", "bf16split")])
+@pytest.mark.parametrize("m,ns", [(1, 1), (65, 127), (64, 129), (129, 0), (255, 2049), (257, 2177), (300, 40_000),
+                                  (513, 8193)])
+def test_gram_edges(sp, prec, kfmt, m, ns):
+    """H against float64, the first rows being the basis; symmetric.  FP32:
+    2,048 sequential roundings; split: the products are exact and the tensor
+    cores' FP32 accumulation truncates, 8,192 x 4 / 16 times."""
+    g = np.random.default_rng(m + ns)
+    n = max(ns, m) + 3
+    K = np.exp(-2 * g.random((m, n)))
+    km, Kref = _kmat(sp, K, kfmt)
+    S = np.zeros(n, dtype=bool)
+    S[g.choice(n, ns, replace=False)] = True
+    kc, _ = _kmat(sp, np.zeros((m, km.ld)), kfmt)
+    _, _, count, _ = sp.spsvm_compact_active(km, _t(S.astype(np.uint8)), None, None, kc)
+    J = np.arange(m)
+    H = sp.spsvm_gram(kc, count, n, km, _t(J), 0.3, prec).cpu().numpy()
+    Ks, KJ = Kref[:, S], Kref[:, J]
+    ref = 0.3 * 0.5 * (KJ + KJ.T) + Ks @ Ks.T
+    assert np.all(np.abs(H - ref) <= 2048 * 2.0 ** -24 * (Ks @ Ks.T) + 1e-12)
+    np.testing.assert_array_equal(H, H.T)
