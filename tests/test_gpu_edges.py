@@ -184,3 +184,30 @@ def test_gram_edges(sp, prec, kfmt, m, ns):
     ref = 0.3 * 0.5 * (KJ + KJ.T) + Ks @ Ks.T
     assert np.all(np.abs(H - ref) <= 2048 * 2.0 ** -24 * (Ks @ Ks.T) + 1e-12)
     np.testing.assert_array_equal(H, H.T)
+
+
+# a cluster of up to 8 blocks per 512 points, each with whole chunks of 32 rows
+@pytest.mark.parametrize("fmt", ["fp32", "bf16split"])
+@pytest.mark.parametrize("n,m", [(1, 1), (511, 33), (513, 257), (1025, 64), (3000, 1000), (80_001, 97)])
+def test_products_over_a_cluster(sp, fmt, n, m):
+    """u = K v (added to u or not) and o = K beta with the flags and stats of
+    the stored o; FP32 chunks of 32 terms, the rest FP64."""
+    g = np.random.default_rng(n + m)
+    km, Kref = _kmat(sp, np.exp(-3 * g.random((m, n))), fmt)
+    v = g.standard_normal(m)
+    u0 = g.standard_normal(n).astype(np.float32)
+    y = np.where(g.random(n) < 0.5, 1.0, -1.0).astype(np.float32)
+    ref, terms = v @ Kref, np.abs(v) @ Kref
+    tol = 33 * 2.0 ** -24 * terms + 2.0 ** -24 * (np.abs(ref) + np.abs(u0))
+    for add in (False, True):
+        u = _t(u0)
+        sp.spsvm_gemv(km, _t(v), u, accumulate=add)
+        assert np.all(np.abs(u.cpu().numpy() - ref - (u0 if add else 0)) <= tol)
+    o = torch.empty(n, dtype=torch.float32, device=DEV)
+    active, stats = sp.spsvm_outputs(km, _t(v), _t(y), o)
+    oh = o.cpu().numpy()
+    assert np.all(np.abs(oh - ref) <= tol)
+    margin = y * oh
+    np.testing.assert_array_equal(active.cpu().numpy(), margin < 1)
+    want = [0.5 * np.sum(np.maximum(0, 1 - margin.astype(np.float64)) ** 2), np.sum(margin <= 0), np.sum(margin < 1)]
+    np.testing.assert_allclose(stats.cpu().numpy(), want, rtol=1e-12)
