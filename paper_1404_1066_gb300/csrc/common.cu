@@ -172,7 +172,9 @@ struct PinnedStage {
 };
 thread_local PinnedStage t_stage;
 
-int read_back_code(cudaStream_t s, const ReadChunk* c, int n, int32_t* code) {
+// Copies the chunks (and with st the word there into *code) to the host
+// through the pinned staging memory and one synchronisation.
+int read_staged(cudaStream_t s, const ReadChunk* c, int n, const int* st, int32_t* code) {
   size_t total = 16;
   for (int k = 0; k < n; ++k) total += (size_t)round_up((int64_t)c[k].bytes, 16);
   if (t_stage.bytes < total) {
@@ -183,8 +185,6 @@ int read_back_code(cudaStream_t s, const ReadChunk* c, int n, int32_t* code) {
     SPSVM_CUDA_TRY(cudaMallocHost(&t_stage.p, want));
     t_stage.bytes = want;
   }
-  WaitCtx w;
-  SPSVM_TRY(wait_ctx(s, &w));
   char* h = static_cast<char*>(t_stage.p);
   size_t off = 16;
   for (int k = 0; k < n; ++k) {
@@ -192,15 +192,22 @@ int read_back_code(cudaStream_t s, const ReadChunk* c, int n, int32_t* code) {
       SPSVM_CUDA_TRY(cudaMemcpyAsync(h + off, c[k].src, c[k].bytes, cudaMemcpyDeviceToHost, s));
     off += (size_t)round_up((int64_t)c[k].bytes, 16);
   }
-  SPSVM_CUDA_TRY(cudaMemcpyAsync(h, w.st, sizeof(int), cudaMemcpyDeviceToHost, s));
+  if (st) SPSVM_CUDA_TRY(cudaMemcpyAsync(h, st, sizeof(int), cudaMemcpyDeviceToHost, s));
   SPSVM_CUDA_TRY(cudaStreamSynchronize(s));
   off = 16;
   for (int k = 0; k < n; ++k) {
     if (c[k].bytes) memcpy(c[k].dst, h + off, c[k].bytes);
     off += (size_t)round_up((int64_t)c[k].bytes, 16);
   }
-  int v = 0;
-  memcpy(&v, h, sizeof(int));
+  if (st) memcpy(code, h, sizeof(int));
+  return SPSVM_OK;
+}
+
+int read_back_code(cudaStream_t s, const ReadChunk* c, int n, int32_t* code) {
+  WaitCtx w;
+  SPSVM_TRY(wait_ctx(s, &w));
+  int32_t v = 0;
+  SPSVM_TRY(read_staged(s, c, n, w.st, &v));
   if (code) *code = v;
   if (v != 0) {
     SPSVM_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(int), s));
@@ -213,6 +220,10 @@ int read_back_code(cudaStream_t s, const ReadChunk* c, int n, int32_t* code) {
 
 int read_back(cudaStream_t s, const ReadChunk* chunks, int n) {
   return read_back_code(s, chunks, n, nullptr);
+}
+
+int read_plain(cudaStream_t s, const ReadChunk* chunks, int n) {
+  return read_staged(s, chunks, n, nullptr, nullptr);
 }
 
 int device_status_on(cudaStream_t s, int32_t* code) { return read_back_code(s, nullptr, 0, code); }

@@ -237,6 +237,8 @@ struct ReadChunk {
   size_t bytes;
 };
 int read_back(cudaStream_t s, const ReadChunk* chunks, int n);
+// The same without the status word (which stays as it is).
+int read_plain(cudaStream_t s, const ReadChunk* chunks, int n);
 
 // spsvm_line_search with Eq. 4's bias in basis slot 0 (point index -1):
 // b0 = &beta_0 on the device, or NULL without a bias.

@@ -211,3 +211,37 @@ def test_products_over_a_cluster(sp, fmt, n, m):
     np.testing.assert_array_equal(active.cpu().numpy(), margin < 1)
     want = [0.5 * np.sum(np.maximum(0, 1 - margin.astype(np.float64)) ** 2), np.sum(margin <= 0), np.sum(margin < 1)]
     np.testing.assert_allclose(stats.cpu().numpy(), want, rtol=1e-12)
+
+
+# one CTA up to 2,048 points, four points a thread in registers and the rest
+# read again, at most one CTA per SM; the first bracket is [0, 2]
+@pytest.mark.parametrize("n", [1, 2048, 2049, 40_001, 400_003])
+@pytest.mark.parametrize("scale", [1.0, 0.13, 0.011, 3.7, 1e-4])
+def test_line_search_finds_the_root(sp, n, scale):
+    """phi'(t) by sorted breakpoints in float64 from the same o and u: its root
+    (t near 1 / scale: inside the first bracket, or past it by up to 8^5) to a
+    few FP32 roundings of its terms over the slope there."""
+    g = np.random.default_rng(n)
+    m = min(n, 40)
+    y = np.where(g.random(n) < 0.5, 1.0, -1.0).astype(np.float32)
+    o = (y * (1 + 0.5 * g.standard_normal(n)) - 0.9 * y * (np.arange(n) == 0)).astype(np.float32)
+    step = np.where(y * o < 1, (y - o) * (1 + 0.3 * g.standard_normal(n)), 0.2 * g.standard_normal(n))
+    u = (scale * step).astype(np.float32)
+    J = np.arange(m)
+    d = scale * 1e-3 * np.abs(g.standard_normal(m)) * np.sign(u[J])   # d' K_JJ d >= 0
+    lam = 1e-3
+    a0, a1 = lam * d @ o[J].astype(np.float64), lam * d @ u[J].astype(np.float64)
+    mm = 1 - (y * o).astype(np.float64)
+    v = (y * u).astype(np.float64)
+    f = lambda t: a0 + a1 * t - np.sum(v * np.maximum(0, mm - t * v))  # noqa: E731
+    t = sp.spsvm_line_search(_t(o), _t(u), _t(y), _t(d), _t(J), lam)
+    if not f(0.0) < 0:
+        assert t == 0.0
+        return
+    lo, hi = 0.0, 2.0 * 8.0 ** 12
+    for _ in range(200):
+        mid = 0.5 * (lo + hi)
+        lo, hi = (mid, hi) if f(mid) < 0 else (lo, mid)
+    slope = a1 + np.sum(np.where(mm - hi * v > 0, v * v, 0))
+    noise = abs(a0) + abs(a1) * hi + np.sum(np.abs(v) * np.maximum(0, np.abs(mm) + hi * np.abs(v)))
+    assert abs(t - hi) <= 8 * 2.0 ** -24 * noise / slope + 1e-6 * hi
