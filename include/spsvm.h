@@ -315,11 +315,12 @@ int spsvm_cholesky_solve(const double* L, int64_t m, int64_t ldh, double* b, voi
  * (row-major); the upper triangle of each 64 x 64 diagonal block holds that
  * block's inverse, transposed.  The factorisation is one launch over
  * 64 x 64 tiles whose bounded waits give up after about a second
- * (spsvm_device_status then reports TIMEOUT).  spsvm_solve_mixed then
- * solves for b (device FP64, m) into x (device FP64, m) with the factor in
- * work.  The first three refinement steps are queued at once (a step's
- * kernels return at once on the device when an earlier step reached tol),
- * then the stream is synchronised once, and once per further step; it
+ * (spsvm_device_status then reports TIMEOUT); the inverses of the factor's
+ * diagonal blocks of up to 1,024 rows follow, also in work.
+ * spsvm_solve_mixed then solves for b (device FP64, m) into x (device FP64,
+ * m) with what work holds.  All refinement steps run in one cooperative
+ * launch (bounded grid barriers), after which the stream is synchronised
+ * once; it
  * returns OK, or SPSVM_ERR_NO_CONVERGE when the residual stops shrinking (by
  * half per step, from the third step on) or max_iter steps do not reach tol
  * (x then holds the last iterate).  iters, backward_error: host, may be

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "refine.h"
 
 namespace spsvm {
 
@@ -462,292 +463,10 @@ __global__ void __launch_bounds__(SV_THREADS) trsv_bwd_onepass(
   if (t == 0) st_release_u32(&flags[k], 1u);
 }
 
-// FP32 one-pass triangular solves whose results travel as self-validating
-// 64-bit words (tag << 32 | float bits; a 64-bit store is single-copy
-// atomic), so a block's result needs no flag, fence or second load.  In each
-// CTA warp 0 alone polls (two words per lane cover a 64-value block), takes
-// up to SV_BATCH published blocks at once into shared memory, and one
-// barrier hands them to the CTA.  A block that gives up publishes with the
-// tag's top bit set; its dependants give up at once.
-constexpr int SV_BATCH = 8;
-
-// A refinement step's kernels return at once when the solve's stop word is
-// set (the backward error was reached, or the refinement failed): the host
-// enqueues several steps ahead and checks once.
-__device__ __forceinline__ bool refine_stopped(const int* stop) {
-  return stop && *reinterpret_cast<const volatile int*>(stop) != 0;
-}
-
-
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// Warp 0: stages the published blocks blk[0], blk[1], ... (up to want, in
-// that order; rows at or past m count as published zeros) into xs until the
-// first one not yet published, waiting (bounded) while not even blk[0] is.
-// Returns the number staged, or -1 when a block is abandoned or the wait
-// runs out.
-__device__ int grab_blocks(const unsigned long long* __restrict__ wt, int64_t m, int64_t first,
-                           int step, int want, unsigned tag, float (*xs)[NB], int code,
-                           const WaitCtx& w) {
-  const uint32_t lim = wait_limit(w, 1u << 20);
-  const int lane = threadIdx.x & 31;
-  const unsigned abt = tag | 0x80000000u;
-  for (uint32_t it = 0;; ++it) {
-    unsigned long long w0[SV_BATCH], w1[SV_BATCH];
-#pragma unroll
-    for (int u = 0; u < SV_BATCH; ++u) {
-      const int64_t base = (first + (int64_t)step * u) * NB;
-      w0[u] = w1[u] = (unsigned long long)tag << 32;
-      if (u < want) {
-        if (base + lane < m) w0[u] = ld_relaxed_u64(wt + base + lane);
-        if (base + 32 + lane < m) w1[u] = ld_relaxed_u64(wt + base + 32 + lane);
-      }
-    }
-    int got = 0;
-    bool ab = false;
-#pragma unroll
-    for (int u = 0; u < SV_BATCH; ++u) {
-      if (u < want && got == u && !ab) {
-        const unsigned h0 = (unsigned)(w0[u] >> 32), h1 = (unsigned)(w1[u] >> 32);
-        ab = __any_sync(0xffffffffu, h0 == abt || h1 == abt);
-        if (!ab && __all_sync(0xffffffffu, h0 == tag && h1 == tag)) {
-          xs[u][lane] = __uint_as_float((unsigned)w0[u]);
-          xs[u][32 + lane] = __uint_as_float((unsigned)w1[u]);
-          ++got;
-        }
-      }
-    }
-    if (ab) return -1;
-    if (got > 0) return got;
-    if (it >= lim) {
-      if (lane == 0) wait_gave_up(w, code);
-      return -1;
-    }
-    if (it >= 8) __nanosleep(32);
-  }
-}
-
-// z = L^{-1} b (FP32).  Thread t: row t / 4 of the block row, columns
-// 16 (t % 4) .. + 15 of each earlier 64-column block.
-__global__ void __launch_bounds__(SV_THREADS) trsv32_fwd(const float* __restrict__ L, int64_t ldh,
-                                                        int64_t m, const float* __restrict__ b,
-                                                        unsigned long long* __restrict__ zt,
-                                                        float* __restrict__ z,
-                                                        unsigned* __restrict__ ticket, unsigned tag,
-                                                        WaitCtx wc, const int* stop) {
-  if (refine_stopped(stop)) return;
-  __shared__ float Li[NB][NB + 1];
-  __shared__ float xs[SV_BATCH][NB];
-  __shared__ float v[NB];
-  __shared__ unsigned k_s;
-  __shared__ int n_s;
-  const int t = threadIdx.x;
-  if (t == 0) k_s = atomicAdd(ticket, 1u);
-  __syncthreads();
-  const int64_t k = k_s;
-  const int64_t r0 = k * NB;
-  const int nb = (int)min64(NB, m - r0);
-  load_diag_inverse(L, ldh, r0, nb, Li);
-  const int r = t >> 2, q = t & 3;
-  const bool row_ok = r < nb;
-  const float* __restrict__ Lrow = L + (r0 + (row_ok ? r : 0)) * ldh + 16 * q;
-  float acc = 0.0f;
-  bool ok = true;
-  // the row's values against block jj (zeros past k); blocks j (a) and
-  // j + 1 (nxt) are loaded a step ahead of their use
-  auto ld = [&](float (&v)[16], int64_t jj) {
-    const bool in = row_ok && jj < k;
-#pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] = in ? __ldg(Lrow + jj * NB + c) : 0.0f;
-  };
-  float a[16], nxt[16];
-  ld(a, 0);
-  ld(nxt, 1);
-  for (int64_t j = 0; j < k;) {
-    if (t < 32) {
-      const int g = grab_blocks(zt, m, j, 1, (int)min64(SV_BATCH, k - j), tag, xs, 221, wc);
-      if (t == 0) n_s = g;
-    }
-    __syncthreads();
-    const int got = n_s;
-    if (got < 0) {
-      ok = false;
-      break;
-    }
-#pragma unroll
-    for (int c = 0; c < 16; ++c) acc = fmaf(a[c], xs[0][16 * q + c], acc);
-    if (got > 1) {
-#pragma unroll
-      for (int c = 0; c < 16; ++c) acc = fmaf(nxt[c], xs[1][16 * q + c], acc);
-    }
-    for (int u = 2; u < got; ++u) {
-#pragma unroll
-      for (int c = 0; c < 16; ++c)
-        acc = fmaf(row_ok ? __ldg(Lrow + (j + u) * NB + c) : 0.0f, xs[u][16 * q + c], acc);
-    }
-    __syncthreads();   // xs free again
-    j += got;
-    if (got == 1) {
-#pragma unroll
-      for (int c = 0; c < 16; ++c) a[c] = nxt[c];
-    } else {
-      ld(a, j);
-    }
-    ld(nxt, j + 1);
-  }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  if (q == 0) v[r] = row_ok ? b[r0 + r] - acc : 0.0f;
-  __syncthreads();
-  float sres = 0.0f;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) sres = fmaf(Li[r][16 * q + c], v[16 * q + c], sres);
-  sres += __shfl_xor_sync(0xffffffffu, sres, 1);
-  sres += __shfl_xor_sync(0xffffffffu, sres, 2);
-  if (q == 0 && row_ok) {
-    z[r0 + r] = sres;
-    st_relaxed_u64(zt + r0 + r, ((unsigned long long)(ok ? tag : (tag | 0x80000000u)) << 32) |
-                                    __float_as_uint(sres));
-  }
-}
-
-// x = L^{-T} z (FP32).  Block rows from the last; thread t: column t % 64 of
-// the block, rows 16 (t / 64) .. + 15 of each later 64-row block.
-__global__ void __launch_bounds__(SV_THREADS) trsv32_bwd(const float* __restrict__ L, int64_t ldh,
-                                                        int64_t m, const float* __restrict__ z,
-                                                        unsigned long long* __restrict__ xt,
-                                                        double* __restrict__ xacc,
-                                                        double* __restrict__ xmax,
-                                                        unsigned* __restrict__ ticket, unsigned tag,
-                                                        WaitCtx wc, const int* stop) {
-  if (refine_stopped(stop)) return;
-  __shared__ float Li[NB][NB + 1];
-  __shared__ float xs[SV_BATCH][NB];
-  __shared__ float part[4][NB];
-  __shared__ float v[NB];
-  __shared__ double xm[2];
-  __shared__ unsigned k_s;
-  __shared__ int n_s;
-  const int t = threadIdx.x;
-  const int64_t B = ceil_div(m, (int64_t)NB);
-  if (t == 0) k_s = atomicAdd(ticket, 1u);
-  __syncthreads();
-  const int64_t k = B - 1 - (int64_t)k_s;
-  const int64_t r0 = k * NB;
-  const int nb = (int)min64(NB, m - r0);
-  load_diag_inverse(L, ldh, r0, nb, Li);
-  const int c = t & (NB - 1), g = t >> 6;
-  const bool col_ok = c < nb;
-  float acc = 0.0f;
-  bool ok = true;
-  // block jj's rows against this block's column (zeros at or before k);
-  // blocks j (a) and j - 1 (nxt) are loaded a step ahead of their use
-  auto ld = [&](float (&v)[16], int64_t jj) {
-    const int64_t rb = jj * NB + 16 * g;
-    const bool live = col_ok && jj > k;
-#pragma unroll
-    for (int rr = 0; rr < 16; ++rr)
-      v[rr] = (live && rb + rr < m) ? __ldg(L + (rb + rr) * ldh + r0 + c) : 0.0f;
-  };
-  float a[16], nxt[16];
-  ld(a, B - 1);
-  ld(nxt, B - 2);
-  for (int64_t j = B - 1; j > k;) {   // later blocks, last first
-    if (t < 32) {
-      const int gb = grab_blocks(xt, m, j, -1, (int)min64(SV_BATCH, j - k), tag, xs, 222, wc);
-      if (t == 0) n_s = gb;
-    }
-    __syncthreads();
-    const int got = n_s;
-    if (got < 0) {
-      ok = false;
-      break;
-    }
-#pragma unroll
-    for (int rr = 0; rr < 16; ++rr) acc = fmaf(a[rr], xs[0][16 * g + rr], acc);
-    if (got > 1) {
-#pragma unroll
-      for (int rr = 0; rr < 16; ++rr) acc = fmaf(nxt[rr], xs[1][16 * g + rr], acc);
-    }
-    for (int u = 2; u < got; ++u) {
-      const int64_t rbu = (j - u) * NB + 16 * g;   // a full block (only the last is partial)
-#pragma unroll
-      for (int rr = 0; rr < 16; ++rr)
-        acc = fmaf(col_ok ? __ldg(L + (rbu + rr) * ldh + r0 + c) : 0.0f, xs[u][16 * g + rr], acc);
-    }
-    __syncthreads();
-    j -= got;
-    if (got == 1) {
-#pragma unroll
-      for (int rr = 0; rr < 16; ++rr) a[rr] = nxt[rr];
-    } else {
-      ld(a, j);
-    }
-    ld(nxt, j - 1);
-  }
-  part[g][c] = acc;
-  __syncthreads();
-  if (t < NB) v[t] = (t < nb) ? z[r0 + t] - (part[0][t] + part[1][t] + part[2][t] + part[3][t]) : 0.0f;
-  __syncthreads();
-  float sres = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) sres = fmaf(Li[16 * g + i][c], v[16 * g + i], sres);
-  part[g][c] = sres;
-  __syncthreads();
-  // publish the block (the chain), then x += the correction in FP64 and
-  // the block's maximum of |x|
-  double am = 0.0;
-  if (t < nb) {
-    const float xv = part[0][t] + part[1][t] + part[2][t] + part[3][t];
-    st_relaxed_u64(xt + r0 + t, ((unsigned long long)(ok ? tag : (tag | 0x80000000u)) << 32) |
-                                    __float_as_uint(xv));
-    const double xn = xacc[r0 + t] + (double)xv;
-    xacc[r0 + t] = xn;
-    am = fabs(xn);
-  }
-  if (t < NB) {   // warps 0 and 1
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) am = fmax(am, __shfl_xor_sync(0xffffffffu, am, o));
-    if ((t & 31) == 0) xm[t >> 5] = am;
-  }
-  __syncthreads();
-  if (t == 0) xmax[k] = fmax(xm[0], xm[1]);
-}
-
 // ---------------------------------------------------------------------------
 // Mixed precision: FP32 factor of H + shift I, FP64 iterative refinement.
 // ---------------------------------------------------------------------------
 constexpr int MX_T = 256;
-
-// FP64 -> FP32 with round to nearest even, from the IEEE-754 encodings with
-// integer operations only (GB300 issues the FP64 conversion instruction at
-// its FP64 rate).  Results below the FP32 normal range flush to signed zero
-// and results above it become infinity (an FP32 factor then breaks down and
-// the caller falls back to FP64).
-__device__ __forceinline__ float f64_to_f32_rn(double v) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
-  const int e = (int)((u >> 52) & 0x7ff) - 1023 + 127;
-  const unsigned long long man = u & 0xfffffffffffffull;
-  if ((int)((u >> 52) & 0x7ff) == 0x7ff)   // inf / nan
-    return __uint_as_float(sign | 0x7f800000u | (man ? 0x400000u : 0u));
-  if (e <= 0) return __uint_as_float(sign);
-  if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
-  const unsigned m23 = (unsigned)(man >> 29);
-  const unsigned rem = (unsigned)(man & 0x1fffffffu);
-  const unsigned up = (rem > 0x10000000u) || (rem == 0x10000000u && (m23 & 1u));
-  unsigned bits = ((unsigned)e << 23) + m23 + up;   // a carry moves into the exponent
-  if (bits >= 0x7f800000u) bits = 0x7f800000u;
-  return __uint_as_float(sign | bits);
-}
 
 // L (FP32, lower triangle) = H + shift I, one block per row (the row's
 // loads all in flight at once); rowsum[r] = sum_c |H_rc + shift [c = r]|,
@@ -1492,89 +1211,6 @@ __global__ void __launch_bounds__(DAG_T, 1) chol32_dag(float* __restrict__ L, in
   }
 }
 
-// r = b - (H + shift I) x (H full and symmetric, FP64), one warp per row,
-// 16-byte loads four deep per lane when H's rows and x are 16-byte aligned;
-// z = (float) r, the next refinement step's right-hand side; block maxima
-// of |r|.
-template <bool VEC>
-__global__ void __launch_bounds__(MX_T) residual_f64(const double* __restrict__ H, int64_t ldh,
-                                                     int64_t m, double shift,
-                                                     const double* __restrict__ b,
-                                                     const double* __restrict__ x,
-                                                     double* __restrict__ r,
-                                                     float* __restrict__ z,
-                                                     double* __restrict__ rmax, const int* stop) {
-  if (refine_stopped(stop)) return;
-  __shared__ double wm[MX_T / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t i = (int64_t)blockIdx.x * (MX_T / 32) + w;
-  double a = 0.0;
-  if (i < m) {
-    const double* __restrict__ Hi = H + i * ldh;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    if (VEC) {
-      const double2* __restrict__ H2 = reinterpret_cast<const double2*>(Hi);
-      const double2* __restrict__ x2 = reinterpret_cast<const double2*>(x);
-      const int64_t half = m >> 1;
-      for (int64_t c = lane; c < half; c += 128) {
-        double2 h0 = make_double2(0, 0), h1 = h0, h2 = h0, h3 = h0;
-        double2 x0 = h0, x1 = h0, y2 = h0, x3 = h0;
-        if (c < half) { h0 = H2[c]; x0 = x2[c]; }
-        if (c + 32 < half) { h1 = H2[c + 32]; x1 = x2[c + 32]; }
-        if (c + 64 < half) { h2 = H2[c + 64]; y2 = x2[c + 64]; }
-        if (c + 96 < half) { h3 = H2[c + 96]; x3 = x2[c + 96]; }
-        s0 = fma(h0.y, x0.y, fma(h0.x, x0.x, s0));
-        s1 = fma(h1.y, x1.y, fma(h1.x, x1.x, s1));
-        s2 = fma(h2.y, y2.y, fma(h2.x, y2.x, s2));
-        s3 = fma(h3.y, x3.y, fma(h3.x, x3.x, s3));
-      }
-      if ((m & 1) && lane == 0) s0 = fma(Hi[m - 1], x[m - 1], s0);
-    } else {
-      for (int64_t c = lane; c < m; c += 128) {
-        s0 = fma(Hi[c], x[c], s0);
-        if (c + 32 < m) s1 = fma(Hi[c + 32], x[c + 32], s1);
-        if (c + 64 < m) s2 = fma(Hi[c + 64], x[c + 64], s2);
-        if (c + 96 < m) s3 = fma(Hi[c + 96], x[c + 96], s3);
-      }
-    }
-    const double s = warp_sum((s0 + s1) + (s2 + s3));
-    if (lane == 0) {
-      const double ri = b[i] - s - shift * x[i];
-      r[i] = ri;
-      z[i] = f64_to_f32_rn(ri);
-      a = fabs(ri);
-    }
-  }
-  if (lane == 0) wm[w] = a;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double mx = 0.0;
-    for (int k = 0; k < MX_T / 32; ++k) mx = fmax(mx, wm[k]);
-    rmax[blockIdx.x] = mx;
-  }
-}
-
-// Block maxima of |v|, and z = (float) v.
-__global__ void __launch_bounds__(MX_T) absmax_blocks(const double* __restrict__ v, int64_t m,
-                                                      double* __restrict__ out, float* __restrict__ z) {
-  __shared__ double wm[MX_T / 32];
-  const int64_t i = (int64_t)blockIdx.x * MX_T + threadIdx.x;
-  double a = 0.0;
-  if (i < m) {
-    a = fabs(v[i]);
-    z[i] = f64_to_f32_rn(v[i]);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = a;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double mx = 0.0;
-    for (int k = 0; k < MX_T / 32; ++k) mx = fmax(mx, wm[k]);
-    out[blockIdx.x] = mx;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Low-rank correction of the FP32 factor.  Between Newton steps of Section
 // 4's reoptimisation the active set changes by a few points, and with it the
@@ -1809,128 +1445,6 @@ __global__ void __launch_bounds__(LR_INV_T) lr_invert(float* __restrict__ C, int
   if (t == 0) *info = 0;
 }
 
-// Partial dot products s_z[a] = sum_{i in slice z} V[i][a] z[i] over slices
-// of LR_ROWS rows (FP32 products and sums): one block per slice and 16
-// columns; thread t: column t % 16, rows t / 16 + 16 q of the slice.
-__global__ void __launch_bounds__(256) lr_dots(const float* __restrict__ V, int64_t ldv, int64_t m,
-                                              const float* __restrict__ z, int64_t ldp,
-                                              float* __restrict__ sp, const int* stop) {
-  if (refine_stopped(stop)) return;
-  __shared__ float part[16][LR_G + 1];
-  const int c = threadIdx.x & 15, rr = threadIdx.x >> 4;
-  const int a = blockIdx.x * LR_G + c;
-  const int64_t lo = (int64_t)blockIdx.y * LR_ROWS, hi = min64(m, lo + LR_ROWS);
-  float f = 0.f;
-  for (int64_t i = lo + rr; i < hi; i += 16) f = fmaf(V[i * ldv + a], z[i], f);
-  part[rr][c] = f;
-  __syncthreads();
-  if (rr == 0) {
-    float v = 0.f;
-    for (int q = 0; q < 16; ++q) v += part[q][c];
-    sp[(int64_t)blockIdx.y * ldp + a] = v;
-  }
-}
-
-// z[i] -= sum_a V[i][a] w[a], w = C^{-1} s with s the sum of the slices'
-// partial dot products (fixed order), computed by every block (k^2
-// multiply-adds, cheap next to a launch).  Sixteen rows per block pass; lane
-// c of a row covers columns c, c + 16, ...
-__global__ void __launch_bounds__(256) lr_update(const float* __restrict__ V, int64_t ldv, int64_t m,
-                                                const float* __restrict__ Ci, int64_t ldc,
-                                                const float* __restrict__ sp, int64_t slices,
-                                                int64_t ldp, int32_t k, float* __restrict__ z,
-                                                const int* stop) {
-  if (refine_stopped(stop)) return;
-  __shared__ float ws[SPSVM_LOWRANK_KMAX];
-  __shared__ float ss[SPSVM_LOWRANK_KMAX];
-  for (int a = threadIdx.x; a < k; a += 256) {
-    double v = 0.0;
-    for (int64_t q = 0; q < slices; ++q) v += (double)sp[q * ldp + a];
-    ss[a] = (float)v;
-  }
-  __syncthreads();
-  for (int a = threadIdx.x; a < k; a += 256) {
-    float v = 0.f;
-    for (int b = 0; b < k; ++b) v = fmaf(Ci[a * ldc + b], ss[b], v);
-    ws[a] = v;
-  }
-  __syncthreads();
-  const int c = threadIdx.x & 15, rr = threadIdx.x >> 4;
-  for (int64_t i0 = (int64_t)blockIdx.x * 16; i0 < m; i0 += (int64_t)gridDim.x * 16) {
-    const int64_t i = i0 + rr;
-    float v = 0.f;
-    if (i < m)
-      for (int a = c; a < k; a += 16) v = fmaf(V[i * ldv + a], ws[a], v);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, 16);
-    if (c == 0 && i < m) z[i] -= v;
-  }
-}
-
-// The refinement's state on the device: stop word (0 running, 1 backward
-// error reached, 2 stagnation, 3 not finite, 4 the FP32 factorisation broke
-// down), steps taken, the last backward error and residual norm.
-struct RefineState {
-  int32_t stop, iters;
-  double be, rprev;
-};
-
-// Maximum of v[0..n) over the block (result in thread 0).
-__device__ double block_max(const double* __restrict__ v, int64_t n, double* sh) {
-  double a = 0.0;
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) a = fmax(a, v[e]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
-  __syncthreads();
-  double r = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r = fmax(r, sh[k]);
-  return r;
-}
-
-// After refinement step `it` (one block of MX_T threads): the norms from the
-// block maxima (at the first step also ||H + shift I|| and ||b||), the
-// normwise backward error ||r|| / (||H + shift I|| ||x|| + ||b||), and the
-// stop word.  Stagnation (the residual norm not halved) counts from the
-// third step, the first two being the FP32 solve and its first correction.
-__global__ void __launch_bounds__(MX_T) refine_decide(
-    const double* __restrict__ xmax, int64_t nx, const double* __restrict__ rmax, int64_t nr,
-    const double* __restrict__ rowmax, int64_t nh, const double* __restrict__ bmax, int64_t nbm,
-    double* __restrict__ norms, const int32_t* __restrict__ finfo, int it, double tol, void* state) {
-  __shared__ double sh[MX_T / 32];
-  __shared__ int stop_s;
-  RefineState* st = static_cast<RefineState*>(state);
-  if (threadIdx.x == 0) stop_s = *reinterpret_cast<const volatile int32_t*>(&st->stop);
-  __syncthreads();
-  if (stop_s) return;
-  if (it == 0) {
-    const double h = block_max(rowmax, nh, sh);
-    const double bb = block_max(bmax, nbm, sh);
-    if (threadIdx.x == 0) {
-      norms[0] = h;
-      norms[1] = bb;
-    }
-  }
-  const double xn = block_max(xmax, nx, sh);
-  const double rn = block_max(rmax, nr, sh);
-  if (threadIdx.x != 0) return;
-  if (finfo && *finfo != 0) {
-    st->stop = 4;
-    return;
-  }
-  const double hn = norms[0], bn = norms[1];
-  const double denom = hn * xn + bn;
-  const double be = denom > 0.0 ? rn / denom : 0.0;
-  st->iters = it + 1;
-  st->be = be;
-  if (!(be == be)) st->stop = 3;
-  else if (be <= tol) st->stop = 1;
-  else if (it >= 2 && rn > 0.5 * st->rprev) st->stop = 2;
-  st->rprev = rn;
-}
-
 }  // namespace
 }  // namespace spsvm
 
@@ -2111,11 +1625,9 @@ extern "C" int spsvm_cholesky_solve(const double* L, int64_t m, int64_t ldh, dou
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int kTicketSteps = 64;   // refinement steps between ticket resets
-
 struct MixedLayout {
-  int64_t ldl, B, nrow_blocks, nvec_blocks;
-  size_t L, sw, sw_bytes, z32, r, rowmax, xmax, rmax, bmax, norms, state, dag, total;
+  int64_t ldl, B;
+  size_t L, W, WT, T, v, z, xs, rowsum, red, state, dag, total;
   int64_t tiles;   // tile rows of the factor
 };
 
@@ -2124,22 +1636,19 @@ MixedLayout mixed_layout(int64_t m) {
   auto al = [](size_t b) { return (size_t)round_up((int64_t)b, (int64_t)256); };
   ly.ldl = round_up(m, (int64_t)4);
   ly.B = ceil_div(m, (int64_t)NB);
-  ly.nrow_blocks = ceil_div(m, (int64_t)(MX_T / 32));
-  ly.nvec_blocks = ceil_div(m, (int64_t)MX_T);
   size_t off = 0;
   ly.L = off;      off += al((size_t)m * ly.ldl * 4);
-  // solve scratch: the forward result (FP32), the tagged words of both
-  // solves, and per-step tickets of the two launches (zeroed once per call)
-  ly.sw = off;     ly.sw_bytes = al((size_t)m * 4) + al((size_t)m * 16) + al((size_t)2 * kTicketSteps * 4);
-  off += ly.sw_bytes;
-  ly.z32 = off;    off += al((size_t)m * 4);
-  ly.r = off;      off += al((size_t)m * 8);
-  ly.rowmax = off; off += al((size_t)m * 8);
-  ly.xmax = off;   off += al((size_t)ly.B * 8);   // per 64-row block of the backward solve
-  ly.rmax = off;   off += al((size_t)ly.nrow_blocks * 8);
-  ly.bmax = off;   off += al((size_t)ly.nvec_blocks * 8);
-  ly.norms = off;  off += al(8 * 8);
-  ly.state = off;  off += al(sizeof(RefineState));
+  // inverses of the factor's diagonal blocks, transposed too, and temporaries
+  ly.W = off;      off += al((size_t)inv_elems(m) * 4);
+  ly.WT = off;     off += al((size_t)inv_elems(m) * 4);
+  ly.T = off;      off += al((size_t)inv_temp_elems(m) * 4);
+  // refinement vectors, row sums, the CTAs' maxima
+  ly.v = off;      off += al((size_t)m * 4);
+  ly.z = off;      off += al((size_t)m * 4);
+  ly.xs = off;     off += al((size_t)m * 4);
+  ly.rowsum = off; off += al((size_t)m * 8);
+  ly.red = off;    off += al((size_t)ceil_div(m, kRefineRows) * 4 * 8);
+  ly.state = off;  off += 256;   // RefineState, and at 128 the barrier's counter
   ly.tiles = ceil_div(m, (int64_t)DT);
   ly.dag = off;    off += al((size_t)(ly.tiles * ly.tiles + 1) * 4);   // tile flags, ticket
   ly.total = off;
@@ -2168,7 +1677,7 @@ extern "C" int spsvm_cholesky_mixed(const double* H, int64_t m, int64_t ldh, dou
   const int64_t T = ly.tiles, ntiles = T * (T + 1) / 2;
   SPSVM_CUDA_TRY(cudaMemsetAsync(dflags, 0, (size_t)(T * T + 1) * 4, s));
   to_f32_shift<<<(unsigned)m, MX_T, 0, s>>>(H, ldh, m, shift, L, ly.ldl,
-                                            reinterpret_cast<double*>(w + ly.rowmax));
+                                            reinterpret_cast<double*>(w + ly.rowsum));
   SPSVM_LAUNCH_CHECK();
   SPSVM_CUDA_TRY(cudaFuncSetAttribute(chol32_dag, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)DAG_SMEM));
@@ -2180,9 +1689,8 @@ extern "C" int spsvm_cholesky_mixed(const double* H, int64_t m, int64_t ldh, dou
   chol32_dag<<<(unsigned)grid, DAG_T, DAG_SMEM, s>>>(
       L, ly.ldl, m, T, dflags, dflags + T * T, info, wc);
   SPSVM_LAUNCH_CHECK();
-  diag_inverse<float><<<(unsigned)ly.B, DI_T, 0, s>>>(L, ly.ldl, m);
-  SPSVM_LAUNCH_CHECK();
-  return SPSVM_OK;
+  return launch_block_inverse(L, ly.ldl, m, reinterpret_cast<float*>(w + ly.W),
+                              reinterpret_cast<float*>(w + ly.WT), reinterpret_cast<float*>(w + ly.T), s);
 }
 
 namespace {
@@ -2203,7 +1711,7 @@ LowRankLayout lowrank_layout(int64_t m, int32_t k) {
   size_t off = 0;
   ly.V = off;      off += al((size_t)B * NB * ly.ldv * 4);
   ly.Ci = off;     off += al((size_t)k * ly.ldv * 4);
-  ly.s = off;      off += al((size_t)ly.slices * ly.ldv * 4);              // partial dots
+  ly.s = off;      off += al((size_t)ceil_div(m, kRefineRows) * ly.ldv * 4);   // partial dots
   ly.cpart = off;  off += al((size_t)ly.slices * ly.ldv * ly.ldv * 8);     // partial V^T V
   ly.flags = off;  off += al((size_t)(B * ly.G + 1) * 4);
   ly.total = off;
@@ -2214,14 +1722,11 @@ struct LowRankView {
   const float* V;
   const float* Ci;
   float* s;
-  int64_t ldv, slices;
-  int32_t k, G;
+  int64_t ldv;
+  int32_t k;
 };
 
 }  // namespace
-
-// Refinement steps queued before the first host check.
-constexpr int kRefineAhead = 3;
 
 static int solve_mixed_impl(const double* H, int64_t m, int64_t ldh, double shift,
                             const double* b, double* x, int32_t max_iter, double tol,
@@ -2239,99 +1744,57 @@ static int solve_mixed_impl(const double* H, int64_t m, int64_t ldh, double shif
   cudaStream_t s = as_stream(stream);
   ProfScope prof(PROF_SOLVE, s, 8.0 * (double)m * m);
   char* w = static_cast<char*>(work);
-  const float* L = reinterpret_cast<const float*>(w + ly.L);
-  float* zw = reinterpret_cast<float*>(w + ly.sw);
-  char* tagged_region = w + ly.sw + round_up(m * 4, (int64_t)256);
-  unsigned long long* zt = reinterpret_cast<unsigned long long*>(tagged_region);
-  unsigned long long* xt = zt + m;
-  unsigned* tickets = reinterpret_cast<unsigned*>(tagged_region + round_up(m * 16, (int64_t)256));
-  const size_t tagged_bytes = (size_t)round_up(m * 16, (int64_t)256) + (size_t)2 * kTicketSteps * 4;
-  float* z32 = reinterpret_cast<float*>(w + ly.z32);
-  double* r = reinterpret_cast<double*>(w + ly.r);
-  double* rowmax = reinterpret_cast<double*>(w + ly.rowmax);
-  double* xmax = reinterpret_cast<double*>(w + ly.xmax);
-  double* rmax = reinterpret_cast<double*>(w + ly.rmax);
-  double* bmax = reinterpret_cast<double*>(w + ly.bmax);
-  double* norms = reinterpret_cast<double*>(w + ly.norms);
-  const unsigned vb = (unsigned)ly.nvec_blocks, rb = (unsigned)ly.nrow_blocks;
-  const bool vec = (ldh % 2) == 0 && (reinterpret_cast<uintptr_t>(H) & 15) == 0 &&
-                   (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   RefineState* state = reinterpret_cast<RefineState*>(w + ly.state);
-  const int* stop = &state->stop;
-  WaitCtx wc;
-  SPSVM_TRY(wait_ctx(s, &wc));
-  SPSVM_CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)m * 8, s));
-  SPSVM_CUDA_TRY(cudaMemsetAsync(tagged_region, 0, tagged_bytes, s));
-  SPSVM_CUDA_TRY(cudaMemsetAsync(state, 0, sizeof(RefineState), s));
-  // block maxima of |b| (||b||_inf) and the first right-hand side z = (float) b
-  absmax_blocks<<<vb, MX_T, 0, s>>>(b, m, bmax, z32);
-  SPSVM_LAUNCH_CHECK();
-  // One refinement step: z = (L L^T)^{-1} r in FP32, x += z (with the
-  // backward solve), r = b - (H + shift I) x in FP64 and the next z =
-  // (float) r, then the norms and the stop word.  Every kernel of a step
-  // returns at once once the stop word is set.
-  auto step = [&](int it) -> int {
-    // tags 1, 2, ... (the tagged words start zeroed); tickets per step
-    const unsigned tag = (unsigned)(it + 1);
-    if (it > 0 && it % kTicketSteps == 0)
-      SPSVM_CUDA_TRY(cudaMemsetAsync(tickets, 0, (size_t)2 * kTicketSteps * 4, s));
-    unsigned* tk = tickets + 2 * (it % kTicketSteps);
-    trsv32_fwd<<<(unsigned)ly.B, SV_THREADS, 0, s>>>(L, ly.ldl, m, z32, zt, zw, tk, tag, wc, stop);
-    SPSVM_LAUNCH_CHECK();
-    if (lr) {   // z <- (I - V C^{-1} V^T) z
-      lr_dots<<<dim3((unsigned)lr->G, (unsigned)lr->slices), 256, 0, s>>>(lr->V, lr->ldv, m, zw,
-                                                                          lr->ldv, lr->s, stop);
-      SPSVM_LAUNCH_CHECK();
-      lr_update<<<(unsigned)min64(ceil_div(m, (int64_t)16), 2 * (int64_t)sm_count()), 256, 0, s>>>(
-          lr->V, lr->ldv, m, lr->Ci, lr->ldv, lr->s, lr->slices, lr->ldv, lr->k, zw, stop);
-      SPSVM_LAUNCH_CHECK();
+  RefineArgs a{};
+  a.L = reinterpret_cast<const float*>(w + ly.L);
+  a.ldl = ly.ldl;
+  a.m = m;
+  a.W = reinterpret_cast<const float*>(w + ly.W);
+  a.WT = reinterpret_cast<const float*>(w + ly.WT);
+  a.H = H;
+  a.ldh = ldh;
+  a.shift = shift;
+  a.b = b;
+  a.x = x;
+  a.v = reinterpret_cast<float*>(w + ly.v);
+  a.z = reinterpret_cast<float*>(w + ly.z);
+  a.xs = reinterpret_cast<float*>(w + ly.xs);
+  a.red = reinterpret_cast<double*>(w + ly.red);
+  a.rowsum = reinterpret_cast<const double*>(w + ly.rowsum);
+  a.finfo = factor_info;
+  a.state = state;
+  a.bar = reinterpret_cast<unsigned*>(w + ly.state + 128);
+  a.max_iter = max_iter;
+  a.tol = tol;
+  if (lr) {
+    a.V = lr->V;
+    a.Ci = lr->Ci;
+    a.sp = lr->s;
+    a.ldv = lr->ldv;
+    a.k = lr->k;
+  }
+  SPSVM_CUDA_TRY(cudaMemsetAsync(state, 0, 256, s));
+  SPSVM_TRY(launch_refine(a, s));
+  RefineState h{};
+  const ReadChunk c{&h, state, sizeof(h)};
+  SPSVM_TRY(read_back(s, &c, 1));
+  if (iters) *iters = h.iters;
+  if (backward_error) *backward_error = h.be;
+  switch (h.stop) {
+    case 1:
+      return SPSVM_OK;
+    case 2:
+      return set_error(SPSVM_ERR_NO_CONVERGE, "solve_mixed: refinement stagnates (backward error %.3g)", h.be);
+    case 3:
+      return set_error(SPSVM_ERR_NO_CONVERGE, "solve_mixed: not finite");
+    case 4: {
+      int32_t fi = 0;
+      const ReadChunk cf{&fi, factor_info, sizeof(fi)};
+      SPSVM_TRY(read_back(s, &cf, 1));
+      return set_error(SPSVM_ERR_NOT_PD, "solve_mixed: the FP32 factorisation broke down at pivot %d", fi - 1);
     }
-    trsv32_bwd<<<(unsigned)ly.B, SV_THREADS, 0, s>>>(L, ly.ldl, m, zw, xt, x, xmax, tk + 1, tag, wc,
-                                                     stop);
-    SPSVM_LAUNCH_CHECK();
-    if (vec)
-      residual_f64<true><<<rb, MX_T, 0, s>>>(H, ldh, m, shift, b, x, r, z32, rmax, stop);
-    else
-      residual_f64<false><<<rb, MX_T, 0, s>>>(H, ldh, m, shift, b, x, r, z32, rmax, stop);
-    SPSVM_LAUNCH_CHECK();
-    refine_decide<<<1, MX_T, 0, s>>>(xmax, ly.B, rmax, ly.nrow_blocks, rowmax, m, bmax,
-                                     ly.nvec_blocks, norms, it <= 1 ? factor_info : nullptr, it, tol,
-                                     state);
-    SPSVM_LAUNCH_CHECK();
-    return SPSVM_OK;
-  };
-  // an FP32 factor reaches FP64 backward error in about three steps: they
-  // are queued before the first host check, later ones one at a time
-  int it = 0;
-  for (; it < max_iter && it < kRefineAhead; ++it) SPSVM_TRY(step(it));
-  for (;;) {
-    RefineState h{};
-    const ReadChunk c{&h, state, sizeof(h)};
-    SPSVM_TRY(read_back(s, &c, 1));
-    if (iters) *iters = h.iters;
-    if (backward_error) *backward_error = h.be;
-    switch (h.stop) {
-      case 1:
-        return SPSVM_OK;
-      case 2:
-        return set_error(SPSVM_ERR_NO_CONVERGE, "solve_mixed: refinement stagnates (backward error %.3g)",
-                         h.be);
-      case 3:
-        return set_error(SPSVM_ERR_NO_CONVERGE, "solve_mixed: not finite");
-      case 4: {
-        int32_t fi = 0;
-        const ReadChunk cf{&fi, factor_info, sizeof(fi)};
-        SPSVM_TRY(read_back(s, &cf, 1));
-        return set_error(SPSVM_ERR_NOT_PD, "solve_mixed: the FP32 factorisation broke down at pivot %d",
-                         fi - 1);
-      }
-      default:
-        break;
-    }
-    if (it >= max_iter)
+    default:
       return set_error(SPSVM_ERR_NO_CONVERGE, "solve_mixed: %d iterations not enough", max_iter);
-    SPSVM_TRY(step(it));
-    ++it;
   }
 }
 
@@ -2409,7 +1872,7 @@ extern "C" int spsvm_solve_lowrank(const double* H, int64_t m, int64_t ldh, cons
   if (lr_bytes < ly.total) return set_error(SPSVM_ERR_OOM, "solve_lowrank: work too small");
   char* w = static_cast<char*>(lr_work);
   LowRankView v{reinterpret_cast<const float*>(w + ly.V), reinterpret_cast<const float*>(w + ly.Ci),
-                reinterpret_cast<float*>(w + ly.s), ly.ldv, ly.slices, k, (int32_t)ly.G};
+                reinterpret_cast<float*>(w + ly.s), ly.ldv, k};
   return solve_mixed_impl(H, m, ldh, 0.0, b, x, max_iter, tol, iters, backward_error, mixed_work,
                           mixed_bytes, &v, nullptr, stream);
 }

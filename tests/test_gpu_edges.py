@@ -245,3 +245,32 @@ def test_line_search_finds_the_root(sp, n, scale):
     slope = a1 + np.sum(np.where(mm - hi * v > 0, v * v, 0))
     noise = abs(a0) + abs(a1) * hi + np.sum(np.abs(v) * np.maximum(0, np.abs(mm) + hi * np.abs(v)))
     assert abs(t - hi) <= 8 * 2.0 ** -24 * noise / slope + 1e-6 * hi
+
+
+# diagonal blocks of 64 rows inverted directly, of 256 by columns, merged to
+# 1,024; more than one such block; 16 columns a tile and 8 rows a CTA
+@pytest.mark.parametrize("m", [2, 64, 66, 129, 255, 256, 257, 320, 513, 1023, 1024, 1025, 1100, 2049, 2500])
+@pytest.mark.parametrize("ldx,shift", [(0, 0.0), (1, 0.5)])
+def test_mixed_solve_over_block_inverses(sp, m, ldx, shift):
+    """Backward error 1e-13 as asked, from H with an even and an odd pitch, H
+    untouched, and the 64 x 64 blocks' inverses beside the factor."""
+    g = np.random.default_rng(m)
+    A = g.standard_normal((m, m + 8)) / np.sqrt(m)
+    Hn = A @ A.T + 0.2 * np.eye(m)
+    buf = torch.zeros((m, m + ldx), dtype=torch.float64, device=DEV)
+    buf[:, :m] = _t(Hn)
+    H, b = buf[:, :m], _t(g.standard_normal(m))
+    info, status, x, iters, be = sp.spsvm_solve_mixed(H, b, shift=shift)
+    assert info == 0 and status == 0 and be <= 1e-13
+    np.testing.assert_array_equal(H.cpu().numpy(), Hn)
+    Hs = Hn + shift * np.eye(m)
+    xn, bn = x.cpu().numpy(), b.cpu().numpy()
+    r = np.max(np.abs(bn - Hs @ xn))
+    assert r <= 2e-13 * (np.max(np.abs(Hs).sum(1)) * np.max(np.abs(xn)) + np.max(np.abs(bn)))
+    info, Lw = sp.spsvm_cholesky_mixed(H, shift=shift)
+    Lw = Lw.cpu().numpy().astype(np.float64)
+    for k in {0, (m - 1) // 64}:
+        D = Lw[64 * k:64 * k + 64, 64 * k:min(m, 64 * k + 64)]
+        low, inv = np.tril(D), np.triu(D, 1).T + np.diag(1 / np.diag(D))
+        c = np.abs(np.linalg.inv(low)) @ np.abs(low)
+        assert np.all(np.abs(inv @ low - np.eye(len(D))) <= 64 * 2.0 ** -24 * c @ c + 1e-12)
