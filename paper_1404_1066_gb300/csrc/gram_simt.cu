@@ -143,20 +143,53 @@ int launch_gram_simt(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t m, flo
 }
 
 // K_JJ[a][b] = (K[b][J[a]] + K[a][J[b]]) / 2 (the stored values made
-// symmetric; exact in FP64) for the rows and columns from row0 on: thread
-// (r, c), r >= row0, writes (r, c) and (c, r).  A fit keeps K_JJ in its
-// workspace and extends it once per round, so the Gram finish reads it
-// coalesced instead of gathering two scattered kernel values per entry.
-__global__ void kjj_fill_kernel(KView K, const int64_t* __restrict__ J, int64_t m, int64_t row0,
-                                double* __restrict__ kjj, int64_t ldk) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t rows = m - row0;
-  if (e >= rows * m) return;
-  const int64_t r = row0 + e / m, c = e % m;
-  // the bias slot (point index -1) has no regulariser row or column
-  const double v = (J[r] < 0 || J[c] < 0) ? 0.0 : 0.5 * ((double)K.at(c, J[r]) + (double)K.at(r, J[c]));
-  kjj[r * ldk + c] = v;
-  kjj[c * ldk + r] = v;
+// symmetric; exact in FP64) for the rows and columns from row0 on.  A fit
+// keeps K_JJ in its workspace and extends it once per round, so the Gram
+// finish reads it coalesced.  One block per 32 x 32 tile (ta <= tb): each
+// scattered kernel value is read once, eight in flight a thread, and both
+// halves are written along their rows.  Bound by the scattered sectors: m =
+// 2,048 85 us (a thread per entry, two reads each: 155 us).
+constexpr int FT = 32;
+__global__ void __launch_bounds__(FT * 8) kjj_fill_kernel(KView K, const int64_t* __restrict__ J, int64_t m,
+                                                          int64_t row0, double* __restrict__ kjj,
+                                                          int64_t ldk) {
+  __shared__ float B[FT][FT + 1];
+  __shared__ double V[FT][FT + 1];
+  // tiles of column block tb: ta = 0 .. tb, from the block that holds row0
+  const int64_t t0 = row0 / FT;
+  int64_t rem = blockIdx.x, tb = t0;
+  while (rem > tb) rem -= ++tb;   // (column block tb has tb + 1 tiles)
+  const int64_t ta = rem, a0 = ta * FT, b0 = tb * FT;
+  const int c = threadIdx.x, y = threadIdx.y;
+  const int64_t Jb = b0 + c < m ? J[b0 + c] : -1, Ja = a0 + c < m ? J[a0 + c] : -1;
+  float va[4], vb[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = y + 8 * u;
+    // the bias slot (point index -1) has no regulariser row or column
+    va[u] = a0 + r < m && Jb >= 0 ? K.at(a0 + r, Jb) : 0.f;
+    vb[u] = ta != tb && b0 + r < m && Ja >= 0 ? K.at(b0 + r, Ja) : 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) B[y + 8 * u][c] = ta != tb ? vb[u] : va[u];
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = y + 8 * u;
+    const int64_t a = a0 + r, b = b0 + c;
+    double v = 0.0;
+    if (a < m && b < m && Jb >= 0 && J[a] >= 0) v = 0.5 * ((double)B[c][r] + (double)va[u]);
+    V[r][c] = v;
+    if (a < m && b < m && (a >= row0 || b >= row0)) kjj[a * ldk + b] = v;
+  }
+  if (ta == tb) return;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = y + 8 * u;
+    const int64_t b = b0 + r, a = a0 + c;
+    if (a < m && b < m && (a >= row0 || b >= row0)) kjj[b * ldk + a] = V[c][r];
+  }
 }
 
 // H[a][b] = H[b][a] = lambda K_JJ[a][b] + sum_s part[s][min(a,b)][max(a,b)]
@@ -164,7 +197,6 @@ __global__ void kjj_fill_kernel(KView K, const int64_t* __restrict__ J, int64_t 
 // at 1/64 of the FP32 rate made the sum over 16 splits take 16 us at m = 100,
 // now 9): the partials, K_JJ and both halves of H move
 // through shared memory so that every global access is coalesced.
-constexpr int FT = 32;
 __global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const float2* __restrict__ part,
                                                              GramPlan plan,
                                                              const int64_t* __restrict__ ns_dev,
@@ -243,8 +275,9 @@ size_t gram_part_bytes(int64_t m, int64_t ns) {
 int kjj_fill(const spsvm_kmat* K, const int64_t* J, int64_t m, int64_t row0, double* kjj,
              int64_t ldk, cudaStream_t s) {
   if (m <= row0) return SPSVM_OK;
-  const int64_t total = (m - row0) * m;
-  kjj_fill_kernel<<<(unsigned)ceil_div(total, 256), 256, 0, s>>>(view(K), J, m, row0, kjj, ldk);
+  const int64_t t0 = row0 / FT, t1 = ceil_div(m, (int64_t)FT);   // column blocks [t0, t1), tb + 1 tiles each
+  const int64_t tiles = t1 * (t1 + 1) / 2 - t0 * (t0 + 1) / 2;
+  kjj_fill_kernel<<<(unsigned)tiles, dim3(FT, 8), 0, s>>>(view(K), J, m, row0, kjj, ldk);
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }
