@@ -79,7 +79,8 @@ __global__ void __launch_bounds__(T::NT, 3) kernel_block_simt(
 }
 
 // Per tile of 128 points: partial sums over i in S of (o_i - y_i) K_ic and
-// K_ic^2 for the tile's candidates, written to part[tile][c] (FP64).  A
+// K_ic^2 for the tile's candidates, written to part[tile][c] as two
+// compensated pairs.  A
 // thread sums 4 points at a time in FP32; everything wider is summed as
 // compensated pairs (an FP64 warp sum per candidate would outweigh the tile's
 // product at small d).
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(T::NT, 3) score_partials_simt(
     const float* __restrict__ X, int64_t n, int64_t d, int64_t ldx,
     const float* __restrict__ norms, const float* __restrict__ y,
     const float* __restrict__ o, const int64_t* __restrict__ idx, int32_t kappa,
-    float gamma, double2* __restrict__ part) {
+    float gamma, float4* __restrict__ part) {
   __shared__ typename T::Smem sm;
   const int64_t i0 = (int64_t)blockIdx.x * T::TN, c0 = (int64_t)blockIdx.y * T::TM;
   simt::FloatRows<VEC> a[T::LA], b[T::LB];
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(T::NT, 3) score_partials_simt(
   }
   const int64_t c = c0 + T::row(mine >> 1);
   if (c < kappa && (NV == 16 || (tx & 1) == 0))
-    reinterpret_cast<double*>(part + (int64_t)blockIdx.x * kappa + c)[mine & 1] = pair_value(hi[0], lo[0]);
+    reinterpret_cast<float2*>(part + (int64_t)blockIdx.x * kappa + c)[mine & 1] = make_float2(hi[0], lo[0]);
 }
 
 // The 32-row tile where it wastes fewer rows, or where 64-row tiles would leave
@@ -172,28 +173,52 @@ bool use_narrow(int64_t n, int64_t m) {
   return m <= 32 || 4 * ceil_div(n, PT) * ceil_div(m, (int64_t)64) < 5 * (int64_t)sm_count();
 }
 
-// g_k = lambda o[c] + sum_tiles G, h_k = lambda + sum_tiles H, delta = g^2/(2h).
-__global__ void score_finish(const double2* __restrict__ part, int64_t tiles, int32_t kappa,
-                             const float* __restrict__ o, const int64_t* __restrict__ idx,
-                             double lambda, double* g, double* h, double* delta) {
-  const int k = blockIdx.x;
-  __shared__ double sh[32];
-  double gs = 0.0, hs = 0.0;
-  for (int64_t t = threadIdx.x; t < tiles; t += blockDim.x) {
-    const double2 p = part[t * kappa + k];
-    gs += p.x;
-    hs += p.y;
+// g_k = lambda o[c] + sum_tiles G, h_k = lambda + sum_tiles H, delta = g^2/(2h),
+// two candidates a block (a whole sector a partial), 256 threads over the
+// partials of each, sums as compensated pairs.  256 candidates: 76 partials
+// (split form, n = 500,000) 5 us; 3,907, one block a candidate in FP64, 12.
+constexpr int SF_C = 2, SF_T = 512;
+__global__ void __launch_bounds__(SF_T) score_finish(const float4* __restrict__ part, int64_t tiles,
+                                                     int32_t kappa, const float* __restrict__ o,
+                                                     const int64_t* __restrict__ idx, double lambda,
+                                                     double* g, double* h, double* delta) {
+  __shared__ float4 sh[SF_T / 32][SF_C];
+  const int c = threadIdx.x % SF_C, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int k = blockIdx.x * SF_C + c;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (k < kappa) {
+    constexpr int STEP = SF_T / SF_C, U = 16;
+    for (int64_t t = threadIdx.x / SF_C; t < tiles; t += U * STEP) {
+      float4 p[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        p[u] = t + u * STEP < tiles ? part[(t + u * STEP) * kappa + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        pair_add(s.x, s.y, make_float2(p[u].x, p[u].y));
+        pair_add(s.z, s.w, make_float2(p[u].z, p[u].w));
+      }
+    }
   }
-  gs = block_sum(gs, sh);
+#pragma unroll
+  for (int x = SF_C; x < 32; x <<= 1) {
+    const float a = __shfl_xor_sync(0xffffffffu, s.x, x), b = __shfl_xor_sync(0xffffffffu, s.y, x);
+    const float d = __shfl_xor_sync(0xffffffffu, s.z, x), e = __shfl_xor_sync(0xffffffffu, s.w, x);
+    pair_add(s.x, s.y, make_float2(a, b));
+    pair_add(s.z, s.w, make_float2(d, e));
+  }
+  if (lane < SF_C) sh[w][c] = s;
   __syncthreads();
-  hs = block_sum(hs, sh);
-  if (threadIdx.x == 0) {
-    const double gg = lambda * (double)o[idx[k]] + gs;
-    const double hh = lambda + hs;
-    g[k] = gg;
-    h[k] = hh;
-    delta[k] = gg * gg / (2.0 * hh);
+  if (threadIdx.x >= SF_C || k >= kappa) return;
+  for (int q = 1; q < SF_T / 32; ++q) {
+    pair_add(s.x, s.y, make_float2(sh[q][c].x, sh[q][c].y));
+    pair_add(s.z, s.w, make_float2(sh[q][c].z, sh[q][c].w));
   }
+  const double gg = lambda * (double)o[idx[k]] + pair_value(s.x, s.y);
+  const double hh = lambda + pair_value(s.z, s.w);
+  g[k] = gg;
+  h[k] = hh;
+  delta[k] = gg * gg / (2.0 * hh);
 }
 
 }  // namespace
@@ -216,7 +241,7 @@ int launch_kernel_block_simt(const spsvm_points* p, const int64_t* idx, int32_t 
 }
 
 static void launch_score_simt(const spsvm_points* p, const float* y, const float* o,
-                              const int64_t* idx, int32_t kappa, float gamma, double2* part,
+                              const int64_t* idx, int32_t kappa, float gamma, float4* part,
                               cudaStream_t s) {
   auto launch = [&](auto tile, auto vec) {
     using T = decltype(tile);
@@ -263,16 +288,15 @@ extern "C" int spsvm_kernel_block(const spsvm_points* p, const int64_t* idx, int
 
 namespace spsvm {
 int launch_score_tc(const spsvm_points* p, const float* y, const float* o, const int64_t* idx,
-                    int32_t kappa, float gamma, double2* part, int64_t tiles, void* zbuf,
+                    int32_t kappa, float gamma, float4* part, int64_t* parts, void* zbuf,
                     size_t zbytes, cudaStream_t s);
-int64_t score_tc_tiles(int64_t n);
+int64_t score_tc_parts(int64_t n, int32_t kappa);
 namespace {
-// per-tile partial sums (tiles of 128 points in both forms), then room for
-// the gathered candidate rows of the tensor-core form
+// partial sums per candidate (of each tile of 128 points in FP32, of each CTA
+// or pair in the tensor-core form), then room for the gathered candidate rows
 size_t score_part_bytes(int64_t n, int32_t kappa) {
-  // the larger of the two forms' tile counts (both tile 128 points today)
-  const int64_t tiles = std::max<int64_t>(ceil_div(n, PT), score_tc_tiles(n));
-  return (size_t)round_up(tiles * (int64_t)kappa * (int64_t)sizeof(double2), 256);
+  const int64_t tiles = std::max<int64_t>(ceil_div(n, PT), score_tc_parts(n, kappa));
+  return (size_t)round_up(tiles * (int64_t)kappa * (int64_t)sizeof(float4), 256);
 }
 }  // namespace
 }  // namespace spsvm
@@ -297,22 +321,21 @@ extern "C" int spsvm_score_candidates(const spsvm_points* p, const float* y, con
     return set_error(SPSVM_ERR_OOM, "score_candidates: scratch %zu < %zu", scratch_bytes, need);
   cudaStream_t s = as_stream(stream);
   ProfScope prof(PROF_SCORE, s, (precision == SPSVM_BF16SPLIT ? 12.0 : 2.0) * (double)p->n * kappa * (double)p->d);
-  double2* part = static_cast<double2*>(scratch);
-  int64_t tiles = ceil_div(p->n, PT);
+  float4* part = static_cast<float4*>(scratch);
+  int64_t parts = ceil_div(p->n, PT);
   if (precision == SPSVM_BF16SPLIT) {
     if (!p->hi || !p->mid || !p->lo)
       return set_error(SPSVM_ERR_ARG, "score_candidates: BF16SPLIT needs split planes");
-    tiles = score_tc_tiles(p->n);
     const size_t pb = score_part_bytes(p->n, kappa);
-    SPSVM_TRY(launch_score_tc(p, y, o, idx, kappa, gamma, part, tiles,
-                              static_cast<char*>(scratch) + pb, scratch_bytes - pb, s));
+    SPSVM_TRY(launch_score_tc(p, y, o, idx, kappa, gamma, part, &parts, static_cast<char*>(scratch) + pb,
+                              scratch_bytes - pb, s));
   } else if (precision == SPSVM_FP32) {
     launch_score_simt(p, y, o, idx, kappa, gamma, part, s);
     SPSVM_LAUNCH_CHECK();
   } else {
     return set_error(SPSVM_ERR_ARG, "score_candidates: bad precision");
   }
-  score_finish<<<kappa, 256, 0, s>>>(part, tiles, kappa, o, idx, lambda, g, h, delta);
+  score_finish<<<(unsigned)ceil_div(kappa, SF_C), SF_T, 0, s>>>(part, parts, kappa, o, idx, lambda, g, h, delta);
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }

@@ -18,9 +18,11 @@
 #include <cudaTypedefs.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "gram.h"
 #include "internal.h"
+#include "simt_tile.h"
 #include "tc_ptx.h"
 
 namespace spsvm {
@@ -28,6 +30,11 @@ namespace spsvm {
 namespace {
 
 using namespace tc;
+using simt::dup2;
+using simt::fma2;
+using simt::mul2;
+using simt::pack2;
+using simt::unpack2;
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   const uint32_t a = smem_u32(p);
@@ -35,64 +42,72 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 }
 
 // ---------------------------------------------------------------------------
-// Kernel block / scores, persistent and warp-specialised.  D[c][i] = z_c . x_i
-// over tiles of 128 basis (or candidate) rows c (MMA M; the rows gathered
-// beforehand into contiguous BF16 planes Z) by 128 points i (MMA N), both
-// operands streamed by TMA through a 3-stage shared-memory ring (32-element
-// K slices, 64-byte swizzle) holding the three planes of each (x = hi + mid
-// + lo, exact for FP32) and multiplied as the six products hi hi, hi mid,
-// mid hi, mid mid, hi lo, lo hi (the three dropped ones are below 2^-24 of
-// |x z|), hi hi into one TMEM accumulator and the rest into a second (the
-// FP32 accumulation's rounding grows with the MMAs a sum takes, and only the
-// few large-term ones then count).  Warp 0 issues the TMA loads, warp 1 the
-// MMAs into one of two tile buffers, warps 2-9 drain the other (TMEM lane c =
-// row c; warps w and w + 4 share a lane quarter and split the 128 columns),
-// so the epilogue of one tile overlaps the MMAs of the next.  Tiles are ordered point-tile major so the CTAs in flight share their
-// X tiles through L2.
+// Kernel block / scores / decision values, persistent and warp-specialised:
+// products x.z over tiles of rows (MMA M) by columns (MMA N), both operands
+// streamed by TMA, each FP32 value as three planes (x = hi + mid + lo, exact)
+// and multiplied as the six products hi hi, hi mid, mid hi, mid mid, hi lo, lo
+// hi (the three dropped ones are below 2^-24 of |x z|), hi hi into one TMEM
+// accumulator and the rest into a second (the FP32 accumulation's rounding
+// grows with the MMAs a sum takes, and only the few large-term ones then
+// count).  Epilogue modes:
+//   STORE   rows the points, columns the basis: the FP32 kernel values (a warp
+//           stores 32 consecutive points of a basis row);
+//   SCORE   rows the candidates, columns the points: the score sums, a
+//           thread's own over its columns of all of the CTA's tiles (kernel
+//           values not stored);
+//   DECIDE  rows the queries, columns the basis: sums of beta K over 32.
+// Basis and candidate rows are gathered into contiguous planes beforehand.
+//
+// Warp 0 issues the TMA loads, warp 1 the MMAs into one of two tile buffers,
+// the other warps drain the other (TMEM lane = row; four lane quarters by
+// groups of 32 columns).  A slot of the shared-memory ring holds one plane of
+// both operands over 64 columns of K, so a chunk starts as soon as its hi
+// planes are there.  With more than 128 rows two CTAs work as a pair (PAIR,
+// cta_group::2) on 256 rows, each staging 128 rows and half of the columns,
+// the even one issuing the MMAs for both: a 128 x 128 MMA of one CTA reads its
+// operands from shared memory at the full 128 bytes a cycle, with loads of 64
+// bytes a cycle on top, the pair reads 96 and loads 47.  Up to 64 columns take
+// a tile of 64 (N), at 128 half of the products would be padding.
+//
+// MMAs on the same plane of the rows stand together, so the rows are read from
+// shared memory three times a step instead of six.  Arrivals of a pair are
+// relaxed (a release waits for the epilogue's global stores).
+// 32,768 queries by 4,096 basis rows, d = 128: 117 us, 1.77 PFLOP/s in the six
+// products (154 us in 128 x 128 tiles of single CTAs with the queries as
+// columns, where each sum over a warp's rows took 31 exchanges).  Scores of 256
+// candidates, n = 500,000: 130 us (157).  Kernel block of 64 rows, n = 500,000:
+// 76 us, 512 MB at 6.7 TB/s (90 us in tiles of 128 basis rows).
 // ---------------------------------------------------------------------------
-constexpr int PK_M = 128;
-constexpr int PK_N = 128;
-constexpr int PK_KC = 32;                                  // K elements per stage (64-byte rows)
-constexpr int PK_WP = PK_N / 2;                            // points per epilogue warp
-constexpr int PK_ACC_COLS = 2 * PK_N;                      // TMEM per tile: large + small terms
-constexpr int PK_STAGES = 3;
-constexpr int PK_PLANE_A = PK_M * PK_KC * 2;               // 8 KB: 128 rows x 32 BF16
-constexpr int PK_PLANE_B = PK_N * PK_KC * 2;               // 8 KB
-constexpr int PK_STAGE = 3 * PK_PLANE_A + 3 * PK_PLANE_B;  // 48 KB
-constexpr int PK_EPI_WARPS = 8;
-constexpr int PK_THREADS = 32 * (2 + PK_EPI_WARPS);
-constexpr int PK_OUT_BOX = 32 * 128;                       // 32 rows x 32 FP32
-constexpr int PK_OUT_OFF = PK_STAGES * PK_STAGE;           // per epilogue warp: two boxes
-constexpr int PK_BAR_OFF = PK_OUT_OFF + PK_EPI_WARPS * 2 * PK_OUT_BOX;
-constexpr int PK_RED_OFF = PK_BAR_OFF + 256;
-constexpr int PK_STAGE_OFF = PK_RED_OFF + 4 * 32 * 8;      // per epilogue warp: 3 x 64 floats
-constexpr int PK_SMEM = PK_STAGE_OFF + PK_EPI_WARPS * 3 * PK_WP * 4 + 1024;   // + alignment slack
-static_assert(PK_SMEM <= 227 * 1024, "kernel block shared memory");
-static_assert(2 * PK_ACC_COLS <= 512, "two tiles of two accumulators fit TMEM");
+constexpr int64_t kScoreUnits = 160;   // CTAs or pairs of a SCORE launch at most
 
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, const void* src) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-          reinterpret_cast<uint64_t>(map)),
-      "r"(x), "r"(y), "r"(smem_u32(src))
-      : "memory");
-}
-__device__ __forceinline__ void bulk_commit() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// Waits until the shared-memory sources of every committed bulk store have been read.
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
+enum KbMode { KB_STORE_F32 = 0, KB_SCORE = 2, KB_DECIDE = 3 };
 
-// Tile order: groups of PK_GROUP consecutive point tiles, each group swept
-// over all basis blocks with the point tile varying fastest.  The CTAs in
-// flight then share a few X tiles through L2 while each basis row receives
-// PK_GROUP x 256 contiguous bytes, so the kernel-matrix writes reach DRAM in
-// long runs.
+constexpr int PK_M = 128;                                  // rows per CTA
+constexpr int PK_KC = 64;                                  // K elements per slot (128-byte rows)
+constexpr int PK_WP = 32;                                  // columns per epilogue warp
+template <bool PAIR, int N>
+struct Kb {
+  static constexpr int CTAS = PAIR ? 2 : 1;
+  static constexpr int M = CTAS * PK_M;                    // rows of a tile
+  static constexpr int ROWS_B = N / CTAS;                  // columns staged per CTA
+  static constexpr int GROUPS = N / PK_WP;
+  static constexpr int EPI_WARPS = 4 * GROUPS;
+  static constexpr int THREADS = 32 * (2 + EPI_WARPS);
+  static constexpr int PLANE_A = PK_M * PK_KC * 2;
+  static constexpr int SLOT = PLANE_A + ROWS_B * PK_KC * 2;
+  static constexpr int SLOTS = 192 * 1024 / SLOT;
+  static constexpr int RED_OFF = SLOTS * SLOT;             // SCORE: the groups' sums
+  static constexpr int BAR_OFF = RED_OFF + (GROUPS - 1) * 128 * 16;
+  static constexpr int STAGE_OFF = BAR_OFF + 512;          // per epilogue warp: 3 x 32 floats
+  static constexpr int SMEM = STAGE_OFF + EPI_WARPS * 3 * PK_WP * 4 + 1024;   // + alignment slack
+  static_assert(SMEM <= 227 * 1024, "kernel block shared memory");
+  static_assert(8 * (2 * SLOTS + 12) + 12 <= 512, "barriers");
+  static_assert(SLOTS >= 6, "two chunks in flight");
+};
+
+// Tile order: groups of PK_GROUP consecutive column tiles, each group swept
+// over all row blocks with the column tile varying fastest, so the CTAs in
+// flight share their tiles of both operands through L2.
 constexpr int64_t PK_GROUP = 32;
 __device__ __forceinline__ void tile_coords(int64_t t, int64_t nCB, int64_t nPT, int& cb,
                                             int64_t& pt) {
@@ -104,302 +119,392 @@ __device__ __forceinline__ void tile_coords(int64_t t, int64_t nCB, int64_t nPT,
   pt = g0 + r % gw;
 }
 
-// Epilogue modes: store the FP32 kernel values, reduce the candidate-score
-// sums without storing them, or reduce the decision values
-// f(x_i) = sum_c beta_c k(z_c, x_i) (Z the basis rows, X the queries) over
-// each warp's 32 basis rows, also without storing the kernel values.
-enum KbMode { KB_STORE_F32 = 0, KB_SCORE = 2, KB_DECIDE = 3 };
-
-
-template <int MODE>
-__global__ void __launch_bounds__(PK_THREADS, 1) kblock_tc_kernel(
-    const __grid_constant__ CUtensorMap map_zhi, const __grid_constant__ CUtensorMap map_zmid,
-    const __grid_constant__ CUtensorMap map_zlo, const __grid_constant__ CUtensorMap map_xhi,
-    const __grid_constant__ CUtensorMap map_xmid, const __grid_constant__ CUtensorMap map_xlo,
-    const __grid_constant__ CUtensorMap map_out, int64_t ldh, int64_t n, int32_t m,
-    const float* __restrict__ norms, const int64_t* __restrict__ idx, float gamma, int64_t row0,
-    const float* __restrict__ y, const float* __restrict__ o, double2* __restrict__ part,
-    int32_t kappa, const float* __restrict__ znorm, const double* __restrict__ beta,
+template <int MODE, bool PAIR, int N>
+__global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
+    const __grid_constant__ CUtensorMap map_ahi, const __grid_constant__ CUtensorMap map_amid,
+    const __grid_constant__ CUtensorMap map_alo, const __grid_constant__ CUtensorMap map_bhi,
+    const __grid_constant__ CUtensorMap map_bmid, const __grid_constant__ CUtensorMap map_blo,
+    int64_t ldh, int64_t ncols, int64_t nrows,
+    const float* __restrict__ colnorm, const float* __restrict__ rownorm,
+    const int64_t* __restrict__ idx, float gamma, float* __restrict__ out, int64_t ld,
+    const float* __restrict__ y,
+    const float* __restrict__ o, float4* __restrict__ part, const double* __restrict__ beta,
     float* __restrict__ dpart, int64_t ldp, WaitCtx wc) {
   constexpr bool SCORE = MODE == KB_SCORE;
   constexpr bool STORE = MODE == KB_STORE_F32;
   constexpr bool DECIDE = MODE == KB_DECIDE;
+  using TL = Kb<PAIR, N>;
+  constexpr int SLOTS = TL::SLOTS, KC = PK_KC, GROUPS = TL::GROUPS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + PK_BAR_OFF);
-  uint64_t* empty = full + PK_STAGES;
-  uint64_t* tfull = empty + PK_STAGES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + TL::BAR_OFF);
+  uint64_t* empty = full + SLOTS;
+  uint64_t* tfull = empty + SLOTS;
   uint64_t* tempty = tfull + 2;
-  uint64_t* redf = tempty + 2;   // per lane quarter: half-tile sums written
-  uint64_t* rede = redf + 4;     // per lane quarter: half-tile sums consumed
+  uint64_t* redf = tempty + 2;   // per lane quarter: the groups' sums written
+  uint64_t* rede = redf + 4;     // per lane quarter: the groups' sums consumed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rede + 4);
-  float2* red = reinterpret_cast<float2*>(smem + PK_RED_OFF);
+  uint32_t* bad = tmem_slot + 1;   // [2], PAIR: a wait had given up before, as each CTA saw it
+  float4* red = reinterpret_cast<float4*>(smem + TL::RED_OFF);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (__syncthreads_or(tid == 0 && *(volatile int*)wc.st != 0)) return;
-  const int64_t nCB = ceil_div((int64_t)m, (int64_t)PK_M);
-  const int64_t nPT = ceil_div(n, (int64_t)PK_N);
+  const uint32_t rank = PAIR ? cluster_rank() : 0u;
+  const int64_t unit = PAIR ? blockIdx.x >> 1 : blockIdx.x, units = PAIR ? gridDim.x >> 1 : gridDim.x;
+  if (!PAIR && __syncthreads_or(tid == 0 && *(volatile int*)wc.st != 0)) return;
+  const int64_t nCB = ceil_div(nrows, (int64_t)TL::M);
+  const int64_t nPT = ceil_div(ncols, (int64_t)N);
   const int64_t T = nCB * nPT;
-  const int nK = (int)(ldh / PK_KC);
-  constexpr uint32_t IDESC = idesc_bf16_f32(PK_M, PK_N);
+  const int nK = (int)(ldh / KC);
+  constexpr uint32_t IDESC = idesc_bf16_f32(TL::M, N);
 
   if (tid == 0) {
-    for (int s = 0; s < PK_STAGES; ++s) {
+    for (int s = 0; s < SLOTS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull[a], 1);
-      mbar_init(&tempty[a], 32 * PK_EPI_WARPS);
+      mbar_init(&tempty[a], TL::CTAS * TL::EPI_WARPS);   // one arrival per epilogue warp
     }
     for (int qd = 0; qd < 4; ++qd) {
-      mbar_init(&redf[qd], 32);
+      mbar_init(&redf[qd], 32 * (GROUPS - 1));
       mbar_init(&rede[qd], 32);
     }
     fence_barrier_init();
-    prefetch_tmap(&map_zhi);
-    prefetch_tmap(&map_zmid);
-    prefetch_tmap(&map_zlo);
-    prefetch_tmap(&map_xhi);
-    prefetch_tmap(&map_xmid);
-    prefetch_tmap(&map_xlo);
-    if (STORE) prefetch_tmap(&map_out);
+    prefetch_tmap(&map_ahi);
+    prefetch_tmap(&map_amid);
+    prefetch_tmap(&map_alo);
+    prefetch_tmap(&map_bhi);
+    prefetch_tmap(&map_bmid);
+    prefetch_tmap(&map_blo);
   }
-  if (warp == 0) tmem_alloc(tmem_slot, 2 * PK_ACC_COLS);
-  fence_before_sync();
-  __syncthreads();
+  bool live = true;
+  if constexpr (PAIR) {
+    __syncwarp();
+    cluster_sync();   // both CTAs run, and their barriers are initialised
+    if (tid == 0) {
+      const uint32_t st = *(volatile int*)wc.st != 0 ? 1u : 0u;
+      st_cluster(map_rank(&bad[rank], 0), st);
+      st_cluster(map_rank(&bad[rank], 1), st);
+    }
+    __syncwarp();
+    if (warp == 0) tmem_alloc_pair(tmem_slot, 4 * N);
+    fence_before_sync();
+    cluster_sync();
+    live = bad[0] == 0 && bad[1] == 0;   // the same in both CTAs
+  } else {
+    if (warp == 0) tmem_alloc(tmem_slot, 4 * N);
+    fence_before_sync();
+    __syncthreads();
+  }
   fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  // for a barrier that threads or MMAs of the other CTA may complete
+  auto wait = [&](uint64_t* bar, uint32_t parity, int code) {
+    return PAIR ? mbar_wait_cluster(bar, parity, wc.st, code, wc.lim) : mbar_wait(bar, parity, wc.st, code, wc.lim);
+  };
 
-  if (warp == 0) {
+  if (!live) {
+  } else if (warp == 0) {
     if (lane == 0) {
-      // ---- TMA producer
+      // ---- TMA producer (of a pair: both CTAs' loads complete on the even one's barrier)
       int64_t q = 0;
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < T && ok; t += gridDim.x) {
+      const CUtensorMap* ma[3] = {&map_ahi, &map_amid, &map_alo};
+      const CUtensorMap* mb[3] = {&map_bhi, &map_bmid, &map_blo};
+      for (int64_t t = unit; t < T && ok; t += units) {
         int cb;
         int64_t pt;
         tile_coords(t, nCB, nPT, cb, pt);
-        for (int kc = 0; kc < nK; ++kc, ++q) {
-          const int s = (int)(q % PK_STAGES);
-          const uint32_t ph = (uint32_t)((q / PK_STAGES) & 1);
-          if (!mbar_wait(&empty[s], ph ^ 1u, wc.st, 21, wc.lim)) {
-            ok = false;
-            break;
+        const int ra = cb * TL::M + (int)rank * PK_M, rb = (int)(pt * N) + (int)rank * TL::ROWS_B;
+        for (int kc = 0; kc < nK && ok; ++kc) {
+#pragma unroll
+          for (int p = 0; p < 3; ++p, ++q) {
+            const int s = (int)(q % SLOTS);
+            if (!wait(&empty[s], (uint32_t)((q / SLOTS) & 1) ^ 1u, 21)) {
+              ok = false;
+              break;
+            }
+            uint8_t* st = smem + s * TL::SLOT;
+            if (rank == 0) mbar_expect_tx(&full[s], TL::CTAS * TL::SLOT);
+            if constexpr (PAIR) {
+              const uint32_t bar = map_rank(&full[s], 0);
+              tma_load_2d_pair(st, ma[p], kc * KC, ra, bar);
+              tma_load_2d_pair(st + TL::PLANE_A, mb[p], kc * KC, rb, bar);
+            } else {
+              tma_load_2d(st, ma[p], kc * KC, ra, &full[s]);
+              tma_load_2d(st + TL::PLANE_A, mb[p], kc * KC, rb, &full[s]);
+            }
           }
-          uint8_t* st = smem + s * PK_STAGE;
-          uint8_t* sb = st + 3 * PK_PLANE_A;
-          mbar_expect_tx(&full[s], PK_STAGE);
-          tma_load_2d(st, &map_zhi, kc * PK_KC, cb * PK_M, &full[s]);
-          tma_load_2d(st + PK_PLANE_A, &map_zmid, kc * PK_KC, cb * PK_M, &full[s]);
-          tma_load_2d(st + 2 * PK_PLANE_A, &map_zlo, kc * PK_KC, cb * PK_M, &full[s]);
-          tma_load_2d(sb, &map_xhi, kc * PK_KC, (int)(pt * PK_N), &full[s]);
-          tma_load_2d(sb + PK_PLANE_B, &map_xmid, kc * PK_KC, (int)(pt * PK_N), &full[s]);
-          tma_load_2d(sb + 2 * PK_PLANE_B, &map_xlo, kc * PK_KC, (int)(pt * PK_N), &full[s]);
         }
       }
       // no copy may be in flight when the block exits
-      for (int64_t r = (q > PK_STAGES ? q - PK_STAGES : 0); r < q; ++r)
-        mbar_wait(&full[r % PK_STAGES], (uint32_t)((r / PK_STAGES) & 1), wc.st, 22, wc.lim);
+      if (rank == 0)
+        for (int64_t r = (q > SLOTS ? q - SLOTS : 0); r < q; ++r)
+          mbar_wait(&full[r % SLOTS], (uint32_t)((r / SLOTS) & 1), wc.st, 22, wc.lim);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- MMA issuer
+    if (rank == 0) {
+      // ---- MMA issuer: the whole warp runs the loop, one lane issues; a wait
+      // counts as run out for all lanes when it has for one
+      auto mma = [&](auto use, uint32_t d, uint32_t a, uint32_t b, uint32_t accumulate) {
+        constexpr int A = decltype(use)::value;
+        if constexpr (PAIR) mma_bf16_pair<A>(d, desc_sw128(a), desc_sw128(b), IDESC, accumulate);
+        else mma_bf16<A>(d, desc_sw128(a), desc_sw128(b), IDESC, accumulate);
+      };
+      const std::integral_constant<int, A_DISCARD> once;
+      const std::integral_constant<int, A_FILL> fill;
+      const std::integral_constant<int, A_USE> use;
+      const std::integral_constant<int, A_LASTUSE> last;
+      auto commit = [&](uint64_t* bar) {
+        if constexpr (PAIR) mma_commit_pair(bar);
+        else mma_commit(bar);
+      };
       int64_t q = 0, j = 0;
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < T && ok; t += gridDim.x, ++j) {
+      for (int64_t t = unit; t < T && ok; t += units, ++j) {
         const int acc = (int)(j & 1);
-        if (!mbar_wait(&tempty[acc], (uint32_t)(((j >> 1) & 1) ^ 1), wc.st, 23, wc.lim)) break;
+        if (!__all_sync(~0u, wait(&tempty[acc], (uint32_t)((j >> 1) & 1) ^ 1u, 23))) break;
         fence_after_sync();
         // hi hi products in one accumulator, the five smaller ones (2^-8 and
         // below) in another: the FP32 accumulation's rounding then grows with
         // the few large-term MMAs only
-        const uint32_t d_big = tmem + acc * PK_ACC_COLS;
-        const uint32_t d_small = d_big + PK_N;
-        for (int kc = 0; kc < nK; ++kc, ++q) {
-          const int s = (int)(q % PK_STAGES);
-          const uint32_t ph = (uint32_t)((q / PK_STAGES) & 1);
-          if (!mbar_wait(&full[s], ph, wc.st, 24, wc.lim)) {
-            ok = false;
-            break;
-          }
-          fence_after_sync();
-          const uint32_t base = smem_u32(smem + s * PK_STAGE);
-          const uint32_t a_hi = base, a_mid = base + PK_PLANE_A, a_lo = base + 2 * PK_PLANE_A;
-          const uint32_t b_hi = base + 3 * PK_PLANE_A, b_mid = b_hi + PK_PLANE_B,
-                         b_lo = b_hi + 2 * PK_PLANE_B;
+        const uint32_t d_big = tmem + acc * 2 * N;
+        const uint32_t d_small = d_big + N;
+        for (int kc = 0; kc < nK && ok; ++kc) {
+          uint32_t a[3], b[3];
+          int slot[3];
 #pragma unroll
-          for (int k = 0; k < PK_KC / 16; ++k) {
-            const uint32_t koff = k * 32;
-            const uint32_t first = (kc | k) != 0 ? 1u : 0u;
-            mma_bf16(d_small, desc_sw64(a_lo + koff), desc_sw64(b_hi + koff), IDESC, first);
-            mma_bf16(d_small, desc_sw64(a_hi + koff), desc_sw64(b_lo + koff), IDESC, 1u);
-            mma_bf16(d_small, desc_sw64(a_mid + koff), desc_sw64(b_mid + koff), IDESC, 1u);
-            mma_bf16(d_small, desc_sw64(a_mid + koff), desc_sw64(b_hi + koff), IDESC, 1u);
-            mma_bf16(d_small, desc_sw64(a_hi + koff), desc_sw64(b_mid + koff), IDESC, 1u);
-            mma_bf16(d_big, desc_sw64(a_hi + koff), desc_sw64(b_hi + koff), IDESC, first);
+          for (int p = 0; p < 3; ++p, ++q) {
+            slot[p] = (int)(q % SLOTS);
+            a[p] = smem_u32(smem + slot[p] * TL::SLOT);
+            b[p] = a[p] + TL::PLANE_A;
+            if (!__all_sync(~0u, mbar_wait(&full[slot[p]], (uint32_t)((q / SLOTS) & 1), wc.st, 24, wc.lim))) {
+              ok = false;
+              break;
+            }
           }
-          mma_commit(&empty[s]);
+          if (!ok) break;
+          fence_after_sync();
+          if (elect_one()) {
+#pragma unroll
+            for (int k = 0; k < KC / 16; ++k) {
+              const uint32_t koff = k * 32, first = (kc | k) != 0 ? 1u : 0u;
+              mma(fill, d_big, a[0] + koff, b[0] + koff, first);
+              mma(use, d_small, a[0] + koff, b[1] + koff, first);
+              mma(last, d_small, a[0] + koff, b[2] + koff, 1u);
+              mma(fill, d_small, a[1] + koff, b[0] + koff, 1u);
+              mma(last, d_small, a[1] + koff, b[1] + koff, 1u);
+              mma(once, d_small, a[2] + koff, b[0] + koff, 1u);
+            }
+            for (int p = 0; p < 3; ++p) commit(&empty[slot[p]]);
+            if (kc == nK - 1) commit(&tfull[acc]);
+          }
+          __syncwarp();
         }
-        mma_commit(&tfull[acc]);
       }
     }
   } else {
-    // ---- epilogue: warp w drains lane quarter w % 4, points half * 64 ..
+    // ---- epilogue: warp w drains lane quarter w % 4, columns group * 32 ..
     const int quarter = warp & 3;
-    const int half = (warp - 2) >> 2;
+    const int group = (warp - 2) >> 2;
     const int c_in = 32 * quarter + lane;
     const float g2 = gamma * 1.4426950408889634f;   // K = 2^(-g2 |x - z|^2)
-    float* stage = reinterpret_cast<float*>(smem + PK_STAGE_OFF) + (warp - 2) * 3 * PK_WP;
-    uint8_t* obox = smem + PK_OUT_OFF + (warp - 2) * 2 * PK_OUT_BOX;
-    int64_t j = 0;
-    for (int64_t t = blockIdx.x; t < T; t += gridDim.x, ++j) {
+    const uint64_t m2 = dup2(-g2), p2 = dup2(2.0f * g2);
+    float* stage = reinterpret_cast<float*>(smem + TL::STAGE_OFF) + (warp - 2) * 3 * PK_WP;
+    // What a lane needs of a tile besides the product: its row's norm, and of
+    // one of the warp's columns the norm, the output and label (SCORE) or the
+    // coefficient (DECIDE); zero outside.  Read a tile ahead.
+    struct Pre {
+      float rn, cn, oi, yi;
+      double b;
+    };
+    auto fetch = [&](int64_t t) {
+      Pre f{0.f, 0.f, 0.f, 0.f, 0.0};
+      if (t >= T) return f;
       int cb;
       int64_t pt;
       tile_coords(t, nCB, nPT, cb, pt);
-      const int64_t c = (int64_t)cb * PK_M + c_in;
-      const bool crow = c < m;
-      const float zn = crow ? (DECIDE ? znorm[c] : norms[idx[c]]) : 0.f;
-      const float bc = DECIDE && crow ? (float)beta[c] : 0.f;
-      const int64_t ib = pt * PK_N + half * PK_WP;
-      const int64_t npts = min64(PK_WP, n - ib);
-      // this warp's 64 points: norms (and for scores the active residual / flag)
-      for (int h2 = 0; h2 < PK_WP / 32; ++h2) {
-        const int jj = h2 * 32 + lane;
-        const int64_t i = ib + jj;
-        const bool in = jj < npts;
-        stage[jj] = in ? norms[i] : 0.f;
+      const int64_t c = (TL::CTAS * (int64_t)cb + rank) * PK_M + c_in;
+      const int64_t i = pt * N + group * PK_WP + lane;
+      if (c < nrows) f.rn = rownorm[SCORE ? idx[c] : c];
+      if (i < ncols) {
+        f.cn = colnorm[STORE ? idx[i] : i];
         if (SCORE) {
-          float r = 0.f, a = 0.f;
-          if (in) {
-            const float oi = o[i], yi = y[i];
-            if (yi * oi < 1.0f) {
-              r = oi - yi;
-              a = 1.f;
-            }
-          }
-          stage[PK_WP + jj] = r;
-          stage[2 * PK_WP + jj] = a;
+          f.oi = o[i];
+          f.yi = y[i];
         }
+        if (DECIDE) f.b = beta[i];
       }
+      return f;
+    };
+    Pre next = fetch(unit);
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);   // SCORE: compensated pairs of this thread's sums
+    int flushes = 0;
+    if (SCORE && group == 0)
+      for (int64_t c = rank * PK_M + c_in; c < nrows; c += TL::M) part[unit * nrows + c] = sum;
+    int64_t j = 0;
+    for (int64_t t = unit; t < T; t += units, ++j) {
+      int cb;
+      int64_t pt;
+      tile_coords(t, nCB, nPT, cb, pt);
+      const int64_t cblock = TL::CTAS * (int64_t)cb + rank;   // this CTA's 128 rows
+      const int64_t c = cblock * PK_M + c_in;
+      const bool crow = c < nrows;
+      const int64_t ib = pt * N + group * PK_WP;
+      const bool any = ib < ncols;   // uniform per warp
+      const float zz = -g2 * next.rn;
+      __syncwarp();   // the stage has been read
+      stage[lane] = next.cn;
+      if (SCORE) {
+        const bool active = next.yi * next.oi < 1.0f && ib + lane < ncols;
+        stage[PK_WP + lane] = active ? next.oi - next.yi : 0.f;
+        stage[2 * PK_WP + lane] = active ? 1.f : 0.f;
+      }
+      if (DECIDE) stage[PK_WP + lane] = (float)next.b;
       __syncwarp();
       const int acc = (int)(j & 1);
-      if (!mbar_wait(&tfull[acc], (uint32_t)((j >> 1) & 1), wc.st, 25, wc.lim)) break;
+      if (!__all_sync(~0u, wait(&tfull[acc], (uint32_t)((j >> 1) & 1), 25))) break;
       fence_after_sync();
-      float gs = 0.f, hs = 0.f;
-      const uint32_t tb = tmem + acc * PK_ACC_COLS + half * PK_WP + ((uint32_t)(32 * quarter) << 16);
-      if (STORE) {
-        // the previous tile's boxes must have been read out before they are rewritten
-        if (lane == 0) bulk_wait_read();
-        __syncwarp();
+      const uint32_t tb = tmem + acc * 2 * N + group * PK_WP + ((uint32_t)(32 * quarter) << 16);
+      uint64_t v[16];   // x.z = large terms + small terms, two columns each
+      {
+        float a[32], b[32];
+        tmem_ld32(tb, a);
+        tmem_ld32(tb + N, b);
+#pragma unroll
+        for (int jj = 0; jj < 16; ++jj)
+          v[jj] = pack2(a[2 * jj] + b[2 * jj], a[2 * jj + 1] + b[2 * jj + 1]);
       }
-      const float zz = -g2 * zn;
-      for (int cc = 0; cc < PK_WP / 32; ++cc) {
-        if (cc * 32 >= npts) break;   // uniform per warp
-        float v[32], w[32];
-        tmem_ld32(tb + cc * 32, v);
-        tmem_ld32(tb + PK_N + cc * 32, w);
+      // the accumulators are in registers: the next tile's MMAs may start
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) {
+        if constexpr (PAIR) mbar_arrive_cluster(map_rank(&tempty[acc], 0));
+        else mbar_arrive(&tempty[acc]);
+      }
+      next = fetch(t + units);
+      float gs = 0.f, hs = 0.f;
+      if (any) {
+        // arg = -g2 * max(|x|^2 + |z|^2 - 2 x.z, 0); columns past the last
+        // carry zero norms here and are not stored or weighted by zero
+        const uint64_t z2 = dup2(zz);
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj) v[jj] += w[jj];   // x.z = large terms + small terms
-        // arg = -g2 * max(|x|^2 + |z|^2 - 2 x.z, 0); points past n carry zero
-        // norms here and are clipped by the store or weighted by zero flags
+        for (int jj = 0; jj < 16; jj += 2) {
+          const ulonglong2 x4 = *reinterpret_cast<const ulonglong2*>(stage + 2 * jj);
 #pragma unroll
-        for (int jj = 0; jj < 32; jj += 4) {
-          const float4 x4 = *reinterpret_cast<const float4*>(stage + cc * 32 + jj);
-          v[jj + 0] = ex2_approx(fminf(fmaf(-g2, x4.x, fmaf(2.0f * g2, v[jj + 0], zz)), 0.0f));
-          v[jj + 1] = ex2_approx(fminf(fmaf(-g2, x4.y, fmaf(2.0f * g2, v[jj + 1], zz)), 0.0f));
-          v[jj + 2] = ex2_approx(fminf(fmaf(-g2, x4.z, fmaf(2.0f * g2, v[jj + 2], zz)), 0.0f));
-          v[jj + 3] = ex2_approx(fminf(fmaf(-g2, x4.w, fmaf(2.0f * g2, v[jj + 3], zz)), 0.0f));
+          for (int h = 0; h < 2; ++h) {
+            uint64_t a = z2;
+            fma2(a, p2, v[jj + h]);
+            fma2(a, m2, h ? x4.y : x4.x);
+            const float2 f = unpack2(a);
+            v[jj + h] = pack2(ex2_approx(fminf(f.x, 0.0f)), ex2_approx(fminf(f.y, 0.0f)));
+          }
         }
         if (STORE) {
-          // 32 FP32 values into box cc of this warp (row = lane, 128-byte
-          // swizzle: 16-byte chunk ch of row r at chunk ch ^ (r & 7))
-          uint8_t* bx = obox + cc * PK_OUT_BOX;
+          float* dst = out + ib * ld + c;
+          const int64_t left = ncols - ib;
+          if (crow) {
 #pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {
-            const int so = lane * 128 + ((ch ^ (lane & 7)) << 4);
-            *reinterpret_cast<float4*>(bx + so) =
-                make_float4(v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
-          }
-        } else if (SCORE) {
-#pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
-            const float kv = v[jj];
-            gs = fmaf(stage[PK_WP + cc * 32 + jj], kv, gs);
-            hs = fmaf(stage[2 * PK_WP + cc * 32 + jj] * kv, kv, hs);
+            for (int jj = 0; jj < 16; ++jj) {
+              const float2 f = unpack2(v[jj]);
+              if (2 * jj < left) dst[2 * jj * ld] = f.x;
+              if (2 * jj + 1 < left) dst[(2 * jj + 1) * ld] = f.y;
+            }
           }
         } else {
-          // beta_c k(z_c, x_i) summed over this warp's 32 basis rows (rows
-          // past m carry beta 0); one partial per (basis block, lane
-          // quarter) and query, summed in a fixed order by the finish
+          // SCORE: the sums of (o - y) K and K^2 over the active columns;
+          // DECIDE: of beta K over the columns; in chains of 8 and 4 terms
+          uint64_t g2s[4] = {0, 0, 0, 0}, h2s[2] = {0, 0};
+          constexpr int CH = SCORE ? 2 : 4;
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj) v[jj] *= bc;
-          const float f = warp_column_sums(v, lane);
-          if (cc * 32 + lane < npts)
-            dpart[((int64_t)cb * 4 + quarter) * ldp + ib + cc * 32 + lane] = f;
+          for (int jj = 0; jj < 16; jj += 2) {
+            const ulonglong2 r4 = *reinterpret_cast<const ulonglong2*>(stage + PK_WP + 2 * jj);
+            fma2(g2s[jj % CH], r4.x, v[jj]);
+            fma2(g2s[jj % CH + 1], r4.y, v[jj + 1]);
+            if (SCORE) {
+              const ulonglong2 a4 = *reinterpret_cast<const ulonglong2*>(stage + 2 * PK_WP + 2 * jj);
+              fma2(h2s[0], mul2(a4.x, v[jj]), v[jj]);
+              fma2(h2s[1], mul2(a4.y, v[jj + 1]), v[jj + 1]);
+            }
+          }
+          const float2 ga = unpack2(g2s[0]), gb = unpack2(g2s[1]), gc = unpack2(g2s[2]), gd = unpack2(g2s[3]);
+          gs = (ga.x + ga.y) + (gb.x + gb.y);
+          if (CH == 4) gs += (gc.x + gc.y) + (gd.x + gd.y);
+          const float2 ha = unpack2(h2s[0]), hb = unpack2(h2s[1]);
+          hs = (ha.x + ha.y) + (hb.x + hb.y);
         }
       }
-      fence_before_sync();
-      mbar_arrive(&tempty[acc]);
-      if (STORE && npts > 0) {
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) {
-          const int x = (int)ib, yrow = (int)(row0 + (int64_t)cb * PK_M + 32 * quarter);
-          // boxes of 32 points; the second starts past n only when npts <= 32
-          tma_store_2d(&map_out, x, yrow, obox);
-          if (npts > 32) tma_store_2d(&map_out, x + 32, yrow, obox + PK_OUT_BOX);
-          bulk_commit();
-        }
-      }
+      // one partial per 32 basis rows and query, summed in a fixed order by
+      // the finish
+      if (DECIDE && crow && any) dpart[ib / PK_WP * ldp + c] = gs;
       if (SCORE) {
-        // the two warps of a lane quarter combine their halves of the tile
-        const uint32_t par = (uint32_t)(j & 1);
-        if (half == 1) {
-          if (!mbar_wait(&rede[quarter], par ^ 1u, wc.st, 26, wc.lim)) break;
-          red[quarter * 32 + lane] = make_float2(gs, hs);
+        pair_add(sum.x, sum.y, gs);
+        pair_add(sum.z, sum.w, hs);
+        const int64_t tn = t + units;   // the next tile's rows are the same: keep the sums
+        if (tn < T) {
+          int cn;
+          int64_t pn;
+          tile_coords(tn, nCB, nPT, cn, pn);
+          if (cn == cb) continue;
+        }
+        // the warps of a lane quarter combine their groups of columns, in order
+        const uint32_t par = (uint32_t)(flushes & 1);
+        ++flushes;
+        if (group > 0) {
+          if (!__all_sync(~0u, mbar_wait(&rede[quarter], par ^ 1u, wc.st, 26, wc.lim))) break;
+          red[(group - 1) * 128 + c_in] = sum;
           mbar_arrive(&redf[quarter]);
         } else {
-          if (!mbar_wait(&redf[quarter], par, wc.st, 27, wc.lim)) break;
-          const float2 r2 = red[quarter * 32 + lane];
+          if (!__all_sync(~0u, mbar_wait(&redf[quarter], par, wc.st, 27, wc.lim))) break;
+          float4 all = crow ? part[unit * nrows + c] : sum;
+          pair_add(all.x, all.y, make_float2(sum.x, sum.y));
+          pair_add(all.z, all.w, make_float2(sum.z, sum.w));
+#pragma unroll
+          for (int g = 0; g < GROUPS - 1; ++g) {
+            const float4 r = red[g * 128 + c_in];
+            pair_add(all.x, all.y, make_float2(r.x, r.y));
+            pair_add(all.z, all.w, make_float2(r.z, r.w));
+          }
           mbar_arrive(&rede[quarter]);
-          if (crow)
-            part[pt * kappa + c] = make_double2((double)gs + (double)r2.x, (double)hs + (double)r2.y);
+          if (crow) part[unit * nrows + c] = all;
         }
+        sum = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      __syncwarp();
     }
-    if (STORE && lane == 0) bulk_wait_all();
   }
   fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
+  if constexpr (PAIR) {
     __syncwarp();
-    fence_after_sync();
-    tmem_dealloc(tmem, 2 * PK_ACC_COLS);
+    cluster_sync();   // no copy, MMA or arrival of the pair is outstanding
+    if (warp == 0) {
+      fence_after_sync();
+      tmem_dealloc_pair(tmem, 4 * N);
+    }
+  } else {
+    __syncthreads();
+    if (warp == 0) {
+      __syncwarp();
+      fence_after_sync();
+      tmem_dealloc(tmem, 4 * N);
+    }
   }
 }
 
-// Z planes: rows idx[0..m) of the three split X planes, zero rows up to m_pad.
+// Rows idx[0..m) of the three split planes, contiguous.
 __global__ void gather_rows_bf16(const uint16_t* __restrict__ Xhi, const uint16_t* __restrict__ Xmid,
                                  const uint16_t* __restrict__ Xlo, int64_t ldh,
-                                 const int64_t* __restrict__ idx, int32_t m, int64_t m_pad,
+                                 const int64_t* __restrict__ idx, int32_t m,
                                  uint16_t* __restrict__ Zhi, uint16_t* __restrict__ Zmid,
                                  uint16_t* __restrict__ Zlo) {
   const int64_t chunks = ldh / 8;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= m_pad * chunks) return;
+  if (e >= m * chunks) return;
   const int64_t r = e / chunks, ch = e % chunks;
-  uint4 vh = make_uint4(0, 0, 0, 0), vm = vh, vl = vh;
-  if (r < m) {
-    const int64_t src = idx[r] * ldh + ch * 8;
-    vh = *reinterpret_cast<const uint4*>(Xhi + src);
-    vm = *reinterpret_cast<const uint4*>(Xmid + src);
-    vl = *reinterpret_cast<const uint4*>(Xlo + src);
-  }
-  *reinterpret_cast<uint4*>(Zhi + r * ldh + ch * 8) = vh;
-  *reinterpret_cast<uint4*>(Zmid + r * ldh + ch * 8) = vm;
-  *reinterpret_cast<uint4*>(Zlo + r * ldh + ch * 8) = vl;
+  const int64_t src = idx[r] * ldh + ch * 8, dst = r * ldh + ch * 8;
+  *reinterpret_cast<uint4*>(Zhi + dst) = *reinterpret_cast<const uint4*>(Xhi + src);
+  *reinterpret_cast<uint4*>(Zmid + dst) = *reinterpret_cast<const uint4*>(Xmid + src);
+  *reinterpret_cast<uint4*>(Zlo + dst) = *reinterpret_cast<const uint4*>(Xlo + src);
 }
 
 // ---------------------------------------------------------------------------
@@ -550,7 +655,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
     // wait for the copies of the last stages so none is in flight at exit
     if (rank == 0)
       for (int64_t q = (issued > GR_STAGES ? issued - GR_STAGES : 0); q < issued; ++q)
-        mbar_wait_cluster(&full[q % GR_STAGES], (uint32_t)((q / GR_STAGES) & 1), wc.st, 12, wc.lim);
+        mbar_wait(&full[q % GR_STAGES], (uint32_t)((q / GR_STAGES) & 1), wc.st, 12, wc.lim);
   } else if (live && warp == 1 && lane == 0 && rank == 0) {
     // ---- MMA issuer
     bool ok = true;
@@ -565,7 +670,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
       for (int64_t q = q0; q < q1; ++q) {
         const int s = (int)(q % GR_STAGES);
         const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
-        if (!mbar_wait_cluster(&full[s], ph, wc.st, 14, wc.lim)) {
+        if (!mbar_wait(&full[s], ph, wc.st, 14, wc.lim)) {
           ok = false;
           break;
         }
@@ -577,13 +682,13 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const uint32_t koff = k * 32;
-          mma_bf16_pair(d, desc_sw128(a_hi + koff), desc_sw128(b_hi + koff), IDESC,
+          mma_bf16_pair<A_FILL>(d, desc_sw128(a_hi + koff), desc_sw128(b_hi + koff), IDESC,
                         (q != q0 || k != 0) ? 1u : 0u);
-          mma_bf16_pair(d, desc_sw128(a_hi + koff), desc_sw128(b_lo + koff), IDESC, 1u);
-          mma_bf16_pair(d, desc_sw128(a_lo + koff), desc_sw128(b_hi + koff), IDESC, 1u);
+          mma_bf16_pair<A_LASTUSE>(d, desc_sw128(a_hi + koff), desc_sw128(b_lo + koff), IDESC, 1u);
+          mma_bf16_pair<A_FILL>(d, desc_sw128(a_lo + koff), desc_sw128(b_hi + koff), IDESC, 1u);
           // lo x lo too: without it the sum is (hi + lo)^T (hi + lo) - lo^T lo,
           // indefinite in the null space of a short K_SJ
-          mma_bf16_pair(d, desc_sw128(a_lo + koff), desc_sw128(b_lo + koff), IDESC, 1u);
+          mma_bf16_pair<A_LASTUSE>(d, desc_sw128(a_lo + koff), desc_sw128(b_lo + koff), IDESC, 1u);
         }
         mma_commit_pair(&empty[s]);
       }
@@ -737,13 +842,13 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const uint32_t koff = k * 32;
-          mma_bf16(d, desc_sw128(a_hi + koff), desc_sw128(b_hi + koff), IDESC,
+          mma_bf16<A_FILL>(d, desc_sw128(a_hi + koff), desc_sw128(b_hi + koff), IDESC,
                    (q != q0 || k != 0) ? 1u : 0u);
-          mma_bf16(d, desc_sw128(a_hi + koff), desc_sw128(b_lo + koff), IDESC, 1u);
-          mma_bf16(d, desc_sw128(a_lo + koff), desc_sw128(b_hi + koff), IDESC, 1u);
+          mma_bf16<A_LASTUSE>(d, desc_sw128(a_hi + koff), desc_sw128(b_lo + koff), IDESC, 1u);
+          mma_bf16<A_FILL>(d, desc_sw128(a_lo + koff), desc_sw128(b_hi + koff), IDESC, 1u);
           // lo x lo too: without it the sum is (hi + lo)^T (hi + lo) - lo^T lo,
           // indefinite in the null space of a short K_SJ
-          mma_bf16(d, desc_sw128(a_lo + koff), desc_sw128(b_lo + koff), IDESC, 1u);
+          mma_bf16<A_LASTUSE>(d, desc_sw128(a_lo + koff), desc_sw128(b_lo + koff), IDESC, 1u);
         }
         mma_commit(&empty[s]);
       }
@@ -803,81 +908,109 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// 2-D map over rows x inner (row pitch `pitch_elems`) of BF16 (or FP32 with
-// f32), box_inner x box_rows boxes of 128 bytes per row, 128-byte swizzle,
-// zero fill outside the tensor.
+// 2-D map over rows x inner (row pitch `pitch_elems`) of BF16, boxes of
+// 64 elements (128 bytes, 128-byte swizzle) x box_rows, zero fill outside the
+// tensor.
 int make_map(CUtensorMap* map, const void* base, int64_t inner, int64_t rows, int64_t pitch_elems,
-             uint32_t box_rows, uint32_t box_inner, bool f32 = false) {
+             uint32_t box_rows) {
   auto fn = encode_fn();
   if (!fn) return set_error(SPSVM_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-  const int64_t esz = f32 ? 4 : 2;
-  const int64_t row_bytes = box_inner * esz;   // 128-byte rows swizzled by 128, 64-byte rows by 64
-  if ((reinterpret_cast<uintptr_t>(base) & 15) || (pitch_elems * esz) % 16 ||
-      (row_bytes != 128 && row_bytes != 64))
-    return set_error(SPSVM_ERR_ARG, "tensor map: base or pitch not 16-byte aligned, or box row not 64/128 bytes");
+  if ((reinterpret_cast<uintptr_t>(base) & 15) || (pitch_elems * 2) % 16)
+    return set_error(SPSVM_ERR_ARG, "tensor map: base or pitch not 16-byte aligned");
   cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)(rows > 0 ? rows : 1)};
-  cuuint64_t strides[1] = {(cuuint64_t)(pitch_elems * esz)};
-  cuuint32_t box[2] = {box_inner, box_rows};
+  cuuint64_t strides[1] = {(cuuint64_t)(pitch_elems * 2)};
+  cuuint32_t box[2] = {64, box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                  const_cast<void*>(base), dims, strides,
-                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return set_error(SPSVM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return SPSVM_OK;
 }
 
-// Extra arguments of the decision mode: basis norms, beta, the partial sums
-// and their row pitch.
-struct DecideArgs {
-  const float* znorm = nullptr;
-  const double* beta = nullptr;
-  float* dpart = nullptr;
-  int64_t ldp = 0;
+// What the modes read and write besides the products of rows A by columns B.
+struct KbArgs {
+  const uint16_t *a_hi, *a_mid, *a_lo, *b_hi, *b_mid, *b_lo;
+  int64_t ldh, nrows, ncols;
+  const float *colnorm, *rownorm;
+  const int64_t* idx;                 // of the columns' (STORE) or rows' (SCORE) norms
+  float gamma;
+  float* out;                         // STORE: the first column's row
+  int64_t ld;
+  const float *y, *o;                 // SCORE
+  float4* part;
+  int64_t* parts;                     // receives the number of partial sums
+  const double* beta;                 // DECIDE
+  float* dpart;
+  int64_t ldp;
 };
 
-// STORE / SCORE: the m rows idx of the points' planes are gathered into zbuf
-// first (zero rows up to a multiple of 128).  DECIDE: zbuf already holds the
-// basis planes (m rows of pitch ldh; the tensor maps zero-fill past m).
-template <int MODE>
-int launch_kb(const spsvm_points* p, const int64_t* idx, int32_t m, float gamma, void* out,
-              int64_t ld, int64_t row0, const float* y, const float* o, double2* part,
-              int32_t kappa, void* zbuf, size_t zbytes, cudaStream_t s,
-              const DecideArgs& da = DecideArgs()) {
-  const int64_t m_pad = round_up(m, (int64_t)PK_M);
-  const int64_t zrows = MODE == KB_DECIDE ? (int64_t)m : m_pad;
-  if (!zbuf || zbytes < (size_t)(zrows * p->ldh * 6))
-    return set_error(SPSVM_ERR_OOM, "BF16SPLIT kernel block: scratch too small for the basis planes");
-  uint16_t* zhi = static_cast<uint16_t*>(zbuf);
-  uint16_t* zmid = zhi + zrows * p->ldh;
-  uint16_t* zlo = zmid + zrows * p->ldh;
-  if (MODE != KB_DECIDE) {
-    const int64_t work = m_pad * (p->ldh / 8);
-    gather_rows_bf16<<<(unsigned)ceil_div(work, (int64_t)256), 256, 0, s>>>(
-        p->hi, p->mid, p->lo, p->ldh, idx, m, m_pad, zhi, zmid, zlo);
-    SPSVM_LAUNCH_CHECK();
-  }
-  CUtensorMap mzh, mzm, mzl, mxh, mxm, mxl, mo;
-  SPSVM_TRY(make_map(&mzh, zhi, p->ldh, zrows, p->ldh, PK_M, PK_KC));
-  SPSVM_TRY(make_map(&mzm, zmid, p->ldh, zrows, p->ldh, PK_M, PK_KC));
-  SPSVM_TRY(make_map(&mzl, zlo, p->ldh, zrows, p->ldh, PK_M, PK_KC));
-  SPSVM_TRY(make_map(&mxh, p->hi, p->ldh, p->n, p->ldh, PK_N, PK_KC));
-  SPSVM_TRY(make_map(&mxm, p->mid, p->ldh, p->n, p->ldh, PK_N, PK_KC));
-  SPSVM_TRY(make_map(&mxl, p->lo, p->ldh, p->n, p->ldh, PK_N, PK_KC));
-  // output rows [0, row0 + m): rows past the basis block are clipped, never written
-  if (MODE == KB_STORE_F32) SPSVM_TRY(make_map(&mo, out, p->n, row0 + m, ld, 32, 32, true));
-  else mo = mxh;
-  auto kern = kblock_tc_kernel<MODE>;
-  SPSVM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM));
-  const int64_t tiles = ceil_div((int64_t)m, (int64_t)PK_M) * ceil_div(p->n, (int64_t)PK_N);
-  const int grid = (int)min64(tiles, (int64_t)sm_count());
+template <int MODE, bool PAIR, int N>
+int launch_kb_as(const KbArgs& a, cudaStream_t s) {
+  using TL = Kb<PAIR, N>;
+  CUtensorMap mah, mam, mal, mbh, mbm, mbl;
+  SPSVM_TRY(make_map(&mah, a.a_hi, a.ldh, a.nrows, a.ldh, PK_M));
+  SPSVM_TRY(make_map(&mam, a.a_mid, a.ldh, a.nrows, a.ldh, PK_M));
+  SPSVM_TRY(make_map(&mal, a.a_lo, a.ldh, a.nrows, a.ldh, PK_M));
+  SPSVM_TRY(make_map(&mbh, a.b_hi, a.ldh, a.ncols, a.ldh, TL::ROWS_B));
+  SPSVM_TRY(make_map(&mbm, a.b_mid, a.ldh, a.ncols, a.ldh, TL::ROWS_B));
+  SPSVM_TRY(make_map(&mbl, a.b_lo, a.ldh, a.ncols, a.ldh, TL::ROWS_B));
+  auto kern = kblock_tc_kernel<MODE, PAIR, N>;
+  SPSVM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::SMEM));
+  constexpr int W = TL::CTAS;
+  const int64_t tiles = ceil_div(a.nrows, (int64_t)TL::M) * ceil_div(a.ncols, (int64_t)N);
   WaitCtx wc;
   SPSVM_TRY(wait_ctx(s, &wc));
-  kern<<<grid, PK_THREADS, PK_SMEM, s>>>(mzh, mzm, mzl, mxh, mxm, mxl, mo, p->ldh, p->n, m,
-                                         p->norms, idx, gamma, row0, y, o, part, kappa, da.znorm,
-                                         da.beta, da.dpart, da.ldp, wc);
+  cudaLaunchConfig_t cfg{};
+  int64_t units = max64(1, min64(tiles, (int64_t)sm_count() / W));
+  if (MODE == KB_SCORE) *a.parts = units = min64(units, kScoreUnits);
+  cfg.gridDim = dim3((unsigned)(W * units));
+  cfg.blockDim = dim3(TL::THREADS);
+  cfg.dynamicSmemBytes = TL::SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = W;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  SPSVM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mah, mam, mal, mbh, mbm, mbl, a.ldh, a.ncols, a.nrows,
+                                    a.colnorm, a.rownorm, a.idx, a.gamma, a.out, a.ld, a.y, a.o, a.part,
+                                    a.beta, a.dpart, a.ldp, wc));
   SPSVM_LAUNCH_CHECK();
+  return SPSVM_OK;
+}
+
+// Pairs once there are rows for both CTAs (fewer fill one CTA, whatever N).
+template <int MODE>
+int launch_kb(const KbArgs& a, cudaStream_t s) {
+  if (a.nrows <= PK_M) return launch_kb_as<MODE, false, 128>(a, s);
+  if (MODE != KB_SCORE && a.ncols <= 64) return launch_kb_as<MODE, true, MODE != KB_SCORE ? 64 : 128>(a, s);
+  return launch_kb_as<MODE, true, 128>(a, s);
+}
+
+}  // namespace
+
+size_t kernel_block_tc_scratch(int64_t m, int64_t ldh) {
+  return (size_t)(round_up(m, (int64_t)PK_M) * ldh * 6);   // three BF16 planes of the rows
+}
+
+namespace {
+
+// The planes of the m points idx, gathered into zbuf.
+int gather_rows(const spsvm_points* p, const int64_t* idx, int32_t m, void* zbuf, size_t zbytes,
+                cudaStream_t s, const uint16_t* (&z)[3]) {
+  if (!zbuf || zbytes < kernel_block_tc_scratch(m, p->ldh))
+    return set_error(SPSVM_ERR_OOM, "BF16SPLIT kernel block: scratch too small for the basis planes");
+  uint16_t* zhi = static_cast<uint16_t*>(zbuf);
+  uint16_t* zmid = zhi + m * p->ldh;
+  uint16_t* zlo = zmid + m * p->ldh;
+  gather_rows_bf16<<<(unsigned)ceil_div(m * (p->ldh / 8), (int64_t)256), 256, 0, s>>>(
+      p->hi, p->mid, p->lo, p->ldh, idx, m, zhi, zmid, zlo);
+  SPSVM_LAUNCH_CHECK();
+  z[0] = zhi;
+  z[1] = zmid;
+  z[2] = zlo;
   return SPSVM_OK;
 }
 
@@ -885,42 +1018,53 @@ int launch_kb(const spsvm_points* p, const int64_t* idx, int32_t m, float gamma,
 
 bool tc_available() { return encode_fn() != nullptr; }
 
-size_t kernel_block_tc_scratch(int64_t m, int64_t ldh) {
-  return (size_t)(round_up(m, (int64_t)PK_M) * ldh * 6);   // three BF16 planes of the rows
-}
-
 int launch_kernel_block_tc(const spsvm_points* p, const int64_t* idx, int32_t m, float gamma,
                            spsvm_kmat* out, int64_t row0, void* scratch, size_t scratch_bytes,
                            cudaStream_t s) {
   if (m == 0 || p->n == 0) return SPSVM_OK;
   if (out->format != SPSVM_FP32 || (out->ld % 8) != 0)
     return set_error(SPSVM_ERR_ARG, "BF16SPLIT kernel block: stores FP32 (ld %% 8 == 0)");
-  return launch_kb<KB_STORE_F32>(p, idx, m, gamma, out->data, out->ld, row0, nullptr, nullptr,
-                                 nullptr, 0, scratch, scratch_bytes, s);
+  const uint16_t* z[3];
+  SPSVM_TRY(gather_rows(p, idx, m, scratch, scratch_bytes, s, z));
+  KbArgs a{p->hi, p->mid, p->lo, z[0], z[1], z[2], p->ldh, p->n, m, p->norms, p->norms, idx, gamma};
+  a.out = static_cast<float*>(out->data) + row0 * out->ld;
+  a.ld = out->ld;
+  return launch_kb<KB_STORE_F32>(a, s);
 }
 
-int64_t score_tc_tiles(int64_t n) { return ceil_div(n, (int64_t)PK_N); }
+// Partial sums per candidate at most: one per CTA or pair of the grid.
+int64_t score_tc_parts(int64_t n, int32_t kappa) {
+  const int64_t rows = kappa > PK_M ? 2 * PK_M : PK_M;
+  return max64(1, min64(ceil_div((int64_t)kappa, rows) * ceil_div(n, (int64_t)128), kScoreUnits));
+}
 
 int launch_score_tc(const spsvm_points* p, const float* y, const float* o, const int64_t* idx,
-                    int32_t kappa, float gamma, double2* part, int64_t tiles, void* zbuf,
+                    int32_t kappa, float gamma, float4* part, int64_t* parts, void* zbuf,
                     size_t zbytes, cudaStream_t s) {
-  (void)tiles;
-  return launch_kb<KB_SCORE>(p, idx, kappa, gamma, nullptr, 0, 0, y, o, part, kappa, zbuf, zbytes, s);
+  const uint16_t* z[3];
+  SPSVM_TRY(gather_rows(p, idx, kappa, zbuf, zbytes, s, z));
+  KbArgs a{z[0], z[1], z[2], p->hi, p->mid, p->lo, p->ldh, kappa, p->n, p->norms, p->norms, idx, gamma};
+  a.y = y;
+  a.o = o;
+  a.part = part;
+  a.parts = parts;
+  return launch_kb<KB_SCORE>(a, s);
 }
 
-int64_t decision_tc_parts(int64_t m) { return 4 * ceil_div(m, (int64_t)PK_M); }
+int64_t decision_tc_parts(int64_t m) { return ceil_div(m, (int64_t)PK_WP); }
 
 int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes, int64_t m,
                        const float* znorm, const double* beta, float gamma, float* dpart,
                        int64_t ldp, cudaStream_t s) {
   if (m == 0 || q->n == 0) return SPSVM_OK;
-  DecideArgs da;
-  da.znorm = znorm;
-  da.beta = beta;
-  da.dpart = dpart;
-  da.ldp = ldp;
-  return launch_kb<KB_DECIDE>(q, nullptr, (int32_t)m, gamma, nullptr, 0, 0, nullptr, nullptr,
-                              nullptr, 0, const_cast<void*>(zplanes), zbytes, s, da);
+  if (!zplanes || zbytes < (size_t)(m * q->ldh * 6))
+    return set_error(SPSVM_ERR_OOM, "BF16SPLIT decision: scratch too small for the basis planes");
+  const uint16_t* z = static_cast<const uint16_t*>(zplanes);
+  KbArgs a{q->hi, q->mid, q->lo, z, z + m * q->ldh, z + 2 * m * q->ldh, q->ldh, q->n, m, znorm, q->norms, nullptr, gamma};
+  a.beta = beta;
+  a.dpart = dpart;
+  a.ldp = ldp;
+  return launch_kb<KB_DECIDE>(a, s);
 }
 
 GramPlan gram_tc_plan(int64_t m, int64_t ns_max) {
@@ -942,8 +1086,8 @@ int launch_gram_tc(const spsvm_kmat* Kc, const int64_t* ns_dev, int64_t ns_max, 
   const int vec = (reinterpret_cast<uintptr_t>(part) & 15) == 0;
   CUtensorMap mh, ml;   // boxes of 128 rows in both kernels
   static_assert(GS_TILE == GR_HALF, "one tensor map for both kernels");
-  SPSVM_TRY(make_map(&mh, hi, Kc->ld, m, Kc->ld, GR_HALF, 64));
-  SPSVM_TRY(make_map(&ml, lo, Kc->ld, m, Kc->ld, GR_HALF, 64));
+  SPSVM_TRY(make_map(&mh, hi, Kc->ld, m, Kc->ld, GR_HALF));
+  SPSVM_TRY(make_map(&ml, lo, Kc->ld, m, Kc->ld, GR_HALF));
   WaitCtx wc;
   SPSVM_TRY(wait_ctx(s, &wc));
   const bool known = ns_hint >= 0;

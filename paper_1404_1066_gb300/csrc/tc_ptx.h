@@ -72,10 +72,13 @@ __device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
 __device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
+// Arrival on a barrier of either CTA and the wait for such arrivals (or for
+// MMAs of either CTA), relaxed: what they order are TMEM accesses and MMAs,
+// by the tcgen05 fences before and after.  A release would wait for all of
+// the thread's global stores first, an acquire drop the SM's L1 lines.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-// mbar_wait for a barrier that the other CTA's threads arrive on.
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, int* status, int code,
                                                   uint32_t limit) {
   const uint32_t lim = limit ? limit : (1u << 23);
@@ -83,7 +86,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity)
@@ -153,16 +156,42 @@ __device__ __forceinline__ void fence_after_sync() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// What an MMA does with the collector buffer of its A operand: a run of MMAs
+// on the same A reads it from shared memory once.
+enum { A_DISCARD, A_FILL, A_USE, A_LASTUSE };
+
 // D[tmem] (+)= A[smem] * B[smem]^T, BF16 inputs, FP32 accumulation.
+template <int A = A_DISCARD>
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+                                   uint32_t idesc, uint32_t accumulate) {
+#define SPSVM_MMA(OP)                                                          \
+  asm volatile(                                                                \
+      "{\n\t.reg .pred p;\n\t"                                                 \
+      "setp.ne.b32 p, %4, 0;\n\t"                                             \
+      "tcgen05.mma.cta_group::1.kind::f16" OP " [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem), \
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                      \
+      : "memory")
+  if constexpr (A == A_FILL) SPSVM_MMA(".collector::a::fill");
+  else if constexpr (A == A_USE) SPSVM_MMA(".collector::a::use");
+  else if constexpr (A == A_LASTUSE) SPSVM_MMA(".collector::a::lastuse");
+  else SPSVM_MMA("");
+#undef SPSVM_MMA
 }
+
+// True in one lane of the (converged) warp, the same one each time.  A loop
+// that the whole warp runs, with only the MMAs under this test, keeps their
+// descriptors in uniform registers; under a lane test each one is moved
+// there first, and issuing takes longer than the MMAs.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, P;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // Arrives on `bar` once every tcgen05 operation issued so far by this thread
 // has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -174,14 +203,21 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 
 // The same over a pair of CTAs: M = 256 (128 rows of A and of D in each CTA),
 // the N rows of B half in each; issued by one thread of the even CTA.
+template <int A = A_DISCARD>
 __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                              uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+                                   uint32_t idesc, uint32_t accumulate) {
+#define SPSVM_MMA(OP)                                                          \
+  asm volatile(                                                                \
+      "{\n\t.reg .pred p;\n\t"                                                 \
+      "setp.ne.b32 p, %4, 0;\n\t"                                             \
+      "tcgen05.mma.cta_group::2.kind::f16" OP " [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem), \
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                      \
+      : "memory")
+  if constexpr (A == A_FILL) SPSVM_MMA(".collector::a::fill");
+  else if constexpr (A == A_USE) SPSVM_MMA(".collector::a::use");
+  else if constexpr (A == A_LASTUSE) SPSVM_MMA(".collector::a::lastuse");
+  else SPSVM_MMA("");
+#undef SPSVM_MMA
 }
 // Arrives on `bar` of both CTAs of the pair once every pair operation issued
 // so far by this thread has completed.
@@ -198,19 +234,6 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
-}
-
-// The same for the 64-byte swizzled layout: rows of 32 BF16 (64 bytes),
-// 8-row groups 512 bytes apart; tile base 512-byte aligned.  Advancing along
-// K by 16 elements adds 32 bytes to the start address.
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;              // leading byte offset (unused for this layout)
-  d |= (uint64_t)(512 >> 4) << 32;     // stride byte offset: next 8-row group
-  d |= (uint64_t)1 << 46;              // descriptor version
-  d |= (uint64_t)4 << 61;              // 64-byte swizzle
-  return d;
 }
 
 // Shared-memory matrix descriptor of a K-major operand in the 128-byte

@@ -149,6 +149,47 @@ def test_fp32_decision_edges(sp, nq, m, d, pad):
     assert np.all(np.abs(f - ref) <= bound @ np.abs(beta) + 2.0 ** -24 * np.abs(ref))
 
 
+# tiles of 128 rows, or of 256 by pairs of CTAs, by 64 or 128 columns; 64
+# features a step; score sums kept over a CTA's tiles of one block of candidates
+@pytest.mark.parametrize("pad", [False, True])
+@pytest.mark.parametrize("n,d,m", [(1, 1, 1), (128, 64, 64), (129, 65, 65), (257, 63, 129), (300, 130, 128),
+                                   (20_000, 33, 64), (40_001, 100, 257), (60_000, 7, 300)])
+def test_split_block_score_and_decision_edges(sp, n, d, m, pad):
+    """Kernel values: three dropped products and the norms, and d / 16
+    truncating accumulations of the large terms; then sums of at most 32 FP32
+    terms in chains of 8, beta rounded to FP32."""
+    X, Xt = _points(n + m, d, n + d, pad)
+    X, Xt, B, Bt = X[:n], Xt[:n], X[n:], Xt[n:]
+    g = np.random.default_rng(m)
+    J = g.choice(n, min(m, n), replace=False)
+    gamma = 0.7 / d
+    P = sp.spsvm_prepare_points(Xt, "bf16split")
+    out = sp.kmat_empty(n, len(J), "fp32")
+    sp.spsvm_kernel_block(P, _t(J), gamma, "bf16split", out)
+    K = O.rbf_kernel(X, X[J], gamma)                # n x m
+    sq = (X.astype(np.float64) ** 2).sum(1)
+    eps = (d / 16 + 8) * 2.0 ** -23 * gamma
+    bound = eps * (sq[:, None] + sq[J][None, :]) + 2e-6
+    assert np.all(np.abs(out.to_float().cpu().numpy().T - K) <= bound)
+
+    y = np.where(g.random(n) < 0.5, 1.0, -1.0).astype(np.float32)
+    o = (y * (1 + 0.5 * g.standard_normal(n))).astype(np.float32)
+    gs, hs, delta = (v.cpu().numpy() for v in
+                     sp.spsvm_score_candidates(P, _t(y), _t(o), _t(J), gamma, 1e-3, "bf16split"))
+    S = (y * o < 1).astype(np.float64)
+    r = S * (o.astype(np.float64) - y)
+    tol = 12 * 2.0 ** -24
+    assert np.all(np.abs(gs - (1e-3 * o[J] + K.T @ r)) <= (bound + tol * K).T @ np.abs(r) + 1e-9)
+    assert np.all(np.abs(hs - (1e-3 + (K * K).T @ S)) <= (2 * bound * K + tol * K * K).T @ S + 1e-9)
+    np.testing.assert_allclose(delta, gs * gs / (2 * hs), rtol=1e-14)
+
+    beta = g.standard_normal(m) * 10.0 ** g.uniform(-6, 6, m)
+    f = sp.spsvm_decision(Bt, _t(beta), Xt, gamma, "bf16split").cpu().numpy()
+    K = O.rbf_kernel(X, B, gamma)
+    bound = eps * (sq[:, None] + (B.astype(np.float64) ** 2).sum(1)[None, :]) + 2e-6
+    assert np.all(np.abs(f - K @ beta) <= (bound + tol * K) @ np.abs(beta) + 1e-30)
+
+
 def test_split_decision_sums_in_pairs(sp):
     """Partials that cancel: 1,024 basis rows (32 partials a query), beta of
     +-1e6 in pairs on the same point; each partial's 32 terms are FP32."""
