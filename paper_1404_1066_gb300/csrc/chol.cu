@@ -1030,8 +1030,10 @@ __device__ __forceinline__ void dag_stage_regs(float (*S)[DP], const float (&acc
 
 // One ticket's work (all threads): a helper's partial (kinds 3 and 4) or a
 // tile below the chain (kind 2).  Uses As, Bs, rd and acc; ends with the
-// tile's publish.
-__device__ __forceinline__ void dag_ticket_work(int kind, int64_t i, int64_t j, float* __restrict__ L,
+// tile's publish.  One copy for both callers: inlined, the chain's first steps
+// spend longer on fetching their instructions (m = 512: 105 us, this 94; m =
+// 128: 32 and 22).
+__device__ __noinline__ void dag_ticket_work(int kind, int64_t i, int64_t j, float* __restrict__ L,
                                                 int64_t ldl, int64_t m, int64_t T,
                                                 unsigned* __restrict__ flags, float (*As)[DT][DP],
                                                 float (*Bs)[DT][DP], float* __restrict__ rd,
