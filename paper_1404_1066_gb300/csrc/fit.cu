@@ -52,28 +52,6 @@ __global__ void sub_kernel(const float* __restrict__ a, const float* __restrict_
     out[i] = a[i] - b[i];
 }
 
-// (K_JJ w)_k from outputs v = K_nJ w read at the basis points: the bias slot
-// (J_k < 0) has no regulariser row, and a bias w_0 (b0) carried by every
-// output is taken off.
-__device__ __forceinline__ double reg_at(const float* __restrict__ v, const int64_t* __restrict__ J,
-                                         int k, const double* __restrict__ b0) {
-  const int64_t j = J[k];
-  if (j < 0) return 0.0;
-  return (double)v[j] - (b0 ? *b0 : 0.0);
-}
-
-// g_k = lambda (K_JJ beta)_k + gs_k ; rhs_k = -g_k
-__global__ void grad_finish(const float* __restrict__ o, const int64_t* __restrict__ J,
-                            const double* __restrict__ gs, int32_t m, double lambda,
-                            double* __restrict__ g, double* __restrict__ rhs,
-                            const double* __restrict__ b0) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= m) return;
-  const double v = lambda * reg_at(o, J, k, b0) + gs[k];
-  g[k] = v;
-  rhs[k] = -v;
-}
-
 // rho_k = -g_k - lambda u[J_k] - ws_k   (residual of H d = -g, H applied exactly)
 __global__ void refine_resid(const double* __restrict__ g, const float* __restrict__ u,
                              const int64_t* __restrict__ J, const double* __restrict__ ws,
@@ -86,59 +64,6 @@ __global__ void refine_resid(const double* __restrict__ g, const float* __restri
 __global__ void axpy_d(double* __restrict__ y, const double* __restrict__ x, double a, int32_t m) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < m) y[k] += a * x[k];
-}
-
-// beta += t d and o += t u with t read on the device (the line search's
-// result, 0 when it found no descent)
-__global__ void axpy_t(double* __restrict__ y, const double* __restrict__ x,
-                       const double* __restrict__ t, int32_t m) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const double a = *t;
-  if (k < m && a != 0.0) y[k] += a * x[k];
-}
-
-__global__ void update_o_t(float* __restrict__ o, const float* __restrict__ u,
-                           const double* __restrict__ t, int64_t n) {
-  const double a = *t;
-  if (a == 0.0) return;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    o[i] = (float)((double)o[i] + a * (double)u[i]);
-}
-
-__global__ void count_diff(const uint8_t* __restrict__ a, const uint8_t* __restrict__ b, int64_t n,
-                           unsigned long long* __restrict__ out) {
-  __shared__ int sh[32];
-  int c = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    c += (a[i] != b[i]);
-  c = block_sum(c, sh);
-  if (threadIdx.x == 0 && c) atomicAdd(out, (unsigned long long)c);
-}
-
-// out[0] = beta^T K_JJ beta ; out[1] = sum g_k^2 ; out[2] = sum r_k^2
-__global__ void small_dots(const double* __restrict__ beta, const float* __restrict__ o,
-                           const int64_t* __restrict__ J, const double* __restrict__ g,
-                           const double* __restrict__ r, int32_t m, double* __restrict__ out,
-                           const double* __restrict__ b0) {
-  __shared__ double sh[32];
-  double a = 0.0, b = 0.0, c = 0.0;
-  for (int k = threadIdx.x; k < m; k += blockDim.x) {
-    a += beta[k] * reg_at(o, J, k, b0);
-    b += g[k] * g[k];
-    c += r[k] * r[k];
-  }
-  a = block_sum(a, sh);
-  __syncthreads();
-  b = block_sum(b, sh);
-  __syncthreads();
-  c = block_sum(c, sh);
-  if (threadIdx.x == 0) {
-    out[0] = a;
-    out[1] = b;
-    out[2] = c;
-  }
 }
 
 // out[0] = ||d||^2, out[1] = ||beta||^2
@@ -529,17 +454,18 @@ struct Fit {
     // Gradient pass on the flags `act`: residuals o - y, compaction with the
     // masked transposed products (w = K_SJ^T (o_S - y_S), r = K_SJ^T y_S;
     // the copy K_SJ is rewritten unless *kc_cond is zero, i.e. unless the
-    // active set is unchanged), gradient and the dots of the stopping test.
-    auto grad_pass = [&](uint8_t* act_f, const unsigned long long* kc_cond) -> int {
-      sub_kernel<<<grid_for(n, tpb), tpb, 0, s>>>(o, y, n, res);
-      SPSVM_LAUNCH_CHECK();
-      SPSVM_TRY(compact_active_impl(&K, act_f, res, y, wsum, r, &Kc, kc_cond, n_active,
-                                    at<int32_t>(L.off_pos), scratch, sb, s));
-      grad_finish<<<mb, tpb, 0, s>>>(o, Jd, wsum, m, op_lambda(), g, rhs, b0());
-      SPSVM_LAUNCH_CHECK();
-      small_dots<<<1, 256, 0, s>>>(beta, o, Jd, g, r, m, dots, b0());
-      SPSVM_LAUNCH_CHECK();
-      return SPSVM_OK;
+    // active set is unchanged), gradient and the dots of the stopping test;
+    // with `step`, the step to those flags and residuals first.
+    unsigned* done_dev = reinterpret_cast<unsigned*>(small + 216);
+    SPSVM_CUDA_TRY(cudaMemsetAsync(done_dev, 0, sizeof(*done_dev), s));
+    auto grad_pass = [&](uint8_t* act_f, const unsigned long long* kc_cond, const StepArgs* step) -> int {
+      if (!step) {
+        sub_kernel<<<grid_for(n, tpb), tpb, 0, s>>>(o, y, n, res);
+        SPSVM_LAUNCH_CHECK();
+      }
+      const GradArgs grad{o, Jd, op_lambda(), beta, b0(), g, rhs, dots, done_dev};
+      return compact_active_impl(&K, act_f, res, y, wsum, r, &Kc, kc_cond, n_active,
+                                 at<int32_t>(L.off_pos), scratch, sb, s, step, &grad);
     };
     // the small area's layout, read back in one copy after each step:
     // [0, 24) loss / errors / |S|, [96, 104) changed flags, [128, 152) dots,
@@ -557,21 +483,10 @@ struct Fit {
     // leaves beta and o as they were and the rest recomputes the same values.
     auto search_and_step = [&](double* t_out) -> int {
       SPSVM_TRY(line_search_async(o, u, y, n, dir, Jd, m, lambda, t_dev, ls_err, scratch, sb, s, b0()));
-      axpy_t<<<mb, tpb, 0, s>>>(beta, dir, t_dev, m);
-      SPSVM_LAUNCH_CHECK();
-      update_o_t<<<grid_for(n, tpb), tpb, 0, s>>>(o, u, t_dev, n);
-      SPSVM_LAUNCH_CHECK();
-      const int nxt = act_cur ^ 1;
-      {
-        spsvm_kmat Kf = kmat();
-        SPSVM_TRY(spsvm_outputs(&Kf, nullptr, y, o, at<uint8_t>(nxt ? L.off_act1 : L.off_act0),
-                                at<double>(L.off_small), scratch, sb, s));
-      }
-      SPSVM_CUDA_TRY(cudaMemsetAsync(ndiff, 0, sizeof(*ndiff), s));
-      count_diff<<<grid_for(n, tpb), tpb, 0, s>>>(at<uint8_t>(L.off_act0), at<uint8_t>(L.off_act1),
-                                                  n, ndiff);
-      SPSVM_LAUNCH_CHECK();
-      SPSVM_TRY(grad_pass(at<uint8_t>(nxt ? L.off_act1 : L.off_act0), ndiff));
+      uint8_t* after = at<uint8_t>(act_cur ? L.off_act0 : L.off_act1);
+      const StepArgs step{t_dev, beta, dir, m, o, u, y, after, at<uint8_t>(act_cur ? L.off_act1 : L.off_act0),
+                          res, at<double>(L.off_small), ndiff};
+      SPSVM_TRY(grad_pass(after, ndiff, &step));
       alignas(8) unsigned char sm_h[kSmallRead];
       SPSVM_TRY(read(sm_h, small, kSmallRead));
       int32_t err = 0;
@@ -583,7 +498,7 @@ struct Fit {
       std::memcpy(t_out, sm_h + 200, sizeof(double));
       return SPSVM_OK;
     };
-    SPSVM_TRY(grad_pass(at<uint8_t>(act_cur ? L.off_act1 : L.off_act0), nullptr));
+    SPSVM_TRY(grad_pass(at<uint8_t>(act_cur ? L.off_act1 : L.off_act0), nullptr, nullptr));
     SPSVM_TRY(read(dh, dots, sizeof(dh)));
     for (int it = 0; it < op.max_newton; ++it) {
       uint8_t* act = at<uint8_t>(act_cur ? L.off_act1 : L.off_act0);

@@ -218,62 +218,234 @@ __global__ void scan_count(const uint8_t* __restrict__ active, const uint8_t* __
   if (threadIdx.x == 0) counts[blockIdx.x] = c;
 }
 
-// Exclusive scan of block counts in one block; writes the total to *total.
-__global__ void scan_blocks(int32_t* __restrict__ counts, int64_t nb, int64_t* __restrict__ total) {
-  __shared__ int32_t sh[1024];
-  __shared__ int64_t carry;
-  if (threadIdx.x == 0) carry = 0;
+// What a block of step_points leaves beside its count of active points.
+struct StepPart {
+  double loss;
+  int32_t err, diff;
+};
+
+// The step of StepArgs over SC_PTS points per block, with the block's count
+// for the scan.  Latency bound: one launch where the updates of beta and o, the
+// flags, their count, the count of changes and the residuals took seven.  FP64
+// would take longer than the rest (64 cycles an instruction and warp): o + t u
+// and the loss are FP32 pairs, about 2^-46 before their last rounding.
+__global__ void __launch_bounds__(SC_T) step_points(StepArgs a, int64_t n, int32_t* __restrict__ counts,
+                                                    StepPart* __restrict__ part) {
+  __shared__ float2 shl[SC_T / 32];
+  __shared__ int shc[SC_T / 32], she[SC_T / 32], shd[SC_T / 32];
+  constexpr int P = SC_PTS / SC_T;
+  const int64_t base = (int64_t)blockIdx.x * SC_PTS + threadIdx.x;
+  const double t = *a.t;
+  float ov[P], uv[P], yv[P];
+  uint8_t bv[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) {   // all in flight together with t
+    const int64_t i = min64(n - 1, base + (int64_t)SC_T * p);
+    ov[p] = a.o[i];
+    uv[p] = a.u[i];
+    yv[p] = a.y[i];
+    bv[p] = a.before[i];
+  }
+  const float th = (float)t, tl = (float)(t - (double)th);
+  float hi = 0.f, lo = 0.f;
+  int c = 0, err = 0, diff = 0;
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int64_t i = base + (int64_t)SC_T * p;
+    if (i >= n) break;
+    float oi = ov[p];
+    const float yi = yv[p];
+    if (t != 0.0) {
+      const float ui = uv[p];
+      const float q = __fmul_rn(th, ui);
+      const float s = __fadd_rn(oi, q);
+      const float b = __fsub_rn(s, oi);
+      const float e = __fadd_rn(__fsub_rn(oi, __fsub_rn(s, b)), __fsub_rn(q, b));
+      const float f = __fmaf_rn(tl, ui, __fmaf_rn(th, ui, -q));
+      oi = __fsub_rn(s, s) == 0.0f ? __fadd_rn(s, __fadd_rn(e, f)) : s;
+      a.o[i] = oi;
+    }
+    const float margin = yi * oi;
+    const bool act = margin < 1.0f;
+    c += act;
+    err += margin <= 0.0f;
+    diff += (bv[p] != 0) != act;
+    a.active[i] = act ? 1 : 0;
+    a.res[i] = oi - yi;
+    if (act) {   // (1 - margin)^2, 1 - margin exact as a pair
+      const float x = __fsub_rn(1.0f, margin);
+      const float b = __fsub_rn(x, 1.0f);
+      const float e = __fadd_rn(__fsub_rn(1.0f, __fsub_rn(x, b)), -__fadd_rn(margin, b));
+      lo = __fmaf_rn(2.0f * x, e, lo);
+      pair_add_sq(hi, lo, x);
+    }
+  }
+  if (t != 0.0)
+    for (int64_t k = (int64_t)blockIdx.x * SC_T + threadIdx.x; k < a.m; k += (int64_t)gridDim.x * SC_T)
+      a.beta[k] += t * a.dir[k];
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, hi, q), ol = __shfl_xor_sync(0xffffffffu, lo, q);
+    pair_add(hi, lo, make_float2(oh, ol));
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  err = __reduce_add_sync(0xffffffffu, err);
+  diff = __reduce_add_sync(0xffffffffu, diff);
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    shl[w] = make_float2(hi, lo);
+    shc[w] = c;
+    she[w] = err;
+    shd[w] = diff;
+  }
   __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < SC_T / 32; ++k) {
+    pair_add(hi, lo, shl[k]);
+    c += shc[k];
+    err += she[k];
+    diff += shd[k];
+  }
+  counts[blockIdx.x] = c;
+  part[blockIdx.x] = StepPart{0.5 * pair_value(hi, lo), err, diff};
+}
+
+// Sums of the blocks' parts, in a fixed order (all threads of one block).
+__device__ void step_sums(const StepPart* __restrict__ part, int64_t nb, int64_t total,
+                          double* __restrict__ stats, unsigned long long* __restrict__ ndiff) {
+  __shared__ double shs[32];
+  __shared__ int shi[32];
+  double loss = 0.0;
+  int err = 0, diff = 0;
+  for (int64_t b = threadIdx.x; b < nb; b += blockDim.x) {
+    loss += part[b].loss;
+    err += part[b].err;
+    diff += part[b].diff;
+  }
+  loss = block_sum(loss, shs);
+  err = block_sum(err, shi);
+  diff = block_sum(diff, shi);
+  if (threadIdx.x == 0) {
+    stats[0] = loss;
+    stats[1] = (double)err;
+    stats[2] = (double)total;
+    *ndiff = (unsigned long long)diff;
+  }
+}
+
+// v summed over the threads before this one, by warps; *total: over the block.
+__device__ __forceinline__ int32_t block_scan(int32_t v, int32_t* __restrict__ sh /* 32 */, int32_t* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  __syncthreads();
+  if (lane == 31) sh[w] = x;
+  __syncthreads();
+  int32_t before = 0, all = 0;
+  for (int k = 0; k < (int)blockDim.x >> 5; ++k) {
+    if (k < w) before += sh[k];
+    all += sh[k];
+  }
+  *total = all;
+  return before + x - v;
+}
+
+// Exclusive scan of block counts in one block; writes the total to *total.
+__global__ void scan_blocks(int32_t* __restrict__ counts, int64_t nb, int64_t* __restrict__ total,
+                            const StepPart* __restrict__ part, double* __restrict__ stats,
+                            unsigned long long* __restrict__ ndiff) {
+  __shared__ int32_t sh[32];
+  int64_t carry = 0;
   for (int64_t b0 = 0; b0 < nb; b0 += blockDim.x) {
     const int64_t b = b0 + threadIdx.x;
     const int32_t v = (b < nb) ? counts[b] : 0;
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-      int32_t add = (threadIdx.x >= (unsigned)off) ? sh[threadIdx.x - off] : 0;
-      __syncthreads();
-      sh[threadIdx.x] += add;
-      __syncthreads();
-    }
-    const int32_t incl = sh[threadIdx.x];
-    if (b < nb) counts[b] = (int32_t)(carry + incl - v);
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry += incl;
-    __syncthreads();
+    int32_t sum;
+    const int32_t excl = block_scan(v, sh, &sum);
+    if (b < nb) counts[b] = (int32_t)(carry + excl);
+    carry += sum;
   }
   if (threadIdx.x == 0) *total = carry;
+  if (part) step_sums(part, nb, carry, stats, ndiff);
 }
 
-__global__ void scan_write(const uint8_t* __restrict__ active, const uint8_t* __restrict__ ref,
-                           int64_t n, const int32_t* __restrict__ offsets, int32_t* __restrict__ pos,
-                           int32_t* __restrict__ list) {
-  __shared__ int32_t sh[SC_PTS];
-  const int64_t base = (int64_t)blockIdx.x * SC_PTS;
+// Positions and the list of the flagged points.  SUM: counts are the blocks'
+// own, which every block sums up to its place itself (up to SC_SUM of them: a
+// launch less), and block 0 writes the total and the step's sums; else they
+// are scanned.
+constexpr int64_t SC_SUM = 1024;
+template <bool SUM>
+__global__ void __launch_bounds__(SC_T) scan_write(const uint8_t* __restrict__ active,
+                                                   const uint8_t* __restrict__ ref, int64_t n,
+                                                   const int32_t* __restrict__ counts,
+                                                   int32_t* __restrict__ pos, int32_t* __restrict__ list,
+                                                   int64_t* __restrict__ total,
+                                                   const StepPart* __restrict__ part,
+                                                   double* __restrict__ stats,
+                                                   unsigned long long* __restrict__ ndiff) {
+  __shared__ int32_t sh[32];
+  __shared__ int32_t off_s;
+  const int64_t i0 = (int64_t)blockIdx.x * SC_PTS + threadIdx.x * 4;
+  int32_t f[4], run = 0, first = 0;
+#pragma unroll
   for (int p = 0; p < 4; ++p) {
-    const int64_t i = base + threadIdx.x * 4 + p;
-    sh[threadIdx.x * 4 + p] = (i < n) ? scan_flag(active, ref, i) : 0;
+    f[p] = i0 + p < n ? scan_flag(active, ref, i0 + p) : 0;
+    run += f[p];
   }
-  __syncthreads();
-  // sequential scan per thread over its 4, then block scan of thread sums
-  int32_t local[4], run = 0;
-  for (int p = 0; p < 4; ++p) { local[p] = run; run += sh[threadIdx.x * 4 + p]; }
-  __shared__ int32_t ts[SC_T];
-  ts[threadIdx.x] = run;
-  __syncthreads();
-  for (int off = 1; off < SC_T; off <<= 1) {
-    int32_t add = (threadIdx.x >= (unsigned)off) ? ts[threadIdx.x - off] : 0;
+  if (SUM) {
+    int32_t c = 0;
+    const int64_t end = blockIdx.x ? blockIdx.x : gridDim.x;   // block 0: the total
+    for (int64_t b = threadIdx.x; b < end; b += SC_T) c += counts[b];
+    c = block_sum(c, sh);
+    if (threadIdx.x == 0) off_s = c;
     __syncthreads();
-    ts[threadIdx.x] += add;
-    __syncthreads();
-  }
-  const int32_t excl = ts[threadIdx.x] - run + offsets[blockIdx.x];
-  for (int p = 0; p < 4; ++p) {
-    const int64_t i = base + threadIdx.x * 4 + p;
-    if (i < n) {
-      if (pos) pos[i] = excl + local[p];
-      if (sh[threadIdx.x * 4 + p]) list[excl + local[p]] = (int32_t)i;   // flagged indices, in order
+    first = off_s;
+    if (blockIdx.x == 0) {
+      if (threadIdx.x == 0) *total = first;
+      if (part) step_sums(part, gridDim.x, first, stats, ndiff);
+      first = 0;
     }
+  } else {
+    first = counts[blockIdx.x];
   }
+  int32_t sum;
+  int32_t at = first + block_scan(run, sh, &sum);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int64_t i = i0 + p;
+    if (i >= n) break;
+    if (pos) pos[i] = at;
+    if (f[p]) list[at] = (int32_t)i;   // flagged indices, in order
+    at += f[p];
+  }
+}
+
+// Positions, list and count of the flagged points; with `step`, the step first
+// and its sums.  The step's parts take `room` (the compaction's partials,
+// written later) while block 0 reads them beside the list's writers, else the
+// list's space.
+int launch_scan(const uint8_t* active, const uint8_t* ref, int64_t n, int32_t* counts, int32_t* pos,
+                int32_t* list, int64_t* total, const StepArgs* step, void* room, cudaStream_t s) {
+  const int64_t sb = ceil_div(n, (int64_t)SC_PTS);
+  StepPart* part = step ? static_cast<StepPart*>(sb <= SC_SUM ? room : list) : nullptr;
+  double* stats = step ? step->stats : nullptr;
+  unsigned long long* ndiff = step ? step->ndiff : nullptr;
+  if (step) step_points<<<(unsigned)sb, SC_T, 0, s>>>(*step, n, counts, part);
+  else scan_count<<<(unsigned)sb, SC_T, 0, s>>>(active, ref, n, counts);
+  SPSVM_LAUNCH_CHECK();
+  if (sb <= SC_SUM) {
+    scan_write<true><<<(unsigned)sb, SC_T, 0, s>>>(active, ref, n, counts, pos, list, total, part, stats, ndiff);
+    SPSVM_LAUNCH_CHECK();
+    return SPSVM_OK;
+  }
+  scan_blocks<<<1, 1024, 0, s>>>(counts, sb, total, part, stats, ndiff);
+  SPSVM_LAUNCH_CHECK();
+  scan_write<false><<<(unsigned)sb, SC_T, 0, s>>>(active, ref, n, counts, pos, list, total, nullptr, nullptr, nullptr);
+  SPSVM_LAUNCH_CHECK();
+  return SPSVM_OK;
 }
 
 // ---- compaction + masked transposed products ---------------------------
@@ -468,21 +640,74 @@ __global__ void __launch_bounds__(CP_T, 3) compact_kernel(
     reinterpret_cast<double*>(part + (int64_t)blockIdx.y * rows + j0 + (k >> 1))[k & 1] = tot;
 }
 
-// Sums the slices' partials in order.
-__global__ void compact_finish(const double2* __restrict__ part, int64_t slices, int64_t rows,
-                               double* w1out, double* w2out, const int64_t* __restrict__ ns_dev) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= rows) return;
+// Sums of the slices' partials, 32 rows a block, eight threads a row that take
+// every eighth slice; with `grad`, the gradient's entries of these rows and,
+// in the block that ends last, the three dots (blocks' parts in order).
+constexpr int CF_G = 8;
+__global__ void __launch_bounds__(32 * CF_G) compact_finish(const double2* __restrict__ part, int64_t slices,
+                                                            int64_t rows, double* w1out, double* w2out,
+                                                            const int64_t* __restrict__ ns_dev, GradArgs grad,
+                                                            double* __restrict__ dpart) {
+  __shared__ double2 sh[CF_G][32];
+  __shared__ bool last_s;
+  const int c = threadIdx.x & 31, q = threadIdx.x >> 5;
+  const int64_t j = (int64_t)blockIdx.x * 32 + c;
   const int64_t ns = *ns_dev;
+  double r = 0.0, be = 0.0;   // read ahead of the sums
+  if (grad.g && q == 0 && j < rows) {
+    const int64_t k = grad.J[j];
+    r = k < 0 ? 0.0 : (double)grad.o[k] - (grad.b0 ? *grad.b0 : 0.0);
+    be = grad.beta[j];
+  }
   const int64_t used = max64(1, ceil_div(ns, cp_slice(ns, slices)));
   double a = 0.0, b = 0.0;
-  for (int64_t s = 0; s < used; ++s) {
-    const double2 p = part[s * rows + j];
-    a += p.x;
-    b += p.y;
+  if (j < rows)
+    for (int64_t s = q; s < used; s += CF_G) {
+      const double2 p = part[s * rows + j];
+      a += p.x;
+      b += p.y;
+    }
+  sh[q][c] = make_double2(a, b);
+  __syncthreads();
+  if (q != 0) return;
+#pragma unroll
+  for (int k = 1; k < CF_G; ++k) {
+    a += sh[k][c].x;
+    b += sh[k][c].y;
   }
-  if (w1out) w1out[j] = a;
-  if (w2out) w2out[j] = b;
+  double x = 0.0, g = 0.0;
+  if (j < rows) {
+    if (w1out) w1out[j] = a;
+    if (w2out) w2out[j] = b;
+    if (grad.g) {
+      g = grad.lambda * r + a;
+      grad.g[j] = g;
+      grad.rhs[j] = -g;
+      x = be * r;
+    }
+  }
+  if (!grad.g) return;
+  const double d0 = warp_sum(x), d1 = warp_sum(g * g), d2 = warp_sum(j < rows ? b * b : 0.0);
+  if (c == 0) {
+    double* d = dpart + 3 * blockIdx.x;
+    d[0] = d0;
+    d[1] = d1;
+    d[2] = d2;
+    __threadfence();
+    last_s = atomicInc(grad.done, gridDim.x - 1) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncwarp();
+  if (!last_s) return;
+  double t[3] = {0.0, 0.0, 0.0};
+  for (int64_t k = c; k < gridDim.x; k += 32)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) t[e] += __ldcg(dpart + 3 * k + e);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    t[e] = warp_sum(t[e]);
+    if (c == 0) grad.dots[e] = t[e];
+  }
 }
 
 // Wt[j][r] = K[j][list[r]] for the k = *k_dev listed points (nothing when
@@ -622,7 +847,8 @@ extern "C" int spsvm_compact_active(const spsvm_kmat* K, const uint8_t* active, 
 int spsvm::compact_active_impl(const spsvm_kmat* K, const uint8_t* active, const float* w1,
                                const float* w2, double* w1out, double* w2out, spsvm_kmat* Kc,
                                const unsigned long long* kc_cond, int64_t* n_active,
-                               int32_t* pos, void* scratch, size_t scratch_bytes, void* stream) {
+                               int32_t* pos, void* scratch, size_t scratch_bytes, void* stream,
+                               const StepArgs* step, const GradArgs* grad) {
   SPSVM_TRY(check_kmat(K, "compact"));
   if (!active || !n_active || !pos) return set_error(SPSVM_ERR_ARG, "compact: NULL pointer");
   if (Kc) {
@@ -648,12 +874,7 @@ int spsvm::compact_active_impl(const spsvm_kmat* K, const uint8_t* active, const
   if (n == 0) {
     SPSVM_CUDA_TRY(cudaMemsetAsync(n_active, 0, sizeof(int64_t), s));
   } else {
-    scan_count<<<(unsigned)sb, SC_T, 0, s>>>(active, nullptr, n, counts);
-    SPSVM_LAUNCH_CHECK();
-    scan_blocks<<<1, 1024, 0, s>>>(counts, sb, n_active);
-    SPSVM_LAUNCH_CHECK();
-    scan_write<<<(unsigned)sb, SC_T, 0, s>>>(active, nullptr, n, counts, pos, list);
-    SPSVM_LAUNCH_CHECK();
+    SPSVM_TRY(launch_scan(active, nullptr, n, counts, pos, list, n_active, step, part, s));
   }
   if (K->rows > 0 && n > 0) {
     const int64_t slices = compact_slices(n, K->rows);
@@ -671,8 +892,10 @@ int spsvm::compact_active_impl(const spsvm_kmat* K, const uint8_t* active, const
                                              kc_cond, s);
     SPSVM_LAUNCH_CHECK();
     if (w1out || w2out) {
-      compact_finish<<<(unsigned)ceil_div(K->rows, 256), 256, 0, s>>>(part, slices, K->rows, w1out,
-                                                                      w2out, n_active);
+      // (the list has been read: its space takes the blocks' dots)
+      compact_finish<<<(unsigned)ceil_div(K->rows, (int64_t)32), 32 * CF_G, 0, s>>>(
+          part, slices, K->rows, w1out, w2out, n_active, grad ? *grad : GradArgs{},
+          reinterpret_cast<double*>(list));
       SPSVM_LAUNCH_CHECK();
     }
   } else if (K->rows > 0) {
@@ -703,12 +926,7 @@ extern "C" int spsvm_active_diff(const spsvm_kmat* K, const uint8_t* active, con
   const int64_t ysplit_max = ceil_div(n, CP_T) < 1024 ? ceil_div(n, CP_T) : 1024;
   int32_t* list = reinterpret_cast<int32_t*>(
       static_cast<char*>(scratch) + round_up(sb * 4, 256) + round_up(ysplit_max * 16, 256));
-  scan_count<<<(unsigned)sb, SC_T, 0, s>>>(active, ref, n, counts);
-  SPSVM_LAUNCH_CHECK();
-  scan_blocks<<<1, 1024, 0, s>>>(counts, sb, total);
-  SPSVM_LAUNCH_CHECK();
-  scan_write<<<(unsigned)sb, SC_T, 0, s>>>(active, ref, n, counts, nullptr, list);
-  SPSVM_LAUNCH_CHECK();
+  SPSVM_TRY(launch_scan(active, ref, n, counts, nullptr, list, total, nullptr, nullptr, s));
   store_count<<<1, 1, 0, s>>>(total, k_dev);
   SPSVM_LAUNCH_CHECK();
   if (kmax > 0 && K->rows > 0) {

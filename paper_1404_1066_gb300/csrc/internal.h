@@ -260,11 +260,46 @@ int solve_mixed_after_factor(const double* H, int64_t m, int64_t ldh, double shi
                              void* work, size_t work_bytes, const int32_t* factor_info,
                              void* stream);
 
+// A Newton step taken on the way into the compaction: with the step length t
+// (device; 0: none) beta += t dir, o += t u, and from the new outputs the
+// active flags, the residuals o - y, stats as of spsvm_outputs and the count
+// of flags that differ from `before`.
+struct StepArgs {
+  const double* t;
+  double* beta;
+  const double* dir;
+  int32_t m;
+  float* o;
+  const float* u;
+  const float* y;
+  uint8_t* active;
+  const uint8_t* before;
+  float* res;
+  double* stats;               // [3]
+  unsigned long long* ndiff;
+};
+// The gradient from the compaction's sums w1out, w2out: g = lambda K_JJ beta +
+// w1out, rhs = -g, dots = {beta' K_JJ beta, |g|^2, |w2out|^2}, with K_JJ beta
+// read from o at the basis points J (< 0: the bias slot, whose row is zero;
+// *b0, if given, is the bias in o).  *done is zero before and after.
+struct GradArgs {
+  const float* o;
+  const int64_t* J;
+  double lambda;
+  const double* beta;
+  const double* b0;
+  double *g, *rhs, *dots;
+  unsigned* done;
+};
+
 // spsvm_compact_active whose K_SJ copy is written only when *kc_cond (read
-// on the device) is nonzero; kc_cond NULL: always.
+// on the device) is nonzero; kc_cond NULL: always.  With `step`, the step
+// comes first (active, w1 and kc_cond being its results), with `grad` the
+// gradient last (w1out and w2out given, and at least one row and point).
 int compact_active_impl(const spsvm_kmat* K, const uint8_t* active, const float* w1,
                         const float* w2, double* w1out, double* w2out, spsvm_kmat* Kc,
                         const unsigned long long* kc_cond, int64_t* n_active, int32_t* pos,
-                        void* scratch, size_t scratch_bytes, void* stream);
+                        void* scratch, size_t scratch_bytes, void* stream,
+                        const StepArgs* step = nullptr, const GradArgs* grad = nullptr);
 
 }  // namespace spsvm

@@ -202,6 +202,31 @@ def test_split_decision_sums_in_pairs(sp):
     assert np.all(np.abs(f - K @ beta) <= 1e6 * K.sum(1) * 8 * 2.0 ** -24)
 
 
+# 1,024 points a block of the step and the scan, which sum up to 1,024 blocks'
+# counts by themselves
+@pytest.mark.parametrize("n", [5, 1024, 1025, 1_048_577])
+def test_step_stats_and_scan(sp, n):
+    """A fit's last record against its outputs: counts exact, the loss (FP32
+    pairs of exact terms) to 1e-10; the compaction's positions and count."""
+    g = np.random.default_rng(n)
+    X = g.standard_normal((n, 2)).astype(np.float32)
+    y = np.where(X[:, 0] + 0.7 * g.standard_normal(n) > 0, 1.0, -1.0).astype(np.float32)
+    J = g.choice(n, 3, replace=False)
+    mdl = sp.spsvm_fit(_t(X), _t(y), 0.8, 0.1, 3, 1e-8, precision="fp32", initial_basis=J, fixed_basis=True)
+    o = mdl.outputs(n).astype(np.float64)
+    last = mdl.history()[-1]
+    S = y * o < 1
+    assert len(mdl.history()) > 1 and last["active"] == S.sum() and last["errors"] == (y * o <= 0).sum()
+    loss = 0.5 * ((1 - y * o)[S] ** 2).sum()
+    assert abs(last["loss"] - loss) <= 1e-10 * loss
+
+    km, _ = _kmat(sp, np.zeros((1, n)), "fp32")
+    kc, _ = _kmat(sp, np.zeros((1, km.ld)), "fp32")
+    _, _, count, pos = sp.spsvm_compact_active(km, _t(S.astype(np.uint8)), None, None, kc)
+    assert int(count.item()) == S.sum()
+    np.testing.assert_array_equal(pos.cpu().numpy(), np.cumsum(S) - S)
+
+
 # FP32: 64 x 32 or 64 x 128 tiles, split form: 256 x 256 tiles of CTA pairs;
 # points in splits of at least 128, FP32 sums of 2,048 (8,192) points
 @pytest.mark.parametrize("prec,kfmt", [("fp32", "fp32"), ("fp32", "bf16split"), ("bf16split", "bf16split")])
