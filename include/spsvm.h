@@ -106,7 +106,7 @@ typedef struct spsvm_kmat {
 typedef struct spsvm_points {
   const float* X;   /* device, n x d row-major, leading dimension ldx */
   int64_t n, d, ldx;
-  float*    norms;  /* device, n: ||x_i||^2 (FP64 accumulation, rounded) */
+  float*    norms;  /* device, n: ||x_i||^2 (summed to about 2^-46, rounded) */
   uint16_t* hi;     /* device, n x ldh, or NULL for SPSVM_FP32 */
   uint16_t* lo;     /* device, n x ldh, or NULL */
   int64_t   ldh;    /* multiple of 64, >= d */
@@ -261,7 +261,8 @@ int spsvm_active_diff(const spsvm_kmat* K, const uint8_t* active, const uint8_t*
  *   H = lambda * K_JJ + Kc^T Kc,   Kc = K_SJ (compacted, rows = basis),
  * where K_JJ[a][b] = K row b at column J[a] (symmetrised).  The
  * contraction over the first ns columns of Kc runs in `precision` with FP32
- * partial sums per slice of 8192 points, combined in FP64.  H: device FP64,
+ * partial sums per slice of 8192 points (SPSVM_FP32: 2048), combined as
+ * compensated pairs.  H: device FP64,
  * m x m, leading dimension ldh, both triangles written.  J: device int64, m.
  * scratch: spsvm_gram_scratch_bytes(m, ns). */
 size_t spsvm_gram_scratch_bytes(int64_t m, int64_t ns);

@@ -454,8 +454,10 @@ int launch_scan(const uint8_t* active, const uint8_t* ref, int64_t n, int32_t* c
 // step through the list of active indices, so every lane carries an active
 // point whatever their density, a row's reads cover a contiguous stretch of
 // K (16 loads in flight per lane) and its writes are whole 128-byte lines.
-// The weighted sums are FP32 over 32 terms, then a compensated pair, and one
-// FP64 reduction per warp.  Bound by HBM: at n = 200,000, 2,048 rows, 43%
+// The weighted sums are compensated pairs: of every product, its rounding
+// included, in short slices (a chain of latencies, where that costs nothing;
+// the gradient of a small fit is as accurate as these sums), else of FP32 sums
+// of eight terms (of 32: 387 us below as well).  One FP64 reduction per warp.  Bound by HBM: at n = 200,000, 2,048 rows, 43%
 // active (1.64 GB read, 0.70 GB written) 0.38 ms, 6.1 TB/s; a thread per point
 // of every row, 57% of them idle, with two-byte writes took 3.36 ms.
 constexpr int CP_T = 256;
@@ -463,7 +465,8 @@ constexpr int CP_WARPS = CP_T / 32;
 constexpr int CP_R = 4;                      // basis rows per warp
 constexpr int CP_ROWS = CP_WARPS * CP_R;     // basis rows per block
 constexpr int CP_Q = 128;                    // compact columns per step
-constexpr int CP_CHUNK = 8;                  // steps summed in FP32 (4 terms each)
+constexpr int CP_CHUNK = 2;                  // steps summed in FP32 (4 terms each)
+constexpr int64_t CP_FINE = 2048;            // columns of a short slice
 constexpr int64_t CP_MIN_SLICE = 1024;       // points per slice that pay its epilogue
 
 // Columns per slice of the compact matrix for ns active points.
@@ -522,6 +525,7 @@ __global__ void __launch_bounds__(CP_T, 3) compact_kernel(
 #pragma unroll
   for (int r = 0; r < CP_R; ++r) f1[r] = f2[r] = h1[r] = h2[r] = l1[r] = l2[r] = 0.f;
   int since = 0;
+  const bool fine = per <= CP_FINE;
   // the next step's indices are read a step ahead (K's loads wait for them)
   int32_t nxt[4];
   auto indices = [&](int64_t q0) {
@@ -567,8 +571,16 @@ __global__ void __launch_bounds__(CP_T, 3) compact_kernel(
         for (int p = 0; p < 4; ++p) v[r][p] = bf_lo(raw[r][p]) + bf_hi(raw[r][p]);
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
-        f1[r] = fmaf(a[p], v[r][p], f1[r]);
-        f2[r] = fmaf(c[p], v[r][p], f2[r]);
+        if (fine) {
+          const float p1 = __fmul_rn(a[p], v[r][p]), p2 = __fmul_rn(c[p], v[r][p]);
+          l1[r] = __fadd_rn(l1[r], __fmaf_rn(a[p], v[r][p], -p1));
+          l2[r] = __fadd_rn(l2[r], __fmaf_rn(c[p], v[r][p], -p2));
+          pair_add(h1[r], l1[r], p1);
+          pair_add(h2[r], l2[r], p2);
+        } else {
+          f1[r] = fmaf(a[p], v[r][p], f1[r]);
+          f2[r] = fmaf(c[p], v[r][p], f2[r]);
+        }
       }
       if (kc_data && j0 + r < rows) {
 #pragma unroll

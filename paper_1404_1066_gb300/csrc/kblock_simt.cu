@@ -290,12 +290,12 @@ namespace spsvm {
 int launch_score_tc(const spsvm_points* p, const float* y, const float* o, const int64_t* idx,
                     int32_t kappa, float gamma, float4* part, int64_t* parts, void* zbuf,
                     size_t zbytes, cudaStream_t s);
-int64_t score_tc_parts(int64_t n, int32_t kappa);
+int64_t score_tc_parts(int64_t n);
 namespace {
-// partial sums per candidate (of each tile of 128 points in FP32, of each CTA
-// or pair in the tensor-core form), then room for the gathered candidate rows
+// partial sums per candidate (of each tile of 128 points in FP32, at most as
+// many in the tensor-core form), then room for the gathered candidate rows
 size_t score_part_bytes(int64_t n, int32_t kappa) {
-  const int64_t tiles = std::max<int64_t>(ceil_div(n, PT), score_tc_parts(n, kappa));
+  const int64_t tiles = std::max<int64_t>(ceil_div(n, PT), score_tc_parts(n));
   return (size_t)round_up(tiles * (int64_t)kappa * (int64_t)sizeof(float4), 256);
 }
 }  // namespace

@@ -53,8 +53,8 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 //   STORE   rows the points, columns the basis: the FP32 kernel values (a warp
 //           stores 32 consecutive points of a basis row);
 //   SCORE   rows the candidates, columns the points: the score sums, a
-//           thread's own over its columns of all of the CTA's tiles (kernel
-//           values not stored);
+//           thread's own over its columns of all of the CTA's tiles, or per
+//           tile where tiles are few (kernel values not stored);
 //   DECIDE  rows the queries, columns the basis: sums of beta K over 32.
 // Basis and candidate rows are gathered into contiguous planes beforehand.
 //
@@ -78,8 +78,6 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 // candidates, n = 500,000: 130 us (157).  Kernel block of 64 rows, n = 500,000:
 // 76 us, 512 MB at 6.7 TB/s (90 us in tiles of 128 basis rows).
 // ---------------------------------------------------------------------------
-constexpr int64_t kScoreUnits = 160;   // CTAs or pairs of a SCORE launch at most
-
 enum KbMode { KB_STORE_F32 = 0, KB_SCORE = 2, KB_DECIDE = 3 };
 
 constexpr int PK_M = 128;                                  // rows per CTA
@@ -128,7 +126,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
     const float* __restrict__ colnorm, const float* __restrict__ rownorm,
     const int64_t* __restrict__ idx, float gamma, float* __restrict__ out, int64_t ld,
     const float* __restrict__ y,
-    const float* __restrict__ o, float4* __restrict__ part, const double* __restrict__ beta,
+    const float* __restrict__ o, float4* __restrict__ part, int per_tile, const double* __restrict__ beta,
     float* __restrict__ dpart, int64_t ldp, WaitCtx wc) {
   constexpr bool SCORE = MODE == KB_SCORE;
   constexpr bool STORE = MODE == KB_STORE_F32;
@@ -341,7 +339,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
     Pre next = fetch(unit);
     float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);   // SCORE: compensated pairs of this thread's sums
     int flushes = 0;
-    if (SCORE && group == 0)
+    if (SCORE && group == 0 && !per_tile)
       for (int64_t c = rank * PK_M + c_in; c < nrows; c += TL::M) part[unit * nrows + c] = sum;
     int64_t j = 0;
     for (int64_t t = unit; t < T; t += units, ++j) {
@@ -442,7 +440,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
         pair_add(sum.x, sum.y, gs);
         pair_add(sum.z, sum.w, hs);
         const int64_t tn = t + units;   // the next tile's rows are the same: keep the sums
-        if (tn < T) {
+        if (tn < T && !per_tile) {
           int cn;
           int64_t pn;
           tile_coords(tn, nCB, nPT, cn, pn);
@@ -457,9 +455,13 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
           mbar_arrive(&redf[quarter]);
         } else {
           if (!__all_sync(~0u, mbar_wait(&redf[quarter], par, wc.st, 27, wc.lim))) break;
-          float4 all = crow ? part[unit * nrows + c] : sum;
-          pair_add(all.x, all.y, make_float2(sum.x, sum.y));
-          pair_add(all.z, all.w, make_float2(sum.z, sum.w));
+          float4* dst = part + (per_tile ? pt : unit) * nrows + c;
+          float4 all = sum;
+          if (crow && !per_tile) {
+            const float4 r = *dst;
+            pair_add(all.x, all.y, make_float2(r.x, r.y));
+            pair_add(all.z, all.w, make_float2(r.z, r.w));
+          }
 #pragma unroll
           for (int g = 0; g < GROUPS - 1; ++g) {
             const float4 r = red[g * 128 + c_in];
@@ -467,7 +469,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
             pair_add(all.z, all.w, make_float2(r.z, r.w));
           }
           mbar_arrive(&rede[quarter]);
-          if (crow) part[unit * nrows + c] = all;
+          if (crow) *dst = all;
         }
         sum = make_float4(0.f, 0.f, 0.f, 0.f);
       }
@@ -962,8 +964,11 @@ int launch_kb_as(const KbArgs& a, cudaStream_t s) {
   WaitCtx wc;
   SPSVM_TRY(wait_ctx(s, &wc));
   cudaLaunchConfig_t cfg{};
-  int64_t units = max64(1, min64(tiles, (int64_t)sm_count() / W));
-  if (MODE == KB_SCORE) *a.parts = units = min64(units, kScoreUnits);
+  const int64_t units = max64(1, min64(tiles, (int64_t)sm_count() / W));
+  // sums per CTA or pair, unless those outnumber the tiles of points
+  const int64_t col_tiles = ceil_div(a.ncols, (int64_t)N);
+  const int per_tile = MODE == KB_SCORE && units > col_tiles;
+  if (MODE == KB_SCORE) *a.parts = per_tile ? col_tiles : units;
   cfg.gridDim = dim3((unsigned)(W * units));
   cfg.blockDim = dim3(TL::THREADS);
   cfg.dynamicSmemBytes = TL::SMEM;
@@ -975,7 +980,7 @@ int launch_kb_as(const KbArgs& a, cudaStream_t s) {
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   SPSVM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mah, mam, mal, mbh, mbm, mbl, a.ldh, a.ncols, a.nrows,
-                                    a.colnorm, a.rownorm, a.idx, a.gamma, a.out, a.ld, a.y, a.o, a.part,
+                                    a.colnorm, a.rownorm, a.idx, a.gamma, a.out, a.ld, a.y, a.o, a.part, per_tile,
                                     a.beta, a.dpart, a.ldp, wc));
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
@@ -1032,11 +1037,8 @@ int launch_kernel_block_tc(const spsvm_points* p, const int64_t* idx, int32_t m,
   return launch_kb<KB_STORE_F32>(a, s);
 }
 
-// Partial sums per candidate at most: one per CTA or pair of the grid.
-int64_t score_tc_parts(int64_t n, int32_t kappa) {
-  const int64_t rows = kappa > PK_M ? 2 * PK_M : PK_M;
-  return max64(1, min64(ceil_div((int64_t)kappa, rows) * ceil_div(n, (int64_t)128), kScoreUnits));
-}
+// Partial sums per candidate at most.
+int64_t score_tc_parts(int64_t n) { return ceil_div(n, (int64_t)128); }
 
 int launch_score_tc(const spsvm_points* p, const float* y, const float* o, const int64_t* idx,
                     int32_t kappa, float gamma, float4* part, int64_t* parts, void* zbuf,
