@@ -83,7 +83,9 @@ enum KbMode { KB_STORE_F32 = 0, KB_SCORE = 2, KB_DECIDE = 3 };
 constexpr int PK_M = 128;                                  // rows per CTA
 constexpr int PK_KC = 64;                                  // K elements per slot (128-byte rows)
 constexpr int PK_WP = 32;                                  // columns per epilogue warp
-template <bool PAIR, int N>
+// RA: rows of A that a CTA stages (64: the MMAs' other rows are whatever lies
+// behind, and are not read back)
+template <bool PAIR, int N, int RA>
 struct Kb {
   static constexpr int CTAS = PAIR ? 2 : 1;
   static constexpr int M = CTAS * PK_M;                    // rows of a tile
@@ -91,7 +93,7 @@ struct Kb {
   static constexpr int GROUPS = N / PK_WP;
   static constexpr int EPI_WARPS = 4 * GROUPS;
   static constexpr int THREADS = 32 * (2 + EPI_WARPS);
-  static constexpr int PLANE_A = PK_M * PK_KC * 2;
+  static constexpr int PLANE_A = RA * PK_KC * 2;
   static constexpr int SLOT = PLANE_A + ROWS_B * PK_KC * 2;
   static constexpr int SLOTS = 192 * 1024 / SLOT;
   static constexpr int RED_OFF = SLOTS * SLOT;             // SCORE: the groups' sums
@@ -101,28 +103,39 @@ struct Kb {
   static_assert(SMEM <= 227 * 1024, "kernel block shared memory");
   static_assert(8 * (2 * SLOTS + 12) + 12 <= 512, "barriers");
   static_assert(SLOTS >= 6, "two chunks in flight");
+  static_assert(SLOT >= PK_M * PK_KC * 2, "the rows that the MMAs read lie in the slot");
 };
 
-// Tile order: groups of PK_GROUP consecutive column tiles, each group swept
-// over all row blocks with the column tile varying fastest, so the CTAs in
-// flight share their tiles of both operands through L2.
+// Tile order: groups of PK_GROUP consecutive column tiles (STORE: row blocks,
+// so that a basis row's values reach DRAM in runs of PK_GROUP x 1 KB), each
+// group swept over all row blocks (column tiles) with the group's own index
+// varying fastest.  The CTAs in flight share tiles of both operands through L2.
 constexpr int64_t PK_GROUP = 32;
-__device__ __forceinline__ void tile_coords(int64_t t, int64_t nCB, int64_t nPT, int& cb,
-                                            int64_t& pt) {
-  const int64_t per = nCB * PK_GROUP;
-  const int64_t g = t / per, r = t % per;
-  const int64_t g0 = g * PK_GROUP;
-  const int64_t gw = min64(PK_GROUP, nPT - g0);   // the last group may be narrower
-  cb = (int)(r / gw);
-  pt = g0 + r % gw;
+template <int MODE, typename I>
+__device__ __forceinline__ void tile_coords_as(I t, I nCB, I nPT, int& cb, int64_t& pt) {
+  constexpr I G = (I)PK_GROUP;
+  const I grouped = MODE == KB_STORE_F32 ? nCB : nPT, other = MODE == KB_STORE_F32 ? nPT : nCB;
+  const I per = other * G;
+  const I g = t / per, r = t - g * per;
+  const I g0 = g * G;
+  const I gw = grouped - g0 < G ? grouped - g0 : G;   // the last group may be narrower
+  const I a = r / gw, b = g0 + (r - a * gw);
+  cb = (int)(MODE == KB_STORE_F32 ? b : a);
+  pt = (int64_t)(MODE == KB_STORE_F32 ? a : b);
+}
+// (64-bit divisions would take as long as a tile's epilogue)
+template <int MODE>
+__device__ __forceinline__ void tile_coords(int64_t t, int64_t nCB, int64_t nPT, int& cb, int64_t& pt) {
+  if (nCB * nPT < (int64_t)1 << 26) tile_coords_as<MODE, uint32_t>((uint32_t)t, (uint32_t)nCB, (uint32_t)nPT, cb, pt);
+  else tile_coords_as<MODE, int64_t>(t, nCB, nPT, cb, pt);
 }
 
-template <int MODE, bool PAIR, int N>
-__global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
+template <int MODE, bool PAIR, int N, int RA>
+__global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
     const __grid_constant__ CUtensorMap map_ahi, const __grid_constant__ CUtensorMap map_amid,
     const __grid_constant__ CUtensorMap map_alo, const __grid_constant__ CUtensorMap map_bhi,
     const __grid_constant__ CUtensorMap map_bmid, const __grid_constant__ CUtensorMap map_blo,
-    int64_t ldh, int64_t ncols, int64_t nrows,
+    int64_t ldh, int64_t ncols, int64_t nrows, int box_a,
     const float* __restrict__ colnorm, const float* __restrict__ rownorm,
     const int64_t* __restrict__ idx, float gamma, float* __restrict__ out, int64_t ld,
     const float* __restrict__ y,
@@ -131,7 +144,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
   constexpr bool SCORE = MODE == KB_SCORE;
   constexpr bool STORE = MODE == KB_STORE_F32;
   constexpr bool DECIDE = MODE == KB_DECIDE;
-  using TL = Kb<PAIR, N>;
+  using TL = Kb<PAIR, N, RA>;
   constexpr int SLOTS = TL::SLOTS, KC = PK_KC, GROUPS = TL::GROUPS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -213,7 +226,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
       for (int64_t t = unit; t < T && ok; t += units) {
         int cb;
         int64_t pt;
-        tile_coords(t, nCB, nPT, cb, pt);
+        tile_coords<MODE>(t, nCB, nPT, cb, pt);
         const int ra = cb * TL::M + (int)rank * PK_M, rb = (int)(pt * N) + (int)rank * TL::ROWS_B;
         for (int kc = 0; kc < nK && ok; ++kc) {
 #pragma unroll
@@ -224,7 +237,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
               break;
             }
             uint8_t* st = smem + s * TL::SLOT;
-            if (rank == 0) mbar_expect_tx(&full[s], TL::CTAS * TL::SLOT);
+            if (rank == 0) mbar_expect_tx(&full[s], TL::CTAS * (uint32_t)(TL::SLOT - (RA - box_a) * 128));
             if constexpr (PAIR) {
               const uint32_t bar = map_rank(&full[s], 0);
               tma_load_2d_pair(st, ma[p], kc * KC, ra, bar);
@@ -316,15 +329,15 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
     struct Pre {
       float rn, cn, oi, yi;
       double b;
-    };
-    auto fetch = [&](int64_t t) {
-      Pre f{0.f, 0.f, 0.f, 0.f, 0.0};
-      if (t >= T) return f;
       int cb;
       int64_t pt;
-      tile_coords(t, nCB, nPT, cb, pt);
-      const int64_t c = (TL::CTAS * (int64_t)cb + rank) * PK_M + c_in;
-      const int64_t i = pt * N + group * PK_WP + lane;
+    };
+    auto fetch = [&](int64_t t) {
+      Pre f{0.f, 0.f, 0.f, 0.f, 0.0, -1, 0};
+      if (t >= T) return f;
+      tile_coords<MODE>(t, nCB, nPT, f.cb, f.pt);
+      const int64_t c = (TL::CTAS * (int64_t)f.cb + rank) * PK_M + c_in;
+      const int64_t i = f.pt * N + group * PK_WP + lane;
       if (c < nrows) f.rn = rownorm[SCORE ? idx[c] : c];
       if (i < ncols) {
         f.cn = colnorm[STORE ? idx[i] : i];
@@ -343,9 +356,8 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
       for (int64_t c = rank * PK_M + c_in; c < nrows; c += TL::M) part[unit * nrows + c] = sum;
     int64_t j = 0;
     for (int64_t t = unit; t < T; t += units, ++j) {
-      int cb;
-      int64_t pt;
-      tile_coords(t, nCB, nPT, cb, pt);
+      const int cb = next.cb;
+      const int64_t pt = next.pt;
       const int64_t cblock = TL::CTAS * (int64_t)cb + rank;   // this CTA's 128 rows
       const int64_t c = cblock * PK_M + c_in;
       const bool crow = c < nrows;
@@ -439,13 +451,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N>::THREADS, 1) kblock_tc_kernel(
       if (SCORE) {
         pair_add(sum.x, sum.y, gs);
         pair_add(sum.z, sum.w, hs);
-        const int64_t tn = t + units;   // the next tile's rows are the same: keep the sums
-        if (tn < T && !per_tile) {
-          int cn;
-          int64_t pn;
-          tile_coords(tn, nCB, nPT, cn, pn);
-          if (cn == cb) continue;
-        }
+        if (next.cb == cb && !per_tile) continue;   // the next tile's rows are the same: keep the sums
         // the warps of a lane quarter combine their groups of columns, in order
         const uint32_t par = (uint32_t)(flushes & 1);
         ++flushes;
@@ -947,17 +953,19 @@ struct KbArgs {
   int64_t ldp;
 };
 
-template <int MODE, bool PAIR, int N>
+template <int MODE, bool PAIR, int N, int RA = PK_M>
 int launch_kb_as(const KbArgs& a, cudaStream_t s) {
-  using TL = Kb<PAIR, N>;
+  using TL = Kb<PAIR, N, RA>;
   CUtensorMap mah, mam, mal, mbh, mbm, mbl;
-  SPSVM_TRY(make_map(&mah, a.a_hi, a.ldh, a.nrows, a.ldh, PK_M));
-  SPSVM_TRY(make_map(&mam, a.a_mid, a.ldh, a.nrows, a.ldh, PK_M));
-  SPSVM_TRY(make_map(&mal, a.a_lo, a.ldh, a.nrows, a.ldh, PK_M));
+  // few rows: only theirs are loaded
+  const int box_a = PAIR || a.nrows >= RA ? RA : (int)round_up(a.nrows, (int64_t)8);
+  SPSVM_TRY(make_map(&mah, a.a_hi, a.ldh, a.nrows, a.ldh, box_a));
+  SPSVM_TRY(make_map(&mam, a.a_mid, a.ldh, a.nrows, a.ldh, box_a));
+  SPSVM_TRY(make_map(&mal, a.a_lo, a.ldh, a.nrows, a.ldh, box_a));
   SPSVM_TRY(make_map(&mbh, a.b_hi, a.ldh, a.ncols, a.ldh, TL::ROWS_B));
   SPSVM_TRY(make_map(&mbm, a.b_mid, a.ldh, a.ncols, a.ldh, TL::ROWS_B));
   SPSVM_TRY(make_map(&mbl, a.b_lo, a.ldh, a.ncols, a.ldh, TL::ROWS_B));
-  auto kern = kblock_tc_kernel<MODE, PAIR, N>;
+  auto kern = kblock_tc_kernel<MODE, PAIR, N, RA>;
   SPSVM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TL::SMEM));
   constexpr int W = TL::CTAS;
   const int64_t tiles = ceil_div(a.nrows, (int64_t)TL::M) * ceil_div(a.ncols, (int64_t)N);
@@ -979,19 +987,26 @@ int launch_kb_as(const KbArgs& a, cudaStream_t s) {
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  SPSVM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mah, mam, mal, mbh, mbm, mbl, a.ldh, a.ncols, a.nrows,
+  SPSVM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mah, mam, mal, mbh, mbm, mbl, a.ldh, a.ncols, a.nrows, box_a,
                                     a.colnorm, a.rownorm, a.idx, a.gamma, a.out, a.ld, a.y, a.o, a.part, per_tile,
                                     a.beta, a.dpart, a.ldp, wc));
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }
 
-// Pairs once there are rows for both CTAs (fewer fill one CTA, whatever N).
+// Tiles of single CTAs where one wave takes them all, half the latency of a
+// pair's (3,000 points by 200 basis rows, d = 128: 8.5 us against 9.6), else
+// pairs.  Scores of up to 64 candidates stage 64 rows, so more points are in
+// flight (64 candidates, n = 100,000, d = 784: 105 us against 111).
 template <int MODE>
 int launch_kb(const KbArgs& a, cudaStream_t s) {
-  if (a.nrows <= PK_M) return launch_kb_as<MODE, false, 128>(a, s);
-  if (MODE != KB_SCORE && a.ncols <= 64) return launch_kb_as<MODE, true, MODE != KB_SCORE ? 64 : 128>(a, s);
-  return launch_kb_as<MODE, true, 128>(a, s);
+  constexpr int NARROW = MODE == KB_SCORE ? 128 : 64;   // (score columns are the points)
+  const bool narrow = a.ncols <= NARROW;
+  const int64_t tiles = ceil_div(a.nrows, (int64_t)PK_M) * ceil_div(a.ncols, (int64_t)(narrow ? NARROW : 128));
+  if (MODE == KB_SCORE && a.nrows <= 64) return launch_kb_as<MODE, false, 128, MODE == KB_SCORE ? 64 : PK_M>(a, s);
+  if (a.nrows <= PK_M || tiles <= sm_count())
+    return narrow ? launch_kb_as<MODE, false, NARROW>(a, s) : launch_kb_as<MODE, false, 128>(a, s);
+  return narrow ? launch_kb_as<MODE, true, NARROW>(a, s) : launch_kb_as<MODE, true, 128>(a, s);
 }
 
 }  // namespace
