@@ -35,10 +35,12 @@ constexpr int kPerCta = 4 * LT; // points that pay another CTA in the barrier
 constexpr int kMaxPasses = 64;  // the search needs at most 1 + 12 + 13
 constexpr int kOne = 16;        // the first grid's point at t = 1
 
-__constant__ double kFirstGrid[LP] = {
-    0.0,   0.25,  0.5,   0.65, 0.75, 0.82,  0.87, 0.91, 0.94, 0.96, 0.97,
-    0.98,  0.986, 0.991, 0.995, 0.998, 1.0, 1.002, 1.005, 1.009, 1.014, 1.02,
-    1.03,  1.04,  1.06,  1.09, 1.13, 1.18,  1.25, 1.35, 1.5,  1.75, 2.0};
+// The points of every grid are FP32 numbers: the sums are taken there, so a
+// point rounded for them alone would shift the root by up to 2^-24.
+__constant__ float kFirstGrid[LP] = {
+    0.0f,   0.25f,  0.5f,   0.65f, 0.75f, 0.82f,  0.87f, 0.91f, 0.94f, 0.96f, 0.97f,
+    0.98f,  0.986f, 0.991f, 0.995f, 0.998f, 1.0f, 1.002f, 1.005f, 1.009f, 1.014f, 1.02f,
+    1.03f,  1.04f,  1.06f,  1.09f, 1.13f, 1.18f,  1.25f, 1.35f, 1.5f,  1.75f, 2.0f};
 
 // Result of the search (CTA 0 writes it).
 struct LsState {
@@ -312,10 +314,11 @@ __global__ void __launch_bounds__(LT, 1) ls_search(const float* __restrict__ o,
         }
       }
       __syncwarp();
-      // points 0 and LC the ends lo and hi, 1 .. LC - 1 even over [A, B]
+      // points 0 and LC the ends lo and hi, 1 .. LC - 1 even over [A, B],
+      // rounded to FP32 (lo and hi are)
       auto grid = [&](double lo, double hi, double A, double B) {
-        T[lane] = lane == 0 ? lo : A + (B - A) * (1.0 / (LC - 2)) * (lane - 1);
-        if (lane == 31) T[31] = B;
+        T[lane] = lane == 0 ? lo : (double)(float)(A + (B - A) * (1.0 / (LC - 2)) * (lane - 1));
+        if (lane == 31) T[31] = (double)(float)B;
         if (lane == 0) T[LC] = hi;
         aimed = A > lo || B < hi;
       };
