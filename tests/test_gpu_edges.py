@@ -153,7 +153,8 @@ def test_fp32_decision_edges(sp, nq, m, d, pad):
 # features a step; score sums kept over a CTA's tiles of one block of candidates
 @pytest.mark.parametrize("pad", [False, True])
 @pytest.mark.parametrize("n,d,m", [(1, 1, 1), (128, 64, 64), (129, 65, 65), (257, 63, 129), (300, 130, 128),
-                                   (20_000, 33, 64), (40_001, 100, 257), (60_000, 7, 300), (600, 33, 300), (5000, 20, 600)])
+                                   (20_000, 33, 64), (40_001, 100, 257), (60_000, 7, 300), (600, 33, 300), (5000, 20, 600),
+                                   (3000, 9, 2000), (33_000, 12, 1100)])
 def test_split_block_score_and_decision_edges(sp, n, d, m, pad):
     """Kernel values: three dropped products and the norms, and d / 16
     truncating accumulations of the large terms; then sums of at most 32 FP32
