@@ -148,6 +148,11 @@ __global__ void __launch_bounds__(128, 1) oz_trailing(const __grid_constant__ CU
   }
   ok = __syncthreads_and(ok);
   const bool got = __syncthreads_and(mbar_wait(done, 0, wc.st, 102, wc.lim)) && ok;
+  if (!got) {   // a wait gave up: no copy or MMA may be in flight when the block ends
+    if (tid == 0) mbar_wait(full, 0, wc.st, 101, 0);
+    mbar_wait(done, 0, wc.st, 102, 0);
+    __syncwarp();
+  }
   fence_after_sync();
   if (got) {
     const int64_t r = r0 + 32 * warp + lane;

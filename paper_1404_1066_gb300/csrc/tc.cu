@@ -42,6 +42,53 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 }
 
 // ---------------------------------------------------------------------------
+// The end of a block after a wait that gave up.  A block must not end, nor free
+// its TMEM, with copies or MMAs of its own in flight; without a give-up the
+// producers' last wait (for the slots to be consumed) and the epilogue's see to
+// that.  The words lie in shared memory, the same in both CTAs of a pair.
+// ---------------------------------------------------------------------------
+struct Leave {
+  uint32_t gave;      // nonzero: a wait gave up
+  uint32_t left[2];   // slots that each CTA's producer has issued loads for
+};
+template <bool PAIR>
+__device__ __forceinline__ void leave_word(uint32_t* w, uint32_t v) {
+  if constexpr (PAIR) {
+    st_cluster(map_rank(w, 0), v);
+    st_cluster(map_rank(w, 1), v);
+  } else {
+    *(volatile uint32_t*)w = v;
+  }
+}
+// Waits (for a second or so each) for all copies and MMAs issued.  Called by all
+// threads after a barrier behind the roles and before another one.  bytes: what
+// one CTA loads per slot; drain: expects the 32 lanes of warp 1 of the even CTA.
+// Where a pair's producers stopped at different slots, the even one's barrier
+// expects exactly the copies that were issued.
+template <bool PAIR, int SLOTS>
+__device__ __noinline__ void settle(uint64_t* full, uint64_t* drain, const Leave* lv, uint32_t bytes,
+                                    uint32_t rank, int* st) {
+  if (threadIdx.x == 0 && rank == 0) {
+    const uint32_t q0 = lv->left[0], q1 = PAIR ? lv->left[1] : q0;
+    const uint32_t top = q0 > q1 ? q0 : q1;
+    for (uint32_t r = top > SLOTS ? top - SLOTS : 0; r < top; ++r) {
+      uint64_t* bar = &full[r % SLOTS];
+      if (r >= q0) mbar_expect_tx(bar, bytes);
+      else if (r >= q1) mbar_complete_tx(bar, bytes);
+      mbar_wait(bar, (r / SLOTS) & 1, st, 28, 0);
+    }
+  }
+  if (threadIdx.x >> 5 == 1) {
+    if (rank == 0) {
+      if constexpr (PAIR) mma_commit_pair(drain);
+      else mma_commit(drain);
+    }
+    mbar_wait(drain, 0, st, 29, 0);
+  }
+  __syncwarp();
+}
+
+// ---------------------------------------------------------------------------
 // Kernel block / scores / decision values, persistent and warp-specialised:
 // products x.z over tiles of rows (MMA M) by columns (MMA N), both operands
 // streamed by TMA, each FP32 value as three planes (x = hi + mid + lo, exact)
@@ -102,7 +149,7 @@ struct Kb {
   static constexpr int STAGE_OFF = BAR_OFF + 512;          // per epilogue warp: 3 x 32 floats
   static constexpr int SMEM = STAGE_OFF + EPI_WARPS * 3 * PK_WP * 4 + 1024;   // + alignment slack
   static_assert(SMEM <= 227 * 1024, "kernel block shared memory");
-  static_assert(8 * (2 * SLOTS + 12) + 12 <= 512, "barriers");
+  static_assert(8 * (2 * SLOTS + 13) + 12 + sizeof(Leave) <= 512, "barriers");
   static_assert(SLOTS >= 6, "two chunks in flight");
   static_assert(SLOT >= PK_M * PK_KC * 2, "the rows that the MMAs read lie in the slot");
 };
@@ -162,8 +209,10 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
   uint64_t* tempty = tfull + 2;
   uint64_t* redf = tempty + 2;   // per lane quarter: the groups' sums written
   uint64_t* rede = redf + 4;     // per lane quarter: the groups' sums consumed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rede + 4);
+  uint64_t* drain = rede + 4;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   uint32_t* bad = tmem_slot + 1;   // [2], PAIR: a wait had given up before, as each CTA saw it
+  Leave* leave = reinterpret_cast<Leave*>(bad + 2);
   float4* red = reinterpret_cast<float4*>(smem + TL::RED_OFF);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -191,6 +240,8 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
       mbar_init(&redf[qd], 32 * (GROUPS - 1));
       mbar_init(&rede[qd], 32);
     }
+    mbar_init(drain, 32);
+    *leave = Leave{0u, {0u, 0u}};
     fence_barrier_init();
     prefetch_tmap(&map_ahi);
     prefetch_tmap(&map_amid);
@@ -220,9 +271,19 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
   }
   fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  // for a barrier that threads or MMAs of the other CTA may complete
+  auto note = [&](bool ok) {   // every wait's outcome goes through this
+    if (!ok) leave_word<PAIR>(&leave->gave, 1u);
+    return ok;
+  };
+  // for a barrier that threads or MMAs of the other CTA may complete; the
+  // producer's acquires, what follows it writes over what the MMAs read
   auto wait = [&](uint64_t* bar, uint32_t parity, int code) {
-    return PAIR ? mbar_wait_cluster(bar, parity, wc.st, code, wc.lim) : mbar_wait(bar, parity, wc.st, code, wc.lim);
+    return note(PAIR ? mbar_wait_cluster<false>(bar, parity, wc.st, code, wc.lim)
+                     : mbar_wait(bar, parity, wc.st, code, wc.lim));
+  };
+  auto wait_free = [&](uint64_t* bar, uint32_t parity, int code) {
+    return note(PAIR ? mbar_wait_cluster<true>(bar, parity, wc.st, code, wc.lim)
+                     : mbar_wait(bar, parity, wc.st, code, wc.lim));
   };
 
   if (!live) {
@@ -242,7 +303,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
 #pragma unroll
           for (int p = 0; p < 3; ++p, ++q) {
             const int s = (int)(q % SLOTS);
-            if (!wait(&empty[s], (uint32_t)((q / SLOTS) & 1) ^ 1u, 21)) {
+            if (!wait_free(&empty[s], (uint32_t)((q / SLOTS) & 1) ^ 1u, 21)) {
               ok = false;
               break;
             }
@@ -259,10 +320,10 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
           }
         }
       }
-      // no copy may be in flight when the block exits
-      if (rank == 0)
-        for (int64_t r = (q > SLOTS ? q - SLOTS : 0); r < q; ++r)
-          mbar_wait(&full[r % SLOTS], (uint32_t)((r / SLOTS) & 1), wc.st, 22, wc.lim);
+      // the last slots consumed: their copies and the MMAs' arrivals here are done
+      for (int64_t r = (q > SLOTS ? q - SLOTS : 0); r < q && ok; ++r)
+        ok = wait_free(&empty[r % SLOTS], (uint32_t)((r / SLOTS) & 1), 22);
+      leave_word<PAIR>(&leave->left[rank], (uint32_t)q);
     }
   } else if (warp == 1) {
     if (rank == 0) {
@@ -300,7 +361,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
             slot[p] = (int)(q % SLOTS);
             a[p] = smem_u32(smem + slot[p] * TL::SLOT);
             b[p] = a[p] + TL::PLANE_A;
-            if (!__all_sync(~0u, mbar_wait(&full[slot[p]], (uint32_t)((q / SLOTS) & 1), wc.st, 24, wc.lim))) {
+            if (!__all_sync(~0u, note(mbar_wait(&full[slot[p]], (uint32_t)((q / SLOTS) & 1), wc.st, 24, wc.lim)))) {
               ok = false;
               break;
             }
@@ -472,11 +533,11 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
         const uint32_t par = (uint32_t)(flushes & 1);
         ++flushes;
         if (group > 0) {
-          if (!__all_sync(~0u, mbar_wait(&rede[quarter], par ^ 1u, wc.st, 26, wc.lim))) break;
+          if (!__all_sync(~0u, note(mbar_wait(&rede[quarter], par ^ 1u, wc.st, 26, wc.lim)))) break;
           red[(group - 1) * 128 + c_in] = sum;
           mbar_arrive(&redf[quarter]);
         } else {
-          if (!__all_sync(~0u, mbar_wait(&redf[quarter], par, wc.st, 27, wc.lim))) break;
+          if (!__all_sync(~0u, note(mbar_wait(&redf[quarter], par, wc.st, 27, wc.lim)))) break;
           float4* dst = part + (per_tile ? pt : unit) * nrows + c;
           float4 all = sum;
           if (crow && !per_tile) {
@@ -498,15 +559,24 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
     }
   }
   fence_before_sync();
+  const uint32_t slot_bytes = (uint32_t)(TL::SLOT - (RA - box_a) * 128);   // of one CTA
   if constexpr (PAIR) {
     __syncwarp();
-    cluster_sync();   // no copy, MMA or arrival of the pair is outstanding
+    cluster_sync();   // no copy, MMA or arrival of the pair is outstanding, or
+    if (*(volatile uint32_t*)&leave->gave) {
+      settle<PAIR, SLOTS>(full, drain, leave, slot_bytes, rank, wc.st);
+      cluster_sync();
+    }
     if (warp == 0) {
       fence_after_sync();
       tmem_dealloc_pair(tmem, 4 * N);
     }
   } else {
     __syncthreads();
+    if (*(volatile uint32_t*)&leave->gave) {
+      settle<PAIR, SLOTS>(full, drain, leave, slot_bytes, 0, wc.st);
+      __syncthreads();
+    }
     if (warp == 0) {
       __syncwarp();
       fence_after_sync();
@@ -601,8 +671,10 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
   uint64_t* empty = full + GR_STAGES;
   uint64_t* accf = empty + GR_STAGES;
   uint64_t* acce = accf + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+  uint64_t* drain = acce + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   uint32_t* bad = tmem_slot + 1;   // [2]: a wait had given up before, as each CTA saw it
+  Leave* leave = reinterpret_cast<Leave*>(bad + 2);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
@@ -637,6 +709,8 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
       mbar_init(&accf[a], 1);
       mbar_init(&acce[a], 2 * 8);   // one arrival per epilogue warp of the pair
     }
+    mbar_init(drain, 32);
+    *leave = Leave{0u, {0u, 0u}};
     fence_barrier_init();
     prefetch_tmap(&map_hi);
     prefetch_tmap(&map_lo);
@@ -655,15 +729,20 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
   fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   const bool live = bad[0] == 0 && bad[1] == 0;   // the same in both CTAs
+  auto note = [&](bool ok) {   // every wait's outcome goes through this
+    if (!ok) leave_word<true>(&leave->gave, 1u);
+    return ok;
+  };
+  const uint32_t bytes = (diag ? 2u : 4u) * GR_PLANE_BYTES;   // a CTA's per stage
 
   if (live && warp == 0 && lane == 0) {
     // ---- TMA producer: both CTAs' loads complete on the even CTA's barrier
-    const uint32_t bytes = (diag ? 2u : 4u) * GR_PLANE_BYTES;
     int64_t issued = 0;
+    bool ok = true;
     for (int64_t q = 0; q < nch; ++q) {
       const int s = (int)(q % GR_STAGES);
       const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
-      if (!mbar_wait_cluster(&empty[s], ph ^ 1u, wc.st, 11, wc.lim)) break;
+      if (!(ok = note(mbar_wait_cluster<true>(&empty[s], ph ^ 1u, wc.st, 11, wc.lim)))) break;
       uint8_t* st = smem + s * GR_STAGE;
       const int x = (int)((c_begin + q) * 64);
       if (rank == 0) mbar_expect_tx(&full[s], 2 * bytes);
@@ -676,17 +755,17 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
       }
       issued = q + 1;
     }
-    // wait for the copies of the last stages so none is in flight at exit
-    if (rank == 0)
-      for (int64_t q = (issued > GR_STAGES ? issued - GR_STAGES : 0); q < issued; ++q)
-        mbar_wait(&full[q % GR_STAGES], (uint32_t)((q / GR_STAGES) & 1), wc.st, 12, wc.lim);
+    // the last stages consumed: their copies and the MMAs' arrivals here are done
+    for (int64_t q = (issued > GR_STAGES ? issued - GR_STAGES : 0); q < issued && ok; ++q)
+      ok = note(mbar_wait_cluster<true>(&empty[q % GR_STAGES], (uint32_t)((q / GR_STAGES) & 1), wc.st, 12, wc.lim));
+    leave_word<true>(&leave->left[rank], (uint32_t)issued);
   } else if (live && warp == 1 && lane == 0 && rank == 0) {
     // ---- MMA issuer
     bool ok = true;
     for (int64_t t = 0; t < nslices && ok; ++t) {
       const int acc = (int)(t & 1);
       const uint32_t use = (uint32_t)((t >> 1) & 1);
-      if (!mbar_wait_cluster(&acce[acc], use ^ 1u, wc.st, 13, wc.lim)) break;
+      if (!note(mbar_wait_cluster<false>(&acce[acc], use ^ 1u, wc.st, 13, wc.lim))) break;
       fence_after_sync();
       const uint32_t d = tmem + acc * GR_TILE;
       const int64_t q0 = t * GR_CHUNKS_PER_SLICE;
@@ -694,7 +773,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
       for (int64_t q = q0; q < q1; ++q) {
         const int s = (int)(q % GR_STAGES);
         const uint32_t ph = (uint32_t)((q / GR_STAGES) & 1);
-        if (!mbar_wait(&full[s], ph, wc.st, 14, wc.lim)) {
+        if (!note(mbar_wait(&full[s], ph, wc.st, 14, wc.lim))) {
           ok = false;
           break;
         }
@@ -730,7 +809,8 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
     for (int64_t t = 0; t < nslices; ++t) {
       const int acc = (int)(t & 1);
       const uint32_t use = (uint32_t)((t >> 1) & 1);
-      if (!mbar_wait_cluster(&accf[acc], use, wc.st, 15, wc.lim)) break;
+      // (all lanes or none: the reads of TMEM are the warp's)
+      if (!__all_sync(~0u, note(mbar_wait_cluster<false>(&accf[acc], use, wc.st, 15, wc.lim)))) break;
       fence_after_sync();
       const uint32_t tbase = tmem + acc * GR_TILE + (warp >= 6 ? GR_HALF : 0) + ((uint32_t)(32 * quarter) << 16);
       for (int cc = 0; cc < GR_HALF / 32; ++cc) {
@@ -749,7 +829,11 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_tc_pair_kernel(
   }
   fence_before_sync();
   __syncwarp();
-  cluster_sync();   // no copy, MMA or arrival of the pair is outstanding
+  cluster_sync();   // no copy, MMA or arrival of the pair is outstanding, or
+  if (*(volatile uint32_t*)&leave->gave) {
+    settle<true, GR_STAGES>(full, drain, leave, bytes, rank, wc.st);
+    cluster_sync();
+  }
   if (warp == 0) {
     fence_after_sync();
     tmem_dealloc_pair(tmem, 2 * GR_TILE);
@@ -778,7 +862,9 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
   uint64_t* empty = full + GS_STAGES;
   uint64_t* accf = empty + GS_STAGES;
   uint64_t* acce = accf + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+  uint64_t* drain = acce + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  Leave* leave = reinterpret_cast<Leave*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (__syncthreads_or(tid == 0 && *(volatile int*)wc.st != 0)) return;
@@ -812,6 +898,8 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
       mbar_init(&accf[a], 1);
       mbar_init(&acce[a], 128);
     }
+    mbar_init(drain, 32);
+    *leave = Leave{0u, {0u, 0u}};
     fence_barrier_init();
     prefetch_tmap(&map_hi);
     prefetch_tmap(&map_lo);
@@ -821,14 +909,19 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  auto note = [&](bool ok) {   // every wait's outcome goes through this
+    if (!ok) leave_word<false>(&leave->gave, 1u);
+    return ok;
+  };
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer
     int64_t issued = 0;
+    bool ok = true;
     for (int64_t q = 0; q < nch; ++q) {
       const int s = (int)(q % GS_STAGES);
       const uint32_t ph = (uint32_t)((q / GS_STAGES) & 1);
-      if (!mbar_wait(&empty[s], ph ^ 1u, wc.st, 11, wc.lim)) break;
+      if (!(ok = note(mbar_wait(&empty[s], ph ^ 1u, wc.st, 11, wc.lim)))) break;
       uint8_t* st = smem + s * GS_STAGE;
       const int x = (int)((c_begin + q) * 64);
       mbar_expect_tx(&full[s], GS_STAGE);
@@ -838,16 +931,17 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
       tma_load_2d(st + 3 * GS_PLANE_BYTES, &map_lo, x, (int)b0, &full[s]);
       issued = q + 1;
     }
-    // wait for the copies of the last stages so none is in flight at exit
-    for (int64_t q = (issued > GS_STAGES ? issued - GS_STAGES : 0); q < issued; ++q)
-      mbar_wait(&full[q % GS_STAGES], (uint32_t)((q / GS_STAGES) & 1), wc.st, 12, wc.lim);
+    // the last stages consumed: their copies and the MMAs' arrivals here are done
+    for (int64_t q = (issued > GS_STAGES ? issued - GS_STAGES : 0); q < issued && ok; ++q)
+      ok = note(mbar_wait(&empty[q % GS_STAGES], (uint32_t)((q / GS_STAGES) & 1), wc.st, 12, wc.lim));
+    leave_word<false>(&leave->left[0], (uint32_t)issued);
   } else if (warp == 1 && lane == 0) {
     // ---- MMA issuer
     bool ok = true;
     for (int64_t t = 0; t < nslices && ok; ++t) {
       const int acc = (int)(t & 1);
       const uint32_t use = (uint32_t)((t >> 1) & 1);
-      if (!mbar_wait(&acce[acc], use ^ 1u, wc.st, 13, wc.lim)) break;
+      if (!note(mbar_wait(&acce[acc], use ^ 1u, wc.st, 13, wc.lim))) break;
       fence_after_sync();
       const uint32_t d = tmem + acc * GS_TILE;
       const int64_t q0 = t * GR_CHUNKS_PER_SLICE;
@@ -855,7 +949,7 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
       for (int64_t q = q0; q < q1; ++q) {
         const int s = (int)(q % GS_STAGES);
         const uint32_t ph = (uint32_t)((q / GS_STAGES) & 1);
-        if (!mbar_wait(&full[s], ph, wc.st, 14, wc.lim)) {
+        if (!note(mbar_wait(&full[s], ph, wc.st, 14, wc.lim))) {
           ok = false;
           break;
         }
@@ -889,7 +983,8 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
     for (int64_t t = 0; t < nslices; ++t) {
       const int acc = (int)(t & 1);
       const uint32_t use = (uint32_t)((t >> 1) & 1);
-      if (!mbar_wait(&accf[acc], use, wc.st, 15, wc.lim)) break;
+      // (all lanes or none: the reads of TMEM are the warp's)
+      if (!__all_sync(~0u, note(mbar_wait(&accf[acc], use, wc.st, 15, wc.lim)))) break;
       fence_after_sync();
       const uint32_t tbase = tmem + acc * GS_TILE + ((uint32_t)(32 * quarter) << 16);
       for (int cc = 0; cc < GS_TILE / 32; ++cc) {
@@ -907,6 +1002,10 @@ __global__ void __launch_bounds__(GS_THREADS, 1) gram_tc_single_kernel(
   }
   fence_before_sync();
   __syncthreads();
+  if (*(volatile uint32_t*)&leave->gave) {
+    settle<false, GS_STAGES>(full, drain, leave, GS_STAGE, 0, wc.st);
+    __syncthreads();
+  }
   if (warp == 0) {
     __syncwarp();
     fence_after_sync();

@@ -72,30 +72,45 @@ __device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
 __device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-// Arrival on a barrier of either CTA and the wait for such arrivals (or for
-// MMAs of either CTA), relaxed: what they order are TMEM accesses and MMAs,
-// by the tcgen05 fences before and after.  A release would wait for all of
-// the thread's global stores first, an acquire drop the SM's L1 lines.
+// Arrival on a barrier of either CTA, relaxed: what it orders are TMEM accesses
+// and MMAs, by the tcgen05 fences before it and after the wait for it.  A
+// release would wait for all of the thread's global stores first.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
+// The wait for arrivals of threads or MMAs of either CTA.  Relaxed where only
+// TMEM accesses and MMAs follow, behind a tcgen05 fence (an acquire would drop
+// the SM's L1 lines); ACQUIRE where shared memory that the MMAs have read is
+// written next, which no tcgen05 fence orders.
+template <bool ACQUIRE>
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, int* status, int code,
                                                   uint32_t limit) {
   const uint32_t lim = limit ? limit : (1u << 23);
   for (uint32_t it = 0; it < lim; ++it) {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
+#define SPSVM_TRY_WAIT(SEM)                                                    \
+  asm volatile(                                                                \
+      "{\n\t.reg .pred p;\n\t"                                                 \
+      "mbarrier.try_wait.parity." SEM ".cluster.shared::cta.b64 p, [%1], %2;\n\t" \
+      "selp.u32 %0, 1, 0, p;\n\t}"                                             \
+      : "=r"(ok)                                                               \
+      : "r"(smem_u32(bar)), "r"(parity)                                        \
+      : "memory")
+    if constexpr (ACQUIRE) SPSVM_TRY_WAIT("acquire");
+    else SPSVM_TRY_WAIT("relaxed");
+#undef SPSVM_TRY_WAIT
     if (ok) return true;
     if (it >= 32) __nanosleep(128);
   }
   atomicCAS(status, 0, code);
   return false;
+}
+// Takes `bytes` off what a barrier's phase still expects (copies that are not
+// going to be issued).
+__device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
 }
 
 // ---- TMA ------------------------------------------------------------------
