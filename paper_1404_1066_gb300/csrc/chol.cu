@@ -1459,7 +1459,7 @@ int chol_tc_panel_update(double* H, int64_t ldh, int64_t m, int64_t k0, const in
 int chol_tc_slice(const double* H, int64_t ldh, int64_t m, int64_t k0, const int32_t* info,
                   void* work, int buf, cudaStream_t s);
 int chol_tc_update(double* H, int64_t ldh, int64_t m, int64_t cbase, int64_t cend,
-                   const int32_t* info, void* work, int buf, cudaStream_t s);
+                   const int32_t* info, void* work, int buf, const WaitCtx& wc, cudaStream_t s);
 int chol_tc_carveout();
 
 namespace {
@@ -1542,6 +1542,8 @@ extern "C" int spsvm_cholesky(double* H, int64_t m, int64_t ldh, int32_t* info, 
                                         (int)cudaSharedmemCarveoutMaxShared));
     SPSVM_CUDA_TRY(cudaFuncSetAttribute(trsm_panel<double>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared));
+    WaitCtx wc;   // waits on either stream are reported on the caller's
+    SPSVM_TRY(wait_ctx(s, &wc));
     SideGuard side;
     SPSVM_TRY(side_acquire(&side.ss));
     side.held = true;
@@ -1565,10 +1567,10 @@ extern "C" int spsvm_cholesky(double* H, int64_t m, int64_t ldh, int32_t* info, 
       SPSVM_TRY(chol_tc_slice(H, ldh, m, k0, info, work, buf, p));
       // the update on s of the previous panel touches the columns updated next
       SPSVM_CUDA_TRY(cudaStreamWaitEvent(p, side.ss.b, 0));
-      SPSVM_TRY(chol_tc_update(H, ldh, m, k0 + 64, k0 + 128, info, work, buf, p));
+      SPSVM_TRY(chol_tc_update(H, ldh, m, k0 + 64, k0 + 128, info, work, buf, wc, p));
       SPSVM_CUDA_TRY(cudaEventRecord(side.ss.a, p));
       SPSVM_CUDA_TRY(cudaStreamWaitEvent(s, side.ss.a, 0));
-      SPSVM_TRY(chol_tc_update(H, ldh, m, k0 + 128, m, info, work, buf, s));
+      SPSVM_TRY(chol_tc_update(H, ldh, m, k0 + 128, m, info, work, buf, wc, s));
       SPSVM_CUDA_TRY(cudaEventRecord(side.ss.b, s));
     }
     // s has waited for everything p did (the last record of a)

@@ -308,9 +308,10 @@ int chol_tc_slice(const double* H, int64_t ldh, int64_t m, int64_t k0, const int
 
 // Trailing update A[r][c] -= sum_l L[r][k0+l] L[c][k0+l] for the columns
 // cbase <= c < cend (cbase >= k0 + 64) and rows r >= c, from the slices in
-// buffer `buf`.
+// buffer `buf`.  wc: the status word of the factorisation's caller, also where s
+// is a stream of the library's own (nobody reads that one's word).
 int chol_tc_update(double* H, int64_t ldh, int64_t m, int64_t cbase, int64_t cend,
-                   const int32_t* info, void* work, int buf, cudaStream_t s) {
+                   const int32_t* info, void* work, int buf, const WaitCtx& wc, cudaStream_t s) {
   const int64_t R = m - cbase;
   if (R <= 0 || cend <= cbase) return SPSVM_OK;
   char* w = static_cast<char*>(work) + buf * slice_buf_bytes(m);
@@ -322,8 +323,6 @@ int chol_tc_update(double* H, int64_t ldh, int64_t m, int64_t cbase, int64_t cen
   SPSVM_CUDA_TRY(cudaFuncSetAttribute(oz_trailing, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       OZ_SMEM));
   dim3 grid((unsigned)ceil_div(cend - cbase, (int64_t)OZ_TN), (unsigned)ceil_div(R, (int64_t)OZ_TM));
-  WaitCtx wc;
-  SPSVM_TRY(wait_ctx(s, &wc));
   oz_trailing<<<grid, 128, OZ_SMEM, s>>>(ma, mb, H, ldh, m, cbase, cend, ex, info, wc);
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;

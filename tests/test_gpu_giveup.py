@@ -39,11 +39,19 @@ def _calls(sp):
         ns = torch.tensor([cols], device="cuda")
         return lambda: sp.spsvm_gram(K, ns, cols, K, torch.arange(rows, device="cuda"), 0.1, "bf16split")
 
+    A = torch.randn(1024, 1100, dtype=torch.float64, device="cuda", generator=g)
+    H = A @ A.T + torch.eye(1024, dtype=torch.float64, device="cuda")
+
+    def factor():
+        L = H.clone()
+        sp.spsvm_cholesky(L)
+        return torch.tril(L)
+
     return {"block": block, "score": score, "decide": decide, "gram_single": gram(200, 20_000),
-            "gram_pair": gram(1500, 40_000)}
+            "gram_pair": gram(1500, 40_000), "factor": factor}
 
 
-@pytest.mark.parametrize("name", ["block", "score", "decide", "gram_single", "gram_pair"])
+@pytest.mark.parametrize("name", ["block", "score", "decide", "gram_single", "gram_pair", "factor"])
 def test_recovers_from_waits_that_give_up(name):
     import paper_1404_1066_gb300 as sp
     lib = sp.load()
