@@ -28,7 +28,10 @@ __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 
 // per BF16 plane.  A warp's load instruction covers 256 contiguous bytes of
 // a row; with a whole chunk of 32 rows in flight per thread this layout
 // streams at the HBM read rate (fewer, wider loads per thread kept fewer
-// bytes in flight).
+// bytes in flight).  kSplitOdd: planes an odd number of elements apart, whose
+// second plane is read singly.
+constexpr int kSplitOdd = 2;
+static_assert(SPSVM_FP32 != kSplitOdd && SPSVM_BF16SPLIT != kSplitOdd, "a form of its own");
 template <int FMT>
 __device__ __forceinline__ void load2(const KView& K, int64_t j, int64_t i, float k[2]) {
   if (FMT == SPSVM_FP32) {
@@ -38,7 +41,9 @@ __device__ __forceinline__ void load2(const KView& K, int64_t j, int64_t i, floa
   } else {
     const uint16_t* base = static_cast<const uint16_t*>(K.data);
     const uint32_t h = *reinterpret_cast<const uint32_t*>(base + j * K.ld + i);
-    const uint32_t l = *reinterpret_cast<const uint32_t*>(base + K.plane + j * K.ld + i);
+    const uint16_t* lo = base + K.plane + j * K.ld + i;
+    const uint32_t l = FMT == kSplitOdd ? (uint32_t)lo[0] | ((uint32_t)lo[1] << 16)
+                                        : *reinterpret_cast<const uint32_t*>(lo);
     k[0] = bf_lo(h) + bf_lo(l);
     k[1] = bf_hi(h) + bf_hi(l);
   }
@@ -770,6 +775,10 @@ cudaError_t gv_launch(Kern kern, int64_t tiles, int cs, cudaStream_t s, Args... 
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
+// The instantiation for K's format.
+#define SPSVM_GV_KERNEL(NAME, K)                             \
+  ((K)->format == SPSVM_FP32 ? NAME<SPSVM_FP32>              \
+                             : ((K)->plane % 2 == 0 ? NAME<SPSVM_BF16SPLIT> : NAME<kSplitOdd>))
 }  // namespace
 }  // namespace spsvm
 
@@ -793,8 +802,8 @@ extern "C" int spsvm_outputs(const spsvm_kmat* K, const double* beta, const floa
   const int64_t blocks = ceil_div(K->n, GV_PTS);
   double* part = stats ? static_cast<double*>(scratch) : nullptr;
   const int cs = beta ? gv_cluster(blocks, K->rows) : 1;
-  SPSVM_CUDA_TRY(gv_launch(K->format == SPSVM_FP32 ? outputs_kernel<SPSVM_FP32> : outputs_kernel<SPSVM_BF16SPLIT>,
-                           blocks, cs, s, view(K), K->rows, K->n, beta, y, o, active, part, 0));
+  SPSVM_CUDA_TRY(gv_launch(SPSVM_GV_KERNEL(outputs_kernel, K), blocks, cs, s, view(K), K->rows, K->n, beta,
+                           y, o, active, part, 0));
   SPSVM_LAUNCH_CHECK();
   if (stats) {
     sum_triples<<<1, 256, 0, s>>>(part, blocks, stats);
@@ -810,9 +819,8 @@ extern "C" int spsvm_gemv(const spsvm_kmat* K, const double* v, float* u, int32_
   if (K->n == 0) return SPSVM_OK;
   const int64_t blocks = ceil_div(K->n, GV_PTS);
   ProfScope prof(PROF_GEMV, as_stream(stream), 4.0 * (double)K->rows * K->n);
-  SPSVM_CUDA_TRY(gv_launch(K->format == SPSVM_FP32 ? gemv_kernel<SPSVM_FP32> : gemv_kernel<SPSVM_BF16SPLIT>,
-                           blocks, gv_cluster(blocks, K->rows), as_stream(stream), view(K), K->rows, K->n,
-                           v, u, accumulate));
+  SPSVM_CUDA_TRY(gv_launch(SPSVM_GV_KERNEL(gemv_kernel, K), blocks, gv_cluster(blocks, K->rows),
+                           as_stream(stream), view(K), K->rows, K->n, v, u, accumulate));
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }

@@ -1,0 +1,55 @@
+"""Inputs that the entry points accept beside the usual ones: kernel matrices
+whose planes lie an odd number of elements apart, active flags of any nonzero
+byte, coefficients past FP32's range, requests of any size."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import spsvm as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _t(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.fixture(scope="module")
+def sp():
+    import paper_1404_1066_gb300 as m
+    return m
+
+
+def _split_kmat(sp, K, gap):
+    """hi / lo planes of K, `gap` elements between them; and the values held."""
+    rows, n = K.shape
+    ld = (n + 7) // 8 * 8
+    plane = rows * ld + gap
+    buf = torch.zeros(2 * plane, dtype=torch.bfloat16, device="cuda")
+    K32 = _t(K.astype(np.float32))
+    hi = K32.to(torch.bfloat16)
+    lo = (K32 - hi.float()).to(torch.bfloat16)
+    buf[:rows * ld].view(rows, ld)[:, :n] = hi
+    buf[plane:plane + rows * ld].view(rows, ld)[:, :n] = lo
+    return sp.KMat(buf, sp.SPSVM_BF16SPLIT, n, rows, ld, plane), (hi.double() + lo.double()).cpu().numpy()
+
+
+# planes an even and an odd number of elements apart; one block of 512 points
+# and a cluster
+@pytest.mark.parametrize("gap", [0, 1, 2, 5])
+@pytest.mark.parametrize("n,m", [(1, 1), (7, 3), (515, 70), (3001, 129)])
+def test_products_with_planes_any_distance_apart(sp, gap, n, m):
+    """u = K v and o = K beta: FP32 chunks of 32 terms, then one rounding."""
+    g = np.random.default_rng(n + gap)
+    km, Kref = _split_kmat(sp, np.exp(-3 * g.random((m, n))), gap)
+    v = g.standard_normal(m)
+    y = np.where(g.random(n) < 0.5, 1.0, -1.0).astype(np.float32)
+    ref = v @ Kref
+    tol = 33 * 2.0 ** -24 * (np.abs(v) @ Kref) + 2.0 ** -24 * np.abs(ref)
+    u = torch.empty(n, dtype=torch.float32, device="cuda")
+    sp.spsvm_gemv(km, _t(v), u)
+    assert np.all(np.abs(u.cpu().numpy() - ref) <= tol)
+    o = torch.empty(n, dtype=torch.float32, device="cuda")
+    active, _ = sp.spsvm_outputs(km, _t(v), _t(y), o)
+    np.testing.assert_array_equal(o.cpu().numpy(), u.cpu().numpy())
+    np.testing.assert_array_equal(active.cpu().numpy(), y * o.cpu().numpy() < 1)
