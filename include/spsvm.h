@@ -231,7 +231,8 @@ int spsvm_gemv(const spsvm_kmat* K, const double* v, float* u, int32_t accumulat
  *             zero-filled up to Kc->n (a multiple of 128);
  *   w1out_j = sum_{i active} w1_i K_ji,  w2out_j = sum_{i active} w2_i K_ji
  *   (each optional: NULL skips it).
- * active: device n bytes; w1, w2: device FP32 n; outputs device FP64.
+ * active: device n bytes (nonzero: active); w1, w2: device FP32 n; outputs
+ * device FP64.
  * n_active: device int64, written with |S|.  Kc must have the format of K
  * (or, for an FP32 K, the two BF16 planes: each value is then split as
  * hi = bf16(v), lo = bf16(v - hi)), the same rows and Kc->n >= |S| rounded
@@ -247,7 +248,8 @@ int spsvm_compact_active(const spsvm_kmat* K, const uint8_t* active,
 /* Change of the active set (Section 4 reoptimisation: between Newton steps
  * the set S of points with y_i o_i < 1 changes by a few points, and the
  * Newton matrix by their kernel rows):
- *   D = {i : active[i] != ref[i]} in increasing i, *k_dev = |D|;
+ *   D = {i : active in one of active and ref (nonzero bytes), not in the
+ *   other} in increasing i, *k_dev = |D|;
  * when |D| <= kmax also Wt[j*ldw + r] = K row j, column D_r (j < K->rows,
  * r < |D|; columns |D|..ldw-1 untouched) and sign[r] = +1 if D_r entered S
  * (active) and -1 if it left.  active, ref: device n bytes; Wt: device FP32,

@@ -204,10 +204,12 @@ __global__ void sum_triples(const double* __restrict__ part, int64_t blocks, dou
 constexpr int SC_T = 256;
 constexpr int SC_PTS = SC_T * 4;
 
-// The scanned flag of point i: active[i], or with ref, active[i] != ref[i].
+// The scanned flag of point i: whether it is active (any nonzero byte), or with
+// ref, whether that differs.
 __device__ __forceinline__ int scan_flag(const uint8_t* __restrict__ active,
                                          const uint8_t* __restrict__ ref, int64_t i) {
-  return ref ? (active[i] != ref[i]) : active[i];
+  const bool a = active[i] != 0;
+  return ref ? (int)(a != (ref[i] != 0)) : (int)a;
 }
 
 __global__ void scan_count(const uint8_t* __restrict__ active, const uint8_t* __restrict__ ref,

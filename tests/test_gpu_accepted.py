@@ -53,3 +53,37 @@ def test_products_with_planes_any_distance_apart(sp, gap, n, m):
     active, _ = sp.spsvm_outputs(km, _t(v), _t(y), o)
     np.testing.assert_array_equal(o.cpu().numpy(), u.cpu().numpy())
     np.testing.assert_array_equal(active.cpu().numpy(), y * o.cpu().numpy() < 1)
+
+
+# flags of one set written as 1, 255 and a mix; up to and past the points that
+# the writers of the list count by themselves
+@pytest.mark.parametrize("n", [1, 1025, 40_000, 1_048_577 + 3])
+def test_active_flags_are_any_nonzero_byte(sp, n):
+    """Count, positions, copies and sums are those of the set; flags that
+    differ only as bytes are no change."""
+    g = np.random.default_rng(n)
+    S = g.random(n) < 0.4
+    K = np.exp(-g.random((2, n)))
+    km = sp.kmat_empty(n, 2, "fp32")
+    km.buf.view(2, km.ld)[:, :n] = _t(K.astype(np.float32))
+    w = _t(g.standard_normal(n).astype(np.float32))
+    outs = []
+    for values in ([1], [255], [1, 2, 128, 255]):
+        act = (S * g.choice(values, n)).astype(np.uint8)
+        kc = sp.kmat_empty(km.ld, 2, "fp32")
+        a, b, count, pos = sp.spsvm_compact_active(km, _t(act), w, w, kc)
+        assert int(count.item()) == S.sum()
+        np.testing.assert_array_equal(pos.cpu().numpy(), np.cumsum(S) - S)
+        outs.append((a.cpu().numpy(), kc.to_float().cpu().numpy()))
+        ref = (S * g.choice([1, 3, 255], n)).astype(np.uint8)
+        changed = g.choice(n, min(n, 3), replace=False)
+        ref[changed] = np.where(S[changed], 0, 255)
+        k, Wt, sign = sp.spsvm_active_diff(km, _t(act), _t(ref), 8)
+        changed.sort()
+        assert k == len(changed)
+        np.testing.assert_array_equal(sign.cpu().numpy(), np.where(S[changed], 1.0, -1.0))
+        np.testing.assert_array_equal(Wt.cpu().numpy(), km.to_float().cpu().numpy()[:, changed])
+    np.testing.assert_array_equal(outs[0][1][:, :S.sum()], K.astype(np.float32)[:, S])
+    for o in outs[1:]:
+        np.testing.assert_array_equal(o[0], outs[0][0])
+        np.testing.assert_array_equal(o[1], outs[0][1])
