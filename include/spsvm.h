@@ -323,10 +323,10 @@ int spsvm_cholesky_solve(const double* L, int64_t m, int64_t ldh, double* b, voi
  * spsvm_solve_mixed then solves for b (device FP64, m) into x (device FP64,
  * m) with what work holds.  All refinement steps run in one cooperative
  * launch (bounded grid barriers), after which the stream is synchronised
- * once; it
- * returns OK, or SPSVM_ERR_NO_CONVERGE when the residual stops shrinking (by
- * half per step, from the third step on) or max_iter steps do not reach tol
- * (x then holds the last iterate).  iters, backward_error: host, may be
+ * once.  It returns OK, or SPSVM_ERR_NO_CONVERGE when the residual stops
+ * shrinking (by half per step, from the third step on), when b, x or the
+ * residual holds a NaN or an infinity, or when max_iter steps do not reach
+ * tol (x then holds the last iterate).  iters, backward_error: host, may be
  * NULL. */
 size_t spsvm_mixed_work_bytes(int64_t m);
 int spsvm_cholesky_mixed(const double* H, int64_t m, int64_t ldh, double shift, int32_t* info,

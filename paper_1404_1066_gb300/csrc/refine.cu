@@ -342,10 +342,10 @@ __device__ __forceinline__ float row_dot(const float* __restrict__ row, const fl
   return warp_sum((f[0] + f[1]) + (f[2] + f[3]));
 }
 
-// Largest of non-negative doubles over the block, by their encodings (valid in
-// thread 0; NaN counts as zero).
+// Maxima of |a| are taken over the encodings, which order NaN above infinity: a
+// vector with a NaN has a NaN for its maximum.
 __device__ __forceinline__ unsigned long long bits_of(double a) {
-  return a == a ? (unsigned long long)__double_as_longlong(fabs(a)) : 0ull;
+  return (unsigned long long)__double_as_longlong(fabs(a));
 }
 __device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
 #pragma unroll
@@ -577,9 +577,9 @@ __global__ void __launch_bounds__(RT, 1) refine_kernel(RefineArgs a, int64_t NI,
       const double rn = __longlong_as_double((long long)q[0]), xn = __longlong_as_double((long long)q[1]);
       const double hn = __longlong_as_double((long long)q[2]), bn = __longlong_as_double((long long)q[3]);
       const double denom = hn * xn + bn;
-      be = denom > 0.0 ? rn / denom : 0.0;
+      be = rn == 0.0 && denom == 0.0 ? 0.0 : rn / denom;
       int s = 0;
-      if (!(be == be)) s = 3;
+      if (!(rn < INFINITY) || !(denom < INFINITY)) s = 3;   // a NaN or an infinity anywhere
       else if (be <= a.tol) s = 1;
       else if (it >= 2 && rn > 0.5 * rprev) s = 2;
       rprev = rn;

@@ -87,3 +87,22 @@ def test_active_flags_are_any_nonzero_byte(sp, n):
     for o in outs[1:]:
         np.testing.assert_array_equal(o[0], outs[0][0])
         np.testing.assert_array_equal(o[1], outs[0][1])
+
+
+# one block of 64 rows, several, and more than one inverse of 1,024 rows
+@pytest.mark.parametrize("m", [3, 130, 1100])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_solve_of_what_is_not_finite_does_not_converge(sp, m, bad):
+    """A NaN or an infinity in b is no solution with backward error zero; b of
+    zeros has one."""
+    SPSVM_ERR_NO_CONVERGE = -4
+    g = np.random.default_rng(m)
+    A = g.standard_normal((m, m + 8)) / np.sqrt(m)
+    H = _t(A @ A.T + 0.5 * np.eye(m))
+    for k in (0, m - 1):
+        b = g.standard_normal(m)
+        b[k] = bad
+        info, status, x, iters, be = sp.spsvm_solve_mixed(H, _t(b))
+        assert info == 0 and status == SPSVM_ERR_NO_CONVERGE and not be <= 1e-13
+    info, status, x, iters, be = sp.spsvm_solve_mixed(H, _t(np.zeros(m)))
+    assert info == 0 and status == 0 and be == 0.0 and torch.all(x == 0)
