@@ -18,7 +18,7 @@ namespace spsvm {
 int64_t decision_tc_parts(int64_t m);
 int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes, int64_t m,
                        const float* znorm, const double* beta, float gamma, float* dpart,
-                       int64_t ldp, DecidePlan* plan, cudaStream_t s);
+                       int64_t ldp, cudaStream_t s);
 
 namespace {
 
@@ -193,20 +193,17 @@ int launch_decision_simt(int cs, const float* B, int64_t m, int64_t ldb, const f
   return SPSVM_OK;
 }
 
-// out[i] = sum over the partials of query i as compensated pairs: each of 8
-// groups of threads sums every 8th partial of 32 queries, the groups are added
-// in order.  Bound by latency: 32,768 queries by 4,096 rows, 12 partials a
-// query, 6 us (9 with one partial per 32 rows, 24 as a thread a query in FP64).
+// out[i] = sum over the P partials of column i as compensated pairs: each of
+// 8 groups of threads sums every 8th partial of 32 columns, the groups are
+// added in order.  L2 bound: 32,768 columns of 128 partials
+// 9 us; one thread a column in FP64 took 24.
 constexpr int DF_G = 8;
-__global__ void __launch_bounds__(32 * DF_G) decision_finish(const float* __restrict__ part, DecidePlan plan,
+__global__ void __launch_bounds__(32 * DF_G) decision_finish(const float* __restrict__ part, int64_t P,
                                                              int64_t ldp, int64_t nq,
                                                              float* __restrict__ out) {
   __shared__ float2 sh[DF_G][32];
   const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * 32 + c;
-  const int64_t first = i / plan.rows * plan.col_tiles;
-  const int64_t P = plan.groups * (decide_unit(first + plan.col_tiles - 1, plan.tiles, plan.units) -
-                                   decide_unit(first, plan.tiles, plan.units) + 1);
   float h = 0.f, l = 0.f;
   if (i < nq) {
     for (int64_t p = g; p < P; p += 8 * DF_G) {
@@ -303,9 +300,8 @@ extern "C" int spsvm_decision(const float* B, int64_t m, int64_t ldb, const doub
       spsvm_points qb{Q + q0 * ldq, cnt, d, ldq, reinterpret_cast<float*>(w + L.off_qn), qp,
                       qp + 2 * L.qc * L.ldh, L.ldh, qp + L.qc * L.ldh};
       SPSVM_TRY(spsvm_prepare_points(&qb, SPSVM_BF16SPLIT, stream));
-      DecidePlan plan{};
-      SPSVM_TRY(launch_decision_tc(&qb, zp, L.z_bytes, m, zb.norms, beta, gamma, part, L.qc, &plan, s));
-      decision_finish<<<(unsigned)ceil_div(cnt, (int64_t)32), 32 * DF_G, 0, s>>>(part, plan, L.qc,
+      SPSVM_TRY(launch_decision_tc(&qb, zp, L.z_bytes, m, zb.norms, beta, gamma, part, L.qc, s));
+      decision_finish<<<(unsigned)ceil_div(cnt, (int64_t)32), 32 * DF_G, 0, s>>>(part, L.parts, L.qc,
                                                                                 cnt, out + q0);
       SPSVM_LAUNCH_CHECK();
     }

@@ -260,18 +260,6 @@ int solve_mixed_after_factor(const double* H, int64_t m, int64_t ldh, double shi
                              void* work, size_t work_bytes, const int32_t* factor_info,
                              void* stream);
 
-// Where the split form's decision partials are: `tiles` in blocks of `rows`
-// queries by col_tiles, unit u of `units` taking the tiles u tiles / units up to
-// (u + 1) tiles / units; a block's units in turn have `groups` partials each.
-struct DecidePlan {
-  int64_t tiles, units, col_tiles;
-  int rows, groups;
-};
-// The unit that has tile t.
-__host__ __device__ inline int64_t decide_unit(int64_t t, int64_t tiles, int64_t units) {
-  return ((t + 1) * units - 1) / tiles;
-}
-
 // A Newton step taken on the way into the compaction: with the step length t
 // (device; 0: none) beta += t dir, o += t u, and from the new outputs the
 // active flags, the residuals o - y, stats as of spsvm_outputs and the count

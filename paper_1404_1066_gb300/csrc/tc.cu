@@ -102,8 +102,7 @@ __device__ __noinline__ void settle(uint64_t* full, uint64_t* drain, const Leave
 //   SCORE   rows the candidates, columns the points: the score sums, a
 //           thread's own over its columns of all of the CTA's tiles, or per
 //           tile where tiles are few (kernel values not stored);
-//   DECIDE  rows the queries, columns the basis: sums of beta K, a thread's
-//           own over its columns of the CTA's consecutive tiles of a row block.
+//   DECIDE  rows the queries, columns the basis: sums of beta K over 32.
 // Basis and candidate rows are gathered into contiguous planes beforehand.
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into one of two tile buffers,
@@ -120,7 +119,7 @@ __device__ __noinline__ void settle(uint64_t* full, uint64_t* drain, const Leave
 // MMAs on the same plane of the rows stand together, so the rows are read from
 // shared memory three times a step instead of six.  Arrivals of a pair are
 // relaxed (a release waits for the epilogue's global stores).
-// 32,768 queries by 4,096 basis rows, d = 128: 115 us, 1.79 PFLOP/s in the six
+// 32,768 queries by 4,096 basis rows, d = 128: 117 us, 1.77 PFLOP/s in the six
 // products (154 us in 128 x 128 tiles of single CTAs with the queries as
 // columns, where each sum over a warp's rows took 31 exchanges).  Scores of 256
 // candidates, n = 500,000: 130 us (157).  Kernel block of 64 rows, n = 500,000:
@@ -158,16 +157,9 @@ struct Kb {
 // so that a basis row's values reach DRAM in runs of PK_GROUP x 1 KB), each
 // group swept over all row blocks (column tiles) with the group's own index
 // varying fastest.  The CTAs in flight share tiles of both operands through L2.
-// DECIDE: row block after row block, a CTA (or pair) taking consecutive tiles.
 constexpr int64_t PK_GROUP = 32;
 template <int MODE, typename I>
 __device__ __forceinline__ void tile_coords_as(I t, I nCB, I nPT, int& cb, int64_t& pt) {
-  if (MODE == KB_DECIDE) {
-    const I a = t / nPT;
-    cb = (int)a;
-    pt = (int64_t)(t - a * nPT);
-    return;
-  }
   constexpr I G = (I)PK_GROUP;
   const I grouped = MODE == KB_STORE_F32 ? nCB : nPT, other = MODE == KB_STORE_F32 ? nPT : nCB;
   const I per = other * G;
@@ -222,8 +214,6 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
   const int64_t nCB = ceil_div(nrows, (int64_t)TL::M);
   const int64_t nPT = ceil_div(ncols, (int64_t)N);
   const int64_t T = nCB * nPT;
-  const int64_t t0 = DECIDE ? unit * T / units : unit, t1 = DECIDE ? (unit + 1) * T / units : T;
-  const int64_t dt = DECIDE ? 1 : units;
   const int nK = (int)(ldh / KC);
   constexpr uint32_t IDESC = idesc_bf16_f32(TL::M, N);
 
@@ -294,7 +284,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
       bool ok = true;
       const CUtensorMap* ma[3] = {&map_ahi, &map_amid, &map_alo};
       const CUtensorMap* mb[3] = {&map_bhi, &map_bmid, &map_blo};
-      for (int64_t t = t0; t < t1 && ok; t += dt) {
+      for (int64_t t = unit; t < T && ok; t += units) {
         int cb;
         int64_t pt;
         tile_coords<MODE>(t, nCB, nPT, cb, pt);
@@ -344,7 +334,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
       };
       int64_t q = 0, j = 0;
       bool ok = true;
-      for (int64_t t = t0; t < t1 && ok; t += dt, ++j) {
+      for (int64_t t = unit; t < T && ok; t += units, ++j) {
         const int acc = (int)(j & 1);
         if (!__all_sync(~0u, wait(&tempty[acc], (uint32_t)((j >> 1) & 1) ^ 1u, 23))) break;
         fence_after_sync();
@@ -405,7 +395,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
     };
     auto fetch = [&](int64_t t) {
       Pre f{0.f, 0.f, 0.f, 0.f, 0.0, -1, 0};
-      if (t >= t1) return f;
+      if (t >= T) return f;
       tile_coords<MODE>(t, nCB, nPT, f.cb, f.pt);
       const int64_t c = (TL::CTAS * (int64_t)f.cb + rank) * PK_M + c_in;
       const int64_t i = f.pt * N + group * PK_WP + lane;
@@ -420,13 +410,13 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
       }
       return f;
     };
-    Pre next = fetch(t0);
-    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);   // compensated pairs of this thread's sums
+    Pre next = fetch(unit);
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);   // SCORE: compensated pairs of this thread's sums
     int flushes = 0;
     if (SCORE && group == 0 && !per_tile)
       for (int64_t c = rank * PK_M + c_in; c < nrows; c += TL::M) part[unit * nrows + c] = sum;
     int64_t j = 0;
-    for (int64_t t = t0; t < t1; t += dt, ++j) {
+    for (int64_t t = unit; t < T; t += units, ++j) {
       const int cb = next.cb;
       const int64_t pt = next.pt;
       const int64_t cblock = TL::CTAS * (int64_t)cb + rank;   // this CTA's 128 rows
@@ -464,7 +454,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
         if constexpr (PAIR) mbar_arrive_cluster(map_rank(&tempty[acc], 0));
         else mbar_arrive(&tempty[acc]);
       }
-      next = fetch(t + dt);
+      next = fetch(t + units);
       float gs = 0.f, hs = 0.f;
       if (any) {
         // arg = -g2 * max(|x|^2 + |z|^2 - 2 x.z, 0); columns past the last
@@ -516,15 +506,9 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
           hs = (ha.x + ha.y) + (hb.x + hb.y);
         }
       }
-      if (DECIDE) {
-        // one partial per group, query and CTA with tiles of its block, summed
-        // in a fixed order by the finish
-        pair_add(sum.x, sum.y, gs);
-        if (next.cb == cb) continue;
-        const int64_t slot = unit - decide_unit(cb * nPT, T, units);
-        if (crow) dpart[(slot * GROUPS + group) * ldp + c] = (float)pair_value(sum.x, sum.y);
-        sum = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+      // one partial per 32 basis rows and query, summed in a fixed order by
+      // the finish
+      if (DECIDE && crow && any) dpart[ib / PK_WP * ldp + c] = gs;
       if (SCORE) {
         pair_add(sum.x, sum.y, gs);
         pair_add(sum.z, sum.w, hs);
@@ -1066,7 +1050,6 @@ struct KbArgs {
   const double* beta;                 // DECIDE
   float* dpart;
   int64_t ldp;
-  DecidePlan* plan;                   // receives where the partials are
 };
 
 template <int MODE, bool PAIR, int N, int RA = PK_M>
@@ -1089,8 +1072,6 @@ int launch_kb_as(const KbArgs& a, cudaStream_t s) {
   SPSVM_TRY(wait_ctx(s, &wc));
   cudaLaunchConfig_t cfg{};
   const int64_t units = max64(1, min64(tiles, (int64_t)sm_count() / W));
-  if (MODE == KB_DECIDE)
-    *a.plan = DecidePlan{tiles, units, ceil_div(a.ncols, (int64_t)N), TL::M, TL::GROUPS};
   // sums per CTA or pair, unless those outnumber the tiles of points
   const int64_t col_tiles = ceil_div(a.ncols, (int64_t)N);
   const int per_tile = MODE == KB_SCORE && units > col_tiles;
@@ -1186,12 +1167,11 @@ int launch_score_tc(const spsvm_points* p, const float* y, const float* o, const
   return launch_kb<KB_SCORE>(a, s);
 }
 
-// (a unit with tiles of a row block has one at least)
-int64_t decision_tc_parts(int64_t m) { return 4 * ceil_div(m, (int64_t)128); }
+int64_t decision_tc_parts(int64_t m) { return ceil_div(m, (int64_t)PK_WP); }
 
 int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes, int64_t m,
                        const float* znorm, const double* beta, float gamma, float* dpart,
-                       int64_t ldp, DecidePlan* plan, cudaStream_t s) {
+                       int64_t ldp, cudaStream_t s) {
   if (m == 0 || q->n == 0) return SPSVM_OK;
   if (!zplanes || zbytes < (size_t)(m * q->ldh * 6))
     return set_error(SPSVM_ERR_OOM, "BF16SPLIT decision: scratch too small for the basis planes");
@@ -1200,7 +1180,6 @@ int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes
   a.beta = beta;
   a.dpart = dpart;
   a.ldp = ldp;
-  a.plan = plan;
   return launch_kb<KB_DECIDE>(a, s);
 }
 

@@ -106,3 +106,23 @@ def test_solve_of_what_is_not_finite_does_not_converge(sp, m, bad):
         assert info == 0 and status == SPSVM_ERR_NO_CONVERGE and not be <= 1e-13
     info, status, x, iters, be = sp.spsvm_solve_mixed(H, _t(np.zeros(m)))
     assert info == 0 and status == 0 and be == 0.0 and torch.all(x == 0)
+
+
+# single CTAs and pairs of them, tiles of 64 and 128 basis rows, a last partial
+# tile, two passes of queries; SIMT tiles of 32 and 128 queries, clusters of 1 to
+# 8 blocks, one to four shares of the features
+@pytest.mark.parametrize("precision", ["bf16split"])
+@pytest.mark.parametrize("m,d", [(1, 3), (40, 17), (65, 64), (300, 130), (600, 784), (2100, 33)])
+def test_decision_value_is_the_same_in_any_request(sp, precision, m, d):
+    """A query's value has the same bits alone, in a small and in a large
+    request, wherever it stands in it."""
+    g = np.random.default_rng(m + d)
+    nq = 40_000
+    Q = _t(g.standard_normal((nq, d)).astype(np.float32))
+    B = _t(g.standard_normal((m, d)).astype(np.float32))
+    beta = _t(g.standard_normal(m) * 10.0 ** g.uniform(-3, 3, m))
+    f = sp.spsvm_decision(B, beta, Q, 0.5 / d, precision).cpu().numpy()
+    for a, b in [(0, 1), (17, 18), (127, 160), (100, 229), (0, 1000), (5, 3005), (20_000, 32_769),
+                 (39_999, 40_000), (3, 40_000)]:
+        part = sp.spsvm_decision(B, beta, Q[a:b], 0.5 / d, precision).cpu().numpy()
+        np.testing.assert_array_equal(part, f[a:b])
