@@ -384,12 +384,14 @@ int spsvm_line_search(const float* o, const float* u, const float* y, int64_t n,
  *   out[i] = sum_{j<m} beta_j exp(-gamma ||q_i - b_j||^2)
  * for query rows q (nq x d, ldq) and basis rows b (m x d, ldb), computed
  * tile by tile without storing the kernel block.  beta FP64; out FP32.
- * SPSVM_FP32: FP32 SIMT dot products, beta_j k summed in FP64.
+ * SPSVM_FP32: FP32 SIMT dot products, beta_j k summed as compensated FP32
+ * pairs (about 2^-46).
  * SPSVM_BF16SPLIT: the kernel block's tensor-core engine (basis rows and
  * queries split into three BF16 planes, six products: the dot products
  * carry FP32-level error), beta_j k summed in FP32 over groups of 32 basis
- * rows and the groups in FP64 in a fixed order (results do not depend on
- * the launch); queries go in passes of at most 32,768.
+ * rows and the groups as compensated FP32 pairs; queries go in passes of at
+ * most 32,768.  Sums have a fixed order in both: a query's value does not
+ * depend on the launch, or on the queries that it comes with.
  * All device.  scratch: spsvm_decision_scratch_bytes(nq, m, d, precision)
  * bytes (SPSVM_BF16SPLIT: the basis planes, one pass of query planes and
  * the partial sums, about m d 6 + min(nq, 32768) (6 d + m / 8) bytes).

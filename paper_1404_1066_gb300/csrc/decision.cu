@@ -1,8 +1,8 @@
 // Decision values f(q) = sum_j beta_j k(q, b_j) (Section 4: the classifier
 // h(x) = w^T phi(x) with w restricted to the basis J), tile by tile, never
-// storing the query-by-basis kernel block.  SPSVM_FP32: plain FP32 SIMT dot
-// products, beta_j k(q, b_j) summed as compensated FP32 pairs and in FP64
-// across threads.  SPSVM_BF16SPLIT: the tensor-core kernel block engine with
+// storing the query-by-basis kernel block.  SPSVM_FP32: FP32 SIMT dot
+// products, beta_j k(q, b_j) summed as compensated FP32 pairs over a tile of 64
+// basis rows and in FP64 over the tiles.  SPSVM_BF16SPLIT: the tensor-core kernel block engine with
 // the basis rows and the queries split into three BF16 planes each, FP32 sums
 // of beta_j k over 32 basis rows per partial, the partials summed as a
 // compensated pair in a fixed order.
@@ -23,8 +23,8 @@ int launch_decision_tc(const spsvm_points* q, const void* zplanes, size_t zbytes
 namespace {
 
 // Basis rows by queries.  The wide tile where there are queries enough to fill
-// the SMs; else 32 queries, half the outputs per thread and the
-// features split over four groups of threads: the loop over features is then
+// the SMs; else 32 queries, half the rows per thread and the features
+// split over four groups of threads: the loop over features is then
 // a latency chain of one warp per sub-partition, which the groups shorten, and
 // blocks that fit an SM twice let every cluster of a small request start at
 // once (with one block per SM not all clusters of 8 found room).
@@ -44,14 +44,49 @@ __global__ void row_norms_kernel(const float* __restrict__ A, int64_t m, int64_t
   if (lane == 0) out[i] = s;
 }
 
-// A cluster of blocks takes one tile of queries; its blocks take the tiles of
-// 64 basis rows in turn and rank 0 adds their sums in rank order, so a small
-// request spreads over the GPU without scratch and its result does not depend
-// on the launch.  beta_j k is summed as compensated pairs with beta_j in two
-// FP32 terms (an FP64 multiply-add and conversion per kernel value, at 1/64 of
-// the FP32 rate, cost more than the dot products at small d).  FP32 ALU bound
-// for many queries, latency of the feature loop for few: 1,000 queries, 512
-// basis rows, d = 784 0.035 ms, where 8 blocks of 128 queries took 0.80 ms.
+// A query's value has the same bits in every request: each sum below has one
+// order, whatever the tile and the cluster.
+//   * A dot product is the sum, in order, of those over up to four shares of the
+//     features (whole steps of 16, at least two): the small tile's
+//     groups take one each, the wide tile keeps the sums so far in shared memory.
+//   * beta_j k over a tile of 64 basis rows: four rows at a time in order, the 16
+//     sums of four joined by fours (q and q + 8 of two neighbours), these in order.
+//   * A query's tiles fall in kLanes lanes, tile t in lane t % kLanes; a lane's
+//     tiles are added in order, then the lanes.  A cluster's blocks take whole
+//     lanes, and rank 0 adds them through distributed shared memory.
+constexpr int kLanes = kMaxCluster;
+// (32 features at least: of 64, one query by 4,096 rows, d = 128 took 80 us
+// instead of 69; of 16, 100,000 queries by 512 rows, d = 64 368 instead of 346)
+__host__ __device__ inline int64_t feature_share(int64_t d) {
+  return max64(2, ceil_div(ceil_div(d, (int64_t)16), (int64_t)4)) * 16;
+}
+
+// Sums of beta_j k.  In pairs (beta_j in two FP32 terms: an FP64 multiply-add and
+// conversion per kernel value, at 1/64 of the FP32 rate, cost more than the dot
+// products at small d).
+struct PairSum {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float bh, float bl, float k) {
+    const float x = __fmul_rn(bh, k);
+    l = __fadd_rn(l, __fmaf_rn(bl, k, __fmaf_rn(bh, k, -x)));
+    pair_add(h, l, x);
+  }
+  __device__ __forceinline__ void join(PairSum o) {   // a.join(b) == b.join(a)
+    l = __fadd_rn(l, o.l);
+    pair_add(h, l, o.h);
+  }
+  __device__ __forceinline__ PairSum shfl_xor(int x) const {
+    PairSum o;
+    o.h = __shfl_xor_sync(0xffffffffu, h, x);
+    o.l = __shfl_xor_sync(0xffffffffu, l, x);
+    return o;
+  }
+  __device__ __forceinline__ double value() const { return pair_value(h, l); }
+};
+// FP32 ALU bound for many queries, latency of the feature loop for few: 1,000
+// queries, 512 basis rows, d = 784 0.037 ms, where 8 blocks of 128 queries took
+// 0.66 ms.  The one order costs the wide tile 3 to 9%: 30,000 queries by 4,096
+// rows, d = 128 1.11 ms, 1.02 with sums in whatever order a block meets them.
 template <class T, bool VB, bool VQ>
 __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
     const float* __restrict__ B, int64_t m, int64_t ldb, const float* __restrict__ bnorm,
@@ -60,9 +95,11 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
   extern __shared__ __align__(16) unsigned char dyn[];
   typename T::Smem* sm = reinterpret_cast<typename T::Smem*>(dyn);
   constexpr int W = T::THREADS / 32;
+  constexpr int RED = T::KG == 1 ? 4 : 16;   // partial sums of a tile per query
   __shared__ float qn[T::TN], bn[T::TM], bh[T::TM], bl[T::TM];
-  __shared__ double tot[T::TN];
-  static_assert(sizeof(typename T::Smem) >= sizeof(float2) * W * T::TN, "partial sums fit the stages");
+  __shared__ PairSum totals[kLanes][T::TN];
+  static_assert(T::TM == 64 && T::TY * T::RM == 64 && T::THREADS >= T::TN, "64 rows a tile, a thread per query");
+  static_assert(sizeof(typename T::Smem) >= sizeof(PairSum) * RED * T::TN, "partial sums fit the stages");
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -86,84 +123,129 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
     const int64_t q = q0 + T::load_row(u);
     b[u].p = q < nq ? Q + q * ldq : nullptr;
   }
-  float sh[8], sl[8];
+  const int64_t share = feature_share(d), tiles = ceil_div(m, (int64_t)T::TM);
+  // sum += the sum over the tile at b0 of query q0 + t (threads below TN), from
+  // the dot products of this thread's rows and columns
+  auto add_tile = [&](PairSum& sum, int64_t b0, auto dots) {
+    using S = PairSum;
+    S* red = reinterpret_cast<S*>(dyn);   // [RED][TN]
+    // four rows from T::row(r0) on, all columns at once (independent chains)
+    auto four = [&](int r0, auto& v, auto col) {
 #pragma unroll
-  for (int c = 0; c < 8; ++c) sh[c] = sl[c] = 0.f;
-  // beta_j k(q, b_j) of basis row j (of the tile at b0) into the 8 queries' sums
-  auto add_row = [&](int64_t b0, int j, const float (&dot)[8]) {
-    if (b0 + j >= m) return;
-    const float zn = bn[j], ch = bh[j], cl2 = bl[j];
+      for (int r = r0; r < r0 + 4; ++r) {
+        const int j = T::row(r);
+        if (b0 + j >= m) continue;
+        const float zn = bn[j], jh = bh[j], jl = bl[j];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const float k = rbf_from_dot(qn[T::col(c)], zn, dot[c], gamma);
-      const float x = __fmul_rn(ch, k);
-      sl[c] = __fadd_rn(sl[c], __fmaf_rn(cl2, k, __fmaf_rn(ch, k, -x)));
-      pair_add(sh[c], sl[c], x);
+        for (int c = 0; c < (int)(sizeof(v) / sizeof(S)); ++c)
+          v[c].add(jh, jl, rbf_from_dot(qn[col(c)], zn, dots(r, c), gamma));
+      }
+    };
+    if constexpr (T::KG == 1) {
+      auto col = [](int c) { return T::col(c); };
+      S s[8], u[8];
+      four(0, s, col);
+      four(4, u, col);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) s[c].join(u[c]);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) s[c].join(s[c].shfl_xor(T::TX));   // the neighbour's
+      if (lane < T::TX)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) red[w * T::TN + T::col(c)] = s[c];
+    } else {
+      auto col = [](int e) { return 4 * T::tx() + ((2 * T::group() + e) & 3) + (T::group() >> 1) * (T::TN / 2); };
+      S s[2];
+      four(0, s, col);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) red[T::ty() * T::TN + col(e)] = s[e];
+    }
+    __syncthreads();
+    if (t < T::TN) {
+      S s;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        if constexpr (T::KG == 1) {
+          s.join(red[p * T::TN + t]);
+        } else {
+          S x = red[2 * p * T::TN + t], y = red[(2 * p + 1) * T::TN + t];
+          x.join(red[(2 * p + 8) * T::TN + t]);
+          y.join(red[(2 * p + 9) * T::TN + t]);
+          x.join(y);
+          s.join(x);
+        }
+      }
+      sum.join(s);
     }
   };
-  for (int64_t b0 = (int64_t)rank * T::TM; b0 < m; b0 += (int64_t)cs * T::TM) {
-    __syncthreads();   // the last tile's norms and coefficients have been read
-    if (t < T::TM) {
-      const int64_t j = b0 + t;
-      const double bj = j < m ? beta[j] : 0.0;
-      bn[t] = j < m ? bnorm[j] : 0.f;
-      bh[t] = (float)bj;
-      bl[t] = (float)(bj - (double)bh[t]);
-    }
+  for (int ln = rank; ln < kLanes; ln += cs) {
+    PairSum sum;        // of query q0 + t over the lane's tiles
+    for (int64_t tile = ln; tile < tiles; tile += kLanes) {
+      const int64_t b0 = tile * T::TM;
+      __syncthreads();   // the last tile's norms, coefficients and sums have been read
+      if (t < T::TM) {
+        const int64_t j = b0 + t;
+        const double bj = j < m ? beta[j] : 0.0;
+        bn[t] = j < m ? bnorm[j] : 0.f;
+        bh[t] = (float)bj;
+        bl[t] = (float)(bj - (double)bh[t]);
+      }
 #pragma unroll
-    for (int u = 0; u < T::LA; ++u) {
-      const int64_t j = b0 + T::load_row(u);
-      a[u].p = j < m ? B + j * ldb : nullptr;
-    }
-    uint64_t acc[T::RM][4];
-    T::block_k(sm, a, b, 0, d, acc);
-    if constexpr (T::KG > 1) {
-      float dot[8];
-      T::combine(sm, acc, dot);
-      add_row(b0, T::row(T::group()), dot);
-    } else {
+      for (int u = 0; u < T::LA; ++u) {
+        const int64_t j = b0 + T::load_row(u);
+        a[u].p = j < m ? B + j * ldb : nullptr;
+      }
+      uint64_t acc[T::RM][4];
+      if constexpr (T::KG > 1) {
+        T::block_k(sm, a, b, 0, d, share, acc);
+        uint64_t v[4];
+        T::combine_cols(sm, acc, v);
+        auto dots = [&](int r, int e) {
+          const float2 x = simt::unpack2(v[r]);
+          return e ? x.y : x.x;
+        };
+        add_tile(sum, b0, dots);
+      } else {
+        // the sums of a whole share are added to those kept
+        ulonglong2* keep = reinterpret_cast<ulonglong2*>(dyn + sizeof(typename T::Smem)) + t;
+        const int steps = (int)(share / T::TK);
+        int left = steps;
+        bool kept = false;
+        auto add_kept = [&](uint64_t (&f)[T::RM][4]) {
 #pragma unroll
-      for (int r = 0; r < T::RM; ++r) {
-        float dot[8];
+          for (int i = 0; i < T::RM * 2; ++i) {
+            const ulonglong2 o = keep[i * T::THREADS];
+            f[i / 2][2 * (i & 1)] = simt::add2(o.x, f[i / 2][2 * (i & 1)]);
+            f[i / 2][2 * (i & 1) + 1] = simt::add2(o.y, f[i / 2][2 * (i & 1) + 1]);
+          }
+        };
+        T::product(*sm, a, b, 0, d, acc, [&](uint64_t (&f)[T::RM][4]) {
+          if (--left > 0) return;
+          left = steps;
+          if (kept) add_kept(f);
+          kept = true;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-          const float2 v = simt::unpack2(acc[r][p]);
-          dot[2 * p] = v.x;
-          dot[2 * p + 1] = v.y;
-        }
-        add_row(b0, T::row(r), dot);
+          for (int i = 0; i < T::RM * 2; ++i) {
+            keep[i * T::THREADS] = make_ulonglong2(f[i / 2][2 * (i & 1)], f[i / 2][2 * (i & 1) + 1]);
+            f[i / 2][2 * (i & 1)] = f[i / 2][2 * (i & 1) + 1] = 0ull;
+          }
+        });
+        if (kept) add_kept(acc);
+        auto dots = [&](int r, int c) {
+          const float2 x = simt::unpack2(acc[r][c / 2]);
+          return c & 1 ? x.y : x.x;
+        };
+        add_tile(sum, b0, dots);
       }
     }
-  }
-  // over the rows: the warp's row groups, the warps in order, the ranks in order
-#pragma unroll
-  for (int o = T::TX; o < 32; o <<= 1)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const float oh = __shfl_xor_sync(0xffffffffu, sh[c], o), ol = __shfl_xor_sync(0xffffffffu, sl[c], o);
-      sl[c] = __fadd_rn(sl[c], ol);
-      pair_add(sh[c], sl[c], oh);
-    }
-  __syncthreads();
-  float2 (*red)[T::TN] = reinterpret_cast<float2 (*)[T::TN]>(dyn);
-  if (lane < T::TX)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) red[w][T::col(c)] = make_float2(sh[c], sl[c]);
-  __syncthreads();
-  if (t < T::TN) {
-    float h = 0.f, l = 0.f;
-#pragma unroll
-    for (int g = 0; g < W; ++g) {
-      l = __fadd_rn(l, red[g][t].y);
-      pair_add(h, l, red[g][t].x);
-    }
-    tot[t] = pair_value(h, l);
+    if (t < T::TN) totals[ln][t] = sum;
   }
   cl.sync();
   if (rank == 0 && t < T::TN && q0 + t < nq) {
-    double s = tot[t];
-    for (int r = 1; r < cs; ++r) s += *cl.map_shared_rank(&tot[t], r);
-    out[q0 + t] = (float)s;
+    PairSum p;
+#pragma unroll
+    for (int ln = 0; ln < kLanes; ++ln) p.join(*cl.map_shared_rank(&totals[ln][t], ln % cs));
+    out[q0 + t] = (float)p.value();
   }
   cl.sync();   // no block leaves while rank 0 reads its sums
 }
@@ -176,6 +258,7 @@ int launch_decision_simt(int cs, const float* B, int64_t m, int64_t ldb, const f
   cfg.gridDim = dim3((unsigned)(ceil_div(nq, T::TN) * cs));
   cfg.blockDim = dim3(T::THREADS);
   cfg.dynamicSmemBytes = T::KG * sizeof(typename T::Smem);
+  if (T::KG == 1 && d > feature_share(d)) cfg.dynamicSmemBytes += sizeof(float) * T::TM * T::TN;
   cfg.stream = s;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;

@@ -28,6 +28,11 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ float2 unpack2(uint64_t v) {
   float2 r;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
@@ -115,10 +120,15 @@ struct Tile {
 
   // acc[r][c / 2] (packed pairs of columns) = the sums over k in [k0, k1) of
   // rows a[], b[] (this thread's staged rows).  All threads; starts with the
-  // stages free and ends with a barrier.
-  template <class RA, class RB>
+  // stages free and ends with a barrier.  step(acc) runs after every TK terms
+  // but the last ones, and may move the sums so far elsewhere.
+  struct NoStep {
+    __device__ __forceinline__ void operator()(uint64_t (&)[RM][RN / 2]) const {}
+  };
+  template <class RA, class RB, class Step = NoStep>
   static __device__ __forceinline__ void product(Smem& sm, const RA (&a)[LA], const RB (&b)[LB],
-                                                 int64_t k0, int64_t k1, uint64_t (&acc)[RM][RN / 2]) {
+                                                 int64_t k0, int64_t k1, uint64_t (&acc)[RM][RN / 2],
+                                                 Step step = Step()) {
 #pragma unroll
     for (int r = 0; r < RM; ++r)
 #pragma unroll
@@ -161,6 +171,7 @@ struct Tile {
       if (more) {
         stage<LA, TM>(sm.A[s ^ 1], va);
         stage<LB, TN>(sm.B[s ^ 1], vb);
+        step(acc);
       }
       sync();
     };
@@ -174,14 +185,21 @@ struct Tile {
     }
   }
 
-  // product over [k0, k1) by the whole block: group g takes the g-th share of
-  // the chunks.  combine then leaves thread (group g, t) with the 8 sums of
-  // row r = g of thread t's outputs, added over the groups in order (KG ==
-  // RM; sm: the groups' stages).  All threads; combine ends with a barrier.
+  // product over [k0, k1) by the whole block: group g takes the g-th share
+  // (share, a multiple of TK, or the chunks evenly).  combine then leaves
+  // thread (group g, t) with the 8 sums of row r = g of thread t's outputs,
+  // added over the groups in order (KG == RM; sm: the groups' stages);
+  // combine_cols with all rows of its columns 2 g, 2 g + 1 (KG == RN / 2).
+  // All threads; both end with a barrier.
   template <class RA, class RB>
   static __device__ __forceinline__ void block_k(Smem* sm, const RA (&a)[LA], const RB (&b)[LB],
                                                  int64_t k0, int64_t k1, uint64_t (&acc)[RM][RN / 2]) {
-    const int64_t share = ceil_div(ceil_div(k1 - k0, (int64_t)TK), (int64_t)KG) * TK;
+    block_k(sm, a, b, k0, k1, ceil_div(ceil_div(k1 - k0, (int64_t)TK), (int64_t)KG) * TK, acc);
+  }
+  template <class RA, class RB>
+  static __device__ __forceinline__ void block_k(Smem* sm, const RA (&a)[LA], const RB (&b)[LB],
+                                                 int64_t k0, int64_t k1, int64_t share,
+                                                 uint64_t (&acc)[RM][RN / 2]) {
     const int64_t g0 = min64(k1, k0 + group() * share);
     product(sm[group()], a, b, g0, min64(k1, g0 + share), acc);
   }
@@ -204,6 +222,24 @@ struct Tile {
         const float4 f = p[(group() * 2 + h) * NT + tid()];
         v[4 * h] += f.x; v[4 * h + 1] += f.y; v[4 * h + 2] += f.z; v[4 * h + 3] += f.w;
       }
+    }
+    __syncthreads();
+  }
+  static __device__ __forceinline__ void combine_cols(Smem* sm, const uint64_t (&acc)[RM][RN / 2],
+                                                      uint64_t (&v)[RM]) {
+    static_assert(KG == RN / 2 && sizeof(Smem) >= sizeof(float) * RM * NT * RN, "a pair of columns per group");
+    uint64_t* mine = reinterpret_cast<uint64_t*>(&sm[group()]);
+#pragma unroll
+    for (int r = 0; r < RM; ++r)
+#pragma unroll
+      for (int p = 0; p < RN / 2; ++p) mine[(r * (RN / 2) + p) * NT + tid()] = acc[r][p];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RM; ++r) {
+      v[r] = reinterpret_cast<const uint64_t*>(&sm[0])[(r * (RN / 2) + group()) * NT + tid()];
+#pragma unroll
+      for (int g = 1; g < KG; ++g)
+        v[r] = add2(v[r], reinterpret_cast<const uint64_t*>(&sm[g])[(r * (RN / 2) + group()) * NT + tid()]);
     }
     __syncthreads();
   }

@@ -111,7 +111,7 @@ def test_solve_of_what_is_not_finite_does_not_converge(sp, m, bad):
 # single CTAs and pairs of them, tiles of 64 and 128 basis rows, a last partial
 # tile, two passes of queries; SIMT tiles of 32 and 128 queries, clusters of 1 to
 # 8 blocks, one to four shares of the features
-@pytest.mark.parametrize("precision", ["bf16split"])
+@pytest.mark.parametrize("precision", ["fp32", "bf16split"])
 @pytest.mark.parametrize("m,d", [(1, 3), (40, 17), (65, 64), (300, 130), (600, 784), (2100, 33)])
 def test_decision_value_is_the_same_in_any_request(sp, precision, m, d):
     """A query's value has the same bits alone, in a small and in a large
