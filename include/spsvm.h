@@ -385,7 +385,7 @@ int spsvm_line_search(const float* o, const float* u, const float* y, int64_t n,
  * for query rows q (nq x d, ldq) and basis rows b (m x d, ldb), computed
  * tile by tile without storing the kernel block.  beta FP64; out FP32.
  * SPSVM_FP32: FP32 SIMT dot products, beta_j k summed as compensated FP32
- * pairs (about 2^-46).
+ * pairs (about 2^-46), or in FP64 where |beta_j| is outside 2^-80 to 2^90.
  * SPSVM_BF16SPLIT: the kernel block's tensor-core engine (basis rows and
  * queries split into three BF16 planes, six products: the dot products
  * carry FP32-level error), beta_j k summed in FP32 over groups of 32 basis

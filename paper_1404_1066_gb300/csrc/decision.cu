@@ -8,6 +8,8 @@
 // compensated pair in a fixed order.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "simt_tile.h"
 
@@ -63,10 +65,11 @@ __host__ __device__ inline int64_t feature_share(int64_t d) {
 
 // Sums of beta_j k.  In pairs (beta_j in two FP32 terms: an FP64 multiply-add and
 // conversion per kernel value, at 1/64 of the FP32 rate, cost more than the dot
-// products at small d).
+// products at small d), or in FP64 for the tiles with a beta_j outside the range
+// where the pairs keep 2^-46 of it.
 struct PairSum {
   float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float bh, float bl, float k) {
+  __device__ __forceinline__ void add(float bh, float bl, double, float k) {
     const float x = __fmul_rn(bh, k);
     l = __fadd_rn(l, __fmaf_rn(bl, k, __fmaf_rn(bh, k, -x)));
     pair_add(h, l, x);
@@ -83,6 +86,22 @@ struct PairSum {
   }
   __device__ __forceinline__ double value() const { return pair_value(h, l); }
 };
+struct WideSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(float, float, double b, float k) { s += b * (double)k; }
+  __device__ __forceinline__ void join(WideSum o) { s += o.s; }
+  __device__ __forceinline__ WideSum shfl_xor(int x) const {
+    WideSum o;
+    o.s = __shfl_xor_sync(0xffffffffu, s, x);
+    return o;
+  }
+  __device__ __forceinline__ double value() const { return s; }
+};
+__device__ __forceinline__ bool beyond_pairs(double b) {
+  const double a = fabs(b);
+  return b != 0.0 && !(a >= 0x1p-80 && a <= 0x1p90);
+}
+
 // FP32 ALU bound for many queries, latency of the feature loop for few: 1,000
 // queries, 512 basis rows, d = 784 0.037 ms, where 8 blocks of 128 queries took
 // 0.66 ms.  The one order costs the wide tile 3 to 9%: 30,000 queries by 4,096
@@ -97,9 +116,12 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
   constexpr int W = T::THREADS / 32;
   constexpr int RED = T::KG == 1 ? 4 : 16;   // partial sums of a tile per query
   __shared__ float qn[T::TN], bn[T::TM], bh[T::TM], bl[T::TM];
-  __shared__ PairSum totals[kLanes][T::TN];
+  __shared__ double bd[T::TM];
+  // [lane][query]: PairSum, or (widel[lane]) WideSum
+  __shared__ __align__(8) unsigned char totals[kLanes * T::TN * 8];
+  __shared__ int widel[kLanes], widet[2];   // widet: per warp that loads a tile's coefficients
   static_assert(T::TM == 64 && T::TY * T::RM == 64 && T::THREADS >= T::TN, "64 rows a tile, a thread per query");
-  static_assert(sizeof(typename T::Smem) >= sizeof(PairSum) * RED * T::TN, "partial sums fit the stages");
+  static_assert(sizeof(typename T::Smem) >= sizeof(double) * RED * T::TN, "partial sums fit the stages");
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -126,8 +148,8 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
   const int64_t share = feature_share(d), tiles = ceil_div(m, (int64_t)T::TM);
   // sum += the sum over the tile at b0 of query q0 + t (threads below TN), from
   // the dot products of this thread's rows and columns
-  auto add_tile = [&](PairSum& sum, int64_t b0, auto dots) {
-    using S = PairSum;
+  auto add_tile = [&](auto& sum, int64_t b0, auto dots) {
+    using S = std::remove_reference_t<decltype(sum)>;
     S* red = reinterpret_cast<S*>(dyn);   // [RED][TN]
     // four rows from T::row(r0) on, all columns at once (independent chains)
     auto four = [&](int r0, auto& v, auto col) {
@@ -136,9 +158,10 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
         const int j = T::row(r);
         if (b0 + j >= m) continue;
         const float zn = bn[j], jh = bh[j], jl = bl[j];
+        const double jd = std::is_same<S, WideSum>::value ? bd[j] : 0.0;
 #pragma unroll
         for (int c = 0; c < (int)(sizeof(v) / sizeof(S)); ++c)
-          v[c].add(jh, jl, rbf_from_dot(qn[col(c)], zn, dots(r, c), gamma));
+          v[c].add(jh, jl, jd, rbf_from_dot(qn[col(c)], zn, dots(r, c), gamma));
       }
     };
     if constexpr (T::KG == 1) {
@@ -180,6 +203,8 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
   };
   for (int ln = rank; ln < kLanes; ln += cs) {
     PairSum sum;        // of query q0 + t over the lane's tiles
+    WideSum wide;       // and over those with a beta_j beyond the pairs
+    bool any = false;   // there was one
     for (int64_t tile = ln; tile < tiles; tile += kLanes) {
       const int64_t b0 = tile * T::TM;
       __syncthreads();   // the last tile's norms, coefficients and sums have been read
@@ -187,8 +212,11 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
         const int64_t j = b0 + t;
         const double bj = j < m ? beta[j] : 0.0;
         bn[t] = j < m ? bnorm[j] : 0.f;
+        bd[t] = bj;
         bh[t] = (float)bj;
         bl[t] = (float)(bj - (double)bh[t]);
+        const bool beyond = __any_sync(0xffffffffu, beyond_pairs(bj));
+        if (lane == 0) widet[w] = beyond;
       }
 #pragma unroll
       for (int u = 0; u < T::LA; ++u) {
@@ -204,7 +232,12 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
           const float2 x = simt::unpack2(v[r]);
           return e ? x.y : x.x;
         };
-        add_tile(sum, b0, dots);
+        if (widet[0] | widet[1]) {
+          add_tile(wide, b0, dots);
+          any = true;
+        } else {
+          add_tile(sum, b0, dots);
+        }
       } else {
         // the sums of a whole share are added to those kept
         ulonglong2* keep = reinterpret_cast<ulonglong2*>(dyn + sizeof(typename T::Smem)) + t;
@@ -235,17 +268,34 @@ __global__ void __launch_bounds__(T::THREADS, T::KG == 1 ? 3 : 2) decision_simt(
           const float2 x = simt::unpack2(acc[r][c / 2]);
           return c & 1 ? x.y : x.x;
         };
-        add_tile(sum, b0, dots);
+        if (widet[0] | widet[1]) {
+          add_tile(wide, b0, dots);
+          any = true;
+        } else {
+          add_tile(sum, b0, dots);
+        }
       }
     }
-    if (t < T::TN) totals[ln][t] = sum;
+    if (t < T::TN) {
+      if (any) wide.s += sum.value();
+      if (any) reinterpret_cast<WideSum*>(totals)[ln * T::TN + t] = wide;
+      else reinterpret_cast<PairSum*>(totals)[ln * T::TN + t] = sum;
+      if (t == 0) widel[ln] = any;
+    }
   }
   cl.sync();
   if (rank == 0 && t < T::TN && q0 + t < nq) {
     PairSum p;
+    WideSum v;
 #pragma unroll
-    for (int ln = 0; ln < kLanes; ++ln) p.join(*cl.map_shared_rank(&totals[ln][t], ln % cs));
-    out[q0 + t] = (float)p.value();
+    for (int ln = 0; ln < kLanes; ++ln) {
+      const int r = ln % cs;
+      if (*cl.map_shared_rank(&widel[ln], r))
+        v.join(cl.map_shared_rank(reinterpret_cast<WideSum*>(totals), r)[ln * T::TN + t]);
+      else
+        p.join(cl.map_shared_rank(reinterpret_cast<PairSum*>(totals), r)[ln * T::TN + t]);
+    }
+    out[q0 + t] = (float)(p.value() + v.s);
   }
   cl.sync();   // no block leaves while rank 0 reads its sums
 }

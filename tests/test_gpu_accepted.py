@@ -126,3 +126,31 @@ def test_decision_value_is_the_same_in_any_request(sp, precision, m, d):
                  (39_999, 40_000), (3, 40_000)]:
         part = sp.spsvm_decision(B, beta, Q[a:b], 0.5 / d, precision).cpu().numpy()
         np.testing.assert_array_equal(part, f[a:b])
+
+
+# one tile and several lanes of tiles, the small and the wide tile
+@pytest.mark.parametrize("nq", [5, 60_000])
+@pytest.mark.parametrize("m", [3, 70, 700])
+def test_coefficients_beyond_fp32(sp, m, nq):
+    """beta_j past FP32's range where the kernel value brings the term back, and
+    as small as FP64 goes, beside ordinary ones.  Kernel values carry the
+    rounding of their exponent (FP32 norms and product) and of the exponential;
+    sums are FP64, or FP32 pairs, then rounded once."""
+    g = np.random.default_rng(m)
+    d, gamma = 4, 1.0
+    B = g.standard_normal((m, d)).astype(np.float32)
+    Q = g.standard_normal((nq, d)).astype(np.float32)
+    beta = g.standard_normal(m)
+    far = g.choice(m, max(1, m // 5), replace=False)
+    B[far] += 4.0 * np.sign(B[far])     # exp(-d2) about 1e-20 to 1e-60
+    beta[far] *= 10.0 ** g.uniform(38, 42, len(far))
+    beta[g.choice(m, m // 4, replace=False)] *= 1e-200
+    f = sp.spsvm_decision(_t(B), _t(beta), _t(Q), gamma, "fp32").cpu().numpy().astype(np.float64)
+    K = O.rbf_kernel(Q, B, gamma)
+    sq = (Q.astype(np.float64) ** 2).sum(1)[:, None] + (B.astype(np.float64) ** 2).sum(1)[None, :]
+    rel = 8 * 2.0 ** -24 * gamma * sq + 2.0 ** -20
+    err = (rel * K + 2.0 ** -149) @ np.abs(beta)
+    ref = K @ beta
+    inside = np.abs(ref) < 1e38
+    assert inside.mean() > 0.5 and np.all(np.isfinite(f[inside]))
+    assert np.all(np.abs(f - ref)[inside] <= (err + 2.0 ** -23 * np.abs(ref) + 1e-44)[inside])
