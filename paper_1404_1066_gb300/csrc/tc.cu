@@ -107,9 +107,9 @@ __device__ __noinline__ void settle(uint64_t* full, uint64_t* drain, const Leave
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into one of two tile buffers,
 // the other warps drain the other (TMEM lane = row; four lane quarters by
-// groups of 32 columns).  A slot of the shared-memory ring holds one plane of
-// both operands over 64 columns of K, so a chunk starts as soon as its hi
-// planes are there.  With more than 128 rows two CTAs work as a pair (PAIR,
+// groups of 32 columns).  A slot of the shared-memory ring holds 64 columns of K
+// of both operands, in one plane (a pair, whose chunk starts as soon as its hi
+// planes are there) or in all three.  With more than 128 rows two CTAs work as a pair (PAIR,
 // cta_group::2) on 256 rows, each staging 128 rows and half of the columns,
 // the even one issuing the MMAs for both: a 128 x 128 MMA of one CTA reads its
 // operands from shared memory at the full 128 bytes a cycle, with loads of 64
@@ -135,13 +135,18 @@ constexpr int PK_WP = 32;                                  // columns per epilog
 template <bool PAIR, int N, int RA>
 struct Kb {
   static constexpr int CTAS = PAIR ? 2 : 1;
+  // Planes per slot.  A single CTA waits once for all three: with a wait for
+  // each, the MMAs of a chunk started late (20,000 points by 128 candidates,
+  // d = 500: 27.8 us so, 31.6 plane by plane)
+  static constexpr int PPS = PAIR ? 1 : 3;
   static constexpr int M = CTAS * PK_M;                    // rows of a tile
   static constexpr int ROWS_B = N / CTAS;                  // columns staged per CTA
   static constexpr int GROUPS = N / PK_WP;
   static constexpr int EPI_WARPS = 4 * GROUPS;
   static constexpr int THREADS = 32 * (2 + EPI_WARPS);
   static constexpr int PLANE_A = RA * PK_KC * 2;
-  static constexpr int SLOT = PLANE_A + ROWS_B * PK_KC * 2;
+  static constexpr int PLANE = PLANE_A + ROWS_B * PK_KC * 2;   // of both operands
+  static constexpr int SLOT = PPS * PLANE;
   static constexpr int SLOTS = 192 * 1024 / SLOT;
   static constexpr int RED_OFF = SLOTS * SLOT;             // SCORE: the groups' sums
   static constexpr int BAR_OFF = RED_OFF + (GROUPS - 1) * 128 * 16;
@@ -149,8 +154,8 @@ struct Kb {
   static constexpr int SMEM = STAGE_OFF + EPI_WARPS * 3 * PK_WP * 4 + 1024;   // + alignment slack
   static_assert(SMEM <= 227 * 1024, "kernel block shared memory");
   static_assert(8 * (2 * SLOTS + 13) + 12 + sizeof(Leave) <= 512, "barriers");
-  static_assert(SLOTS >= 6, "two chunks in flight");
-  static_assert(SLOT >= PK_M * PK_KC * 2, "the rows that the MMAs read lie in the slot");
+  static_assert(SLOTS * PPS >= 6, "two chunks in flight");
+  static_assert(PLANE >= PK_M * PK_KC * 2, "the rows that the MMAs read lie in the slot");
 };
 
 // Tile order: groups of PK_GROUP consecutive column tiles (STORE: row blocks,
@@ -192,7 +197,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
   constexpr bool STORE = MODE == KB_STORE_F32;
   constexpr bool DECIDE = MODE == KB_DECIDE;
   using TL = Kb<PAIR, N, RA>;
-  constexpr int SLOTS = TL::SLOTS, KC = PK_KC, GROUPS = TL::GROUPS;
+  constexpr int SLOTS = TL::SLOTS, KC = PK_KC, PPS = TL::PPS, GROUPS = TL::GROUPS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + TL::BAR_OFF);
@@ -276,6 +281,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
                      : mbar_wait(bar, parity, wc.st, code, wc.lim));
   };
 
+  const uint32_t slot_bytes = (uint32_t)(TL::SLOT - PPS * (RA - box_a) * 128);   // of one CTA
   if (!live) {
   } else if (warp == 0) {
     if (lane == 0) {
@@ -291,21 +297,24 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
         const int ra = cb * TL::M + (int)rank * PK_M, rb = (int)(pt * N) + (int)rank * TL::ROWS_B;
         for (int kc = 0; kc < nK && ok; ++kc) {
 #pragma unroll
-          for (int p = 0; p < 3; ++p, ++q) {
+          for (int p = 0; p < 3; p += PPS, ++q) {
             const int s = (int)(q % SLOTS);
             if (!wait_free(&empty[s], (uint32_t)((q / SLOTS) & 1) ^ 1u, 21)) {
               ok = false;
               break;
             }
-            uint8_t* st = smem + s * TL::SLOT;
-            if (rank == 0) mbar_expect_tx(&full[s], TL::CTAS * (uint32_t)(TL::SLOT - (RA - box_a) * 128));
-            if constexpr (PAIR) {
-              const uint32_t bar = map_rank(&full[s], 0);
-              tma_load_2d_pair(st, ma[p], kc * KC, ra, bar);
-              tma_load_2d_pair(st + TL::PLANE_A, mb[p], kc * KC, rb, bar);
-            } else {
-              tma_load_2d(st, ma[p], kc * KC, ra, &full[s]);
-              tma_load_2d(st + TL::PLANE_A, mb[p], kc * KC, rb, &full[s]);
+            if (rank == 0) mbar_expect_tx(&full[s], TL::CTAS * slot_bytes);
+#pragma unroll
+            for (int e = 0; e < PPS; ++e) {
+              uint8_t* st = smem + s * TL::SLOT + e * TL::PLANE;
+              if constexpr (PAIR) {
+                const uint32_t bar = map_rank(&full[s], 0);
+                tma_load_2d_pair(st, ma[p + e], kc * KC, ra, bar);
+                tma_load_2d_pair(st + TL::PLANE_A, mb[p + e], kc * KC, rb, bar);
+              } else {
+                tma_load_2d(st, ma[p + e], kc * KC, ra, &full[s]);
+                tma_load_2d(st + TL::PLANE_A, mb[p + e], kc * KC, rb, &full[s]);
+              }
             }
           }
         }
@@ -347,10 +356,13 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
           uint32_t a[3], b[3];
           int slot[3];
 #pragma unroll
-          for (int p = 0; p < 3; ++p, ++q) {
+          for (int p = 0; p < 3; p += PPS, ++q) {
             slot[p] = (int)(q % SLOTS);
-            a[p] = smem_u32(smem + slot[p] * TL::SLOT);
-            b[p] = a[p] + TL::PLANE_A;
+#pragma unroll
+            for (int e = 0; e < PPS; ++e) {
+              a[p + e] = smem_u32(smem + slot[p] * TL::SLOT) + e * TL::PLANE;
+              b[p + e] = a[p + e] + TL::PLANE_A;
+            }
             if (!__all_sync(~0u, note(mbar_wait(&full[slot[p]], (uint32_t)((q / SLOTS) & 1), wc.st, 24, wc.lim)))) {
               ok = false;
               break;
@@ -369,7 +381,7 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
               mma(last, d_small, a[1] + koff, b[1] + koff, 1u);
               mma(once, d_small, a[2] + koff, b[0] + koff, 1u);
             }
-            for (int p = 0; p < 3; ++p) commit(&empty[slot[p]]);
+            for (int p = 0; p < 3; p += PPS) commit(&empty[slot[p]]);
             if (kc == nK - 1) commit(&tfull[acc]);
           }
           __syncwarp();
@@ -543,7 +555,6 @@ __global__ void __launch_bounds__(Kb<PAIR, N, RA>::THREADS, 1) kblock_tc_kernel(
     }
   }
   fence_before_sync();
-  const uint32_t slot_bytes = (uint32_t)(TL::SLOT - (RA - box_a) * 128);   // of one CTA
   if constexpr (PAIR) {
     __syncwarp();
     cluster_sync();   // no copy, MMA or arrival of the pair is outstanding, or
