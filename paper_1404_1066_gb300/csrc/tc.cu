@@ -1104,17 +1104,30 @@ int launch_kb_as(const KbArgs& a, cudaStream_t s) {
   return SPSVM_OK;
 }
 
-// Tiles of single CTAs where one wave takes them all, half the latency of a
-// pair's (3,000 points by 200 basis rows, d = 128: 8.5 us against 9.6), else
-// pairs.  Scores of up to 64 candidates stage 64 rows, so more points are in
-// flight (64 candidates, n = 100,000, d = 784: 105 us against 111).
+// Single CTAs where their tiles cost less than a pair's, which take 256 rows and
+// a microsecond more to start:
+//   * up to 128 rows, or one wave of tiles (3,000 points by 200 basis rows, d =
+//     128: 8.8 us against 10.3);
+//   * three or five blocks of 128 rows, of which pairs would compute four or six
+//     (300 candidates, d = 20: n = 500,000 154 us against 176, n = 20,000 17.5
+//     against 19.3; 600: 205 against 270; seven blocks, d = 128 115 against 104);
+//   * a few waves at small d, where the MMAs are not the bound (200 candidates, n =
+//     20,000, d = 20: 15.3 us against 15.8; kernel block of 12,000 points by 512
+//     rows, d = 30: 12.0 against 13.4), and every kernel block that its stores
+//     bound (500,000 by 512, d = 54: 210 us against 214).
+// Else pairs (256 candidates, n = 500,000, d = 128: 130 us against 143; 100,000
+// queries by 4,096 rows: 418 against 454).  Scores of up to 64 candidates stage 64
+// rows, which leaves more of the ring to the points.
 template <int MODE>
 int launch_kb(const KbArgs& a, cudaStream_t s) {
   constexpr int NARROW = MODE == KB_SCORE ? 128 : 64;   // (score columns are the points)
   const bool narrow = a.ncols <= NARROW;
-  const int64_t tiles = ceil_div(a.nrows, (int64_t)PK_M) * ceil_div(a.ncols, (int64_t)(narrow ? NARROW : 128));
+  const int64_t blocks = ceil_div(a.nrows, (int64_t)PK_M);
+  const int64_t tiles = blocks * ceil_div(a.ncols, (int64_t)(narrow ? NARROW : 128));
+  constexpr bool STORE = MODE == KB_STORE_F32;
+  const int waves = a.ldh == 64 || (STORE && a.ldh == 128) ? 4 : 1;
   if (MODE == KB_SCORE && a.nrows <= 64) return launch_kb_as<MODE, false, 128, MODE == KB_SCORE ? 64 : PK_M>(a, s);
-  if (a.nrows <= PK_M || tiles <= sm_count())
+  if (blocks == 1 || blocks == 3 || blocks == 5 || tiles <= waves * (int64_t)sm_count() || (STORE && a.ldh == 64))
     return narrow ? launch_kb_as<MODE, false, NARROW>(a, s) : launch_kb_as<MODE, false, 128>(a, s);
   return narrow ? launch_kb_as<MODE, true, NARROW>(a, s) : launch_kb_as<MODE, true, 128>(a, s);
 }
