@@ -93,13 +93,14 @@ __device__ __forceinline__ void row_products(const KView& K, int64_t rows, int64
 // Where the points alone leave SMs idle (a block takes 512), a cluster of
 // blocks shares a tile of points: rank r sums the r-th share of the rows, in
 // whole chunks, and rank 0 adds the ranks' sums in order through distributed
-// shared memory.  HBM (or L2) bound: n = 30,000, 1,024 rows (123 MB) 29 us, 116
+// shared memory.  HBM (or L2) bound: n = 30,000, 1,024 rows (123 MB) 28 us, 114
 // with 59 blocks.
 constexpr int GV_CLUSTER = 8;
 template <int FMT>
 __device__ __forceinline__ bool cluster_products(const KView& K, int64_t rows, int64_t n,
                                                  const double* __restrict__ v, int64_t i, float* vs,
-                                                 double (*red)[GV_P], double acc[GV_P]) {
+                                                 double acc[GV_P]) {
+  __shared__ double red[GV_T][GV_P];
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int64_t per = ceil_div(ceil_div(rows, (int64_t)GV_CHUNK), (int64_t)cs) * GV_CHUNK;
@@ -108,7 +109,6 @@ __device__ __forceinline__ bool cluster_products(const KView& K, int64_t rows, i
   if (FMT == SPSVM_FP32) Kr.data = static_cast<const float*>(K.data) + j0 * K.ld;
   else Kr.data = static_cast<const uint16_t*>(K.data) + j0 * K.ld;
   row_products<FMT>(Kr, min64(rows, j0 + per) - j0, n, v + j0, i, vs, acc);
-  if (cs == 1) return true;
 #pragma unroll
   for (int p = 0; p < GV_P; ++p) red[threadIdx.x][p] = acc[p];
   cl.sync();
@@ -120,19 +120,34 @@ __device__ __forceinline__ bool cluster_products(const KView& K, int64_t rows, i
   return rank == 0;
 }
 
+// The thread's products over all rows; false in the blocks of a cluster that
+// have given theirs away.  CL: a cluster per tile of points.
+template <int FMT, bool CL>
+__device__ __forceinline__ bool tile_products(const KView& K, int64_t rows, int64_t n,
+                                              const double* __restrict__ v, int64_t i, float* vs,
+                                              double acc[GV_P]) {
+  if constexpr (CL) return cluster_products<FMT>(K, rows, n, v, i, vs, acc);
+  row_products<FMT>(K, rows, n, v, i, vs, acc);
+  return true;
+}
+template <bool CL>
+__device__ __forceinline__ int64_t tile_of_block() {
+  if constexpr (CL) return blockIdx.x / cg::this_cluster().num_blocks();
+  return blockIdx.x;
+}
+
 // o = K beta (or given), active flags, per-block loss / errors / |S|.
-template <int FMT>
+template <int FMT, bool CL>
 __global__ void __launch_bounds__(GV_T) outputs_kernel(
     KView K, int64_t rows, int64_t n, const double* __restrict__ beta,
     const float* __restrict__ y, float* __restrict__ o, uint8_t* __restrict__ active,
     double* __restrict__ part, int accumulate) {
   __shared__ float vs[GV_BETA];
   __shared__ double sh[32];
-  __shared__ double red[GV_T][GV_P];
-  const int64_t tile = blockIdx.x / cg::this_cluster().num_blocks();
+  const int64_t tile = tile_of_block<CL>();
   const int64_t i = (tile * GV_T + threadIdx.x) * GV_P;
   double acc[GV_P];
-  if (beta && !cluster_products<FMT>(K, rows, n, beta, i, vs, red, acc)) return;
+  if (beta && !tile_products<FMT, CL>(K, rows, n, beta, i, vs, acc)) return;
   double loss = 0.0, err = 0.0, act = 0.0;
   {
 #pragma unroll
@@ -172,15 +187,14 @@ __global__ void __launch_bounds__(GV_T) outputs_kernel(
   }
 }
 
-template <int FMT>
+template <int FMT, bool CL>
 __global__ void __launch_bounds__(GV_T) gemv_kernel(KView K, int64_t rows, int64_t n,
                                                     const double* __restrict__ v,
                                                     float* __restrict__ u, int accumulate) {
   __shared__ float vs[GV_BETA];
-  __shared__ double red[GV_T][GV_P];
-  const int64_t i = ((int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * GV_T + threadIdx.x) * GV_P;
+  const int64_t i = (tile_of_block<CL>() * GV_T + threadIdx.x) * GV_P;
   double acc[GV_P];
-  if (!cluster_products<FMT>(K, rows, n, v, i, vs, red, acc)) return;
+  if (!tile_products<FMT, CL>(K, rows, n, v, i, vs, acc)) return;
 #pragma unroll
   for (int p = 0; p < GV_P; ++p) {
     const int64_t ii = i + p;
@@ -754,13 +768,23 @@ __global__ void store_count(const int64_t* __restrict__ total, int32_t* __restri
 
 namespace spsvm {
 namespace {
-// Blocks per tile of points: enough for four blocks per SM, each with a chunk
-// of rows at least.
-int gv_cluster(int64_t tiles, int64_t rows) {
+// Blocks per tile of points: two, four or eight while SMs would be idle or nearly
+// so, and a block keeps rows enough to pay the cluster's barriers: 32 up to a block
+// for every other SM, 64 up to two blocks per SM, then 128; the outputs, whose
+// epilogue one block in each cluster runs, 64 up to one block per SM, then 192.
+// 30,000 points by 1,024 rows: u = K v 28 us, one block a tile 114; 100,000 by 128: 7.8, two blocks
+// of 64 rows 7.3, four 10.3 (outputs 14.8, 17.1 and 25.4); 60,000 by 256: 9.2 with two, 9.8
+// with four, 12.3 with one (outputs 17.5, 21.3, 17.0).
+int gv_cluster(int64_t tiles, int64_t rows, bool outputs) {
+  const int64_t sms = sm_count();
   int cs = 1;
-  while (2 * cs <= GV_CLUSTER && tiles * cs < 4 * (int64_t)sm_count() &&
-         2 * cs <= ceil_div(rows, (int64_t)GV_CHUNK))
+  while (2 * cs <= GV_CLUSTER && tiles * cs < (outputs ? 2 : 4) * sms) {
+    const int64_t after = 2 * cs * tiles;
+    const int64_t least = outputs ? (after <= sms ? 64 : 192)
+                                  : (2 * after <= sms ? 32 : (after <= 2 * sms ? 64 : 128));
+    if (rows < 2 * cs * least) break;
     cs *= 2;
+  }
   return cs;
 }
 template <class Kern, class... Args>
@@ -769,6 +793,7 @@ cudaError_t gv_launch(Kern kern, int64_t tiles, int cs, cudaStream_t s, Args... 
   cfg.gridDim = dim3((unsigned)(tiles * cs));
   cfg.blockDim = dim3(GV_T);
   cfg.stream = s;
+  if (cs == 1) return cudaLaunchKernelEx(&cfg, kern, args...);
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = (unsigned)cs;
@@ -777,10 +802,10 @@ cudaError_t gv_launch(Kern kern, int64_t tiles, int cs, cudaStream_t s, Args... 
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
-// The instantiation for K's format.
-#define SPSVM_GV_KERNEL(NAME, K)                             \
-  ((K)->format == SPSVM_FP32 ? NAME<SPSVM_FP32>              \
-                             : ((K)->plane % 2 == 0 ? NAME<SPSVM_BF16SPLIT> : NAME<kSplitOdd>))
+// The instantiation for K's format and the cluster.
+#define SPSVM_GV_KERNEL(NAME, K, CL)                             \
+  ((K)->format == SPSVM_FP32 ? NAME<SPSVM_FP32, CL>              \
+                             : ((K)->plane % 2 == 0 ? NAME<SPSVM_BF16SPLIT, CL> : NAME<kSplitOdd, CL>))
 }  // namespace
 }  // namespace spsvm
 
@@ -803,9 +828,9 @@ extern "C" int spsvm_outputs(const spsvm_kmat* K, const double* beta, const floa
   ProfScope prof(PROF_OUTPUTS, s, beta ? 4.0 * (double)K->rows * K->n : 9.0 * K->n);
   const int64_t blocks = ceil_div(K->n, GV_PTS);
   double* part = stats ? static_cast<double*>(scratch) : nullptr;
-  const int cs = beta ? gv_cluster(blocks, K->rows) : 1;
-  SPSVM_CUDA_TRY(gv_launch(SPSVM_GV_KERNEL(outputs_kernel, K), blocks, cs, s, view(K), K->rows, K->n, beta,
-                           y, o, active, part, 0));
+  const int cs = beta ? gv_cluster(blocks, K->rows, true) : 1;
+  auto kern = cs > 1 ? SPSVM_GV_KERNEL(outputs_kernel, K, true) : SPSVM_GV_KERNEL(outputs_kernel, K, false);
+  SPSVM_CUDA_TRY(gv_launch(kern, blocks, cs, s, view(K), K->rows, K->n, beta, y, o, active, part, 0));
   SPSVM_LAUNCH_CHECK();
   if (stats) {
     sum_triples<<<1, 256, 0, s>>>(part, blocks, stats);
@@ -821,8 +846,9 @@ extern "C" int spsvm_gemv(const spsvm_kmat* K, const double* v, float* u, int32_
   if (K->n == 0) return SPSVM_OK;
   const int64_t blocks = ceil_div(K->n, GV_PTS);
   ProfScope prof(PROF_GEMV, as_stream(stream), 4.0 * (double)K->rows * K->n);
-  SPSVM_CUDA_TRY(gv_launch(SPSVM_GV_KERNEL(gemv_kernel, K), blocks, gv_cluster(blocks, K->rows),
-                           as_stream(stream), view(K), K->rows, K->n, v, u, accumulate));
+  const int cs = gv_cluster(blocks, K->rows, false);
+  auto kern = cs > 1 ? SPSVM_GV_KERNEL(gemv_kernel, K, true) : SPSVM_GV_KERNEL(gemv_kernel, K, false);
+  SPSVM_CUDA_TRY(gv_launch(kern, blocks, cs, as_stream(stream), view(K), K->rows, K->n, v, u, accumulate));
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }
