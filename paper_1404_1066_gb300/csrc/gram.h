@@ -8,8 +8,11 @@ namespace spsvm {
 constexpr int64_t GRAM_SLICE = 8192;
 
 // Both forms split the active points evenly over at most kGramMaxSplits
-// partial matrices of at least a quantum of points: in the FP32 form about
-// what a partial matrix costs to write and add, in the split form a slice.
+// partial matrices (or, where a wave of blocks takes more, one for each slice of
+// GRAM_SLICE points: matrices of few tiles on many points, m = 64, ns = 400,000
+// in split form 109 us, 445 with 16) of at least a quantum of points: in
+// the FP32 form about what a partial matrix costs to write and add, in the split
+// form a slice.
 // Their number is read on the device, so the last splits may be empty (they
 // are neither written nor read).
 constexpr int64_t kGramQuantumSimt = 128;
@@ -19,11 +22,15 @@ __host__ __device__ __forceinline__ int64_t gram_split_points(int64_t ns, int64_
   return max64(quantum, round_up(ceil_div(ns, splits), (int64_t)128));
 }
 
+inline int64_t gram_most_splits(int64_t tiles, int64_t slots, int64_t ns_max) {
+  return max64(kGramMaxSplits, min64(slots / max64(1, tiles), ceil_div(ns_max, GRAM_SLICE)));
+}
+
 // The fewest splits, from `least`, that fill whole waves of `slots` blocks to
 // `good`, else those that fill them best.
 inline int64_t gram_splits(int64_t tiles, int64_t slots, int64_t least, double good, int64_t ns_max,
                            int64_t quantum) {
-  const int64_t most = max64(1, min64(kGramMaxSplits, ceil_div(ns_max, quantum)));
+  const int64_t most = max64(1, min64(gram_most_splits(tiles, slots, ns_max), ceil_div(ns_max, quantum)));
   int64_t best = min64(max64(1, least), most);
   double be = 0.0;
   for (int64_t s = best; s <= most; ++s) {

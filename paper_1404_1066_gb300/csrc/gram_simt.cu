@@ -193,10 +193,11 @@ __global__ void __launch_bounds__(FT * 8) kjj_fill_kernel(KView K, const int64_t
 }
 
 // H[a][b] = H[b][a] = lambda K_JJ[a][b] + sum_s part[s][min(a,b)][max(a,b)]
-// over 32 x 32 upper tiles (the partials are compensated FP32 pairs: FP64 adds
-// at 1/64 of the FP32 rate made the sum over 16 splits take 16 us at m = 100,
-// now 9): the partials, K_JJ and both halves of H move
-// through shared memory so that every global access is coalesced.
+// over 32 x 32 upper tiles (the partials are compensated FP32 pairs: an FP64 add
+// has 1/64 of their rate): the partials, K_JJ and both halves of H move through
+// shared memory so that every global access is coalesced.  Bound by the latency
+// of the partials: 62 splits at m = 64 take 28 us more than one, 66 when only a
+// split's four rows were in flight.
 __global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const float2* __restrict__ part,
                                                              GramPlan plan,
                                                              const int64_t* __restrict__ ns_dev,
@@ -218,17 +219,29 @@ __global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const float2* __res
   const int64_t splits = max64(1, ceil_div(ns, gram_split_points(ns, plan.splits(ns), quantum)));
   const int c = threadIdx.x;
   const int64_t b = b0 + c;
-  // the thread's four rows together: their partials are independent loads
+  // the thread's four rows of eight splits are read together (zeros past the
+  // last), and added in order
+  constexpr int KS = 8;
   float h[FT / 8], l[FT / 8];
+  const float2* src[FT / 8];
 #pragma unroll
-  for (int u = 0; u < FT / 8; ++u) h[u] = l[u] = 0.f;
-#pragma unroll 4
-  for (int64_t k = 0; k < splits; ++k)
+  for (int u = 0; u < FT / 8; ++u) {
+    const int64_t a = a0 + threadIdx.y + 8 * u;
+    h[u] = l[u] = 0.f;
+    src[u] = a < m && b < m ? part + a * ldp + b : nullptr;
+  }
+  for (int64_t k0 = 0; k0 < splits; k0 += KS) {
+    float2 v[KS][FT / 8];
 #pragma unroll
-    for (int u = 0; u < FT / 8; ++u) {
-      const int64_t a = a0 + threadIdx.y + 8 * u;
-      if (a < m && b < m) pair_add(h[u], l[u], part[k * ldp * ldp + a * ldp + b]);
-    }
+    for (int k = 0; k < KS; ++k)
+#pragma unroll
+      for (int u = 0; u < FT / 8; ++u)
+        v[k][u] = src[u] && k0 + k < splits ? src[u][(k0 + k) * ldp * ldp] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < KS; ++k)
+#pragma unroll
+      for (int u = 0; u < FT / 8; ++u) pair_add(h[u], l[u], v[k][u]);
+  }
 #pragma unroll
   for (int u = 0; u < FT / 8; ++u) {
     const int r = threadIdx.y + 8 * u;

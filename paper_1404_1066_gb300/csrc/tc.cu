@@ -1211,7 +1211,7 @@ GramPlan gram_tc_plan(int64_t m, int64_t ns_max) {
   const int64_t sms = sm_count();
   const int64_t T1 = ceil_div(m, (int64_t)GS_TILE), T2 = ceil_div(m, (int64_t)GR_TILE);
   GramPlan p;
-  p.s_single = min64(sms / max64(1, T1 * (T1 + 1) / 2), min64(kGramMaxSplits, ceil_div(ns_max, kGramQuantumTc)));
+  p.s_single = min64(sms / max64(1, T1 * (T1 + 1) / 2), ceil_div(ns_max, kGramQuantumTc));
   p.s_pair = gram_splits(max64(1, T2 * (T2 + 1) / 2), max64(1, sms / 2), 1, 0.9, ns_max, kGramQuantumTc);
   return p;
 }
