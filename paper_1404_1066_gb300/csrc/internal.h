@@ -110,23 +110,6 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Column sums of a warp's 32 x 32 block (lane = row, v[j] = column j): after
-// five exchange steps, each halving the columns a lane holds and summing
-// the pair, lane l holds the sum of column l (31 shuffles in all).
-__device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
-#pragma unroll
-  for (int h = 16; h >= 1; h >>= 1) {
-    const bool upper = (lane & h) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const float give = upper ? v[k] : v[k + h];
-      const float keep = upper ? v[k + h] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
-    }
-  }
-  return v[0];
-}
-
 // Sum carried as an unevaluated pair hi + lo of FP32 values (Knuth's exact
 // two-term addition): (hi, lo) += x keeps about 2^-46 of the sum.  GB300
 // issues FP64 adds and conversions at 1/64 of the FP32 rate, and these six
@@ -165,6 +148,54 @@ __device__ __forceinline__ float warp_pair_sum(float hi, float lo) {
 __device__ __forceinline__ void pair_add(float& hi, float& lo, float2 p) {
   lo = __fadd_rn(lo, p.y);
   pair_add(hi, lo, p.x);
+}
+
+// Column sums of a warp's 32 x 32 block (lane = row, v[j] = column j) as
+// compensated pairs: after five exchange steps, each halving the columns a lane
+// holds and summing the pair, lane l holds the sum of column l.  The first two
+// steps, over four lanes, round in FP32, the others keep what they round off (of
+// terms of one sign most of an FP32 sum's error comes from its last steps).
+__device__ __forceinline__ float2 warp_column_sums(float (&v)[32], int lane) {
+#pragma unroll
+  for (int h = 16; h >= 8; h >>= 1) {
+    const bool upper = (lane & h) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const float give = upper ? v[k] : v[k + h];
+      const float keep = upper ? v[k + h] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+    }
+  }
+  float lo[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) lo[k] = 0.f;
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1) {
+    const bool upper = (lane & h) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const float gh = upper ? v[k] : v[k + h], gl = upper ? lo[k] : lo[k + h];
+      float kh = upper ? v[k + h] : v[k], kl = upper ? lo[k + h] : lo[k];
+      const float oh = __shfl_xor_sync(0xffffffffu, gh, h);
+      const float ol = h < 4 ? __shfl_xor_sync(0xffffffffu, gl, h) : 0.f;
+      pair_add(kh, kl, make_float2(oh, ol));
+      v[k] = kh;
+      lo[k] = kl;
+    }
+  }
+  return make_float2(v[0], lo[0]);
+}
+// The same of one column, in every lane.
+__device__ __forceinline__ float2 warp_column_sum(float v) {
+#pragma unroll
+  for (int o = 16; o >= 8; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  float lo = 0.f;
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, v, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
+    pair_add(v, lo, make_float2(oh, ol));
+  }
+  return make_float2(v, lo);
 }
 
 // Block sum (blockDim.x multiple of 32, <= 1024); result valid in thread 0.
