@@ -1811,9 +1811,9 @@ extern "C" int spsvm_solve_mixed(const double* H, int64_t m, int64_t ldh, double
 }
 
 // spsvm_solve_mixed right after spsvm_cholesky_mixed, without a host read of
-// the factorisation's info in between: the first refinement check reads it
-// and returns SPSVM_ERR_NOT_PD when the FP32 factorisation broke down (the
-// refinement's results are then discarded).
+// the factorisation's info in between: the refinement's launch reads it at its
+// start and ends there when the FP32 factorisation broke down
+// (SPSVM_ERR_NOT_PD).
 int spsvm::solve_mixed_after_factor(const double* H, int64_t m, int64_t ldh, double shift,
                                     const double* b, double* x, int32_t max_iter, double tol,
                                     void* work, size_t work_bytes, const int32_t* factor_info,

@@ -630,7 +630,7 @@ struct Fit {
           // error; H is kept, so a failure costs no Gram rebuild
           mixed = false;
           if (op.solver == SPSVM_SOLVE_MIXED) {
-            // the factorisation's info is read at the refinement's first check
+            // the factorisation's info is read at the start of the refinement
             SPSVM_TRY(spsvm_cholesky_mixed(H, m, ldH, shift, info, mixw, L.mix_bytes, s));
             const int rc = solve_mixed_after_factor(H, m, ldH, shift, rhs, dir, kMixedIters,
                                                     kMixedTol, mixw, L.mix_bytes, info, s);

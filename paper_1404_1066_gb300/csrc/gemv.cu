@@ -3,7 +3,8 @@
 //   * u = K_nJ v (line-search direction);
 //   * active-set compaction K_SJ with the masked transposed products
 //     K_SJ^T w (gradient and Newton right-hand side of Eq. 4).
-// Products are FP32; every 32 terms the running sum is promoted to FP64.
+// Products are FP32.  The first two promote the running sum to FP64 every 32
+// terms, the compaction keeps its sums as compensated FP32 pairs.
 #include <cooperative_groups.h>
 
 #include "internal.h"
@@ -141,7 +142,7 @@ template <int FMT, bool CL>
 __global__ void __launch_bounds__(GV_T) outputs_kernel(
     KView K, int64_t rows, int64_t n, const double* __restrict__ beta,
     const float* __restrict__ y, float* __restrict__ o, uint8_t* __restrict__ active,
-    double* __restrict__ part, int accumulate) {
+    double* __restrict__ part) {
   __shared__ float vs[GV_BETA];
   __shared__ double sh[32];
   const int64_t tile = tile_of_block<CL>();
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(GV_T) outputs_kernel(
       if (ii >= n) break;
       float oi;
       if (beta) {
-        oi = accumulate ? (float)((double)o[ii] + acc[p]) : (float)acc[p];
+        oi = (float)acc[p];
         o[ii] = oi;
       } else {
         oi = o[ii];
@@ -830,7 +831,7 @@ extern "C" int spsvm_outputs(const spsvm_kmat* K, const double* beta, const floa
   double* part = stats ? static_cast<double*>(scratch) : nullptr;
   const int cs = beta ? gv_cluster(blocks, K->rows, true) : 1;
   auto kern = cs > 1 ? SPSVM_GV_KERNEL(outputs_kernel, K, true) : SPSVM_GV_KERNEL(outputs_kernel, K, false);
-  SPSVM_CUDA_TRY(gv_launch(kern, blocks, cs, s, view(K), K->rows, K->n, beta, y, o, active, part, 0));
+  SPSVM_CUDA_TRY(gv_launch(kern, blocks, cs, s, view(K), K->rows, K->n, beta, y, o, active, part));
   SPSVM_LAUNCH_CHECK();
   if (stats) {
     sum_triples<<<1, 256, 0, s>>>(part, blocks, stats);

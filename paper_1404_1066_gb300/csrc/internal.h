@@ -284,8 +284,8 @@ int line_search_async(const float* o, const float* u, const float* y, int64_t n,
                       const int64_t* J, int32_t m, double lambda, double* t_dev, int32_t* err_dev,
                       void* scratch, size_t scratch_bytes, void* stream, const double* b0);
 
-// spsvm_solve_mixed right after spsvm_cholesky_mixed with its info word
-// read at the first refinement check (SPSVM_ERR_NOT_PD when it is nonzero).
+// spsvm_solve_mixed right after spsvm_cholesky_mixed, whose info word the
+// refinement reads at its start (SPSVM_ERR_NOT_PD when it is nonzero).
 int solve_mixed_after_factor(const double* H, int64_t m, int64_t ldh, double shift,
                              const double* b, double* x, int32_t max_iter, double tol,
                              void* work, size_t work_bytes, const int32_t* factor_info,

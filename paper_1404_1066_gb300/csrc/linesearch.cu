@@ -16,10 +16,6 @@
 // n = 30,000 25 us, n = 500,000 41 us; with a uniform grid on the bracket
 // (32-fold a pass), counts by shared atomics with FP64 divisions and two
 // barriers over 304 CTAs a pass it took 103 us and 150.
-#include <cmath>
-#include <mutex>
-#include <vector>
-
 #include "internal.h"
 
 namespace spsvm {

@@ -17,7 +17,6 @@
 //     compensated pairs.
 #include <cudaTypedefs.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "gram.h"
