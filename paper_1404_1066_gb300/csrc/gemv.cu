@@ -787,18 +787,19 @@ namespace spsvm {
 namespace {
 // Blocks per tile of points: two, four or eight while SMs would be idle or nearly
 // so, and a block keeps rows enough to pay the cluster's barriers: 32 up to a block
-// for every other SM, 64 up to two blocks per SM, then 128; the outputs, whose
+// for every other SM, 64 up to three blocks per SM, then 128; the outputs, whose
 // epilogue one block in each cluster runs, 64 up to one block per SM, then 192.
-// 30,000 points by 1,024 rows: u = K v 28 us, one block a tile 114; 100,000 by 128: 7.8, two blocks
-// of 64 rows 7.3, four 10.3 (outputs 14.8, 17.1 and 25.4); 60,000 by 256: 9.2 with two, 9.8
-// with four, 12.3 with one (outputs 17.5, 21.3, 17.0).
+// 30,000 points by 1,024 rows: u = K v 28 us, one block a tile 114.  From L2,
+// 100,000 by 128: two blocks of 64 rows 7.3, one 7.8, four 10.3 (from HBM 20.7, 25.1
+// and 21.8; outputs 17.1, 14.8 and 25.4); 60,000 by 256: two 9.2, four 9.8, one 12.3
+// (outputs 17.5, 21.3 and 17.0).
 int gv_cluster(int64_t tiles, int64_t rows, bool outputs) {
   const int64_t sms = sm_count();
   int cs = 1;
   while (2 * cs <= GV_CLUSTER && tiles * cs < (outputs ? 2 : 4) * sms) {
     const int64_t after = 2 * cs * tiles;
     const int64_t least = outputs ? (after <= sms ? 64 : 192)
-                                  : (2 * after <= sms ? 32 : (after <= 2 * sms ? 64 : 128));
+                                  : (2 * after <= sms ? 32 : (after <= 3 * sms ? 64 : 128));
     if (rows < 2 * cs * least) break;
     cs *= 2;
   }
