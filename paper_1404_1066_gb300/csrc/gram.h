@@ -9,8 +9,8 @@ constexpr int64_t GRAM_SLICE = 8192;
 
 // Both forms split the active points evenly over at most kGramMaxSplits
 // partial matrices (or, where a wave of blocks takes more, one for each slice of
-// GRAM_SLICE points: matrices of few tiles on many points, m = 64, ns = 400,000
-// in split form 109 us, 445 with 16) of at least a quantum of points: in
+// GRAM_SLICE points: matrices of few tiles on many points, m = 64, ns = 200,000
+// in split form 93 us, 239 with 16) of at least a quantum of points: in
 // the FP32 form about what a partial matrix costs to write and add, in the split
 // form a slice.
 // Their number is read on the device, so the last splits may be empty (they

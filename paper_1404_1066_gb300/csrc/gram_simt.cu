@@ -196,9 +196,11 @@ __global__ void __launch_bounds__(FT * 8) kjj_fill_kernel(KView K, const int64_t
 // over 32 x 32 upper tiles (the partials are compensated FP32 pairs: an FP64 add
 // has 1/64 of their rate): the partials, K_JJ and both halves of H move through
 // shared memory so that every global access is coalesced.  Bound by the latency
-// of the partials: 62 splits at m = 64 take 28 us more than one, 66 when only a
-// split's four rows were in flight.
-__global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const float2* __restrict__ part,
+// of the partials while the blocks leave SMs to spare (then eight splits are in
+// flight a thread: 62 splits at m = 64 take 14 us more than one, 66 with one in
+// flight), else by HBM (two, which leaves registers for six blocks an SM).
+template <int KS>
+__global__ void __launch_bounds__(FT * 8, KS == 8 ? 2 : 6) gram_finish_kernel(const float2* __restrict__ part,
                                                              GramPlan plan,
                                                              const int64_t* __restrict__ ns_dev,
                                                              int64_t quantum, int64_t ldp,
@@ -219,9 +221,8 @@ __global__ void __launch_bounds__(FT * 8) gram_finish_kernel(const float2* __res
   const int64_t splits = max64(1, ceil_div(ns, gram_split_points(ns, plan.splits(ns), quantum)));
   const int c = threadIdx.x;
   const int64_t b = b0 + c;
-  // the thread's four rows of eight splits are read together (zeros past the
-  // last), and added in order
-  constexpr int KS = 8;
+  // the thread's four rows of KS splits are read together (zeros past the last),
+  // and added in order
   float h[FT / 8], l[FT / 8];
   const float2* src[FT / 8];
 #pragma unroll
@@ -270,8 +271,9 @@ int launch_gram_finish(const float2* part, const GramPlan& plan, const int64_t* 
                        const double* kjj, int64_t ldk, int64_t m, double lambda, double* H, int64_t ldh,
                        cudaStream_t s) {
   const int64_t T = ceil_div(m, (int64_t)FT);
-  gram_finish_kernel<<<(unsigned)(T * (T + 1) / 2), dim3(FT, 8), 0, s>>>(part, plan, ns_dev, quantum, ldp,
-                                                                         kjj, ldk, m, lambda, H, ldh);
+  const int64_t blocks = T * (T + 1) / 2;
+  auto kern = blocks <= sm_count() ? gram_finish_kernel<8> : gram_finish_kernel<2>;
+  kern<<<(unsigned)blocks, dim3(FT, 8), 0, s>>>(part, plan, ns_dev, quantum, ldp, kjj, ldk, m, lambda, H, ldh);
   SPSVM_LAUNCH_CHECK();
   return SPSVM_OK;
 }
