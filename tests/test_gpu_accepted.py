@@ -34,10 +34,10 @@ def _split_kmat(sp, K, gap):
     return sp.KMat(buf, sp.SPSVM_BF16SPLIT, n, rows, ld, plane), (hi.double() + lo.double()).cpu().numpy()
 
 
-# planes an even and an odd number of elements apart; one block of 512 points
-# and a cluster
+# planes an even and an odd number of elements apart; one block of 512 points,
+# clusters, and more blocks than six per SM
 @pytest.mark.parametrize("gap", [0, 1, 2, 5])
-@pytest.mark.parametrize("n,m", [(1, 1), (7, 3), (515, 70), (3001, 129)])
+@pytest.mark.parametrize("n,m", [(1, 1), (7, 3), (515, 70), (3001, 129), (500_001, 3)])
 def test_products_with_planes_any_distance_apart(sp, gap, n, m):
     """u = K v and o = K beta: FP32 chunks of 32 terms, then one rounding."""
     g = np.random.default_rng(n + gap)
